@@ -838,11 +838,9 @@ __device__ __forceinline__ void pair2_sym(float2 dx, float2 dy, float2 dz, float
         c2f = mul2(mul2(ri, ri2), fma2(bc2(-k.kf3), ri2, one));
     }
     const float2 dlxy = fma2(dx, lx, mul2(dy, ly));
-    const float2 Df = fma2(dz, lz, dlxy);
     const float2 dmxy = fma2(dx, mx, mul2(dy, my));
-    const float2 Dfm = fma2(dz, mz, dmxy);
     if (!WALL) {
-        const float2 sl = mul2(c2f, Df), sm = mul2(c2f, Dfm);
+        const float2 sl = mul2(c2f, fma2(dz, lz, dlxy)), sm = mul2(c2f, fma2(dz, mz, dmxy));
         ux = fma2(c1f, lx, fma2(sl, dx, ux));
         uy = fma2(c1f, ly, fma2(sl, dy, uy));
         uz = fma2(c1f, lz, fma2(sl, dz, uz));
@@ -865,28 +863,20 @@ __device__ __forceinline__ void pair2_sym(float2 dx, float2 dy, float2 dz, float
     const float2 A4w2n = mul2(w2, bc2(-k.wa4));
     const float2 cc = fma2(s, cI, c1f);
     const float2 g = fma2(Rz, fma2(cRR, bc2(-2.f), fma2(A4w2n, bc2(-1.f), bc2(-2.f))), h2);
-    const float2 s3cRR = mul2(s3, cRR), s3g = mul2(s3, g), s3h2 = mul2(s3, h2);
-    const float2 s3A = mul2(s3, mul2(A4w2n, Rz)), s3phi = mul2(s3, mul2(w, fma2(yz, bc2(-2.f), bc2(k.wi2))));
-    {
-        const float2 Di = fma2(Rz, lz, dlxy);
-        const float2 sdl = mul2(c2f, Df);
-        const float2 P = fma2(s3cRR, Di, mul2(s3g, lz));
-        const float2 Q = fma2(s3h2, Df, fma2(s3A, Di, mul2(s3phi, lz)));
-        const float2 pp = add2(sdl, P);
-        ux = fma2(cc, lx, fma2(pp, dx, ux));
-        uy = fma2(cc, ly, fma2(pp, dy, uy));
-        uz = fma2(cc, lz, fma2(sdl, dz, fma2(P, Rz, add2(uz, Q))));
-    }
-    {
-        const float2 Di = fma2(Rz, mz, dmxy);
-        const float2 cd = fma2(c2f, Dfm, mul2(s3h2, mz));
-        const float2 P = fma2(s3cRR, Di, mul2(s3A, mz));
-        const float2 Q = fma2(s3g, Di, mul2(s3phi, mz));
-        const float2 pp = add2(cd, P);
-        vx = fma2(cc, mx, fma2(pp, dx, vx));
-        vy = fma2(cc, my, fma2(pp, dy, vy));
-        vz = fma2(cc, mz, fma2(cd, dz, fma2(P, Rz, add2(vz, Q))));
-    }
+    const float2 phi = mul2(w, fma2(yz, bc2(-2.f), bc2(k.wi2)));
+    const float2 E = fma2(s3, cRR, c2f);
+    const float2 Pc = fma2(c2f, dz, mul2(mul2(s3, cRR), Rz));
+    const float2 P1 = fma2(s3, g, Pc);
+    const float2 P2 = fma2(s3, fma2(A4w2n, Rz, h2), Pc);
+    const float2 M33 = fma2(dz, P2, fma2(s3, fma2(Rz, fma2(add2(cRR, A4w2n), h2, g), phi), cc));
+    const float2 q = fma2(E, dlxy, mul2(P1, lz));
+    ux = fma2(cc, lx, fma2(q, dx, ux));
+    uy = fma2(cc, ly, fma2(q, dy, uy));
+    uz = fma2(P2, dlxy, fma2(M33, lz, uz));
+    const float2 p = fma2(E, dmxy, mul2(P2, mz));
+    vx = fma2(cc, mx, fma2(p, dx, vx));
+    vy = fma2(cc, my, fma2(p, dy, vy));
+    vz = fma2(P1, dmxy, fma2(M33, mz, vz));
 }
 
 // Symmetric mixed product on tile pairs of 128 blobs (the SymItem list of

@@ -124,11 +124,9 @@ __device__ __forceinline__ void pair_sym_df(df dx, df dy, df dz, df rxy2, df r2,
     df c1f, c2f;
     free_coefs_df(r2, k, c1f, c2f);
     const df dlxy = df_fma(dx, lx, df_mul(dy, ly));
-    const df Df = df_fma(dz, lz, dlxy);
     const df dmxy = df_fma(dx, mx, df_mul(dy, my));
-    const df Dfm = df_fma(dz, mz, dmxy);
     if (!WALL) {
-        const df sl = df_mul(c2f, Df), sm = df_mul(c2f, Dfm);
+        const df sl = df_mul(c2f, df_fma(dz, lz, dlxy)), sm = df_mul(c2f, df_fma(dz, mz, dmxy));
         ux = df_fma(c1f, lx, df_fma(sl, dx, ux));
         uy = df_fma(c1f, ly, df_fma(sl, dy, uy));
         uz = df_fma(c1f, lz, df_fma(sl, dz, uz));
@@ -143,38 +141,31 @@ __device__ __forceinline__ void pair_sym_df(df dx, df dy, df dz, df rxy2, df r2,
     const df c1 = df_fma(h2, nx3, k.wc1);
     const df c2 = df_fma(Rz2, k.w2a2, k.wc2);
     const df c3 = df_mul(Rz2, k.wc3);
-    const df x1 = df_fma(w, c3, c2);
+    const df wc3 = df_mul(w, c3);
+    const df x1 = df_add(wc3, c2);
     const df cI = df_fma(w, df_fma(w, x1, c1), df{-1.0f, 0.0f});
-    const df y = df_fma(w, c3, x1);
-    const df yz = df_fma(w, c3, y);
+    const df y = df_add(wc3, x1);
+    const df yz = df_add(wc3, y);
     const df cRR = df_add(df_scale2(df_mul(w2, y), -2.0f), df_add(df_mul_f(cI, -3.0f), df{-4.0f, 0.0f}));
     const df A4w2n = df_mul(w2, k.nwa4);
     const df inner = df_add(df_add(df_scale2(cRR, -2.0f), df{-2.0f, 0.0f}), df_neg(A4w2n));
     const df g = df_fma(Rz, inner, h2);
     const df phi = df_mul(w, df_add(df_scale2(yz, -2.0f), k.wi2));
     const df cc = df_fma(s, cI, c1f);
-    const df s3cRR = df_mul(s3, cRR), s3g = df_mul(s3, g), s3h2 = df_mul(s3, h2);
-    const df s3A = df_mul(s3, df_mul(A4w2n, Rz)), s3phi = df_mul(s3, phi);
-    {
-        const df Di = df_fma(Rz, lz, dlxy);
-        const df sdl = df_mul(c2f, Df);
-        const df P = df_fma(s3cRR, Di, df_mul(s3g, lz));
-        const df Q = df_fma(s3h2, Df, df_fma(s3A, Di, df_mul(s3phi, lz)));
-        const df pp = df_add(sdl, P);
-        ux = df_fma(cc, lx, df_fma(pp, dx, ux));
-        uy = df_fma(cc, ly, df_fma(pp, dy, uy));
-        uz = df_fma(cc, lz, df_fma(sdl, dz, df_fma(P, Rz, df_add(uz, Q))));
-    }
-    {
-        const df Di = df_fma(Rz, mz, dmxy);
-        const df cd = df_fma(c2f, Dfm, df_mul(s3h2, mz));
-        const df P = df_fma(s3cRR, Di, df_mul(s3A, mz));
-        const df Q = df_fma(s3g, Di, df_mul(s3phi, mz));
-        const df pp = df_add(cd, P);
-        vx = df_fma(cc, mx, df_fma(pp, dx, vx));
-        vy = df_fma(cc, my, df_fma(pp, dy, vy));
-        vz = df_fma(cc, mz, df_fma(cd, dz, df_fma(P, Rz, df_add(vz, Q))));
-    }
+    const df s3cRR = df_mul(s3, cRR);
+    const df E = df_add(s3cRR, c2f);
+    const df Pc = df_fma(c2f, dz, df_mul(s3cRR, Rz));
+    const df P1 = df_fma(s3, g, Pc);
+    const df P2 = df_fma(s3, df_fma(A4w2n, Rz, h2), Pc);
+    const df M33 = df_fma(dz, P2, df_fma(s3, df_fma(Rz, df_fma(df_add(cRR, A4w2n), h2, g), phi), cc));
+    const df q = df_fma(E, dlxy, df_mul(P1, lz));
+    ux = df_fma(cc, lx, df_fma(q, dx, ux));
+    uy = df_fma(cc, ly, df_fma(q, dy, uy));
+    uz = df_fma(P2, dlxy, df_fma(M33, lz, uz));
+    const df p = df_fma(E, dmxy, df_mul(P2, mz));
+    vx = df_fma(cc, mx, df_fma(p, dx, vx));
+    vy = df_fma(cc, my, df_fma(p, dy, vy));
+    vz = df_fma(P1, dmxy, df_fma(M33, mz, vz));
 }
 
 __device__ __forceinline__ df df_shfl(df x, int src) {

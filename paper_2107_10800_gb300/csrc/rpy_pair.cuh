@@ -215,12 +215,17 @@ __device__ __forceinline__ void pair_wall_r2(T dx, T dy, T dz, T rxy2, T r2, T R
 // pair_wall_r2 is
 //   cc I + c2f d d^T + s^3 cRR R R^T + s^3 g R e3^T
 //        + s^3 e3 (h2 d^T - (20/3) a^4 w^2 Rz R^T) + s^3 phi e3 e3^T,
-// g = Rz inner + h2, phi = w (c2-term of Q), so the transpose multiplies mu
-// with the d, R and e3 coefficients
-//   c2f (d . mu) + s^3 h2 mu_3,  s^3 cRR (R . mu) - (20/3) s^3 a^4 w^2 Rz mu_3,
-//   s^3 g (R . mu) + s^3 phi mu_3.
-// The coefficients are shared; the second direction costs about 20
-// operations against about 60 for a separate evaluation.
+// g = Rz inner + h2, phi = w (c2-term of Q).  d and R share their lateral
+// part (dx, dy), so the tensor has only five distinct factors:
+//   lateral block  cc I + E (dx, dy)(dx, dy)^T,  E  = c2f + s^3 cRR
+//   column 3       (dx, dy) P1,  P1 = c2f dz + s^3 (cRR Rz + g)
+//   row 3          (dx, dy) P2,  P2 = c2f dz + s^3 (cRR Rz + h2 - (20/3) a^4 w^2 Rz)
+//   M33 = cc + dz P2 + s^3 (Rz (h2 (cRR - (20/3) a^4 w^2) + g) + phi)
+// (the last with Rz - dz = h2), and either direction is ten multiply-adds:
+//   t = (dx, dy) . f_lat,  q = E t + P f_3,  lateral cc f + (dx, dy) q,
+//   third P' t + M33 f_3, with (P, P') = (P1, P2) forward and (P2, P1) for
+// the transpose.  FP64-issue-bound: about 79 FP64 operations per unordered
+// pair (91 when d, R and e3 terms were applied one by one).
 template <class T>
 __device__ __forceinline__ void pair_wall_sym(T dx, T dy, T dz, T rxy2, T r2, T Rz, T h2, T nx3, T lx, T ly,
                                               T lz, T mx, T my, T mz, const RpyK<T>& k, T& ux, T& uy, T& uz,
@@ -241,29 +246,25 @@ __device__ __forceinline__ void pair_wall_sym(T dx, T dy, T dz, T rxy2, T r2, T 
     const T A4w2n = w2 * -k.wa4;                // -20/3 a^4 w^2
     const T cc = fma(s, cI, c1f);
     const T g = fma(Rz, fma(cRR, (T)-2, fma(A4w2n, (T)-1, (T)-2)), h2);
-    const T s3cRR = s3 * cRR, s3g = s3 * g, s3h2 = s3 * h2;
-    const T s3A = s3 * (A4w2n * Rz), s3phi = s3 * (w * fma(yz, (T)-2, k.wi2));
+    const T phi = w * fma(yz, (T)-2, k.wi2);
+    const T E = fma(s3, cRR, c2f);
+    const T Pc = fma(c2f, dz, (s3 * cRR) * Rz);
+    const T P1 = fma(s3, g, Pc);
+    const T P2 = fma(s3, fma(A4w2n, Rz, h2), Pc);
+    const T M33 = fma(dz, P2, fma(s3, fma(Rz, fma(cRR + A4w2n, h2, g), phi), cc));
     {   // u += M_ij lambda
-        const T dlxy = fma(dx, lx, dy * ly);
-        const T Df = fma(dz, lz, dlxy), Di = fma(Rz, lz, dlxy);
-        const T sdl = c2f * Df;
-        const T P = fma(s3cRR, Di, s3g * lz);
-        const T Q = fma(s3h2, Df, fma(s3A, Di, s3phi * lz));
-        const T pp = sdl + P;
-        ux = fma(cc, lx, fma(pp, dx, ux));
-        uy = fma(cc, ly, fma(pp, dy, uy));
-        uz = fma(cc, lz, fma(sdl, dz, fma(P, Rz, uz + Q)));
+        const T t = fma(dx, lx, dy * ly);
+        const T q = fma(E, t, P1 * lz);
+        ux = fma(cc, lx, fma(q, dx, ux));
+        uy = fma(cc, ly, fma(q, dy, uy));
+        uz = fma(P2, t, fma(M33, lz, uz));
     }
     {   // v += M_ij^T mu
-        const T dmxy = fma(dx, mx, dy * my);
-        const T Df = fma(dz, mz, dmxy), Di = fma(Rz, mz, dmxy);
-        const T cd = fma(c2f, Df, s3h2 * mz);
-        const T P = fma(s3cRR, Di, s3A * mz);
-        const T Q = fma(s3g, Di, s3phi * mz);
-        const T pp = cd + P;
-        vx = fma(cc, mx, fma(pp, dx, vx));
-        vy = fma(cc, my, fma(pp, dy, vy));
-        vz = fma(cc, mz, fma(cd, dz, fma(P, Rz, vz + Q)));
+        const T t = fma(dx, mx, dy * my);
+        const T q = fma(E, t, P2 * mz);
+        vx = fma(cc, mx, fma(q, dx, vx));
+        vy = fma(cc, my, fma(q, dy, vy));
+        vz = fma(P1, t, fma(M33, mz, vz));
     }
 }
 
