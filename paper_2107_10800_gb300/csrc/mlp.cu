@@ -333,99 +333,151 @@ __global__ void k_flow_rhs(int Nb, const int* __restrict__ body_of_blob, const d
 }
 
 // --------------------------------------------------------- FP32 training ---
-// C[r][o] = sum_i A[r][i] W[o][i] + b[o]; Z = C, Aout = relu(C) (or C)
-__global__ void __launch_bounds__(256)
-k_linear_fwd(const float* __restrict__ A, const float* __restrict__ W, const float* __restrict__ b,
-             float* __restrict__ Z, float* __restrict__ Aout, int n, int in, int out, int relu) {
-    __shared__ float As[32][33];
-    __shared__ float Ws[32][33];
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 32 x 8
-    const int r0 = blockIdx.y * 32, o0 = blockIdx.x * 32;
-    float acc[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int k0 = 0; k0 < in; k0 += 32) {
-        for (int e = threadIdx.x; e < 32 * 32; e += 256) {
-            const int rr = e / 32, kk = e % 32;
-            As[rr][kk] = (r0 + rr < n && k0 + kk < in) ? A[(size_t)(r0 + rr) * in + k0 + kk] : 0.f;
-            Ws[rr][kk] = (o0 + rr < out && k0 + kk < in) ? W[(size_t)(o0 + rr) * in + k0 + kk] : 0.f;
-        }
-        __syncthreads();
-        for (int kk = 0; kk < 32; ++kk) {
-            const float w = Ws[tx][kk];
-            for (int q = 0; q < 4; ++q) acc[q] = fmaf(As[ty + 8 * q][kk], w, acc[q]);
-        }
-        __syncthreads();
+// The three products of a layer on one tiled kernel, C[m][n] = sum_k A B:
+//   forward  C[r][o] = sum_i A[r][i] W[o][i]   (both operands k-contiguous)
+//   xgrad    C[r][i] = sum_o dZ[r][o] W[o][i]  (first k-contiguous)
+//   wgrad    C[o][i] = sum_r dZ[r][o] A[r][i]  (neither)
+// A block of 256 threads forms a 16 R x 16 R tile of C, R x R entries per
+// thread in paired FP32 lanes, from k-slices of 16 staged k-major in shared
+// memory; the next slice's global loads are in flight while a slice is
+// multiplied.  R = 4 (64 x 64 tiles: 16 multiply-adds per two 16-byte shared
+// loads) once such tiles fill the SMs, R = 2 (32 x 32 tiles) for the mini-
+// batches of the training loop, whose 64 x 64 tiles would leave most SMs idle.
+// wgrad's sum runs over the samples: it is split over blockIdx.z into chunks
+// of samples whose partial gradients k_sum_grad adds in a fixed order (one
+// block per 32 x 32 tile with the whole sum took 537 us per layer at 4,096
+// samples, 88 % of loss and gradient).  FP32 throughout.
+constexpr int kGemmK = 16;
+
+enum { kGemmFwd = 0, kGemmXgrad = 1, kGemmWgrad = 2 };
+
+// slice [k0, k0 + 16) of an operand into S[k][m] (kc: rows of length ld are
+// contiguous in k, else in m); entries outside [0, m_end) x [0, k_end) are
+// zero.  ld, m_end (k-major) and k_end (k-contiguous) are multiples of 4.
+template <int R, bool KC>
+__device__ __forceinline__ float4 gemm_fetch(const float* __restrict__ P, int ld, int m0, int m_end, int k0,
+                                             int k_end) {
+    const int t = threadIdx.x;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (t >= 64 * R) return v;
+    if (KC) {
+        const int m = m0 + t / 4, k = k0 + 4 * (t % 4);
+        if (m < m_end && k < k_end) v = *reinterpret_cast<const float4*>(P + (size_t)m * ld + k);
+    } else {
+        const int k = k0 + t / (4 * R), m = m0 + 4 * (t % (4 * R));
+        if (m < m_end && k < k_end) v = *reinterpret_cast<const float4*>(P + (size_t)k * ld + m);
     }
-    const int o = o0 + tx;
-    if (o >= out) return;
-    for (int q = 0; q < 4; ++q) {
-        const int r = r0 + ty + 8 * q;
-        if (r >= n) continue;
-        const float z = acc[q] + b[o];
-        Z[(size_t)r * out + o] = z;
-        Aout[(size_t)r * out + o] = relu ? fmaxf(z, 0.f) : z;
+    return v;
+}
+
+template <int R, bool KC>
+__device__ __forceinline__ void gemm_store(float (*S)[16 * R + 4], float4 v) {
+    const int t = threadIdx.x;
+    if (t >= 64 * R) return;
+    if (KC) {
+        const int m = t / 4, k = 4 * (t % 4);
+        S[k][m] = v.x; S[k + 1][m] = v.y; S[k + 2][m] = v.z; S[k + 3][m] = v.w;
+    } else {
+        *reinterpret_cast<float4*>(&S[t / (4 * R)][4 * (t % (4 * R))]) = v;
     }
 }
 
-// gW[o][i] = sum_r dZ[r][o] A[r][i];  gb[o] = sum_r dZ[r][o]
-__global__ void __launch_bounds__(256)
-k_linear_wgrad(const float* __restrict__ dZ, const float* __restrict__ A, float* __restrict__ gW,
-               float* __restrict__ gb, int n, int in, int out) {
-    __shared__ float Ds[32][33];
-    __shared__ float As[32][33];
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const int o0 = blockIdx.y * 32, i0 = blockIdx.x * 32;
-    float acc[4] = {0.f, 0.f, 0.f, 0.f};
-    float bacc = 0.f;
-    for (int r0 = 0; r0 < n; r0 += 32) {
-        for (int e = threadIdx.x; e < 32 * 32; e += 256) {
-            const int rr = e / 32, cc = e % 32;
-            Ds[rr][cc] = (r0 + rr < n && o0 + cc < out) ? dZ[(size_t)(r0 + rr) * out + o0 + cc] : 0.f;
-            As[rr][cc] = (r0 + rr < n && i0 + cc < in) ? A[(size_t)(r0 + rr) * in + i0 + cc] : 0.f;
-        }
-        __syncthreads();
-        for (int rr = 0; rr < 32; ++rr) {
-            const float a = As[rr][tx];
-            for (int q = 0; q < 4; ++q) acc[q] = fmaf(Ds[rr][ty + 8 * q], a, acc[q]);
-            if (blockIdx.x == 0 && ty == 0) bacc += Ds[rr][tx];
-        }
-        __syncthreads();
+// R consecutive floats of shared memory as pairs
+template <int R>
+__device__ __forceinline__ void gemm_row(const float* p, float2* o) {
+    if (R == 4) {
+        const float4 v = *reinterpret_cast<const float4*>(p);
+        o[0] = make_float2(v.x, v.y);
+        o[R / 2 - 1] = make_float2(v.z, v.w);
+    } else {
+        o[0] = *reinterpret_cast<const float2*>(p);
     }
-    const int i = i0 + tx;
-    for (int q = 0; q < 4; ++q) {
-        const int o = o0 + ty + 8 * q;
-        if (o < out && i < in) gW[(size_t)o * in + i] = acc[q];
-    }
-    if (blockIdx.x == 0 && ty == 0 && o0 + tx < out) gb[o0 + tx] = bacc;
 }
 
-// dA[r][i] = sum_o dZ[r][o] W[o][i]; then dZprev = dA * (Zprev > 0)
+// C is M x N over k in [0, K) (wgrad: in chunks of `chunk` per blockIdx.z,
+// chunk z written at C + z * zstride).  forward: + bias[n], ReLU when act is
+// set; xgrad: zero where act[m][n] <= 0; wgrad: blocks of blockIdx.x = 0 also
+// write the row sums of the first operand at C + bias_off + m (the bias
+// gradient).
+template <int MODE, int R>
 __global__ void __launch_bounds__(256)
-k_linear_xgrad(const float* __restrict__ dZ, const float* __restrict__ W, const float* __restrict__ Zprev,
-               float* __restrict__ dZprev, int n, int in, int out) {
-    __shared__ float Ds[32][33];
-    __shared__ float Ws[32][33];
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const int r0 = blockIdx.y * 32, i0 = blockIdx.x * 32;
-    float acc[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int o0 = 0; o0 < out; o0 += 32) {
-        for (int e = threadIdx.x; e < 32 * 32; e += 256) {
-            const int rr = e / 32, cc = e % 32;
-            Ds[rr][cc] = (r0 + rr < n && o0 + cc < out) ? dZ[(size_t)(r0 + rr) * out + o0 + cc] : 0.f;
-            Ws[rr][cc] = (o0 + rr < out && i0 + cc < in) ? W[(size_t)(o0 + rr) * in + i0 + cc] : 0.f;
-        }
-        __syncthreads();
-        for (int oo = 0; oo < 32; ++oo) {
-            const float w = Ws[oo][tx];
-            for (int q = 0; q < 4; ++q) acc[q] = fmaf(Ds[ty + 8 * q][oo], w, acc[q]);
-        }
-        __syncthreads();
+k_gemm32(const float* __restrict__ A, const float* __restrict__ B, const float* __restrict__ bias,
+         const float* __restrict__ act, float* __restrict__ C, int M, int N, int K, int relu, int chunk,
+         size_t zstride, int bias_off) {
+    am::dep_wait();
+    constexpr bool AK = MODE != kGemmWgrad, BK = MODE == kGemmFwd;
+    __shared__ __align__(16) float As[2][kGemmK][16 * R + 4];
+    __shared__ __align__(16) float Bs[2][kGemmK][16 * R + 4];
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    const int m0 = blockIdx.y * 16 * R, n0 = blockIdx.x * 16 * R;
+    const int kb = MODE == kGemmWgrad ? blockIdx.z * chunk : 0;
+    const int ke = MODE == kGemmWgrad ? min(K, kb + chunk) : K;
+    const int lda = AK ? K : M, ldb = BK ? K : N;
+    float2 acc[R][R / 2];
+    float rs[R];
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+        rs[i] = 0.f;
+#pragma unroll
+        for (int j = 0; j < R / 2; ++j) acc[i][j] = make_float2(0.f, 0.f);
     }
-    const int i = i0 + tx;
-    if (i >= in) return;
-    for (int q = 0; q < 4; ++q) {
-        const int r = r0 + ty + 8 * q;
-        if (r < n) dZprev[(size_t)r * in + i] = Zprev[(size_t)r * in + i] > 0.f ? acc[q] : 0.f;
+    const bool row_sums = MODE == kGemmWgrad && blockIdx.x == 0;
+    float4 va = gemm_fetch<R, AK>(A, lda, m0, M, kb, ke), vb = gemm_fetch<R, BK>(B, ldb, n0, N, kb, ke);
+    int buf = 0;
+    for (int k0 = kb; k0 < ke; k0 += kGemmK, buf ^= 1) {
+        gemm_store<R, AK>(As[buf], va);
+        gemm_store<R, BK>(Bs[buf], vb);
+        __syncthreads();
+        if (k0 + kGemmK < ke) {
+            va = gemm_fetch<R, AK>(A, lda, m0, M, k0 + kGemmK, ke);
+            vb = gemm_fetch<R, BK>(B, ldb, n0, N, k0 + kGemmK, ke);
+        }
+#pragma unroll
+        for (int k = 0; k < kGemmK; ++k) {
+            float2 a2[R / 2], b2[R / 2];
+            gemm_row<R>(&As[buf][k][R * ty], a2);
+            gemm_row<R>(&Bs[buf][k][R * tx], b2);
+#pragma unroll
+            for (int i = 0; i < R; ++i) {
+                const float a = i & 1 ? a2[i / 2].y : a2[i / 2].x;
+                if (MODE == kGemmWgrad) rs[i] += a;
+#pragma unroll
+                for (int j = 0; j < R / 2; ++j) acc[i][j] = __ffma2_rn(make_float2(a, a), b2[j], acc[i][j]);
+            }
+        }
+        // the other buffer is stored next; this one is free again after the
+        // following iteration's barrier
     }
+    float* Cz = C + (MODE == kGemmWgrad ? blockIdx.z * zstride : 0);
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+        const int m = m0 + R * ty + i;
+        if (m >= M) continue;
+        if (row_sums && tx == 0) Cz[bias_off + m] = rs[i];
+#pragma unroll
+        for (int j = 0; j < R; ++j) {
+            const int n = n0 + R * tx + j;
+            if (n >= N) continue;
+            float v = j & 1 ? acc[i][j / 2].y : acc[i][j / 2].x;
+            if (MODE == kGemmFwd) {
+                v += bias[n];
+                if (relu) v = fmaxf(v, 0.f);
+            } else if (MODE == kGemmXgrad) {
+                v = act[(size_t)m * N + n] > 0.f ? v : 0.f;
+            }
+            Cz[(size_t)m * N + n] = v;
+        }
+    }
+}
+
+// g = the sum over the sample chunks of the partial gradients
+__global__ void k_sum_grad(const float* __restrict__ part, float* __restrict__ g, int np, int chunks) {
+    am::dep_wait();
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= np) return;
+    float s = 0.f;
+    for (int z = 0; z < chunks; ++z) s += part[(size_t)z * np + e];
+    g[e] = s;
 }
 
 __global__ void k_normalize(const float* __restrict__ X, const float* __restrict__ mu,
@@ -490,6 +542,8 @@ __global__ void k_normalize_bf16(const float* __restrict__ X, const float* __res
 }  // namespace
 
 // ===================================================================== model
+constexpr int kWgradChunks = 16;  // most sample chunks of the weight gradient
+
 struct am_mlp {
     float *d_p = nullptr, *d_m = nullptr, *d_v = nullptr, *d_g = nullptr;
     __nv_bfloat16* d_wbf = nullptr;
@@ -497,13 +551,14 @@ struct am_mlp {
     int adam_t = 0;
     int cap = 0;
     float *d_X = nullptr, *d_T = nullptr, *d_bx = nullptr, *d_bt = nullptr, *d_dz0 = nullptr, *d_dz1 = nullptr;
-    float* d_z[NLAYER + 1] = {};
+    float* d_gpart = nullptr;  // kWgradChunks partial gradients
+    float* d_zout = nullptr;  // the last layer's output
     float* d_a[NLAYER + 1] = {};
     __nv_bfloat16 *d_h0 = nullptr, *d_h1 = nullptr;
     int* d_rows = nullptr;
     int* d_flag = nullptr;  // tensor-core wait timeouts of the standalone prediction
     double* d_loss = nullptr;
-    int data_n = 0;
+    int data_cap = 0;  // samples that d_X, d_T and d_rows hold
     cudaStream_t st = nullptr;
     bool bf_valid = false;
 };
@@ -524,11 +579,12 @@ int mlp_fail(int code, const std::string& m) {
 int ensure_cap(am_mlp* m, int n) {
     if (n <= m->cap) return AM_OK;
     for (int l = 0; l <= NLAYER; ++l) {
-        if (m->d_z[l]) cudaFree(m->d_z[l]);
         if (m->d_a[l]) cudaFree(m->d_a[l]);
-        MCK(cudaMalloc(&m->d_z[l], (size_t)n * WIDTH * sizeof(float)));
         MCK(cudaMalloc(&m->d_a[l], (size_t)n * WIDTH * sizeof(float)));
     }
+    if (m->d_zout) cudaFree(m->d_zout);
+    MCK(cudaMalloc(&m->d_zout, (size_t)n * OUT * sizeof(float)));
+    if (!m->d_gpart) MCK(cudaMalloc(&m->d_gpart, kWgradChunks * n_params_total() * sizeof(float)));
     for (float** p : {&m->d_dz0, &m->d_dz1, &m->d_bx, &m->d_bt}) {
         if (*p) cudaFree(*p);
         MCK(cudaMalloc(p, (size_t)n * WIDTH * sizeof(float)));
@@ -544,40 +600,65 @@ int ensure_cap(am_mlp* m, int n) {
 const float* W_of(const am_mlp* m, int l) { return m->d_p + layer_w_off(l); }
 const float* b_of(const am_mlp* m, int l) { return m->d_p + layer_w_off(l) + (size_t)kDims[l + 1] * kDims[l]; }
 
-// forward (FP32) of n rows already in X (device) into the activation buffers
+// one product of a layer: 64 x 64 tiles where they fill the SMs
+template <int MODE>
+void gemm32(am_mlp* m, const float* A, const float* B, const float* bias, const float* act, float* C, int M, int N,
+            int K, int relu, int chunk, int chunks, size_t zstride, int bias_off) {
+    const long long big = (long long)((M + 63) / 64) * ((N + 63) / 64) * chunks;
+    const int R = big >= am::num_sms() ? 4 : 2;
+    const dim3 grid((N + 16 * R - 1) / (16 * R), (M + 16 * R - 1) / (16 * R), chunks);
+    if (R == 4)
+        am::launch_dep(k_gemm32<MODE, 4>, grid, dim3(256), 0, m->st, A, B, bias, act, C, M, N, K, relu, chunk, zstride,
+                       bias_off);
+    else
+        am::launch_dep(k_gemm32<MODE, 2>, grid, dim3(256), 0, m->st, A, B, bias, act, C, M, N, K, relu, chunk, zstride,
+                       bias_off);
+    am::count_launch();
+}
+
+// forward (FP32) of n rows already in X (device) into the activation
+// buffers; the last layer's output in d_zout
 void forward32(am_mlp* m, const float* X, int n) {
-    cudaStream_t s = m->st;
-    k_normalize<<<(n * FEAT + 255) / 256, 256, 0, s>>>(X, m->d_mu, m->d_sd, m->d_a[0], n);
+    k_normalize<<<(n * FEAT + 255) / 256, 256, 0, m->st>>>(X, m->d_mu, m->d_sd, m->d_a[0], n);
     am::count_launch();
     for (int l = 0; l < NLAYER; ++l) {
-        dim3 grid((kDims[l + 1] + 31) / 32, (n + 31) / 32);
-        k_linear_fwd<<<grid, 256, 0, s>>>(m->d_a[l], W_of(m, l), b_of(m, l), m->d_z[l + 1], m->d_a[l + 1], n,
-                                           kDims[l], kDims[l + 1], l < NLAYER - 1 ? 1 : 0);
-        am::count_launch();
+        const bool last = l == NLAYER - 1;
+        gemm32<kGemmFwd>(m, m->d_a[l], W_of(m, l), b_of(m, l), nullptr, last ? m->d_zout : m->d_a[l + 1], n,
+                         kDims[l + 1], kDims[l], last ? 0 : 1, 0, 1, 0, 0);
     }
+}
+
+// samples per partial gradient: at most kWgradChunks chunks of whole k-slices,
+// of at least 64 samples
+int wgrad_chunk(int n) {
+    const int c = std::max(64, (n + kWgradChunks - 1) / kWgradChunks);
+    return (c + kGemmK - 1) / kGemmK * kGemmK;
 }
 
 // loss and gradient (into d_g) of n rows (X, T device); loss added to d_loss
 void backward32(am_mlp* m, const float* X, const float* T, int n) {
     cudaStream_t s = m->st;
     forward32(m, X, n);
-    k_loss_grad<<<(n * OUT + 255) / 256, 256, 0, s>>>(m->d_z[NLAYER], T, m->d_sdo, m->d_dz0, n, m->d_loss);
+    k_loss_grad<<<(n * OUT + 255) / 256, 256, 0, s>>>(m->d_zout, T, m->d_sdo, m->d_dz0, n, m->d_loss);
     am::count_launch();
     float* dz = m->d_dz0;
     float* dzp = m->d_dz1;
+    const int chunk = wgrad_chunk(n), chunks = (n + chunk - 1) / chunk;
+    const size_t np = n_params_total();
+    float* part = chunks > 1 ? m->d_gpart : m->d_g;
     for (int l = NLAYER - 1; l >= 0; --l) {
         const int in = kDims[l], out = kDims[l + 1];
-        float* gW = m->d_g + layer_w_off(l);
-        float* gb = gW + (size_t)out * in;
-        dim3 gw((in + 31) / 32, (out + 31) / 32);
-        k_linear_wgrad<<<gw, 256, 0, s>>>(dz, m->d_a[l], gW, gb, n, in, out);
-        am::count_launch();
+        gemm32<kGemmWgrad>(m, dz, m->d_a[l], nullptr, nullptr, part + layer_w_off(l), out, in, n, 0, chunk, chunks, np,
+                           out * in);
         if (l > 0) {
-            dim3 gx((in + 31) / 32, (n + 31) / 32);
-            k_linear_xgrad<<<gx, 256, 0, s>>>(dz, W_of(m, l), m->d_z[l], dzp, n, in, out);
-            am::count_launch();
+            gemm32<kGemmXgrad>(m, dz, W_of(m, l), nullptr, m->d_a[l], dzp, n, in, out, 0, 0, 1, 0, 0);
             std::swap(dz, dzp);
         }
+    }
+    if (chunks > 1) {
+        am::launch_dep(k_sum_grad, dim3(((int)np + 255) / 256), dim3(256), 0, s, (const float*)part, m->d_g, (int)np,
+                       chunks);
+        am::count_launch();
     }
 }
 
@@ -662,12 +743,11 @@ extern "C" AM_API void am_mlp_destroy(am_mlp* m) {
     for (void* p : {(void*)m->d_p, (void*)m->d_m, (void*)m->d_v, (void*)m->d_g, (void*)m->d_wbf, (void*)m->d_mu,
                     (void*)m->d_sd, (void*)m->d_sdo, (void*)m->d_X, (void*)m->d_T, (void*)m->d_bx, (void*)m->d_bt,
                     (void*)m->d_dz0, (void*)m->d_dz1, (void*)m->d_h0, (void*)m->d_h1, (void*)m->d_rows,
-                    (void*)m->d_loss, (void*)m->d_flag})
+                    (void*)m->d_loss, (void*)m->d_flag, (void*)m->d_gpart})
         if (p) cudaFree(p);
-    for (int l = 0; l <= NLAYER; ++l) {
-        if (m->d_z[l]) cudaFree(m->d_z[l]);
+    for (int l = 0; l <= NLAYER; ++l)
         if (m->d_a[l]) cudaFree(m->d_a[l]);
-    }
+    if (m->d_zout) cudaFree(m->d_zout);
     delete m;
 }
 
@@ -701,18 +781,23 @@ extern "C" AM_API int am_mlp_set_norm(am_mlp* m, const float* mu, const float* s
     return AM_OK;
 }
 
+// The samples in the model's device buffers, which grow to the largest set
+// and stay (freeing and allocating them on every call synchronised the device
+// three times)
 static int upload_data(am_mlp* m, const float* X, const float* T, int n) {
-    if (m->d_X) cudaFree(m->d_X);
-    if (m->d_T) cudaFree(m->d_T);
-    if (m->d_rows) cudaFree(m->d_rows);
-    m->d_X = m->d_T = nullptr;
-    m->d_rows = nullptr;
-    MCK(cudaMalloc(&m->d_X, (size_t)n * FEAT * sizeof(float)));
-    MCK(cudaMalloc(&m->d_T, (size_t)std::max(n, 1) * OUT * sizeof(float)));
-    MCK(cudaMalloc(&m->d_rows, (size_t)n * sizeof(int)));
+    if (n > m->data_cap) {
+        for (void* p : {(void*)m->d_X, (void*)m->d_T, (void*)m->d_rows})
+            if (p) cudaFree(p);
+        m->d_X = m->d_T = nullptr;
+        m->d_rows = nullptr;
+        m->data_cap = 0;
+        MCK(cudaMalloc(&m->d_X, (size_t)n * FEAT * sizeof(float)));
+        MCK(cudaMalloc(&m->d_T, (size_t)n * OUT * sizeof(float)));
+        MCK(cudaMalloc(&m->d_rows, (size_t)n * sizeof(int)));
+        m->data_cap = n;
+    }
     MCK(cudaMemcpyAsync(m->d_X, X, (size_t)n * FEAT * sizeof(float), cudaMemcpyHostToDevice, m->st));
     if (T) MCK(cudaMemcpyAsync(m->d_T, T, (size_t)n * OUT * sizeof(float), cudaMemcpyHostToDevice, m->st));
-    m->data_n = n;
     return AM_OK;
 }
 
@@ -787,7 +872,7 @@ extern "C" AM_API int am_mlp_predict(am_mlp* m, const float* X, int n, int bf16,
         predict_bf16(m, m->d_X, n, dY, m->d_flag);
     } else {
         forward32(m, m->d_X, n);
-        MCK(cudaMemcpyAsync(dY, m->d_z[NLAYER], (size_t)n * OUT * sizeof(float), cudaMemcpyDeviceToDevice, m->st));
+        MCK(cudaMemcpyAsync(dY, m->d_zout, (size_t)n * OUT * sizeof(float), cudaMemcpyDeviceToDevice, m->st));
         k_scale_out<<<(n * OUT + 255) / 256, 256, 0, m->st>>>(dY, m->d_sdo, n);
         am::count_launch();
     }
