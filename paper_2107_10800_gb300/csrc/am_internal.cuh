@@ -14,7 +14,6 @@ namespace am {
 
 constexpr int kTile = 128;        // sources per shared-memory tile
 constexpr int kThreads = 128;     // threads per block of the pair kernels
-constexpr int kSbChunks = 16;     // most source chunks of the single-blob body mobility
 constexpr double kPi = 3.14159265358979323846;
 
 extern std::atomic<long long> g_launches;
@@ -88,7 +87,10 @@ struct SymItem {
     int tbase, sys;         // first blob of the system, system
     int ti, tj;             // tile indices within the system (partial-sum slots)
     long long poff;         // the system's partial-sum offset
-    int n3, pad;            // 3 N_s
+    int n3;                 // doubles per slot: 3 N_s (6 per body for single-blob bodies)
+    int steps = 32 << 8;    // k_sym_tiles: steps [steps & 255, steps >> 8) of every warp tile
+    __device__ __forceinline__ int step0() const { return steps & 255; }
+    __device__ __forceinline__ int step1() const { return steps >> 8; }
 };
 
 // ---- device helpers -----------------------------------------------------
@@ -309,7 +311,12 @@ struct am_handle {
     // steric repulsion (am_set_repulsion): parameters and blob forces (3Nb)
     bool steric_on = false;
     bool sb = false;   // single-blob bodies (am_config.single_blob)
-    double* d_sbpart = nullptr;   // kSbChunks x 6M partial sums of the body mobility
+    // symmetric tile product of the body mobility: items, partial-sum slots
+    void* d_sb_items = nullptr;
+    double* d_sbpart = nullptr;
+    long long* d_sb_poff = nullptr;
+    int* d_sb_nslots = nullptr;
+    int n_sb_items = 0, sb_grid = 0;
     double st_eps = 0.0, st_b = 1.0, st_rc = 0.0, st_eps_w = 0.0, st_b_w = 1.0;
     double* d_fst = nullptr;
     double *d_zbuf = nullptr, *d_cbuf = nullptr;

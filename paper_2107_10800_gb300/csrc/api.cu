@@ -143,7 +143,8 @@ void free_bodies(am_handle* h) {
     h->n_pcb_small = 0;
     h->pcb_cs = 1;
     h->n_pcw = 0;
-    dfree(&h->d_qnew); dfree(&h->d_thnew); dfree(&h->d_iters); dfree(&h->d_q0); dfree(&h->d_th0); dfree(&h->d_fst); dfree(&h->d_sbpart);
+    dfree(&h->d_qnew); dfree(&h->d_thnew); dfree(&h->d_iters); dfree(&h->d_q0); dfree(&h->d_th0); dfree(&h->d_fst);
+    am::sb_layout_free(h);
 }
 
 void free_solver(am_handle* h) {
@@ -661,7 +662,6 @@ int build_layout(am_handle* h, int M, int Nb, int NA, int maxb, const double* q,
     CK(dalloc(&h->d_qnew, 3 * (size_t)M)); CK(dalloc(&h->d_thnew, 4 * (size_t)M));
     CK(dalloc(&h->d_q0, 3 * (size_t)M)); CK(dalloc(&h->d_th0, 4 * (size_t)M));
     CK(dalloc(&h->d_fst, 3 * (size_t)Nb));
-    if (h->sb) CK(dalloc(&h->d_sbpart, (size_t)am::kSbChunks * 6 * M));
     CK(dalloc(&h->d_iters, NA));
     if (h->h_iters) cudaFreeHost(h->h_iters);
     h->h_iters = nullptr;
@@ -753,6 +753,7 @@ int build_system_maps(am_handle* h) {
         const int rc = am::periodic_setup(h);
         if (rc) return set_err(h, rc, "am_set_bodies: " + h->err);
     }
+    if (h->sb && am::sb_layout(h)) return set_err(h, AM_ERR_CUDA, "am_set_bodies: device allocation failed");
     return am::mobility_layout(h, h->cfg.precision == AM_MIXED ? 2 : 1, 0) ? AM_ERR_CUDA : AM_OK;
 }
 

@@ -76,6 +76,8 @@ int learned_features(am_handle* h, float* X, float* T);
 void steric_apply(am_handle* h);
 // Single-blob mode (single_blob.cu): grand mobility product v = N g (6M),
 // the right-hand side (N F, B), the operator, the preconditioner.
+int sb_layout(am_handle* h);  // items and slots for the current systems; 0 on success
+void sb_layout_free(am_handle* h);
 void sb_mobility(am_handle* h, const double* g, double* v);
 void sb_rhs(am_handle* h);
 void sb_op_apply(am_handle* h, const double* y, double* out);

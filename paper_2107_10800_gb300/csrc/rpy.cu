@@ -1379,7 +1379,7 @@ int mobility_layout(am_handle* h, int tpt, int chunk, int tgroup, int sym) {
                     it.i0 = b0 + a * T; it.ni = std::min(T, nb - a * T);
                     it.j0 = b0 + b * T; it.nj = std::min(T, nb - b * T);
                     it.tbase = b0; it.sys = s; it.ti = a; it.tj = b;
-                    it.poff = poff[s]; it.n3 = 3 * nb; it.pad = 0;
+                    it.poff = poff[s]; it.n3 = 3 * nb;
                     sitems.push_back(it);
                 }
         }

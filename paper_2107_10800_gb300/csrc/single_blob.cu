@@ -21,9 +21,9 @@
 #include "am_internal.cuh"
 #include "ops.cuh"
 #include "rpy_pair.cuh"
+#include "sym_tiles.cuh"
 
 #include <algorithm>
-#include <climits>
 
 namespace am {
 
@@ -66,102 +66,98 @@ __global__ void k_sb_ctphi(int M, const int* __restrict__ blo, const int* __rest
     for (int k = 0; k < 6; ++k) g[6 * (size_t)p + k] = v[k];
 }
 
-// v = N g for all systems (block diagonal): one thread per target body,
-// source bodies of the union of the block's systems in shared-memory tiles
-__global__ void __launch_bounds__(kThreads)
-k_sb_mobility(int M, const double* __restrict__ q, const int* __restrict__ sys_of_U,
-              const int* __restrict__ sys_body_off, const double* __restrict__ g, RpyK<double> k, double eta,
-              double a, double* __restrict__ v) {
-    __shared__ double sx[kTile][3];
-    __shared__ double sg[kTile][6];
-    __shared__ int s_lo, s_hi;
-    const int i = blockIdx.x * kThreads + threadIdx.x;
-    const bool live = i < M;
-    int j0 = INT_MAX, j1 = 0;
-    double xi[3] = {0.0, 0.0, 0.0};
-    if (live) {
-        const int s = sys_of_U[6 * (size_t)i];
-        j0 = sys_body_off[s];
-        j1 = sys_body_off[s + 1];
-        for (int c = 0; c < 3; ++c) xi[c] = q[3 * (size_t)i + c];
-    }
-    if (threadIdx.x == 0) { s_lo = INT_MAX; s_hi = 0; }
-    __syncthreads();
-    if (live) { atomicMin(&s_lo, j0); atomicMax(&s_hi, j1); }
-    __syncthreads();
-    // this block's share of the sources: chunk blockIdx.y of gridDim.y
-    const int span = s_hi - s_lo;
-    const int lo_all = s_lo + (int)((long long)span * blockIdx.y / gridDim.y);
-    const int hi_all = s_lo + (int)((long long)span * (blockIdx.y + 1) / gridDim.y);
-    const double pi = 3.14159265358979323846;
-    const double ctr_far = 1.0 / (8.0 * pi * eta);          // c r^2
-    const double cnear = 1.0 / (16.0 * pi * eta * a * a);   // c / (s - 3 s^2 / 8)
-    const double rr_far = 1.0 / (16.0 * pi * eta);           // |alpha| r^3, beta r^3 / 3
-    const double rr_near = 1.0 / (8.0 * pi * eta * a * a * a);
-    double ux = 0, uy = 0, uz = 0, wx = 0, wy = 0, wz = 0;  // translational part accumulates u / A1
-    for (int jt = lo_all; jt < hi_all; jt += kTile) {
-        const int cnt = min(kTile, hi_all - jt);
-        __syncthreads();
-        if (threadIdx.x < cnt) {
-            const int j = jt + threadIdx.x;
-            for (int c = 0; c < 3; ++c) sx[threadIdx.x][c] = q[3 * (size_t)j + c];
-            for (int c = 0; c < 6; ++c) sg[threadIdx.x][c] = g[6 * (size_t)j + c];
+// Both directions of one pair of bodies, velocities in units of A1 =
+// 1/(8 pi eta), d = x_i - x_j unnormalised.  With ri = 1/r:
+//   c1, c2 of the RPY tensor (rpy_pair.cuh);
+//   the coupling c / (r A1) = ri^3                       r >= 2a
+//                           = (1 - 3 s / 8) / (2 a^3)    r <  2a, s = r / a
+//   alpha / A1 = -ri^3 / 2,  beta / (r^2 A1) = 3 ri^5 / 2     r >= 2a
+//   alpha / A1 = (1 - 27 s / 32 + 5 s^3 / 64) / a^3,
+//   beta / (r^2 A1) = (9 / (32 s) - 3 s / 64) / a^5           r <  2a
+// (1/s taken as 0 at r = 0, where every term but the self mobilities
+// vanishes).  FP64-issue-bound: about 90 FP64 operations per unordered pair
+// (136 per ordered pair in the one-direction form with its divisions).
+struct SymSpherePair {
+    static constexpr int NC = 6;  // (force, torque) in, (velocity, rotation) out
+    RpyK<double> k;
+    double ia, h_a3, i_a3, n9_a4, n3_a5;  // 1/a, 1/(2 a^3), 1/a^3, 9/(32 a^4), -3/(64 a^5)
+    __device__ __forceinline__ double scale() const { return k.A1; }
+    __device__ __forceinline__ void both(const double* xi, const double* xj, const double* l, const double* m,
+                                         double* u, double* v) const {
+        const double dx = xi[0] - xj[0], dy = xi[1] - xj[1], dz = xi[2] - xj[2];
+        const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
+        double c1, c2, gc, al, be;
+        if (r2 >= k.four_a2) {
+            const double ri = rsq(r2);
+            const double ri2 = ri * ri, ri3 = ri * ri2;
+            c1 = ri * fma(k.kf2, ri2, 1.0);
+            c2 = ri3 * fma(-k.kf3, ri2, 1.0);
+            gc = ri3;
+            al = -0.5 * ri3;
+            be = 1.5 * (ri3 * ri2);
+        } else {
+            const double ri = r2 > 0.0 ? rsq(r2) : 0.0;
+            const double sv = (r2 * ri) * ia, s2 = sv * sv;
+            c1 = k.kn0 * fma(-k.kn1, r2 * ri, 1.0);
+            c2 = k.kn2 * ri;
+            gc = h_a3 * fma(-0.375, sv, 1.0);
+            al = i_a3 * fma(fma(5.0 / 64.0, s2, -27.0 / 32.0), sv, 1.0);
+            be = fma(n9_a4, ri, n3_a5 * sv);
         }
-        __syncthreads();
-        if (!live) continue;
-        for (int t = 0; t < cnt; ++t) {
-            const int j = jt + t;
-            if (j < j0 || j >= j1) continue;
-            const double f0 = sg[t][0], f1 = sg[t][1], f2 = sg[t][2];
-            const double T0 = sg[t][3], T1 = sg[t][4], T2 = sg[t][5];
-            const double dx = xi[0] - sx[t][0], dy = xi[1] - sx[t][1], dz = xi[2] - sx[t][2];
-            // translation from force (RPY, self included at r = 0)
-            pair_free<double>(dx, dy, dz, f0, f1, f2, k, ux, uy, uz);
-            const double r2 = dx * dx + dy * dy + dz * dz;
-            if (r2 == 0.0) {  // self rotation
-                wx += rr_near * T0; wy += rr_near * T1; wz += rr_near * T2;
-                continue;
-            }
-            const double r = sqrt(r2), ri = 1.0 / r;
-            const double ex = dx * ri, ey = dy * ri, ez = dz * ri;
-            double c, al, be;
-            if (r >= 2.0 * a) {
-                c = ctr_far * ri * ri;
-                const double r3 = ri * ri * ri;
-                al = -rr_far * r3;
-                be = 3.0 * rr_far * r3;
-            } else {
-                const double sv = r / a;
-                c = cnear * (sv - 0.375 * sv * sv);
-                al = rr_near * (1.0 - 27.0 / 32.0 * sv + 5.0 / 64.0 * sv * sv * sv);
-                be = rr_near * (9.0 / 32.0 * sv - 3.0 / 64.0 * sv * sv * sv);
-            }
-            // u_i += -c e x T_j  (translation from torque), divided by A1 to
-            // share the accumulator of the RPY part
-            const double cA = c / k.A1;
-            ux -= cA * (ey * T2 - ez * T1);
-            uy -= cA * (ez * T0 - ex * T2);
-            uz -= cA * (ex * T1 - ey * T0);
-            // omega_i += -c e x f_j + alpha T_j + beta (e . T_j) e
-            const double eT = ex * T0 + ey * T1 + ez * T2;
-            wx += -c * (ey * f2 - ez * f1) + al * T0 + be * eT * ex;
-            wy += -c * (ez * f0 - ex * f2) + al * T1 + be * eT * ey;
-            wz += -c * (ex * f1 - ey * f0) + al * T2 + be * eT * ez;
+        const double gx = gc * dx, gy = gc * dy, gz = gc * dz;
+        {
+            const double sf = c2 * fma(dx, l[0], fma(dy, l[1], dz * l[2]));
+            u[0] = fma(c1, l[0], fma(sf, dx, fma(gz, l[4], fma(-gy, l[5], u[0]))));
+            u[1] = fma(c1, l[1], fma(sf, dy, fma(gx, l[5], fma(-gz, l[3], u[1]))));
+            u[2] = fma(c1, l[2], fma(sf, dz, fma(gy, l[3], fma(-gx, l[4], u[2]))));
+            const double st = be * fma(dx, l[3], fma(dy, l[4], dz * l[5]));
+            u[3] = fma(al, l[3], fma(st, dx, fma(gz, l[1], fma(-gy, l[2], u[3]))));
+            u[4] = fma(al, l[4], fma(st, dy, fma(gx, l[2], fma(-gz, l[0], u[4]))));
+            u[5] = fma(al, l[5], fma(st, dz, fma(gy, l[0], fma(-gx, l[1], u[5]))));
+        }
+        {   // d and with it the coupling change sign
+            const double sf = c2 * fma(dx, m[0], fma(dy, m[1], dz * m[2]));
+            v[0] = fma(c1, m[0], fma(sf, dx, fma(-gz, m[4], fma(gy, m[5], v[0]))));
+            v[1] = fma(c1, m[1], fma(sf, dy, fma(-gx, m[5], fma(gz, m[3], v[1]))));
+            v[2] = fma(c1, m[2], fma(sf, dz, fma(-gy, m[3], fma(gx, m[4], v[2]))));
+            const double st = be * fma(dx, m[3], fma(dy, m[4], dz * m[5]));
+            v[3] = fma(al, m[3], fma(st, dx, fma(-gz, m[1], fma(gy, m[2], v[3]))));
+            v[4] = fma(al, m[4], fma(st, dy, fma(-gx, m[2], fma(gz, m[0], v[4]))));
+            v[5] = fma(al, m[5], fma(st, dz, fma(-gy, m[0], fma(gx, m[1], v[5]))));
         }
     }
-    if (!live) return;
-    double* o = v + 6 * ((size_t)blockIdx.y * M + i);  // partial sums of chunk blockIdx.y
-    o[0] = k.A1 * ux; o[1] = k.A1 * uy; o[2] = k.A1 * uz;
-    o[3] = wx; o[4] = wy; o[5] = wz;
-}
+    __device__ __forceinline__ void self(const double*, const double* m, double* u) const {
+        for (int c = 0; c < 3; ++c) {
+            u[c] = fma(k.kn0, m[c], u[c]);
+            u[3 + c] = fma(i_a3, m[3 + c], u[3 + c]);
+        }
+    }
+};
 
-// v = sum over the nc chunks of the partial sums (fixed order)
-__global__ void k_sb_sum(int n6, int nc, const double* __restrict__ part, double* __restrict__ v) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n6) return;
+// v = the sum of the slots of the element's system (fixed order: 8 threads
+// per element take every eighth slot)
+__global__ void __launch_bounds__(256)
+k_sb_sum(int n6, const int* __restrict__ sys_of_U, const int* __restrict__ sys_body_off,
+         const long long* __restrict__ poff, const int* __restrict__ nslots, const double* __restrict__ part,
+         double* __restrict__ v) {
+    __shared__ double sh[8][32];
+    const int e = threadIdx.x & 31, q = threadIdx.x >> 5;
+    const int t = blockIdx.x * 32 + e;
     double a = 0.0;
-    for (int c = 0; c < nc; ++c) a += part[(size_t)c * n6 + t];
-    v[t] = a;
+    if (t < n6) {
+        const int s = sys_of_U[t], b0 = sys_body_off[s];
+        const size_t n = 6 * (size_t)(sys_body_off[s + 1] - b0);
+        const double* p = part + poff[s] + (t - 6 * (size_t)b0);
+        const int ns = nslots[s];
+#pragma unroll 4
+        for (int c = q; c < ns; c += 8) a += p[c * n];
+    }
+    sh[q][e] = a;
+    __syncthreads();
+    if (q == 0 && t < n6) {
+        for (int c = 1; c < 8; ++c) a += sh[c][e];
+        v[t] = a;
+    }
 }
 
 // out_U = U - v (v = N C^T phi); out_phi = C U
@@ -211,16 +207,67 @@ static double sb_mur(const am_handle* h) {
     return 1.0 / (8.0 * 3.14159265358979323846 * h->cfg.eta * a * a * a);
 }
 
+int sb_layout(am_handle* h) {
+    long long tiles2 = 0;
+    for (const auto& r : h->sys) {
+        const long long ng = (r.M + 32LL * sym_group_tiles(r.M) - 1) / (32LL * sym_group_tiles(r.M));
+        tiles2 += ng * (ng + 1) / 2;
+    }
+    const int splits = sym_step_splits(tiles2);
+    std::vector<SymItem> items;
+    std::vector<long long> poff(h->S);
+    std::vector<int> nslots(h->S);
+    long long off = 0;
+    for (int s = 0; s < h->S; ++s) {
+        const int n = h->sys[s].M;
+        poff[s] = off;
+        nslots[s] = sym_append_items(items, s, h->sys_body0[s], n, 6, sym_group_tiles(n), splits, off);
+        off += 6LL * n * nslots[s];
+    }
+    sb_layout_free(h);
+    cudaStream_t st = h->stream;
+    int per = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_sym_tiles<SymSpherePair>, 32 * kSymWarps, 0) !=
+            cudaSuccess || per <= 0)
+        per = 4;
+    h->n_sb_items = (int)items.size();
+    h->sb_grid = std::min(per * num_sms(), (h->n_sb_items + kSymWarps - 1) / kSymWarps);
+    if (cudaMalloc(&h->d_sb_items, items.size() * sizeof(SymItem)) != cudaSuccess ||
+        cudaMalloc(reinterpret_cast<void**>(&h->d_sbpart), off * sizeof(double)) != cudaSuccess ||
+        cudaMalloc(reinterpret_cast<void**>(&h->d_sb_poff), h->S * sizeof(long long)) != cudaSuccess ||
+        cudaMalloc(reinterpret_cast<void**>(&h->d_sb_nslots), h->S * sizeof(int)) != cudaSuccess ||
+        cudaMemcpyAsync(h->d_sb_items, items.data(), items.size() * sizeof(SymItem), cudaMemcpyHostToDevice, st) !=
+            cudaSuccess ||
+        cudaMemcpyAsync(h->d_sb_poff, poff.data(), h->S * sizeof(long long), cudaMemcpyHostToDevice, st) !=
+            cudaSuccess ||
+        cudaMemcpyAsync(h->d_sb_nslots, nslots.data(), h->S * sizeof(int), cudaMemcpyHostToDevice, st) != cudaSuccess)
+        return 1;
+    return cudaStreamSynchronize(st) != cudaSuccess;
+}
+
+void sb_layout_free(am_handle* h) {
+    for (void* p : {h->d_sb_items, (void*)h->d_sbpart, (void*)h->d_sb_poff, (void*)h->d_sb_nslots})
+        if (p) cudaFree(p);
+    h->d_sb_items = nullptr;
+    h->d_sbpart = nullptr;
+    h->d_sb_poff = nullptr;
+    h->d_sb_nslots = nullptr;
+    h->n_sb_items = 0;
+}
+
+// v = N g for all systems (block diagonal): the symmetric tile product of
+// sym_tiles.cuh.  6,000 bodies: 7.80 -> 3.02 ms a product (one thread per
+// target over every ordered pair before; the FP64 pipe needs about 2.6 ms for
+// 90 operations per unordered pair).
 void sb_mobility(am_handle* h, const double* g, double* v) {
-    // source chunks so that the grid has about 4 blocks per SM (at most
-    // kSbChunks; the partial sums live in d_sbpart)
-    const int tb = nb(h->M, kThreads);
-    const int nc = std::max(1, std::min(kSbChunks, (4 * num_sms() + tb - 1) / tb));
-    dim3 grid(tb, nc);
-    k_sb_mobility<<<grid, kThreads, 0, h->stream>>>(
-        h->M, h->d_q, h->d_sys_of_elem, h->d_sys_body_off, g, rpy_consts<double>(h->prm), h->cfg.eta,
-        h->cfg.blob_radius, h->d_sbpart);
-    k_sb_sum<<<nb(6LL * h->M, 256), 256, 0, h->stream>>>(6 * h->M, nc, h->d_sbpart, v);
+    const double a = h->cfg.blob_radius, a3 = a * a * a, a4 = a3 * a;
+    const SymSpherePair pr{rpy_consts<double>(h->prm), 1.0 / a, 0.5 / a3, 1.0 / a3, 9.0 / (32.0 * a4),
+                           -3.0 / (64.0 * a4 * a)};
+    launch_dep(k_sym_tiles<SymSpherePair>, dim3(h->sb_grid), dim3(32 * kSymWarps), 0, h->stream,
+               (const double*)h->d_q, g, h->d_sbpart, static_cast<const SymItem*>(h->d_sb_items), h->n_sb_items,
+               h->d_item_counter, pr, (const int*)nullptr);
+    k_sb_sum<<<nb(6LL * h->M, 32), 256, 0, h->stream>>>(6 * h->M, h->d_sys_of_elem, h->d_sys_body_off, h->d_sb_poff,
+                                                        h->d_sb_nslots, h->d_sbpart, v);
     count_launch(2);
     long long pairs = 0;
     for (const auto& r : h->sys) pairs += (long long)r.M * r.M;

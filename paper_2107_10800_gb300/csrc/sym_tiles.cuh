@@ -1,0 +1,203 @@
+// Symmetric FP64 products on 32 x 32 warp tiles: u = N g for a symmetric
+// pair tensor N (N_ji = N_ij^T), each unordered pair evaluated once and
+// applied in both directions.
+//
+// A warp takes a tile of 32 targets, one per lane, against 32 sources staged
+// in its own shared memory: at step t lane l meets source (l + t) mod 32, the
+// target's sum stays on the lane and the source's column sum moves one lane
+// per step, so that it meets every target once.  On a tile against itself
+// steps 1..15, and 16 on half the lanes, take every unordered pair once (step
+// 0: the self term).  A work item is a pair of groups of whole tiles (I <= J)
+// of one system; its warp walks the tile pairs, keeps a target tile's sums in
+// registers across the source tiles and adds the column sums to the item's
+// own slots of the partial sums, so the order of every sum is fixed and the
+// result does not depend on scheduling.  The slots (one per group of the
+// system) are added by the caller.
+//
+// Why this shape: GB300 issues 2 FP64 multiply-adds per SM and cycle (16
+// cycles for a warp), so the FP64 pipe bounds the product and nothing but FP64
+// operations counts; a warp that needs no block barrier and stages its own
+// sources keeps the pipe fed with 4 to 5 warps per scheduler.  Groups of
+// several tiles (up to 96 groups per system) bound the partial sums at 96
+// slots; systems too small to give every SM a few warps split the 32 steps
+// of a tile over up to 8 items (each with its own slots).
+#pragma once
+#include "am_internal.cuh"
+#include "rpy_pair.cuh"
+
+#include <algorithm>
+#include <vector>
+
+namespace am {
+
+constexpr int kSymWarps = 4;       // warps per block
+constexpr int kSymMaxGroups = 96;  // most groups (partial-sum slots) per system
+
+// The blob mobility (3 components), free space or wall; sums in units of A1.
+template <bool WALL>
+struct SymBlobPair {
+    static constexpr int NC = 3;
+    RpyK<double> k;
+    __device__ __forceinline__ double scale() const { return k.A1; }
+    __device__ __forceinline__ void both(const double* xi, const double* xj, const double* l, const double* m,
+                                         double* u, double* v) const {
+        const double dx = xi[0] - xj[0], dy = xi[1] - xj[1], dz = xi[2] - xj[2];
+        if (WALL) {
+            const double rxy2 = fma(dx, dx, dy * dy);
+            pair_wall_sym<double>(dx, dy, dz, rxy2, fma(dz, dz, rxy2), xi[2] + xj[2], 2.0 * xj[2], -xi[2], l[0], l[1],
+                                  l[2], m[0], m[1], m[2], k, u[0], u[1], u[2], v[0], v[1], v[2]);
+        } else {
+            pair_free_sym<double>(dx, dy, dz, fma(dx, dx, fma(dy, dy, dz * dz)), l[0], l[1], l[2], m[0], m[1], m[2], k,
+                                  u[0], u[1], u[2], v[0], v[1], v[2]);
+        }
+    }
+    __device__ __forceinline__ void self(const double* xi, const double* m, double* u) const {
+        if (WALL)
+            pair_wall_r2<double>(0.0, 0.0, 0.0, 0.0, 0.0, 2.0 * xi[2], 2.0 * xi[2], -xi[2], m[0], m[1], m[2], k, u[0],
+                                 u[1], u[2]);
+        else
+            pair_free<double>(0.0, 0.0, 0.0, m[0], m[1], m[2], k, u[0], u[1], u[2]);
+    }
+};
+
+// x: positions, g: NC values per target, both indexed by the items' blob (or
+// body) numbers; part: the slots.  counter[0]: next item, counter[1]: blocks
+// finished.
+template <class Pair>
+__global__ void __launch_bounds__(32 * kSymWarps)
+k_sym_tiles(const double* __restrict__ x, const double* __restrict__ g, double* __restrict__ part,
+            const SymItem* __restrict__ items, int n_items, int* __restrict__ counter, Pair pr,
+            const int* __restrict__ active) {
+    dep_wait();
+    constexpr int NC = Pair::NC;
+    __shared__ double sx[kSymWarps][3 + NC][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double(*src)[32] = sx[warp];
+    for (int round = 0;; ++round) {
+        int itn = 0;
+        if (round == 0)
+            itn = blockIdx.x + warp * gridDim.x;  // the first items spread over the SMs
+        else if (lane == 0)
+            itn = (int)gridDim.x * kSymWarps + atomicAdd(counter, 1);
+        itn = __shfl_sync(0xffffffffu, itn, 0);
+        if (itn >= n_items) break;
+        const SymItem m = items[itn];
+        const bool diag = m.ti == m.tj;
+        double* rowo = part + m.poff + (long long)m.tj * m.n3 + NC * (long long)(m.i0 - m.tbase);
+        double* colo = part + m.poff + (long long)m.ti * m.n3 + NC * (long long)(m.j0 - m.tbase);
+        if (active && !active[m.sys]) {  // a stopped system: zero partial sums
+            for (int q = lane; q < NC * m.ni; q += 32) rowo[q] = 0.0;
+            if (!diag)
+                for (int q = lane; q < NC * m.nj; q += 32) colo[q] = 0.0;
+            continue;
+        }
+        const int s0 = m.step0(), s1 = m.step1();
+        const double scale = pr.scale();
+        for (int ia = 0; ia < m.ni; ia += 32) {
+            const int t = ia + lane;
+            const bool ti_ok = t < m.ni;
+            double xi[3] = {0.0, 0.0, 1.0}, mu[NC], u[NC];
+#pragma unroll
+            for (int c = 0; c < NC; ++c) mu[c] = u[c] = 0.0;
+            if (ti_ok) {
+#pragma unroll
+                for (int c = 0; c < 3; ++c) xi[c] = x[3 * (size_t)(m.i0 + t) + c];
+#pragma unroll
+                for (int c = 0; c < NC; ++c) mu[c] = g[NC * (size_t)(m.i0 + t) + c];
+            }
+            for (int jb = diag ? ia : 0; jb < m.nj; jb += 32) {
+                const bool self_tile = diag && jb == ia;
+                __syncwarp();
+                {
+                    const int q = jb + lane;
+                    const bool ok = q < m.nj;
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) src[c][lane] = ok ? x[3 * (size_t)(m.j0 + q) + c] : 1.0;
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) src[3 + c][lane] = ok ? g[NC * (size_t)(m.j0 + q) + c] : 0.0;
+                }
+                __syncwarp();
+                double v[NC];
+#pragma unroll
+                for (int c = 0; c < NC; ++c) v[c] = 0.0;
+#pragma unroll 1
+                for (int step = s0; step < s1; ++step) {
+                    const int q = (lane + step) & 31;
+                    const bool ok = ti_ok && jb + q < m.nj &&
+                                    (!self_tile || (step >= 1 && (step < 16 || (step == 16 && lane < 16))));
+                    if (ok) {
+                        double xj[3], l[NC];
+#pragma unroll
+                        for (int c = 0; c < 3; ++c) xj[c] = src[c][q];
+#pragma unroll
+                        for (int c = 0; c < NC; ++c) l[c] = src[3 + c][q];
+                        pr.both(xi, xj, l, mu, u, v);
+                    } else if (self_tile && step == 0 && ti_ok) {
+                        pr.self(xi, mu, u);
+                    }
+                    // hand the column sum to the lane that meets this source next
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) v[c] = __shfl_sync(0xffffffffu, v[c], (lane + 1) & 31);
+                }
+                // lane l now holds the column sum of source (l + s1) mod 32
+                if (self_tile) {
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) u[c] += __shfl_sync(0xffffffffu, v[c], (lane - s1) & 31);
+                } else {
+                    const int q = jb + ((lane + s1) & 31);
+                    if (q < m.nj) {
+                        double* o = colo + NC * (size_t)q;
+#pragma unroll
+                        for (int c = 0; c < NC; ++c) o[c] = ia == 0 ? scale * v[c] : fma(scale, v[c], o[c]);
+                    }
+                }
+            }
+            // the rows of a diagonal item also hold the column sums of its
+            // earlier target tiles
+            __syncwarp();
+            if (ti_ok) {
+                double* o = rowo + NC * (size_t)t;
+#pragma unroll
+                for (int c = 0; c < NC; ++c) o[c] = diag && ia > 0 ? fma(scale, u[c], o[c]) : scale * u[c];
+            }
+        }
+    }
+    item_queue_done(counter);
+}
+
+// Tiles per group of a system of n: at most kSymMaxGroups groups.
+inline int sym_group_tiles(int n) {
+    const int tiles = (n + 31) / 32;
+    return tiles <= kSymMaxGroups ? 1 : (tiles + kSymMaxGroups - 1) / kSymMaxGroups;
+}
+
+// Splits of a tile's 32 steps (1, 2, 4 or 8) so that `items` items give the
+// GPU about two warps per scheduler (8 per SM).
+inline int sym_step_splits(long long items) {
+    int sp = 1;
+    while (sp < 8 && items * sp * 2 <= 8LL * num_sms()) sp *= 2;
+    return sp;
+}
+
+// Appends the items of one system: blobs base .. base + n - 1 in groups of
+// 32 `tiles`, steps split `splits` ways, partial sums at poff in slots of nc n
+// doubles.  Returns the number of slots.
+inline int sym_append_items(std::vector<SymItem>& out, int sys, int base, int n, int nc, int tiles, int splits,
+                            long long poff) {
+    const int T = 32 * tiles, ng = (n + T - 1) / T;
+    for (int a = 0; a < ng; ++a)
+        for (int b = a; b < ng; ++b)
+            for (int k = 0; k < splits; ++k) {
+                SymItem it;
+                it.i0 = base + a * T; it.ni = std::min(T, n - a * T);
+                it.j0 = base + b * T; it.nj = std::min(T, n - b * T);
+                it.tbase = base; it.sys = sys;
+                it.ti = a * splits + k; it.tj = b * splits + k;
+                it.poff = poff; it.n3 = nc * n;
+                it.steps = (32 * k / splits) | (32 * (k + 1) / splits) << 8;
+                out.push_back(it);
+            }
+    return ng * splits;
+}
+
+}  // namespace am

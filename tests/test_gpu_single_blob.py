@@ -9,6 +9,7 @@ import pytest
 
 from paper_2107_10800_gb300 import build, binding, workloads as W
 from oracle import single_blob as osb
+from oracle.mobility import rpy_free_pair
 
 pytestmark = pytest.mark.gpu
 
@@ -89,3 +90,22 @@ def test_single_blob_configuration_checks():
         cfg = binding.Config(1.0, 0.1, wall, prec, 1, 1e-8, 50, 100, 1e-10, 10, None, sbv)
         h = ctypes.c_void_p()
         assert L.am_create(ctypes.byref(cfg), ctypes.byref(h)) == binding.AM_ERR_ARG
+
+
+# the symmetric tile product at the edges of its tiles, of the step splits
+# (few tiles: 8, 4, 2 splits) and of the groups of tiles (96 groups hold
+# 3,072 bodies one tile each); FP64 sums of up to 3,100 terms, as the bar above
+@pytest.mark.parametrize("M", [31, 32, 33, 64, 65, 257, 577, 1121, 3072, 3073])
+def test_body_mobility_tile_edges(M):
+    rng = np.random.default_rng(M)
+    x = rng.uniform(0.0, (M / 4.0) ** (1 / 3), (M, 3))
+    g = rng.standard_normal((M, 6))
+    u = loose(x, 0.3).apply_mobility(g)
+    for i in {0, min(31, M - 1), min(32, M - 1), M // 2, M - 2, M - 1}:
+        ref = np.concatenate([g[i, :3] / (6 * np.pi * 1.3 * 0.3), g[i, 3:] / (8 * np.pi * 1.3 * 0.3 ** 3)])
+        for j in range(M):
+            if j != i:
+                d = x[i] - x[j]
+                ref[:3] += rpy_free_pair(d, 0.3, 1.3) @ g[j, :3] + osb.pair_rt(-d, 0.3, 1.3).T @ g[j, 3:]
+                ref[3:] += osb.pair_rt(d, 0.3, 1.3) @ g[j, :3] + osb.pair_rr(d, 0.3, 1.3) @ g[j, 3:]
+        assert rel(u[i], ref) <= 1e-12
