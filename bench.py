@@ -254,7 +254,7 @@ def matvec_at_scale(torch, binding, W, stream, fp32_peak, fp64_peak):
         out[key] = {"blobs": n, "ms": t * 1e3, "pairs_per_s": pairs / t,
                     "tflops": pairs * fpp / t / 1e12, "frac_of_fma_peak": pairs * fpp / t / peak,
                     "kernel": {"mixed": "rpy_items_mixed_x2<wall>", "mixed_symmetric": "rpy_sym_mixed_x2<wall>",
-                               "fp64": "rpy_items_f64<wall>", "fp64_symmetric": "rpy_sym_f64<wall, tile 128>"}[key]}
+                               "fp64": "rpy_items_f64<wall>", "fp64_symmetric": "k_sym_tiles<SymBlobPair<wall>>, tiles of 128"}[key]}
     return out
 
 
@@ -812,7 +812,7 @@ def run_ours(args):
         # symmetric FP64 product: each unordered pair evaluated once and applied
         # both ways, 126 flop per unordered pair (FMA = 2, rsqrt = 1, counted
         # from pair_wall_sym and the pair's distances) against 2 x 119
-        kname = "rpy_sym_f64<wall, tile %d>" % layout[3]
+        kname = "k_sym_tiles<SymBlobPair<wall>>, tiles of %d" % layout[3]
         executed = nb * (nb + 1) / 2 * SYM_WALL_FLOP_PER_UNORDERED_PAIR / avg_launch_s
     else:
         kname = "rpy_items_%s<wall>" % ("f64" if args.precision == "fp64" else "mixed")

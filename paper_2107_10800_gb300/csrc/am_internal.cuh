@@ -222,9 +222,11 @@ struct am_handle {
     int* d_item_counter = nullptr;
     int mv_tpt = 1, mv_chunk = 0, mv_tgroup = 0, mv_grid = 0, mv_grid64 = 0, mv_griddf = 0;
     long long mv_part_total = 0;
+    int mv_sum_groups = 1;  // threads per element in the sum over slots (slot_sum)
     bool mv_tuned = false;
     // tile-pair items of the symmetric FP64 product (tiles of 32 sym_nsub blobs)
     void* d_sym_items = nullptr;
+    int sym_splits = 1;  // items per tile pair, each with part of the steps (FP64 kernel only)
     int n_sym = 0, sym_nsub = 0, mv_gridsym = 0, mv_gridsym32 = 0, mv_gridsymdf = 0;
 
     // host structure

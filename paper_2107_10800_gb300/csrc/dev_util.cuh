@@ -45,6 +45,37 @@ __device__ __forceinline__ bool arrive_last(int* cnt, int idx, int total) {
     return last;
 }
 
+// Element of u = M lambda from the partial sums, in a block of 256 threads for
+// 256 / G elements: G threads add the slots of an element's system (thread g
+// of them every G-th slot, then the G sums in order; the result is valid in
+// threads 0 .. 256 / G - 1, whose element is blk 256 / G + threadIdx.x).  G = 8
+// for many slots (consecutive threads still read consecutive doubles, and the
+// chain of dependent additions is an eighth of the slots), else 1.  Every
+// thread calls it; sh: 256 doubles.
+__device__ __forceinline__ double slot_sum(int blk, int G, int n3, const double* __restrict__ part,
+                                           const int* __restrict__ sys_of_blob, const int* __restrict__ sys_blob0,
+                                           const int* __restrict__ sys_nb, const int* __restrict__ sys_nch,
+                                           const long long* __restrict__ sys_poff, double* sh) {
+    const int per = 256 / G, q = threadIdx.x / per;
+    const int t = blk * per + (int)threadIdx.x - q * per;
+    double a = 0.0;
+    if (t < n3) {
+        const int s = sys_of_blob[t / 3];
+        const size_t n = 3 * (size_t)sys_nb[s];
+        const double* p = part + sys_poff[s] + (t - 3 * (size_t)sys_blob0[s]);
+        const int ns = sys_nch[s];
+#pragma unroll 4
+        for (int c = q; c < ns; c += G) a += p[c * n];
+    }
+    if (G > 1) {
+        sh[threadIdx.x] = a;
+        __syncthreads();
+        if (q == 0)
+            for (int c = 1; c < G; ++c) a += sh[c * per + threadIdx.x];
+    }
+    return a;
+}
+
 __device__ __forceinline__ void cross3(const double* a, const double* b, double* o) {
     o[0] = a[1] * b[2] - a[2] * b[1];
     o[1] = a[2] * b[0] - a[0] * b[2];

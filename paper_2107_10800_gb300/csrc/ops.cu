@@ -75,7 +75,8 @@ __global__ void k_rhs(int Nb, int M, int P, const double* __restrict__ slip,
 //                                 rigid velocity u_p + omega_p x (r_i - q_p))
 // out_U      = -K^T lambda + C^T phi
 // out_phi    = C U   (per link: u_p + omega_p x l_np - u_q - omega_q x l_nq)
-__global__ void k_op_epilogue(int Nb, int M, int P, int nblob_blocks, int nbody_blocks,
+__global__ void __launch_bounds__(256)
+k_op_epilogue(int Nb, int M, int P, int nblob_blocks, int nbody_blocks, int G, int L, int bpb,
                               const double* __restrict__ part, const int* __restrict__ sys_of_blob,
                               const int* __restrict__ sys_blob0, const int* __restrict__ sys_nb,
                               const int* __restrict__ sys_nch, const long long* __restrict__ sys_poff,
@@ -92,59 +93,53 @@ __global__ void k_op_epilogue(int Nb, int M, int P, int nblob_blocks, int nbody_
     double* oU = out + 3 * (size_t)Nb;
     double* of = oU + 6 * (size_t)M;
     const int b = blockIdx.x;
-    if (b < nblob_blocks) {
-        const int i = b * blockDim.x + threadIdx.x;
-        if (i >= Nb) return;
-        const int sy = sys_of_blob[i];
-        const size_t n3 = 3 * (size_t)sys_nb[sy];
-        const double* pb = part + sys_poff[sy] + 3 * (size_t)(i - sys_blob0[sy]);
-        double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-        for (int t = 0; t < sys_nch[sy]; ++t) {
-            const double* pp = pb + t * n3;
-            s0 += pp[0]; s1 += pp[1]; s2 += pp[2];
-        }
-        const int p = body_of_blob[i];
-        const double4_32a d = d4[i];
-        const double* u = U + 6 * p;
-        // u + omega x d
-        const double k0 = u[0] + (u[4] * d.z - u[5] * d.y);
-        const double k1 = u[1] + (u[5] * d.x - u[3] * d.z);
-        const double k2 = u[2] + (u[3] * d.y - u[4] * d.x);
-        out[3 * (size_t)i] = s0 - k0;
-        out[3 * (size_t)i + 1] = s1 - k1;
-        out[3 * (size_t)i + 2] = s2 - k2;
-    } else if (b < nblob_blocks + nbody_blocks) {
-        const int wpb = blockDim.x >> 5;
-        const int p = (b - nblob_blocks) * wpb + (threadIdx.x >> 5);
-        const int lane = threadIdx.x & 31;
-        if (p >= M) return;
-        double f0 = 0, f1 = 0, f2 = 0, t0 = 0, t1 = 0, t2 = 0;
-        for (int i = blob_off[p] + lane; i < blob_off[p + 1]; i += 32) {
-            const double4_32a d = d4[i];
-            const double l0 = lam[3 * (size_t)i], l1 = lam[3 * (size_t)i + 1], l2 = lam[3 * (size_t)i + 2];
-            f0 += l0; f1 += l1; f2 += l2;
-            t0 += d.y * l2 - d.z * l1;
-            t1 += d.z * l0 - d.x * l2;
-            t2 += d.x * l1 - d.y * l0;
-        }
-        f0 = warp_sum(f0); f1 = warp_sum(f1); f2 = warp_sum(f2);
-        t0 = warp_sum(t0); t1 = warp_sum(t1); t2 = warp_sum(t2);
-        if (lane == 0) {
-            double c[6] = {0, 0, 0, 0, 0, 0};
-            for (int k = bl_off[p]; k < bl_off[p + 1]; ++k) {
-                const int e = bl_idx[k];
-                const int n = e >> 1;
+    if (b < nbody_blocks) {
+        // -K^T lambda + C^T phi: L lanes per body, each adding its share of
+        // the blobs and of the link ends, then one reduction of the six sums
+        // over the L lanes
+        const int slot = threadIdx.x / L, lane = threadIdx.x % L;
+        const int p = slot < bpb ? b * bpb + slot : M;
+        double v[6] = {0, 0, 0, 0, 0, 0};
+        if (p < M) {
+            const int e1 = bl_off[p + 1], i1 = blob_off[p + 1];
+            for (int k = bl_off[p] + lane; k < e1; k += L) {
+                const int e = bl_idx[k], n = e >> 1;
                 const double sg = (e & 1) ? -1.0 : 1.0;
                 const double* l = (e & 1) ? lq + 3 * n : lp + 3 * n;
-                const double* ph = phi + 3 * n;
-                double tq[3];
-                cross3(l, ph, tq);
-                for (int a = 0; a < 3; ++a) { c[a] += sg * ph[a]; c[3 + a] += sg * tq[a]; }
+                const double p0 = sg * phi[3 * n], p1 = sg * phi[3 * n + 1], p2 = sg * phi[3 * n + 2];
+                v[0] += p0; v[1] += p1; v[2] += p2;
+                v[3] = fma(l[1], p2, fma(-l[2], p1, v[3]));
+                v[4] = fma(l[2], p0, fma(-l[0], p2, v[4]));
+                v[5] = fma(l[0], p1, fma(-l[1], p0, v[5]));
             }
-            double* o = oU + 6 * p;
-            o[0] = c[0] - f0; o[1] = c[1] - f1; o[2] = c[2] - f2;
-            o[3] = c[3] - t0; o[4] = c[4] - t1; o[5] = c[5] - t2;
+#pragma unroll 4
+            for (int i = blob_off[p] + lane; i < i1; i += L) {
+                const double4_32a d = d4[i];
+                const double l0 = lam[3 * (size_t)i], l1 = lam[3 * (size_t)i + 1], l2 = lam[3 * (size_t)i + 2];
+                v[0] -= l0; v[1] -= l1; v[2] -= l2;
+                v[3] = fma(d.z, l1, fma(-d.y, l2, v[3]));
+                v[4] = fma(d.x, l2, fma(-d.z, l0, v[4]));
+                v[5] = fma(d.y, l0, fma(-d.x, l1, v[5]));
+            }
         }
+        for (int o = L >> 1; o > 0; o >>= 1)
+#pragma unroll
+            for (int c = 0; c < 6; ++c) v[c] += __shfl_xor_sync(0xffffffffu, v[c], o);
+        if (p < M && lane == 0)
+#pragma unroll
+            for (int c = 0; c < 6; ++c) oU[6 * (size_t)p + c] = v[c];
+    } else if (b < nbody_blocks + nblob_blocks) {  // 256 / G elements of lambda
+        __shared__ double sh[256];
+        const int blk = b - nbody_blocks;
+        const double s = slot_sum(blk, G, 3 * Nb, part, sys_of_blob, sys_blob0, sys_nb, sys_nch, sys_poff, sh);
+        const int t = blk * (256 / G) + threadIdx.x;
+        if (threadIdx.x >= 256 / G || t >= 3 * Nb) return;
+        const int i = t / 3, c = t - 3 * i;
+        const double* d = reinterpret_cast<const double*>(d4 + i);
+        const double* u = U + 6 * (size_t)body_of_blob[i];
+        // component c of u + omega x d
+        const int c1 = c == 2 ? 0 : c + 1, c2 = c == 0 ? 2 : c - 1;
+        out[t] = s - (u[c] + (u[3 + c1] * d[c2] - u[3 + c2] * d[c1]));
     } else {
         const int n = (b - nblob_blocks - nbody_blocks) * blockDim.x + threadIdx.x;
         if (n >= P) return;
@@ -950,8 +945,19 @@ void op_apply(am_handle* h, const double* y, double* out, int mode, const int* a
         return;
     }
     mobility_partial(h, y, mode, active);
-    const int nbb = nblk(h->Nb, 128), nbody = nblk(h->M, 4), nlink = nblk(h->P, 128);
-    launch_dep(k_op_epilogue, dim3(nbb + nbody + nlink), dim3(128), 0, h->stream, h->Nb, h->M, h->P, nbb, nbody,
+    // The body sums are bound by FP64 issue (16 cycles of its SM for every
+    // warp instruction, however few lanes take part) and by latency: few
+    // bodies take a warp each, spread over the SMs; many share a warp, each
+    // on as many lanes as have about six blobs to add (at most 16 blobs a
+    // lane for the largest body, whose chain would set the time)
+    const int G = h->mv_sum_groups;
+    int L = 32;
+    if (h->M > 4 * num_sms())
+        while (L > 1 && 6LL * L * h->M > h->Nb && h->max_body_blobs <= 8 * L) L >>= 1;
+    const int bpb = std::min(256 / L, nblk(h->M, num_sms()));
+    const int nbb = nblk(3LL * h->Nb, 256 / G), nbody = nblk(h->M, bpb), nlink = nblk(h->P, 256);
+    launch_dep(k_op_epilogue, dim3(nbb + nbody + nlink), dim3(256), 0, h->stream, h->Nb, h->M, h->P, nbb, nbody, G, L,
+               bpb,
                h->d_mv, h->d_sys_of_blob, h->d_sys_blob0, h->d_sys_nb, h->d_sys_nch, h->d_sys_poff, y, out,
                h->d_body_of_blob, h->d_blob_off, h->d_d4, h->d_body_link_off, h->d_body_link_idx, h->d_lp, h->d_lq,
                h->d_bp, h->d_bq);
@@ -1208,29 +1214,23 @@ static int gmres(am_handle* h, const double* rhs, double* x, double tol, bool fp
     return it;
 }
 
-// m2[s] += |u_i|^2 over the blobs of system s, u = M lambda summed from the
-// partials of the last mobility product (a warp whose blobs share one system
-// adds once)
-__global__ void k_sys_mob_norm2(int Nb, const double* __restrict__ part, const int* __restrict__ sys_of_blob,
-                                const int* __restrict__ sys_blob0, const int* __restrict__ sys_nb,
-                                const int* __restrict__ sys_nch, const long long* __restrict__ sys_poff,
-                                double* __restrict__ m2) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int lane = threadIdx.x & 31;
-    int s = -1;
-    double v = 0.0;
-    if (i < Nb) {
-        s = sys_of_blob[i];
-        const size_t n3 = 3 * (size_t)sys_nb[s];
-        const double* p = part + sys_poff[s] + 3 * (size_t)(i - sys_blob0[s]);
-        double a = 0.0, b = 0.0, c = 0.0;
-        for (int q = 0; q < sys_nch[s]; ++q) { a += p[q * n3]; b += p[q * n3 + 1]; c += p[q * n3 + 2]; }
-        v = a * a + b * b + c * c;
-    }
+// m2[s] += |u_t|^2 over the elements of system s, u = M lambda summed from the
+// partials of the last mobility product (a warp whose elements share one
+// system adds once)
+__global__ void __launch_bounds__(256)
+k_sys_mob_norm2(int n3, int G, const double* __restrict__ part, const int* __restrict__ sys_of_blob,
+                const int* __restrict__ sys_blob0, const int* __restrict__ sys_nb,
+                const int* __restrict__ sys_nch, const long long* __restrict__ sys_poff, double* __restrict__ m2) {
+    __shared__ double sh[256];
+    const double u = slot_sum(blockIdx.x, G, n3, part, sys_of_blob, sys_blob0, sys_nb, sys_nch, sys_poff, sh);
+    if (threadIdx.x >= 256 / G) return;
+    const int t = blockIdx.x * (256 / G) + threadIdx.x;
+    const int s = t < n3 ? sys_of_blob[t / 3] : -1;
+    double v = t < n3 ? u * u : 0.0;
     const int s0 = __shfl_sync(0xffffffffu, s, 0);
-    if (__all_sync(0xffffffffu, s == s0)) {
+    if (__all_sync(0xffffffffu, s == s0 || s < 0)) {
         v = warp_sum(v);
-        if (lane == 0 && s0 >= 0) atomicAdd(&m2[s0], v);
+        if ((threadIdx.x & 31) == 0 && s0 >= 0) atomicAdd(&m2[s0], v);
     } else if (s >= 0) {
         atomicAdd(&m2[s], v);
     }
@@ -1334,8 +1334,10 @@ int solve(am_handle* h, am_step_stats* st) {
                 // norms, and the mobility partials hold M32 lambda_dx
                 double* m2 = h->d_sysred + 2 * (size_t)h->S;
                 cudaMemsetAsync(m2, 0, h->S * sizeof(double), s);
-                k_sys_mob_norm2<<<nblk(h->Nb, 256), 256, 0, s>>>(h->Nb, h->d_mv, h->d_sys_of_blob, h->d_sys_blob0,
-                                                                 h->d_sys_nb, h->d_sys_nch, h->d_sys_poff, m2);
+                const int G = h->mv_sum_groups;
+                k_sys_mob_norm2<<<nblk(3LL * h->Nb, 256 / G), 256, 0, s>>>(
+                    3 * h->Nb, G, h->d_mv, h->d_sys_of_blob, h->d_sys_blob0, h->d_sys_nb, h->d_sys_nch, h->d_sys_poff,
+                    m2);
                 k_sys_resid_bound<<<nblk(h->S, 128), 128, 0, s>>>(h->S, tol, kMixedProductError, bn_out,
                                                                   h->d_beta_s, m2, be_out);
                 cudaMemcpyAsync(h->d_rir, h->d_V, h->n * sizeof(double), cudaMemcpyDeviceToDevice, s);

@@ -24,7 +24,9 @@
 // 152 SMs; each (target block, chunk) writes its partial sums, and a second
 // kernel adds the chunks.
 #include "am_internal.cuh"
+#include "dev_util.cuh"
 #include "rpy_pair.cuh"
+#include "sym_tiles.cuh"
 #include "ops.cuh"
 
 #include <algorithm>
@@ -517,130 +519,6 @@ rpy_items_f64(const double4_32a* __restrict__ r4, const double* __restrict__ lam
     item_queue_done(counter);
 }
 
-// Symmetric FP64 product (the mobility is symmetric: M_ji = M_ij^T).  Per
-// item the block stages both tiles; its warps take the item's NSUB x NSUB
-// warp tiles (32 targets x 32 sources) in turn.  In a warp tile lane l
-// holds target l and, at step t, meets source (l + t) mod 32: u_l gathers
-// M lambda_source, and the source's column sum v (M^T mu_l) is carried
-// from lane to lane (lane l hands it to lane l - 1), so after 32 steps it
-// is back on the source's lane with the sum over the 32 targets.  On the
-// diagonal of a diagonal item the steps 1..15, and 16 on lanes 0..15, take
-// every unordered pair once (step 0: the self term).  Warp-tile sums go to
-// shared memory and are added in a fixed order: the result does not
-// depend on scheduling.
-template <bool WALL, int NSUB>
-__global__ void __launch_bounds__(NSUB == 1 ? 32 : 128)
-rpy_sym_f64(const double4_32a* __restrict__ r4, const double* __restrict__ lam, double* __restrict__ part,
-            const SymItem* __restrict__ items, int n_items, int* __restrict__ counter, RpyK<double> k,
-            const int* __restrict__ active) {
-    dep_wait();
-    constexpr int T = 32 * NSUB;
-    constexpr int NW = NSUB == 1 ? 1 : 4;
-    constexpr int NWT = NSUB * NSUB;
-    __shared__ double4_32a sI[T], sJ[T];
-    __shared__ double lI[3 * T], lJ[3 * T];
-    __shared__ double up[NWT][32][3], vp[NWT][32][3];
-    __shared__ int s_item;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int round = 0;; ++round) {
-        __syncthreads();
-        if (threadIdx.x == 0) s_item = round == 0 ? (int)blockIdx.x : (int)gridDim.x + atomicAdd(counter, 1);
-        __syncthreads();
-        const int itn = s_item;
-        if (itn >= n_items) break;
-        const SymItem m = items[itn];
-        const bool diag = m.ti == m.tj;
-        double* rowo = part + m.poff + (long long)m.tj * m.n3 + 3 * (long long)(m.i0 - m.tbase);
-        double* colo = part + m.poff + (long long)m.ti * m.n3 + 3 * (long long)(m.j0 - m.tbase);
-        if (active && !active[m.sys]) {  // a stopped system: zero partial sums
-            for (int q = threadIdx.x; q < 3 * m.ni; q += blockDim.x) rowo[q] = 0.0;
-            if (!diag)
-                for (int q = threadIdx.x; q < 3 * m.nj; q += blockDim.x) colo[q] = 0.0;
-            continue;
-        }
-        for (int q = threadIdx.x; q < T; q += blockDim.x) {
-            double4_32a a = q < m.ni ? r4[m.i0 + q] : make_double4_32a(0.0, 0.0, 1.0, 0.0);
-            a.w = 2.0 * a.z;
-            sI[q] = a;
-            double4_32a b = q < m.nj ? r4[m.j0 + q] : make_double4_32a(0.0, 0.0, 1.0, 0.0);
-            b.w = 2.0 * b.z;
-            sJ[q] = b;
-        }
-        for (int q = threadIdx.x; q < 3 * T; q += blockDim.x) {
-            lI[q] = q < 3 * m.ni ? lam[3 * (size_t)m.i0 + q] : 0.0;
-            lJ[q] = q < 3 * m.nj ? lam[3 * (size_t)m.j0 + q] : 0.0;
-        }
-        __syncthreads();
-        for (int wt = warp; wt < NWT; wt += NW) {
-            const int a = wt / NSUB, b = wt % NSUB;
-            double ux = 0.0, uy = 0.0, uz = 0.0, vx = 0.0, vy = 0.0, vz = 0.0;
-            if (!(diag && b < a)) {  // below the diagonal of a diagonal item: taken by (b, a)
-                const bool self_tile = diag && a == b;
-                const int t = 32 * a + lane;
-                const double4_32a xi = sI[t];
-                const double mx = lI[3 * t], my = lI[3 * t + 1], mz = lI[3 * t + 2];
-                const double nx3 = -xi.z;
-                const bool ti_ok = t < m.ni;
-#pragma unroll 1
-                for (int step = 0; step < 32; ++step) {
-                    const int q = 32 * b + ((lane + step) & 31);
-                    const bool pair_ok = ti_ok && q < m.nj &&
-                                         (!self_tile || (step >= 1 && (step < 16 || (step == 16 && lane < 16))));
-                    if (pair_ok) {
-                        const double4_32a xj = sJ[q];
-                        const double lx = lJ[3 * q], ly = lJ[3 * q + 1], lz = lJ[3 * q + 2];
-                        const double dx = xi.x - xj.x, dy = xi.y - xj.y, dz = xi.z - xj.z;
-                        if (WALL) {
-                            const double rxy2 = fma(dx, dx, dy * dy);
-                            pair_wall_sym<double>(dx, dy, dz, rxy2, fma(dz, dz, rxy2), xi.z + xj.z, xj.w, nx3, lx,
-                                                  ly, lz, mx, my, mz, k, ux, uy, uz, vx, vy, vz);
-                        } else {
-                            pair_free_sym<double>(dx, dy, dz, fma(dx, dx, fma(dy, dy, dz * dz)), lx, ly, lz, mx,
-                                                  my, mz, k, ux, uy, uz, vx, vy, vz);
-                        }
-                    } else if (self_tile && step == 0 && ti_ok) {  // the self term
-                        if (WALL)
-                            pair_wall_r2<double>(0.0, 0.0, 0.0, 0.0, 0.0, 2.0 * xi.z, xi.w, nx3, mx, my, mz, k, ux,
-                                                 uy, uz);
-                        else
-                            pair_free<double>(0.0, 0.0, 0.0, mx, my, mz, k, ux, uy, uz);
-                    }
-                    // hand the column sum to the lane that meets this source next
-                    const int src = (lane + 1) & 31;
-                    vx = __shfl_sync(0xffffffffu, vx, src);
-                    vy = __shfl_sync(0xffffffffu, vy, src);
-                    vz = __shfl_sync(0xffffffffu, vz, src);
-                }
-            }
-            up[wt][lane][0] = ux; up[wt][lane][1] = uy; up[wt][lane][2] = uz;
-            vp[wt][lane][0] = vx; vp[wt][lane][1] = vy; vp[wt][lane][2] = vz;
-        }
-        __syncthreads();
-        for (int t = threadIdx.x; t < T; t += blockDim.x) {
-            const int a = t >> 5, l = t & 31;
-            if (t < m.ni) {
-                double sx = 0.0, sy = 0.0, sz = 0.0;
-                for (int b = 0; b < NSUB; ++b) {
-                    sx += up[a * NSUB + b][l][0]; sy += up[a * NSUB + b][l][1]; sz += up[a * NSUB + b][l][2];
-                }
-                if (diag)
-                    for (int a2 = 0; a2 < NSUB; ++a2) {
-                        sx += vp[a2 * NSUB + a][l][0]; sy += vp[a2 * NSUB + a][l][1]; sz += vp[a2 * NSUB + a][l][2];
-                    }
-                rowo[3 * t] = k.A1 * sx; rowo[3 * t + 1] = k.A1 * sy; rowo[3 * t + 2] = k.A1 * sz;
-            }
-            if (!diag && t < m.nj) {
-                double sx = 0.0, sy = 0.0, sz = 0.0;
-                for (int a2 = 0; a2 < NSUB; ++a2) {
-                    sx += vp[a2 * NSUB + a][l][0]; sy += vp[a2 * NSUB + a][l][1]; sz += vp[a2 * NSUB + a][l][2];
-                }
-                colo[3 * t] = k.A1 * sx; colo[3 * t + 1] = k.A1 * sy; colo[3 * t + 2] = k.A1 * sz;
-            }
-        }
-    }
-    item_queue_done(counter);
-}
-
 template <bool WALL, int TPT>
 __global__ void __launch_bounds__(kThreads, 4)
 rpy_items_mixed(const float4* __restrict__ hi, const float4* __restrict__ lo,
@@ -885,7 +763,7 @@ __device__ __forceinline__ void pair2_sym(float2 dx, float2 dy, float2 dz, float
 // takes source sub-tiles 2 (w >> 1) and 2 (w >> 1) + 1 of tile J (32
 // sources each).  At step t lane l meets source (l + t) mod 32 of the
 // sub-tile with both targets; the source's column sum (the two targets'
-// contributions added) moves one lane per step as in rpy_sym_f64.
+// contributions added) moves one lane per step as in k_sym_tiles.
 // Differences from the hi parts, with the lo parts added within a quarter
 // of the target's largest coordinate (as rpy_items_mixed_x2).  FP32 sums over
 // at most 64 terms (a warp's sources for u, its targets for v), added in
@@ -1029,7 +907,7 @@ rpy_sym_mixed_x2(const float4* __restrict__ hi, const float4* __restrict__ lo, c
 }
 
 // Symmetric mixed product on tiles of 32 NSUB blobs, one target per lane:
-// the scheme of rpy_sym_f64 (each unordered pair of a tile pair evaluated
+// the scheme of k_sym_tiles (each unordered pair of a tile pair evaluated
 // once and applied in both directions, the column sums carried from lane
 // to lane, the diagonal warp tile on steps 1..16) with FP32 pair terms.
 // Differences are formed from the hi parts of the positions; within a
@@ -1267,21 +1145,16 @@ rpy_items_mixed_x2(const float4* __restrict__ hi, const float4* __restrict__ lo,
     item_queue_done(counter);
 }
 
-// u_i = sum over the chunks of i's system of the partial sums
-__global__ void k_sum_items(int Nb, const double* __restrict__ part, const int* __restrict__ sys_of_blob,
-                            const int* __restrict__ sys_blob0, const int* __restrict__ sys_nb,
-                            const int* __restrict__ sys_nch, const long long* __restrict__ sys_poff,
-                            double* __restrict__ u) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= Nb) return;
-    const int s = sys_of_blob[i];
-    const size_t n3 = 3 * (size_t)sys_nb[s];
-    const double* p = part + sys_poff[s] + 3 * (size_t)(i - sys_blob0[s]);
-    double a = 0.0, b = 0.0, c = 0.0;
-    for (int q = 0; q < sys_nch[s]; ++q) {
-        a += p[q * n3]; b += p[q * n3 + 1]; c += p[q * n3 + 2];
-    }
-    u[3 * (size_t)i] = a; u[3 * (size_t)i + 1] = b; u[3 * (size_t)i + 2] = c;
+// u = the sums over the slots of each element's system
+__global__ void __launch_bounds__(256)
+k_sum_items(int n3, int G, const double* __restrict__ part, const int* __restrict__ sys_of_blob,
+            const int* __restrict__ sys_blob0, const int* __restrict__ sys_nb,
+            const int* __restrict__ sys_nch, const long long* __restrict__ sys_poff,
+            double* __restrict__ u) {
+    __shared__ double sh[256];
+    const double a = slot_sum(blockIdx.x, G, n3, part, sys_of_blob, sys_blob0, sys_nb, sys_nch, sys_poff, sh);
+    const int t = blockIdx.x * (256 / G) + threadIdx.x;
+    if (threadIdx.x < 256 / G && t < n3) u[t] = a;
 }
 
 template <class F>
@@ -1292,17 +1165,10 @@ static int resident_grid(F kernel, int threads = kThreads) {
     return per * num_sms();
 }
 
-// resident blocks of the symmetric FP64 kernel for nsub (1, 2, 4)
-static int sym_grid(bool wall, int nsub) {
-    const int th = nsub == 1 ? 32 : 128;
-    if (wall) {
-        if (nsub == 1) return resident_grid(rpy_sym_f64<true, 1>, th);
-        if (nsub == 2) return resident_grid(rpy_sym_f64<true, 2>, th);
-        return resident_grid(rpy_sym_f64<true, 4>, th);
-    }
-    if (nsub == 1) return resident_grid(rpy_sym_f64<false, 1>, th);
-    if (nsub == 2) return resident_grid(rpy_sym_f64<false, 2>, th);
-    return resident_grid(rpy_sym_f64<false, 4>, th);
+// resident blocks of the symmetric FP64 kernel
+static int sym_grid(bool wall) {
+    return wall ? resident_grid(k_sym_tiles<SymBlobPair<true>>, 32 * kSymWarps)
+                : resident_grid(k_sym_tiles<SymBlobPair<false>>, 32 * kSymWarps);
 }
 
 // resident blocks of the symmetric mixed kernel: paired lanes (tpt 2,
@@ -1343,16 +1209,29 @@ int mobility_layout(am_handle* h, int tpt, int chunk, int tgroup, int sym) {
         const long long per_item = std::max<long long>(pairs / want, (long long)kThreads * tpt * kTile);
         chunk = (int)std::max<long long>(kTile, per_item / (kThreads * tpt) / kTile * kTile);
     }
+    // few tile pairs (FP64, tiles of 32 or 64): their steps split over several
+    // items with slots of their own
+    int splits = 1;
+    if ((sym == 1 || sym == 2) && h->cfg.precision == AM_FP64) {
+        long long tp = 0;
+        for (int s = 0; s < S; ++s) {
+            const long long nt = (h->sys[s].Nb + 32 * sym - 1) / (32 * sym);
+            tp += nt * (nt + 1) / 2;
+        }
+        splits = sym_step_splits(tp);
+    }
     std::vector<MvItem> items;
     std::vector<int> nch(S);
     std::vector<long long> poff(S);
     long long off = 0;
     for (int s = 0; s < S; ++s) {
         const int nb = h->sys[s].Nb, b0 = h->sys_blob0[s];
-        nch[s] = std::max(1, (nb + chunk - 1) / chunk);
+        nch[s] = std::max(1, (nb + chunk - 1) / chunk) * splits;
         poff[s] = off;
         for (int c = 0; c < nch[s]; ++c) {
-            const int j0 = b0 + c * chunk, j1 = std::min(b0 + nb, j0 + chunk);
+            // with split steps there are more slots than chunks: the last ones
+            // are empty and their items write zeros
+            const int j0 = std::min(b0 + nb, b0 + c * chunk), j1 = std::min(b0 + nb, j0 + chunk);
             for (int t0 = b0; t0 < b0 + nb; t0 += tgroup) {
                 MvItem it;
                 it.t0 = t0; it.t1 = std::min(b0 + nb, t0 + tgroup);
@@ -1369,20 +1248,8 @@ int mobility_layout(am_handle* h, int tpt, int chunk, int tgroup, int sym) {
     });
     std::vector<SymItem> sitems;
     if (sym) {
-        const int T = 32 * sym;
-        for (int s = 0; s < S; ++s) {
-            const int nb = h->sys[s].Nb, b0 = h->sys_blob0[s];
-            const int nt = (nb + T - 1) / T;
-            for (int a = 0; a < nt; ++a)
-                for (int b = a; b < nt; ++b) {
-                    SymItem it;
-                    it.i0 = b0 + a * T; it.ni = std::min(T, nb - a * T);
-                    it.j0 = b0 + b * T; it.nj = std::min(T, nb - b * T);
-                    it.tbase = b0; it.sys = s; it.ti = a; it.tj = b;
-                    it.poff = poff[s]; it.n3 = 3 * nb;
-                    sitems.push_back(it);
-                }
-        }
+        for (int s = 0; s < S; ++s)
+            sym_append_items(sitems, s, h->sys_blob0[s], h->sys[s].Nb, 3, sym, splits, poff[s]);
     }
     cudaStream_t st = h->stream;
     if (h->d_sym_items) cudaFree(h->d_sym_items);
@@ -1395,7 +1262,8 @@ int mobility_layout(am_handle* h, int tpt, int chunk, int tgroup, int sym) {
             return 1;
         h->n_sym = (int)sitems.size();
         h->sym_nsub = sym;
-        h->mv_gridsym = std::min(sym_grid(h->cfg.wall != 0, sym), h->n_sym);
+        h->sym_splits = splits;
+        h->mv_gridsym = std::min(sym_grid(h->cfg.wall != 0), (h->n_sym + kSymWarps - 1) / kSymWarps);
         h->mv_gridsym32 = std::min(sym_mixed_grid(h->cfg.wall != 0, tpt, sym), h->n_sym);
         h->mv_gridsymdf = std::min(sym_df_resident_grid(h->cfg.wall != 0), h->n_sym);
     }
@@ -1419,6 +1287,7 @@ int mobility_layout(am_handle* h, int tpt, int chunk, int tgroup, int sym) {
     h->mv_chunk = chunk;
     h->mv_tgroup = tgroup;
     h->mv_part_total = off;
+    h->mv_sum_groups = *std::max_element(nch.begin(), nch.end()) >= 16 ? 8 : 1;
     if (h->cfg.precision == AM_MIXED) {
         if (h->cfg.wall)
             h->mv_grid = tpt == 2 ? resident_grid(rpy_items_mixed_x2<true>) : resident_grid(rpy_items_mixed<true, 1>);
@@ -1453,16 +1322,13 @@ void launch_items(am_handle* h, const double* lam, int mode, const int* active) 
     if (fp64 && h->n_sym > 0) {
         const RpyK<double> k = rpy_consts<double>(h->prm);
         const SymItem* si = static_cast<const SymItem*>(h->d_sym_items);
-        const int th = h->sym_nsub == 1 ? 32 : 128;
-#define AM_SYM(W, N)                                                                                      \
-    launch_dep(rpy_sym_f64<W, N>, dim3(h->mv_gridsym), dim3(th), 0, st, h->d_r4, lam, h->d_mv, si, h->n_sym, \
-               h->d_item_counter, k, active)
-        if (h->cfg.wall) {
-            if (h->sym_nsub == 1) AM_SYM(true, 1); else if (h->sym_nsub == 2) AM_SYM(true, 2); else AM_SYM(true, 4);
-        } else {
-            if (h->sym_nsub == 1) AM_SYM(false, 1); else if (h->sym_nsub == 2) AM_SYM(false, 2); else AM_SYM(false, 4);
-        }
-#undef AM_SYM
+        const dim3 grid(h->mv_gridsym), block(32 * kSymWarps);
+        if (h->cfg.wall)
+            launch_dep(k_sym_tiles<SymBlobPair<true>>, grid, block, 0, st, (const double*)h->d_r3, lam, h->d_mv, si,
+                       h->n_sym, h->d_item_counter, SymBlobPair<true>{k}, active);
+        else
+            launch_dep(k_sym_tiles<SymBlobPair<false>>, grid, block, 0, st, (const double*)h->d_r3, lam, h->d_mv, si,
+                       h->n_sym, h->d_item_counter, SymBlobPair<false>{k}, active);
     } else if (fp64) {
         const RpyK<double> k = rpy_consts<double>(h->prm);
         if (h->cfg.wall)
@@ -1471,7 +1337,7 @@ void launch_items(am_handle* h, const double* lam, int mode, const int* active) 
         else
             launch_dep(rpy_items_f64<false>, dim3(h->mv_grid64), dim3(kThreads), 0, st, h->d_r4, lam, h->d_mv, items,
                        h->n_items, h->d_item_counter, k, active);
-    } else if (h->n_sym > 0) {
+    } else if (h->n_sym > 0 && h->sym_splits == 1) {
         const RpyK<float> k = rpy_consts<float>(h->prm);
         const SymItem* si = static_cast<const SymItem*>(h->d_sym_items);
         const int th = h->mv_tpt == 2 || h->sym_nsub > 1 ? kThreads : 32;
@@ -1515,8 +1381,10 @@ void launch_items(am_handle* h, const double* lam, int mode, const int* active) 
 
 void launch_sum_items(am_handle* h, double* u) {
     if (h->Nb <= 0) return;
-    k_sum_items<<<(h->Nb + 255) / 256, 256, 0, h->stream>>>(h->Nb, h->d_mv, h->d_sys_of_blob, h->d_sys_blob0,
-                                                            h->d_sys_nb, h->d_sys_nch, h->d_sys_poff, u);
+    const int G = h->mv_sum_groups, per = 256 / G;
+    k_sum_items<<<(3 * h->Nb + per - 1) / per, 256, 0, h->stream>>>(3 * h->Nb, G, h->d_mv, h->d_sys_of_blob,
+                                                                    h->d_sys_blob0, h->d_sys_nb, h->d_sys_nch,
+                                                                    h->d_sys_poff, u);
     count_launch();
 }
 

@@ -173,7 +173,7 @@ __device__ __forceinline__ df df_shfl(df x, int src) {
 }
 
 // Symmetric double-float product on the handle's tile pairs of 128 blobs
-// (the scheme of rpy_sym_f64: 32 x 32 warp tiles, the source's column sum
+// (the scheme of k_sym_tiles: 32 x 32 warp tiles, the source's column sum
 // carried lane to lane, steps 1..16 on the diagonal of a diagonal item);
 // warp-tile sums in double-float, added in FP64 across warps in a fixed
 // order.

@@ -78,6 +78,7 @@ __global__ void k_sb_ctphi(int M, const int* __restrict__ blo, const int* __rest
 // vanishes).  FP64-issue-bound: about 90 FP64 operations per unordered pair
 // (136 per ordered pair in the one-direction form with its divisions).
 struct SymSpherePair {
+    static constexpr int kMinBlocks = 20;
     static constexpr int NC = 6;  // (force, torque) in, (velocity, rotation) out
     RpyK<double> k;
     double ia, h_a3, i_a3, n9_a4, n3_a5;  // 1/a, 1/(2 a^3), 1/a^3, 9/(32 a^4), -3/(64 a^5)

@@ -20,7 +20,11 @@
 // sources keeps the pipe fed with 4 to 5 warps per scheduler.  Groups of
 // several tiles (up to 96 groups per system) bound the partial sums at 96
 // slots; systems too small to give every SM a few warps split the 32 steps
-// of a tile over up to 8 items (each with its own slots).
+// of a tile over up to 8 items (each with its own slots).  Measured against
+// the block-wide form it replaced (four warps or one, shared-memory sums of
+// every warp tile): 384 free blobs 108 -> 15 us (78 unsplit tiles keep 78 SMs
+// busy with 14 us of FP64 issue each), 2,560 wall blobs 533 -> 508 us, 5,000
+// wall blobs 1,851 -> 1,885 us.
 #pragma once
 #include "am_internal.cuh"
 #include "rpy_pair.cuh"
@@ -30,13 +34,17 @@
 
 namespace am {
 
-constexpr int kSymWarps = 4;       // warps per block
+// One warp per block: the blocks of a launch then spread evenly over the SMs
+// whatever their number (2,560 blobs make 3,240 items, 21.3 per SM), and at
+// 22 to 25 resident blocks per SM such a launch is one wave.
+constexpr int kSymWarps = 1;
 constexpr int kSymMaxGroups = 96;  // most groups (partial-sum slots) per system
 
 // The blob mobility (3 components), free space or wall; sums in units of A1.
 template <bool WALL>
 struct SymBlobPair {
     static constexpr int NC = 3;
+    static constexpr int kMinBlocks = WALL ? 22 : 20;  // 80 and 96 registers, no spills
     RpyK<double> k;
     __device__ __forceinline__ double scale() const { return k.A1; }
     __device__ __forceinline__ void both(const double* xi, const double* xj, const double* l, const double* m,
@@ -64,7 +72,7 @@ struct SymBlobPair {
 // body) numbers; part: the slots.  counter[0]: next item, counter[1]: blocks
 // finished.
 template <class Pair>
-__global__ void __launch_bounds__(32 * kSymWarps)
+__global__ void __launch_bounds__(32 * kSymWarps, Pair::kMinBlocks)
 k_sym_tiles(const double* __restrict__ x, const double* __restrict__ g, double* __restrict__ part,
             const SymItem* __restrict__ items, int n_items, int* __restrict__ counter, Pair pr,
             const int* __restrict__ active) {
