@@ -330,8 +330,11 @@ AM_API int am_apply_precond(am_handle* h, const double* r, double* z);
  *   d_lambda   3n doubles, blob forces
  *   d_u        3n doubles, output velocities (overwritten)
  *   precision  AM_FP64 or AM_MIXED
- *   d_work     scratch of at least am_rpy_matvec_workspace(n, precision)
- *              bytes, 256-byte aligned; contents are overwritten
+ *   d_work     scratch of am_rpy_matvec_workspace(n, precision) bytes,
+ *              256-byte aligned; contents are overwritten.  At least
+ *              am_rpy_matvec_rows_workspace(n, n, precision) bytes are
+ *              needed; with less than the former an FP64 product takes a
+ *              slower form without its partial sums
  *   stream     cudaStream_t or NULL (legacy default stream)
  * Asynchronous on `stream`.  Errors: AM_ERR_ARG (n < 0, eta or a <= 0, NULL
  * pointer with n > 0, workspace too small or misaligned), AM_ERR_CUDA. */
@@ -364,7 +367,7 @@ AM_API size_t am_rpy_matvec_rows_workspace(int n, int nrows, int precision);
  * am_rpy_matvec); the scratch lives in a fixed device array of
  * AM_NOALLOC_SCRATCH_BYTES inside the library, which every GPU that loads
  * the library holds until the process exits.
- *  - Limit: n must satisfy am_rpy_matvec_workspace(n, precision) <=
+ *  - Limit: n must satisfy am_rpy_matvec_rows_workspace(n, n, precision) <=
  *    AM_NOALLOC_SCRATCH_BYTES, evaluated with the device of the call
  *    current (the source split, and with it the scratch, depends on the
  *    SM count); on a 152-SM GB300 that is n <= about 150,000 blobs for

@@ -33,29 +33,14 @@ struct RpyParams {
 };
 RpyParams make_params(double eta, double a);
 
-// Source splitting of the all-pairs product: grid (target blocks, splits).
-struct Split { int splits; int chunk; int tpt; };
-Split choose_split(int n, int precision);
-Split choose_split_rows(int n, int nt, int precision);
-
-// ---- mobility product launchers (rpy.cu) ------------------------------
-// FP64: r4 = (x, y, z, 0) per blob.  Mixed: hi/lo float4 positions.
-// Writes partial sums part[s][3n] for s < splits.
-void launch_rpy_partial_f64_rows(const double4_32a* r4, const double* lam, double* part, int n, int t0, int nt,
-                                 const Split& sp, const RpyParams& prm, int wall, cudaStream_t st);
-void launch_rpy_partial_mixed_rows(const float4* hi, const float4* lo, const double* lam, double* part, int n,
-                                   int t0, int nt, const Split& sp, const RpyParams& prm, int wall,
-                                   cudaStream_t st);
-void launch_rpy_partial_f64(const double4_32a* r4, const double* lam, double* part,
-                            int n, const Split& sp, const RpyParams& prm, int wall,
-                            cudaStream_t st);
-void launch_rpy_partial_mixed(const float4* hi, const float4* lo, const double* lam,
-                              double* part, int n, const Split& sp,
-                              const RpyParams& prm, int wall, cudaStream_t st);
-void launch_pack_positions(const double* r3, double4_32a* r4, float4* hi, float4* lo,
-                           int n, cudaStream_t st);
-void launch_sum_partials(const double* part, double* u, int n, int splits,
-                         cudaStream_t st);
+// ---- stateless mobility products (rpy.cu) ------------------------------
+// Least scratch of a product of nt targets against n sources, and the scratch
+// of the whole product that lets it take its fastest form.
+size_t least_workspace(int n, int nt, int precision);
+size_t product_workspace(int n, int precision);
+// u = rows t0 .. t0 + nt - 1 of M(r) lambda, device pointers, on `st`.
+cudaError_t product(const double* r, const double* lam, double* u, int n, int t0, int nt, double eta, double a,
+                    int wall, int precision, void* work, size_t bytes, cudaStream_t st);
 
 // Control block of a device-side Arnoldi cycle.
 struct ArnoldiCtrl {
@@ -222,6 +207,8 @@ struct am_handle {
     int* d_item_counter = nullptr;
     int mv_tpt = 1, mv_chunk = 0, mv_tgroup = 0, mv_grid = 0, mv_grid64 = 0, mv_griddf = 0;
     long long mv_part_total = 0;
+    float4* d_lf = nullptr;  // forces as floats (paired-lane symmetric product)
+    bool mv_pairs = false;   // the slots of the last product hold float pairs
     int mv_sum_groups = 1;  // threads per element in the sum over slots (slot_sum)
     bool mv_tuned = false;
     // tile-pair items of the symmetric FP64 product (tiles of 32 sym_nsub blobs)
@@ -304,7 +291,6 @@ struct am_handle {
     am::PeriodicPlan* per = nullptr;
     long long per_nnz = 0;
     int per_status = 0;
-    am::Split split{1, 0, 1};
 
     // device: step
     double *d_qnew = nullptr, *d_thnew = nullptr, *d_corr = nullptr, *d_red = nullptr;

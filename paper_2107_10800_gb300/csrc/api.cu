@@ -137,7 +137,7 @@ void free_bodies(am_handle* h) {
     dfree(&h->d_asm_body_off); dfree(&h->d_asm_body_idx); dfree(&h->d_body_local);
     dfree(&h->d_r4); dfree(&h->d_d4); dfree(&h->d_rhi); dfree(&h->d_rlo); dfree(&h->d_r3);
     dfree(&h->d_minv); dfree(&h->d_pcwork); dfree(&h->d_Y); dfree(&h->d_Nt); dfree(&h->d_minv_off);
-    dfree(&h->d_pc_w); dfree(&h->d_pc_Uhat); dfree(&h->d_mv);
+    dfree(&h->d_pc_w); dfree(&h->d_pc_Uhat); dfree(&h->d_mv); dfree(&h->d_lf);
     dfree(&h->d_pcw_body); dfree(&h->d_pcw_chunk); dfree(&h->d_pcw_off); dfree(&h->d_ytp); dfree(&h->d_pcb_cnt);
     dfree(&h->d_pcb_list);
     h->n_pcb_small = 0;

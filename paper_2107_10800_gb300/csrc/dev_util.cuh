@@ -25,6 +25,15 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
     return sh[32];
 }
 
+// hi + lo += t with Knuth's TwoSum (rounding error of hi + t kept in lo):
+// the compensated accumulation of the mixed kernels' sums
+__device__ __forceinline__ void two_sum_acc(float& hi, float& lo, float t) {
+    const float s = __fadd_rn(hi, t);
+    const float v = __fsub_rn(s, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, v)), __fsub_rn(t, v)));
+    hi = s;
+}
+
 // Arrival count of the blocks that share a reduction: every block that has
 // written its partial results calls it (all threads); true in every thread
 // of the block that completes cnt[idx] = total, which then reads the
@@ -45,14 +54,36 @@ __device__ __forceinline__ bool arrive_last(int* cnt, int idx, int total) {
     return last;
 }
 
+// The sum of slots q, q + G, .. of one element (p: its value in slot 0, n
+// values per slot).  pairs: a slot value is a compensated (hi, lo) pair of
+// floats; they are added as such (a conversion is FP64 work).
+__device__ __forceinline__ double slot_run(const double* __restrict__ p, size_t n, int q, int ns, int G, bool pairs) {
+    if (pairs) {
+        const float2* f = reinterpret_cast<const float2*>(p);
+        float h = 0.f, l = 0.f;
+#pragma unroll 4
+        for (int c = q; c < ns; c += G) {
+            const float2 v = f[c * n];
+            two_sum_acc(h, l, v.x);
+            l += v.y;
+        }
+        return (double)h + (double)l;
+    }
+    double a = 0.0;
+#pragma unroll 4
+    for (int c = q; c < ns; c += G) a += p[c * n];
+    return a;
+}
+
 // Element of u = M lambda from the partial sums, in a block of 256 threads for
 // 256 / G elements: G threads add the slots of an element's system (thread g
 // of them every G-th slot, then the G sums in order; the result is valid in
 // threads 0 .. 256 / G - 1, whose element is blk 256 / G + threadIdx.x).  G = 8
 // for many slots (consecutive threads still read consecutive doubles, and the
-// chain of dependent additions is an eighth of the slots), else 1.  Every
-// thread calls it; sh: 256 doubles.
-__device__ __forceinline__ double slot_sum(int blk, int G, int n3, const double* __restrict__ part,
+// chain of dependent additions is an eighth of the slots), else 1.  scale !=
+// 0: the slots hold float pairs in units of it.  Every thread calls it; sh:
+// 256 doubles.
+__device__ __forceinline__ double slot_sum(int blk, int G, double scale, int n3, const double* __restrict__ part,
                                            const int* __restrict__ sys_of_blob, const int* __restrict__ sys_blob0,
                                            const int* __restrict__ sys_nb, const int* __restrict__ sys_nch,
                                            const long long* __restrict__ sys_poff, double* sh) {
@@ -63,9 +94,7 @@ __device__ __forceinline__ double slot_sum(int blk, int G, int n3, const double*
         const int s = sys_of_blob[t / 3];
         const size_t n = 3 * (size_t)sys_nb[s];
         const double* p = part + sys_poff[s] + (t - 3 * (size_t)sys_blob0[s]);
-        const int ns = sys_nch[s];
-#pragma unroll 4
-        for (int c = q; c < ns; c += G) a += p[c * n];
+        a = slot_run(p, n, q, sys_nch[s], G, scale != 0.0);
     }
     if (G > 1) {
         sh[threadIdx.x] = a;
@@ -73,6 +102,7 @@ __device__ __forceinline__ double slot_sum(int blk, int G, int n3, const double*
         if (q == 0)
             for (int c = 1; c < G; ++c) a += sh[c * per + threadIdx.x];
     }
+    if (scale != 0.0) a *= scale;
     return a;
 }
 

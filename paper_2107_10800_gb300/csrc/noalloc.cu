@@ -1,7 +1,7 @@
 // am_rpy_matvec_noalloc: the blob mobility product for callers that cannot
-// allocate device memory.  Same kernels and source split as am_rpy_matvec;
-// the scratch (packed positions and per-chunk partial sums) is a fixed
-// device array of this file instead of a caller workspace.
+// allocate device memory.  The same product as am_rpy_matvec with a fixed
+// device array of this file as its scratch: the symmetric product where its
+// partial sums fit in it, else the cluster product, which needs none.
 #include "am_internal.cuh"
 
 #include <string>
@@ -19,8 +19,6 @@ int fail(int code, const std::string& msg) {
     am::set_thread_error(msg);
     return code;
 }
-
-size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
 
 // Device address of the scratch array on the current device.  The host-side
 // name of a __device__ array is not a device address, so it is looked up with
@@ -48,7 +46,7 @@ extern "C" AM_API int am_rpy_matvec_noalloc(const double* d_r, const double* d_l
         return fail(AM_ERR_ARG, "am_rpy_matvec_noalloc: unknown precision");
     if (n == 0) return AM_OK;
     if (!d_r || !d_lambda || !d_u) return fail(AM_ERR_ARG, "am_rpy_matvec_noalloc: NULL pointer");
-    const size_t need = am_rpy_matvec_workspace(n, precision);
+    const size_t need = am::least_workspace(n, n, precision);
     if (need > AM_NOALLOC_SCRATCH_BYTES)
         return fail(AM_ERR_ARG, "am_rpy_matvec_noalloc: n = " + std::to_string(n) + " needs " +
                                     std::to_string(need) + " bytes of scratch, more than the " +
@@ -57,25 +55,8 @@ extern "C" AM_API int am_rpy_matvec_noalloc(const double* d_r, const double* d_l
     void* base = nullptr;
     int rc = scratch_address(&base);
     if (rc) return rc;
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    am::Split sp = am::choose_split(n, precision);
-    am::RpyParams prm = am::make_params(eta, a);
-    char* w = static_cast<char*>(base);
-    if (precision == AM_MIXED) {
-        float4* hi = reinterpret_cast<float4*>(w);
-        float4* lo = reinterpret_cast<float4*>(w + align256((size_t)n * sizeof(float4)));
-        double* part = reinterpret_cast<double*>(w + 2 * align256((size_t)n * sizeof(float4)));
-        am::launch_pack_positions(d_r, nullptr, hi, lo, n, st);
-        am::launch_rpy_partial_mixed(hi, lo, d_lambda, part, n, sp, prm, wall, st);
-        am::launch_sum_partials(part, d_u, n, sp.splits, st);
-    } else {
-        double4_32a* r4 = reinterpret_cast<double4_32a*>(w);
-        double* part = reinterpret_cast<double*>(w + align256((size_t)n * sizeof(double4_32a)));
-        am::launch_pack_positions(d_r, r4, nullptr, nullptr, n, st);
-        am::launch_rpy_partial_f64(r4, d_lambda, part, n, sp, prm, wall, st);
-        am::launch_sum_partials(part, d_u, n, sp.splits, st);
-    }
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = am::product(d_r, d_lambda, d_u, n, 0, n, eta, a, wall, precision, base,
+                                      AM_NOALLOC_SCRATCH_BYTES, static_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return fail(AM_ERR_CUDA, cudaGetErrorString(e));
     return AM_OK;
 }

@@ -76,7 +76,7 @@ __global__ void k_rhs(int Nb, int M, int P, const double* __restrict__ slip,
 // out_U      = -K^T lambda + C^T phi
 // out_phi    = C U   (per link: u_p + omega_p x l_np - u_q - omega_q x l_nq)
 __global__ void __launch_bounds__(256)
-k_op_epilogue(int Nb, int M, int P, int nblob_blocks, int nbody_blocks, int G, int L, int bpb,
+k_op_epilogue(int Nb, int M, int P, int nblob_blocks, int nbody_blocks, int G, double scale, int L, int bpb,
                               const double* __restrict__ part, const int* __restrict__ sys_of_blob,
                               const int* __restrict__ sys_blob0, const int* __restrict__ sys_nb,
                               const int* __restrict__ sys_nch, const long long* __restrict__ sys_poff,
@@ -131,7 +131,7 @@ k_op_epilogue(int Nb, int M, int P, int nblob_blocks, int nbody_blocks, int G, i
     } else if (b < nbody_blocks + nblob_blocks) {  // 256 / G elements of lambda
         __shared__ double sh[256];
         const int blk = b - nbody_blocks;
-        const double s = slot_sum(blk, G, 3 * Nb, part, sys_of_blob, sys_blob0, sys_nb, sys_nch, sys_poff, sh);
+        const double s = slot_sum(blk, G, scale, 3 * Nb, part, sys_of_blob, sys_blob0, sys_nb, sys_nch, sys_poff, sh);
         const int t = blk * (256 / G) + threadIdx.x;
         if (threadIdx.x >= 256 / G || t >= 3 * Nb) return;
         const int i = t / 3, c = t - 3 * i;
@@ -956,8 +956,8 @@ void op_apply(am_handle* h, const double* y, double* out, int mode, const int* a
         while (L > 1 && 6LL * L * h->M > h->Nb && h->max_body_blobs <= 8 * L) L >>= 1;
     const int bpb = std::min(256 / L, nblk(h->M, num_sms()));
     const int nbb = nblk(3LL * h->Nb, 256 / G), nbody = nblk(h->M, bpb), nlink = nblk(h->P, 256);
-    launch_dep(k_op_epilogue, dim3(nbb + nbody + nlink), dim3(256), 0, h->stream, h->Nb, h->M, h->P, nbb, nbody, G, L,
-               bpb,
+    launch_dep(k_op_epilogue, dim3(nbb + nbody + nlink), dim3(256), 0, h->stream, h->Nb, h->M, h->P, nbb, nbody, G,
+               slot_scale(h), L, bpb,
                h->d_mv, h->d_sys_of_blob, h->d_sys_blob0, h->d_sys_nb, h->d_sys_nch, h->d_sys_poff, y, out,
                h->d_body_of_blob, h->d_blob_off, h->d_d4, h->d_body_link_off, h->d_body_link_idx, h->d_lp, h->d_lq,
                h->d_bp, h->d_bq);
@@ -1218,11 +1218,11 @@ static int gmres(am_handle* h, const double* rhs, double* x, double tol, bool fp
 // partials of the last mobility product (a warp whose elements share one
 // system adds once)
 __global__ void __launch_bounds__(256)
-k_sys_mob_norm2(int n3, int G, const double* __restrict__ part, const int* __restrict__ sys_of_blob,
+k_sys_mob_norm2(int n3, int G, double scale, const double* __restrict__ part, const int* __restrict__ sys_of_blob,
                 const int* __restrict__ sys_blob0, const int* __restrict__ sys_nb,
                 const int* __restrict__ sys_nch, const long long* __restrict__ sys_poff, double* __restrict__ m2) {
     __shared__ double sh[256];
-    const double u = slot_sum(blockIdx.x, G, n3, part, sys_of_blob, sys_blob0, sys_nb, sys_nch, sys_poff, sh);
+    const double u = slot_sum(blockIdx.x, G, scale, n3, part, sys_of_blob, sys_blob0, sys_nb, sys_nch, sys_poff, sh);
     if (threadIdx.x >= 256 / G) return;
     const int t = blockIdx.x * (256 / G) + threadIdx.x;
     const int s = t < n3 ? sys_of_blob[t / 3] : -1;
@@ -1336,8 +1336,8 @@ int solve(am_handle* h, am_step_stats* st) {
                 cudaMemsetAsync(m2, 0, h->S * sizeof(double), s);
                 const int G = h->mv_sum_groups;
                 k_sys_mob_norm2<<<nblk(3LL * h->Nb, 256 / G), 256, 0, s>>>(
-                    3 * h->Nb, G, h->d_mv, h->d_sys_of_blob, h->d_sys_blob0, h->d_sys_nb, h->d_sys_nch, h->d_sys_poff,
-                    m2);
+                    3 * h->Nb, G, slot_scale(h), h->d_mv, h->d_sys_of_blob, h->d_sys_blob0, h->d_sys_nb, h->d_sys_nch,
+                    h->d_sys_poff, m2);
                 k_sys_resid_bound<<<nblk(h->S, 128), 128, 0, s>>>(h->S, tol, kMixedProductError, bn_out,
                                                                   h->d_beta_s, m2, be_out);
                 cudaMemcpyAsync(h->d_rir, h->d_V, h->n * sizeof(double), cudaMemcpyDeviceToDevice, s);

@@ -49,6 +49,9 @@ int df_resident_grid(bool wall);
 int sym_df_resident_grid(bool wall);
 void launch_items_df(am_handle* h, const double* lam);
 void launch_sum_items(am_handle* h, double* u);
+// unit of the partial sums of the last product when its slots hold float
+// pairs (paired-lane mixed product), else 0 (doubles)
+inline double slot_scale(const am_handle* h) { return h->mv_pairs ? h->prm.inv8pieta : 0.0; }
 int mobility_autotune(am_handle* h);
 // Periodic box (periodic.cu): parameters and buffers for the handle's box,
 // tolerance and blob count; cell list and real-space pair blocks of the

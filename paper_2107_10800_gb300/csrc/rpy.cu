@@ -18,14 +18,15 @@
 // (derived from Blake's image system by applying (1 + a^2/6 lap_x)
 // (1 + a^2/6 lap_y), which is exact for blobs whose centres are above a).
 //
-// Layout: one thread per target blob, 128 targets per block; sources are
-// staged through shared memory 128 at a time; the sources are split into
-// `splits` contiguous chunks (grid.y) so that small systems still fill the
-// 152 SMs; each (target block, chunk) writes its partial sums, and a second
-// kernel adds the chunks.
+// Stateless products (am_rpy_matvec and its variants): clusters of few targets
+// without partial sums (rpy_small.cuh), or, for the whole FP64 product, each
+// unordered pair once in tiles (sym_tiles.cuh); `product` has the rule.  The
+// products of a handle: work items of one or several systems, below.
 #include "am_internal.cuh"
 #include "dev_util.cuh"
 #include "rpy_pair.cuh"
+#include "rpy_pair2.cuh"
+#include "rpy_small.cuh"
 #include "sym_tiles.cuh"
 #include "ops.cuh"
 
@@ -63,257 +64,40 @@ RpyParams make_params(double eta, double a) {
     return p;
 }
 
-Split choose_split(int n, int precision) { return choose_split_rows(n, n, precision); }
-
-// n sources, nt targets
-Split choose_split_rows(int n, int nt, int precision) {
-    Split s{1, std::max(n, 1), 1};
-    if (n <= 0 || nt <= 0) return s;
-    const int want = 4 * num_sms();  // blocks to fill the GPU
-    // two targets per thread once one source chunk already fills the GPU
-    if (precision == AM_MIXED && (nt + 2 * kThreads - 1) / (2 * kThreads) >= want) s.tpt = 2;
-    const int tiles = (n + kTile - 1) / kTile;
-    const int tblocks = (nt + kThreads * s.tpt - 1) / (kThreads * s.tpt);
-    const int splits = std::max(1, std::min(tiles, (want + tblocks - 1) / tblocks));
-    const int per = (tiles + splits - 1) / splits;  // tiles per chunk
-    s.chunk = per * kTile;
-    s.splits = (n + s.chunk - 1) / s.chunk;
-    return s;
-}
-
-template <bool WALL>
-__global__ void __launch_bounds__(kThreads)
-rpy_partial_f64(const double4_32a* __restrict__ r4, const double* __restrict__ lam,
-                double* __restrict__ part, int n, int chunk, RpyK<double> k, int t0, int nt) {
-    __shared__ double4_32a sr[kTile];
-    __shared__ double sl[3 * kTile];
-    // targets t0 .. t0 + nt - 1 against sources 0 .. n - 1
-    const int it = blockIdx.x * kThreads + threadIdx.x;
-    const int i = t0 + it;
-    const int j0 = blockIdx.y * chunk;
-    const int j1 = min(n, j0 + chunk);
-    double4_32a ri = (it < nt) ? r4[i] : make_double4_32a(0.0, 0.0, 1.0, 0.0);
-    const double nx3 = -ri.z;
-    double ux = 0.0, uy = 0.0, uz = 0.0;
-    for (int jt = j0; jt < j1; jt += kTile) {
-        const int cnt = min(kTile, j1 - jt);
-        __syncthreads();
-        if (threadIdx.x < cnt) {
-            double4_32a v = r4[jt + threadIdx.x];
-            v.w = 2.0 * v.z;  // twice the source height, for the wall term
-            sr[threadIdx.x] = v;
-        }
-        for (int q = threadIdx.x; q < 3 * cnt; q += kThreads) sl[q] = lam[3 * (size_t)jt + q];
-        __syncthreads();
-#pragma unroll 2
-        for (int q = 0; q < cnt; ++q) {
-            const double4_32a rj = sr[q];
-            const double lx = sl[3 * q], ly = sl[3 * q + 1], lz = sl[3 * q + 2];
-            const double dx = ri.x - rj.x, dy = ri.y - rj.y, dz = ri.z - rj.z;
-            if (WALL) {
-                const double rxy2 = fma(dx, dx, dy * dy);
-                pair_wall_r2<double>(dx, dy, dz, rxy2, fma(dz, dz, rxy2), ri.z + rj.z, rj.w, nx3, lx, ly, lz, k,
-                                     ux, uy, uz);
-            } else {
-                pair_free<double>(dx, dy, dz, lx, ly, lz, k, ux, uy, uz);
-            }
-        }
-    }
-    if (it < nt) {
-        double* o = part + (size_t)blockIdx.y * 3 * nt + 3 * (size_t)it;
-        o[0] = k.A1 * ux; o[1] = k.A1 * uy; o[2] = k.A1 * uz;
-    }
-}
-
-// sources per FP32 partial sum of the mixed kernels before it is added to
-// the tile's compensated (hi, lo) sums
-constexpr int kSumBlock = 16;
-
-// hi + lo += t with Knuth's TwoSum (rounding error of hi + t kept in lo):
-// the compensated accumulation of the tile sums of the mixed kernels
-__device__ __forceinline__ void two_sum_acc(float& hi, float& lo, float t) {
-    const float s = __fadd_rn(hi, t);
-    const float v = __fsub_rn(s, hi);
-    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, v)), __fsub_rn(t, v)));
-    hi = s;
-}
-
-// Positions as hi + lo float pairs (hi = float(x), lo = float(x - hi)).  A
-// pair's difference is first formed from hi alone; within a radius of a
-// quarter of the target's largest coordinate, where the rounding of hi
-// (1.2e-7 |x|) would exceed 5e-7 of the distance, the lo parts are added,
-// which keeps FP32 relative accuracy of nearby differences anywhere in the
-// domain.  Pair terms and the sum over one tile are FP32; tile sums are
-// folded into FP64.  TPT targets per thread share each shared-memory load.
-template <bool WALL, int TPT>
-__global__ void __launch_bounds__(kThreads, 4)
-rpy_partial_mixed(const float4* __restrict__ hi, const float4* __restrict__ lo,
-                  const double* __restrict__ lam, double* __restrict__ part, int n,
-                  int chunk, RpyK<float> k, int t0, int nt) {
-    __shared__ float4 sh[kTile];
-    __shared__ float4 so[kTile];
-    __shared__ float4 sl[kTile];
-    const int j0 = blockIdx.y * chunk;
-    const int j1 = min(n, j0 + chunk);
-    float4 hi_i[TPT], lo_i[TPT];
-    float near2[TPT];
-    double U[TPT][3];
-#pragma unroll
-    for (int t = 0; t < TPT; ++t) {
-        const int it = (blockIdx.x * TPT + t) * kThreads + threadIdx.x;
-        const int i = t0 + it;
-        hi_i[t] = (it < nt) ? hi[i] : make_float4(0.f, 0.f, 1.f, 0.f);
-        lo_i[t] = (it < nt) ? lo[i] : make_float4(0.f, 0.f, 0.f, 0.f);
-        const float nr = 0.25f * fmaxf(fabsf(hi_i[t].x), fmaxf(fabsf(hi_i[t].y), fabsf(hi_i[t].z)));
-        near2[t] = nr * nr;
-        U[t][0] = U[t][1] = U[t][2] = 0.0;
-    }
-    for (int jt = j0; jt < j1; jt += kTile) {
-        const int cnt = min(kTile, j1 - jt);
-        __syncthreads();
-        if (threadIdx.x < cnt) {
-            const int j = jt + threadIdx.x;
-            const float4 hj = hi[j];
-            sh[threadIdx.x] = make_float4(hj.x, hj.y, hj.z, 2.f * hj.z);  // .w: twice the height
-            so[threadIdx.x] = lo[j];
-            sl[threadIdx.x] = make_float4((float)lam[3 * (size_t)j], (float)lam[3 * (size_t)j + 1],
-                                          (float)lam[3 * (size_t)j + 2], 0.f);
-        }
-        __syncthreads();
-        // pair terms summed in FP32 over blocks of kSumBlock sources, each block
-        // added to the tile's (hi, lo) sums by TwoSum, the tile folded into FP64
-        float th[TPT][3], tl[TPT][3];
-#pragma unroll
-        for (int t = 0; t < TPT; ++t)
-            for (int c = 0; c < 3; ++c) th[t][c] = tl[t][c] = 0.f;
-        for (int q0 = 0; q0 < cnt; q0 += kSumBlock) {
-        const int qe = min(cnt, q0 + kSumBlock);
-        float u[TPT][3];
-#pragma unroll
-        for (int t = 0; t < TPT; ++t) u[t][0] = u[t][1] = u[t][2] = 0.f;
-#pragma unroll 2
-        for (int q = q0; q < qe; ++q) {
-            const float4 h = sh[q];
-            const float4 l = sl[q];
-#pragma unroll
-            for (int t = 0; t < TPT; ++t) {
-                float dx = hi_i[t].x - h.x, dy = hi_i[t].y - h.y, dz = hi_i[t].z - h.z;
-                float rxy2 = fmaf(dx, dx, dy * dy);
-                float r2 = fmaf(dz, dz, rxy2);
-                if (r2 < near2[t]) {
-                    const float4 o = so[q];
-                    dx += lo_i[t].x - o.x;
-                    dy += lo_i[t].y - o.y;
-                    dz += lo_i[t].z - o.z;
-                    rxy2 = fmaf(dx, dx, dy * dy);
-                    r2 = fmaf(dz, dz, rxy2);
-                }
-                if (WALL)
-                    pair_wall_r2<float>(dx, dy, dz, rxy2, r2, hi_i[t].z + h.z, h.w, -hi_i[t].z, l.x, l.y, l.z, k,
-                                        u[t][0], u[t][1], u[t][2]);
-                else
-                    pair_free_r2<float>(dx, dy, dz, r2, l.x, l.y, l.z, k, u[t][0], u[t][1], u[t][2]);
-            }
-        }
-#pragma unroll
-        for (int t = 0; t < TPT; ++t)
-            for (int c = 0; c < 3; ++c) two_sum_acc(th[t][c], tl[t][c], u[t][c]);
-        }
-#pragma unroll
-        for (int t = 0; t < TPT; ++t)
-            for (int c = 0; c < 3; ++c) U[t][c] += (double)th[t][c] + (double)tl[t][c];
-    }
-#pragma unroll
-    for (int t = 0; t < TPT; ++t) {
-        const int it = (blockIdx.x * TPT + t) * kThreads + threadIdx.x;
-        if (it < nt) {
-            double* o = part + (size_t)blockIdx.y * 3 * nt + 3 * (size_t)it;
-            o[0] = k.A1 * U[t][0]; o[1] = k.A1 * U[t][1]; o[2] = k.A1 * U[t][2];
-        }
-    }
-}
-
-__global__ void pack_positions(const double* __restrict__ r3, double4_32a* __restrict__ r4,
-                               float4* __restrict__ hi, float4* __restrict__ lo, int n) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
+// positions as hi + lo float pairs
+__global__ void k_pack_positions(const double* __restrict__ r3, float4* __restrict__ hi, float4* __restrict__ lo,
+                                 int n) {
+    dep_wait();
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    double x = r3[3 * (size_t)i], y = r3[3 * (size_t)i + 1], z = r3[3 * (size_t)i + 2];
-    if (r4) r4[i] = make_double4_32a(x, y, z, 0.0);
-    if (hi) {
-        float hx = (float)x, hy = (float)y, hz = (float)z;
-        hi[i] = make_float4(hx, hy, hz, 0.f);
-        lo[i] = make_float4((float)(x - hx), (float)(y - hy), (float)(z - hz), 0.f);
+    const double x = r3[3 * (size_t)i], y = r3[3 * (size_t)i + 1], z = r3[3 * (size_t)i + 2];
+    const float hx = (float)x, hy = (float)y, hz = (float)z;
+    hi[i] = make_float4(hx, hy, hz, 0.f);
+    lo[i] = make_float4((float)(x - hx), (float)(y - hy), (float)(z - hz), 0.f);
+}
+
+// forces as floats
+__global__ void k_pack_forces(const double* __restrict__ lam, float4* __restrict__ lf, int n) {
+    dep_wait();
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n)
+        lf[i] = make_float4((float)lam[3 * (size_t)i], (float)lam[3 * (size_t)i + 1], (float)lam[3 * (size_t)i + 2], 0.f);
+}
+
+// u = the sum of the slots, 32 elements a block (8 threads per element)
+__global__ void __launch_bounds__(256)
+k_sum_slots(const double* __restrict__ part, double* __restrict__ u, int n3, int slots) {
+    dep_wait();
+    __shared__ double sh[256];
+    const int q = threadIdx.x >> 5, t = blockIdx.x * 32 + (threadIdx.x & 31);
+    double a = 0.0;
+    if (t < n3) a = slot_run(part + t, n3, q, slots, 8, false);
+    sh[threadIdx.x] = a;
+    __syncthreads();
+    if (q == 0 && t < n3) {
+        for (int c = 1; c < 8; ++c) a += sh[32 * c + threadIdx.x];
+        u[t] = a;
     }
-}
-
-__global__ void sum_partials(const double* __restrict__ part, double* __restrict__ u,
-                             int n3, int splits) {
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n3) return;
-    double s = 0.0;
-    for (int t = 0; t < splits; ++t) s += part[(size_t)t * n3 + k];
-    u[k] = s;
-}
-
-
-// Targets t0 .. t0 + nt - 1 against all n sources; partial sums of split c
-// at part[c * 3 nt + 3 (i - t0)].
-void launch_rpy_partial_f64_rows(const double4_32a* r4, const double* lam, double* part, int n, int t0, int nt,
-                                 const Split& sp, const RpyParams& prm, int wall, cudaStream_t st) {
-    if (n <= 0 || nt <= 0) return;
-    dim3 grid((nt + kThreads - 1) / kThreads, sp.splits);
-    const RpyK<double> k = rpy_consts<double>(prm);
-    if (wall)
-        rpy_partial_f64<true><<<grid, kThreads, 0, st>>>(r4, lam, part, n, sp.chunk, k, t0, nt);
-    else
-        rpy_partial_f64<false><<<grid, kThreads, 0, st>>>(r4, lam, part, n, sp.chunk, k, t0, nt);
-    count_launch();
-}
-
-void launch_rpy_partial_mixed_rows(const float4* hi, const float4* lo, const double* lam, double* part, int n,
-                                   int t0, int nt, const Split& sp, const RpyParams& prm, int wall,
-                                   cudaStream_t st) {
-    if (n <= 0 || nt <= 0) return;
-    const RpyK<float> k = rpy_consts<float>(prm);
-    const int per = kThreads * sp.tpt;
-    dim3 grid((nt + per - 1) / per, sp.splits);
-    if (sp.tpt == 2) {
-        if (wall)
-            rpy_partial_mixed<true, 2><<<grid, kThreads, 0, st>>>(hi, lo, lam, part, n, sp.chunk, k, t0, nt);
-        else
-            rpy_partial_mixed<false, 2><<<grid, kThreads, 0, st>>>(hi, lo, lam, part, n, sp.chunk, k, t0, nt);
-    } else {
-        if (wall)
-            rpy_partial_mixed<true, 1><<<grid, kThreads, 0, st>>>(hi, lo, lam, part, n, sp.chunk, k, t0, nt);
-        else
-            rpy_partial_mixed<false, 1><<<grid, kThreads, 0, st>>>(hi, lo, lam, part, n, sp.chunk, k, t0, nt);
-    }
-    count_launch();
-}
-
-void launch_rpy_partial_f64(const double4_32a* r4, const double* lam, double* part, int n,
-                            const Split& sp, const RpyParams& prm, int wall, cudaStream_t st) {
-    launch_rpy_partial_f64_rows(r4, lam, part, n, 0, n, sp, prm, wall, st);
-}
-
-void launch_rpy_partial_mixed(const float4* hi, const float4* lo, const double* lam, double* part,
-                              int n, const Split& sp, const RpyParams& prm, int wall,
-                              cudaStream_t st) {
-    launch_rpy_partial_mixed_rows(hi, lo, lam, part, n, 0, n, sp, prm, wall, st);
-}
-
-void launch_pack_positions(const double* r3, double4_32a* r4, float4* hi, float4* lo, int n,
-                           cudaStream_t st) {
-    if (n <= 0) return;
-    pack_positions<<<(n + 255) / 256, 256, 0, st>>>(r3, r4, hi, lo, n);
-    count_launch();
-}
-
-void launch_sum_partials(const double* part, double* u, int n, int splits, cudaStream_t st) {
-    if (n <= 0) return;
-    int n3 = 3 * n;
-    sum_partials<<<(n3 + 255) / 256, 256, 0, st>>>(part, u, n3, splits);
-    count_launch();
 }
 
 }  // namespace am
@@ -325,7 +109,6 @@ int fail(int code, const char* msg) {
     t_err = msg;
     return code;
 }
-size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
 }  // namespace
 
 namespace am {
@@ -334,11 +117,7 @@ void set_thread_error(const std::string& msg) { t_err = msg; }
 }
 
 extern "C" AM_API size_t am_rpy_matvec_workspace(int n, int precision) {
-    if (n <= 0) return 0;
-    am::Split sp = am::choose_split(n, precision);
-    size_t pos = (precision == AM_MIXED) ? 2 * align256((size_t)n * sizeof(float4))
-                                         : align256((size_t)n * sizeof(double4_32a));
-    return pos + align256((size_t)sp.splits * 3 * n * sizeof(double));
+    return n > 0 ? am::product_workspace(n, precision) : 0;
 }
 
 extern "C" AM_API int am_rpy_matvec(const double* d_r, const double* d_lambda, double* d_u, int n,
@@ -351,39 +130,18 @@ extern "C" AM_API int am_rpy_matvec(const double* d_r, const double* d_lambda, d
         return fail(AM_ERR_ARG, "am_rpy_matvec: unknown precision");
     if (n == 0) return AM_OK;
     if (!d_r || !d_lambda || !d_u || !d_work) return fail(AM_ERR_ARG, "am_rpy_matvec: NULL pointer");
-    if (work_bytes < am_rpy_matvec_workspace(n, precision))
+    if (work_bytes < am::least_workspace(n, n, precision))
         return fail(AM_ERR_ARG, "am_rpy_matvec: workspace too small");
     if (reinterpret_cast<uintptr_t>(d_work) % 256 != 0)
         return fail(AM_ERR_ARG, "am_rpy_matvec: workspace not 256-byte aligned");
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    am::Split sp = am::choose_split(n, precision);
-    am::RpyParams prm = am::make_params(eta, a);
-    char* w = static_cast<char*>(d_work);
-    if (precision == AM_MIXED) {
-        float4* hi = reinterpret_cast<float4*>(w);
-        float4* lo = reinterpret_cast<float4*>(w + align256((size_t)n * sizeof(float4)));
-        double* part = reinterpret_cast<double*>(w + 2 * align256((size_t)n * sizeof(float4)));
-        am::launch_pack_positions(d_r, nullptr, hi, lo, n, st);
-        am::launch_rpy_partial_mixed(hi, lo, d_lambda, part, n, sp, prm, wall, st);
-        am::launch_sum_partials(part, d_u, n, sp.splits, st);
-    } else {
-        double4_32a* r4 = reinterpret_cast<double4_32a*>(w);
-        double* part = reinterpret_cast<double*>(w + align256((size_t)n * sizeof(double4_32a)));
-        am::launch_pack_positions(d_r, r4, nullptr, nullptr, n, st);
-        am::launch_rpy_partial_f64(r4, d_lambda, part, n, sp, prm, wall, st);
-        am::launch_sum_partials(part, d_u, n, sp.splits, st);
-    }
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = am::product(d_r, d_lambda, d_u, n, 0, n, eta, a, wall, precision, d_work, work_bytes,
+                                      static_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return fail(AM_ERR_CUDA, cudaGetErrorString(e));
     return AM_OK;
 }
 
 extern "C" AM_API size_t am_rpy_matvec_rows_workspace(int n, int nrows, int precision) {
-    if (n <= 0 || nrows <= 0) return 0;
-    am::Split sp = am::choose_split_rows(n, nrows, precision);
-    size_t pos = (precision == AM_MIXED) ? 2 * align256((size_t)n * sizeof(float4))
-                                         : align256((size_t)n * sizeof(double4_32a));
-    return pos + align256((size_t)sp.splits * 3 * nrows * sizeof(double));
+    return am::least_workspace(n, nrows, precision);
 }
 
 extern "C" AM_API int am_rpy_matvec_rows(const double* d_r, const double* d_lambda, double* d_u, int n, int row0,
@@ -397,29 +155,12 @@ extern "C" AM_API int am_rpy_matvec_rows(const double* d_r, const double* d_lamb
         return fail(AM_ERR_ARG, "am_rpy_matvec_rows: unknown precision");
     if (n == 0 || nrows == 0) return AM_OK;
     if (!d_r || !d_lambda || !d_u || !d_work) return fail(AM_ERR_ARG, "am_rpy_matvec_rows: NULL pointer");
-    if (work_bytes < am_rpy_matvec_rows_workspace(n, nrows, precision))
+    if (work_bytes < am::least_workspace(n, nrows, precision))
         return fail(AM_ERR_ARG, "am_rpy_matvec_rows: workspace too small");
     if (reinterpret_cast<uintptr_t>(d_work) % 256 != 0)
         return fail(AM_ERR_ARG, "am_rpy_matvec_rows: workspace not 256-byte aligned");
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    am::Split sp = am::choose_split_rows(n, nrows, precision);
-    am::RpyParams prm = am::make_params(eta, a);
-    char* w = static_cast<char*>(d_work);
-    if (precision == AM_MIXED) {
-        float4* hi = reinterpret_cast<float4*>(w);
-        float4* lo = reinterpret_cast<float4*>(w + align256((size_t)n * sizeof(float4)));
-        double* part = reinterpret_cast<double*>(w + 2 * align256((size_t)n * sizeof(float4)));
-        am::launch_pack_positions(d_r, nullptr, hi, lo, n, st);
-        am::launch_rpy_partial_mixed_rows(hi, lo, d_lambda, part, n, row0, nrows, sp, prm, wall, st);
-        am::launch_sum_partials(part, d_u, nrows, sp.splits, st);
-    } else {
-        double4_32a* r4 = reinterpret_cast<double4_32a*>(w);
-        double* part = reinterpret_cast<double*>(w + align256((size_t)n * sizeof(double4_32a)));
-        am::launch_pack_positions(d_r, r4, nullptr, nullptr, n, st);
-        am::launch_rpy_partial_f64_rows(r4, d_lambda, part, n, row0, nrows, sp, prm, wall, st);
-        am::launch_sum_partials(part, d_u, nrows, sp.splits, st);
-    }
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = am::product(d_r, d_lambda, d_u, n, row0, nrows, eta, a, wall, precision, d_work, work_bytes,
+                                      static_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return fail(AM_ERR_CUDA, cudaGetErrorString(e));
     return AM_OK;
 }
@@ -622,79 +363,6 @@ rpy_items_mixed(const float4* __restrict__ hi, const float4* __restrict__ lo,
     item_queue_done(counter);
 }
 
-// ---- paired FP32 arithmetic: two targets per thread in the lanes of float2
-// registers (__ffma2_rn and friends: one instruction for both targets), the
-// source values in shared memory already duplicated and negated so that one
-// 128-bit load gives ready register pairs.
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 bc2(float v) { return make_float2(v, v); }
-__device__ __forceinline__ float2 rsq2(float2 a) { return make_float2(rsq(a.x), rsq(a.y)); }
-
-// (hi, lo) += t exactly in each lane (Knuth's TwoSum of hi and t, the
-// rounding error added to lo): the compensated accumulation of the tile sums
-__device__ __forceinline__ void two_sum_acc2(float2& hi, float2& lo, float2 t) {
-    const float2 m1 = bc2(-1.f);
-    const float2 s = add2(hi, t);
-    const float2 v = fma2(hi, m1, s);                          // s - hi
-    const float2 e = add2(fma2(fma2(v, m1, s), m1, hi),        // hi - (s - v)
-                          fma2(v, m1, t));                      // + (t - v)
-    hi = s;
-    lo = add2(lo, e);
-}
-
-// Free-space pair plus wall image in both lanes: pair_wall_r2 of
-// rpy_pair.cuh (same operations in the same order), with the free-space
-// coefficients of the far branch; pairs closer than 2a in either lane take
-// free_coefs per lane.  nx3 = -x3 per lane.
-template <bool WALL>
-__device__ __forceinline__ void pair2(float2 dx, float2 dy, float2 dz, float2 rxy2, float2 r2, float2 Rz, float2 h2,
-                                      float2 nx3, float2 lx, float2 ly, float2 lz, const RpyK<float>& k,
-                                      float2& ux, float2& uy, float2& uz) {
-    const float2 one = bc2(1.f);
-    float2 c1f, c2f;
-    if (r2.x < k.four_a2 || r2.y < k.four_a2) {
-        free_coefs<float>(r2.x, k, c1f.x, c2f.x);
-        free_coefs<float>(r2.y, k, c1f.y, c2f.y);
-    } else {
-        const float2 ri = rsq2(r2);
-        const float2 ri2 = mul2(ri, ri);
-        c1f = mul2(ri, fma2(bc2(k.kf2), ri2, one));
-        c2f = mul2(mul2(ri, ri2), fma2(bc2(-k.kf3), ri2, one));
-    }
-    const float2 dlxy = fma2(dx, lx, mul2(dy, ly));
-    const float2 Df = fma2(dz, lz, dlxy);
-    const float2 sdl = mul2(c2f, Df);
-    if (!WALL) {
-        ux = fma2(c1f, lx, fma2(sdl, dx, ux));
-        uy = fma2(c1f, ly, fma2(sdl, dy, uy));
-        uz = fma2(c1f, lz, fma2(sdl, dz, uz));
-        return;
-    }
-    const float2 Rz2 = mul2(Rz, Rz);
-    const float2 Di = fma2(Rz, lz, dlxy);
-    const float2 s = rsq2(add2(rxy2, Rz2));
-    const float2 w = mul2(s, s), s3 = mul2(s, w), w2 = mul2(w, w);
-    const float2 c1 = fma2(h2, nx3, bc2(k.wc1));
-    const float2 c2 = fma2(Rz2, bc2(k.w2a2), bc2(k.wc2));
-    const float2 c3 = mul2(Rz2, bc2(k.wc3));
-    const float2 x1 = fma2(w, c3, c2);
-    const float2 cI = fma2(w, fma2(w, x1, c1), bc2(-1.f));
-    const float2 y = fma2(w, c3, x1);
-    const float2 yz = fma2(w, c3, y);
-    const float2 cRR = fma2(mul2(w2, y), bc2(-2.f), fma2(cI, bc2(-3.f), bc2(-4.f)));
-    const float2 A4w2n = mul2(w2, bc2(-k.wa4));
-    const float2 inner = fma2(cRR, bc2(-2.f), fma2(A4w2n, bc2(-1.f), bc2(-2.f)));
-    const float2 P = mul2(s3, fma2(cRR, Di, mul2(fma2(Rz, inner, h2), lz)));
-    const float2 Q = mul2(s3, fma2(h2, Df, fma2(mul2(A4w2n, Rz), Di, mul2(mul2(w, fma2(yz, bc2(-2.f), bc2(k.wi2))), lz))));
-    const float2 cc = fma2(s, cI, c1f);
-    const float2 pp = add2(sdl, P);
-    ux = fma2(cc, lx, fma2(pp, dx, ux));
-    uy = fma2(cc, ly, fma2(pp, dy, uy));
-    uz = fma2(cc, lz, fma2(sdl, dz, fma2(P, Rz, add2(uz, Q))));
-}
-
 // Both directions of a pair in paired FP32 lanes: u += M lambda_src for two
 // targets (the lanes), and v += M^T mu for the source from each target (v.x
 // from the first, v.y from the second; the caller adds them).  The
@@ -757,30 +425,35 @@ __device__ __forceinline__ void pair2_sym(float2 dx, float2 dy, float2 dz, float
     vz = fma2(P1, dmxy, fma2(M33, mz, vz));
 }
 
-// Symmetric mixed product on tile pairs of 128 blobs (the SymItem list of
-// the handle, tiles of 128): warp w holds 64 targets of tile I, two per lane
-// in the lanes of float2 registers (targets 64 (w & 1) + l and + 32), and
-// takes source sub-tiles 2 (w >> 1) and 2 (w >> 1) + 1 of tile J (32
-// sources each).  At step t lane l meets source (l + t) mod 32 of the
-// sub-tile with both targets; the source's column sum (the two targets'
-// contributions added) moves one lane per step as in k_sym_tiles.
-// Differences from the hi parts, with the lo parts added within a quarter
-// of the target's largest coordinate (as rpy_items_mixed_x2).  FP32 sums over
-// at most 64 terms (a warp's sources for u, its targets for v), added in
-// FP64 across warps in a fixed order.  Diagonal items (I = J) take every
-// ordered pair in one direction (the self term included), no column sums.
+// Symmetric mixed product on tiles of 128 blobs: items are pairs of groups of
+// whole tiles, walked tile pair by tile pair.  Warp w holds 64 targets of tile
+// I, two per lane in the lanes of float2 registers (targets 64 (w & 1) + l and
+// + 32), and takes source sub-tiles 2 (w >> 1) and 2 (w >> 1) + 1 of tile J (32
+// sources each).  At step t lane l meets source (l + t) mod 32 of the sub-tile
+// with both targets; the source's column sum (the two targets' contributions
+// added) moves one lane per step as in k_sym_tiles.  Differences from the hi
+// parts, with the lo parts added within a quarter of the target's largest
+// coordinate (as rpy_items_mixed_x2).  FP32 sums over at most 64 terms (a
+// warp's sources for u, its targets for v), added across warps and tiles to
+// compensated (hi, lo) float pairs in a fixed order: the targets' in shared
+// memory, the sources' in the item's slots, which hold such pairs in units of
+// A1.  No FP64 work: sums and forces folded through the FP64 pipe (2 lanes per
+// SM and cycle) cost a tenth of the kernel.  A tile against itself meets every
+// ordered pair (the self term included) and drops the column sums: a second,
+// one-direction form of the pair in the loop cost 6 to 12 % by its code size.
 template <bool WALL>
 __global__ void __launch_bounds__(kThreads, 4)
-rpy_sym_mixed_x2(const float4* __restrict__ hi, const float4* __restrict__ lo, const double* __restrict__ lam,
-                 double* __restrict__ part, const SymItem* __restrict__ items, int n_items, int* __restrict__ counter,
-                 RpyK<float> k, const int* __restrict__ active) {
+rpy_sym_mixed_x2(const float4* __restrict__ hi, const float4* __restrict__ lo, const float4* __restrict__ lf,
+                 double* __restrict__ part, const SymItem* __restrict__ items,
+                 int n_items, int* __restrict__ counter, RpyK<float> k, const int* __restrict__ active) {
     dep_wait();
     constexpr int T = 128;
     __shared__ float4 sq[3][T];   // sources: (-hx, -hx, -hy, -hy), (2hz, 2hz, lz, lz), (lx, lx, ly, ly)
     __shared__ float4 so[T];      // (-ox, -ox, -oy, -oy)
     __shared__ float2 soz[T];     // (-oz, -oz)
-    __shared__ double up[4][64][3];     // row sums of each warp's 64 targets
-    __shared__ double vp[4][2][32][3];  // column sums of each warp's two sub-tiles
+    __shared__ float2 acc[3][T];       // row sums of the tile's targets: (hi, lo)
+    __shared__ float up[4][3][64];     // row sums of each warp's 64 targets over a tile of sources
+    __shared__ float vp[4][2][3][32];  // column sums of each warp's two sub-tiles
     __shared__ int s_item;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int th = warp & 1;            // target half of tile I
@@ -793,113 +466,130 @@ rpy_sym_mixed_x2(const float4* __restrict__ hi, const float4* __restrict__ lo, c
         if (itn >= n_items) break;
         const SymItem m = items[itn];
         const bool diag = m.ti == m.tj;
-        double* rowo = part + m.poff + (long long)m.tj * m.n3 + 3 * (long long)(m.i0 - m.tbase);
-        double* colo = part + m.poff + (long long)m.ti * m.n3 + 3 * (long long)(m.j0 - m.tbase);
+        float2* slots = reinterpret_cast<float2*>(part);
+        float2* rowo = slots + m.poff + (long long)m.tj * m.n3 + 3 * (long long)(m.i0 - m.tbase);
+        float2* colo = slots + m.poff + (long long)m.ti * m.n3 + 3 * (long long)(m.j0 - m.tbase);
         if (active && !active[m.sys]) {
-            for (int q = threadIdx.x; q < 3 * m.ni; q += blockDim.x) rowo[q] = 0.0;
+            for (int q = threadIdx.x; q < 3 * m.ni; q += blockDim.x) rowo[q] = bc2(0.f);
             if (!diag)
-                for (int q = threadIdx.x; q < 3 * m.nj; q += blockDim.x) colo[q] = 0.0;
+                for (int q = threadIdx.x; q < 3 * m.nj; q += blockDim.x) colo[q] = bc2(0.f);
             continue;
         }
-        {   // stage the sources of tile J (one per thread)
-            const int q = threadIdx.x;
-            const bool ok = q < m.nj;
-            const float4 h = ok ? hi[m.j0 + q] : make_float4(0.f, 0.f, 1.f, 0.f);
-            const float4 o = ok ? lo[m.j0 + q] : make_float4(0.f, 0.f, 0.f, 0.f);
-            const float lx = ok ? (float)lam[3 * (size_t)(m.j0 + q)] : 0.f;
-            const float ly = ok ? (float)lam[3 * (size_t)(m.j0 + q) + 1] : 0.f;
-            const float lz = ok ? (float)lam[3 * (size_t)(m.j0 + q) + 2] : 0.f;
-            sq[0][q] = make_float4(-h.x, -h.x, -h.y, -h.y);
-            sq[1][q] = make_float4(2.f * h.z, 2.f * h.z, lz, lz);
-            sq[2][q] = make_float4(lx, lx, ly, ly);
-            so[q] = make_float4(-o.x, -o.x, -o.y, -o.y);
-            soz[q] = make_float2(-o.z, -o.z);
-        }
-        __syncthreads();
-        const int t0 = 64 * th + lane, t1 = t0 + 32;
-        const bool ok0 = t0 < m.ni, ok1 = t1 < m.ni;
-        const float4 h0 = ok0 ? hi[m.i0 + t0] : make_float4(0.f, 0.f, 1.f, 0.f);
-        const float4 h1 = ok1 ? hi[m.i0 + t1] : make_float4(0.f, 0.f, 1.f, 0.f);
-        const float4 l0 = ok0 ? lo[m.i0 + t0] : make_float4(0.f, 0.f, 0.f, 0.f);
-        const float4 l1 = ok1 ? lo[m.i0 + t1] : make_float4(0.f, 0.f, 0.f, 0.f);
-        const float2 HX = make_float2(h0.x, h1.x), HY = make_float2(h0.y, h1.y), HZ = make_float2(h0.z, h1.z);
-        const float2 LX = make_float2(l0.x, l1.x), LY = make_float2(l0.y, l1.y), LZ = make_float2(l0.z, l1.z);
-        const float2 NX3 = make_float2(-h0.z, -h1.z);
-        const float n0 = 0.25f * fmaxf(fabsf(h0.x), fmaxf(fabsf(h0.y), fabsf(h0.z)));
-        const float n1 = 0.25f * fmaxf(fabsf(h1.x), fmaxf(fabsf(h1.y), fabsf(h1.z)));
-        const float near2x = n0 * n0, near2y = n1 * n1;
-        // the targets' forces for the column sums (zero for missing targets)
-        float2 MX = bc2(0.f), MY = bc2(0.f), MZ = bc2(0.f);
-        if (ok0) {
-            MX.x = (float)lam[3 * (size_t)(m.i0 + t0)];
-            MY.x = (float)lam[3 * (size_t)(m.i0 + t0) + 1];
-            MZ.x = (float)lam[3 * (size_t)(m.i0 + t0) + 2];
-        }
-        if (ok1) {
-            MX.y = (float)lam[3 * (size_t)(m.i0 + t1)];
-            MY.y = (float)lam[3 * (size_t)(m.i0 + t1) + 1];
-            MZ.y = (float)lam[3 * (size_t)(m.i0 + t1) + 2];
-        }
-        float2 ux = bc2(0.f), uy = bc2(0.f), uz = bc2(0.f);
-        for (int sbi = 0; sbi < 2; ++sbi) {
-            const int sb = sb0 + sbi;
-            float vx = 0.f, vy = 0.f, vz = 0.f;  // column sum of source 32 sb + ((lane + t) & 31)
+        for (int ia = 0; ia < m.ni; ia += T) {
+            const int t0 = ia + 64 * th + lane, t1 = t0 + 32;
+            const bool ok0 = t0 < m.ni, ok1 = t1 < m.ni;
+            const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
+            const float4 h0 = ok0 ? hi[m.i0 + t0] : make_float4(0.f, 0.f, 1.f, 0.f);
+            const float4 h1 = ok1 ? hi[m.i0 + t1] : make_float4(0.f, 0.f, 1.f, 0.f);
+            const float4 l0 = ok0 ? lo[m.i0 + t0] : none, l1 = ok1 ? lo[m.i0 + t1] : none;
+            const float2 HX = make_float2(h0.x, h1.x), HY = make_float2(h0.y, h1.y), HZ = make_float2(h0.z, h1.z);
+            const float2 LX = make_float2(l0.x, l1.x), LY = make_float2(l0.y, l1.y), LZ = make_float2(l0.z, l1.z);
+            const float2 NX3 = make_float2(-h0.z, -h1.z);
+            const float n0 = 0.25f * fmaxf(fabsf(h0.x), fmaxf(fabsf(h0.y), fabsf(h0.z)));
+            const float n1 = 0.25f * fmaxf(fabsf(h1.x), fmaxf(fabsf(h1.y), fabsf(h1.z)));
+            const float near2x = n0 * n0, near2y = n1 * n1;
+            // the targets' forces for the column sums (zero for missing targets)
+            const float4 f0 = ok0 ? lf[m.i0 + t0] : none, f1 = ok1 ? lf[m.i0 + t1] : none;
+            const float2 MX = make_float2(f0.x, f1.x), MY = make_float2(f0.y, f1.y), MZ = make_float2(f0.z, f1.z);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) acc[c][threadIdx.x] = bc2(0.f);
+            for (int jb = diag ? ia : 0; jb < m.nj; jb += T) {
+                const bool dtile = diag && jb == ia;
+                __syncthreads();
+                {   // stage the sources of the tile (one per thread)
+                    const int q = threadIdx.x;
+                    const bool ok = jb + q < m.nj;
+                    const int i = m.j0 + jb + q;
+                    const float4 h = ok ? hi[i] : make_float4(0.f, 0.f, 1.f, 0.f);
+                    const float4 o = ok ? lo[i] : none, f = ok ? lf[i] : none;
+                    sq[0][q] = make_float4(-h.x, -h.x, -h.y, -h.y);
+                    sq[1][q] = make_float4(2.f * h.z, 2.f * h.z, f.z, f.z);
+                    sq[2][q] = make_float4(f.x, f.x, f.y, f.y);
+                    so[q] = make_float4(-o.x, -o.x, -o.y, -o.y);
+                    soz[q] = make_float2(-o.z, -o.z);
+                }
+                __syncthreads();
+                float2 ux = bc2(0.f), uy = bc2(0.f), uz = bc2(0.f);
+#pragma unroll 1
+                for (int sbi = 0; sbi < 2; ++sbi) {
+                    const int sb = sb0 + sbi;
+                    float vx = 0.f, vy = 0.f, vz = 0.f;  // column sum of source 32 sb + ((lane + t) & 31)
 #pragma unroll 2
-            for (int t = 0; t < 32; ++t) {
-                const int q = 32 * sb + (diag ? t : ((lane + t) & 31));
-                const float4 v0 = sq[0][q], v1 = sq[1][q], v2 = sq[2][q];
-                const float2 h2 = make_float2(v1.x, v1.y);
-                float2 dx = add2(HX, make_float2(v0.x, v0.y));
-                float2 dy = add2(HY, make_float2(v0.z, v0.w));
-                float2 dz = fma2(h2, bc2(-0.5f), HZ);
-                const float2 Rz = fma2(h2, bc2(0.5f), HZ);
-                float2 rxy2 = fma2(dx, dx, mul2(dy, dy));
-                float2 r2 = fma2(dz, dz, rxy2);
-                if (r2.x < near2x || r2.y < near2y) {
-                    const float4 o = so[q];
-                    dx = add2(dx, add2(LX, make_float2(o.x, o.y)));
-                    dy = add2(dy, add2(LY, make_float2(o.z, o.w)));
-                    dz = add2(dz, add2(LZ, soz[q]));
-                    rxy2 = fma2(dx, dx, mul2(dy, dy));
-                    r2 = fma2(dz, dz, rxy2);
+                    for (int t = 0; t < 32; ++t) {
+                        const int q = 32 * sb + ((lane + t) & 31);
+                        const float4 v0 = sq[0][q], v1 = sq[1][q], v2 = sq[2][q];
+                        const float2 h2 = make_float2(v1.x, v1.y);
+                        float2 dx = add2(HX, make_float2(v0.x, v0.y));
+                        float2 dy = add2(HY, make_float2(v0.z, v0.w));
+                        float2 dz = fma2(h2, bc2(-0.5f), HZ);
+                        const float2 Rz = fma2(h2, bc2(0.5f), HZ);
+                        float2 rxy2 = fma2(dx, dx, mul2(dy, dy));
+                        float2 r2 = fma2(dz, dz, rxy2);
+                        if (r2.x < near2x || r2.y < near2y) {
+                            const float4 o = so[q];
+                            dx = add2(dx, add2(LX, make_float2(o.x, o.y)));
+                            dy = add2(dy, add2(LY, make_float2(o.z, o.w)));
+                            dz = add2(dz, add2(LZ, soz[q]));
+                            rxy2 = fma2(dx, dx, mul2(dy, dy));
+                            r2 = fma2(dz, dz, rxy2);
+                        }
+                        const float2 lxs = make_float2(v2.x, v2.y), lys = make_float2(v2.z, v2.w),
+                                     lzs = make_float2(v1.z, v1.w);
+                        float2 cx = bc2(0.f), cy = bc2(0.f), cz = bc2(0.f);
+                        pair2_sym<WALL>(dx, dy, dz, rxy2, r2, Rz, h2, NX3, lxs, lys, lzs, MX, MY, MZ, k, ux, uy, uz,
+                                        cx, cy, cz);
+                        vx += cx.x + cx.y;
+                        vy += cy.x + cy.y;
+                        vz += cz.x + cz.y;
+                        const int src = (lane + 1) & 31;
+                        vx = __shfl_sync(0xffffffffu, vx, src);
+                        vy = __shfl_sync(0xffffffffu, vy, src);
+                        vz = __shfl_sync(0xffffffffu, vz, src);
+                    }
+                    vp[warp][sbi][0][lane] = vx;
+                    vp[warp][sbi][1][lane] = vy;
+                    vp[warp][sbi][2][lane] = vz;
                 }
-                const float2 lxs = make_float2(v2.x, v2.y), lys = make_float2(v2.z, v2.w),
-                             lzs = make_float2(v1.z, v1.w);
-                if (diag) {
-                    pair2<WALL>(dx, dy, dz, rxy2, r2, Rz, h2, NX3, lxs, lys, lzs, k, ux, uy, uz);
-                } else {
-                    float2 cx = bc2(0.f), cy = bc2(0.f), cz = bc2(0.f);
-                    pair2_sym<WALL>(dx, dy, dz, rxy2, r2, Rz, h2, NX3, lxs, lys, lzs, MX, MY, MZ, k, ux, uy, uz,
-                                    cx, cy, cz);
-                    vx += cx.x + cx.y;
-                    vy += cy.x + cy.y;
-                    vz += cz.x + cz.y;
-                    const int src = (lane + 1) & 31;
-                    vx = __shfl_sync(0xffffffffu, vx, src);
-                    vy = __shfl_sync(0xffffffffu, vy, src);
-                    vz = __shfl_sync(0xffffffffu, vz, src);
+                up[warp][0][lane] = ux.x; up[warp][1][lane] = uy.x; up[warp][2][lane] = uz.x;
+                up[warp][0][32 + lane] = ux.y; up[warp][1][32 + lane] = uy.y; up[warp][2][32 + lane] = uz.y;
+                __syncthreads();
+                const int t = threadIdx.x;
+                {   // target t: half t >> 6, entry t & 63 of warps t >> 6 and + 2
+                    const int hh = t >> 6, j = t & 63;
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) {
+                        float2 a = acc[c][t];
+                        two_sum_acc(a.x, a.y, up[hh][c][j]);
+                        two_sum_acc(a.x, a.y, up[hh + 2][c][j]);
+                        acc[c][t] = a;
+                    }
+                }
+                if (!dtile && jb + t < m.nj) {  // source t: sub-tile sb = t >> 5 of warps 2 (sb >> 1) and + 1
+                    const int sb = t >> 5, l = t & 31, wa = 2 * (sb >> 1), si = sb & 1;
+                    float2* o = colo + 3 * (size_t)(jb + t);
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) {
+                        float2 a = ia == 0 ? bc2(0.f) : o[c];
+                        two_sum_acc(a.x, a.y, vp[wa][si][c][l]);
+                        two_sum_acc(a.x, a.y, vp[wa + 1][si][c][l]);
+                        o[c] = a;
+                    }
                 }
             }
-            vp[warp][sbi][lane][0] = vx;
-            vp[warp][sbi][lane][1] = vy;
-            vp[warp][sbi][lane][2] = vz;
-        }
-        up[warp][lane][0] = ux.x; up[warp][lane][1] = uy.x; up[warp][lane][2] = uz.x;
-        up[warp][32 + lane][0] = ux.y; up[warp][32 + lane][1] = uy.y; up[warp][32 + lane][2] = uz.y;
-        __syncthreads();
-        {
+            // the rows of a diagonal item also hold the column sums of its
+            // earlier target tiles
             const int t = threadIdx.x;
-            if (t < m.ni) {  // target t: half t >> 6, row t & 63 of warps th and th + 2
-                const int hh = t >> 6, j = t & 63;
-                rowo[3 * t] = k.A1 * (up[hh][j][0] + up[hh + 2][j][0]);
-                rowo[3 * t + 1] = k.A1 * (up[hh][j][1] + up[hh + 2][j][1]);
-                rowo[3 * t + 2] = k.A1 * (up[hh][j][2] + up[hh + 2][j][2]);
-            }
-            if (!diag && t < m.nj) {  // source t: sub-tile sb = t >> 5 of warps 2 (sb >> 1) and + 1
-                const int sb = t >> 5, l = t & 31, wa = 2 * (sb >> 1), si = sb & 1;
-                colo[3 * t] = k.A1 * (vp[wa][si][l][0] + vp[wa + 1][si][l][0]);
-                colo[3 * t + 1] = k.A1 * (vp[wa][si][l][1] + vp[wa + 1][si][l][1]);
-                colo[3 * t + 2] = k.A1 * (vp[wa][si][l][2] + vp[wa + 1][si][l][2]);
+            if (ia + t < m.ni) {
+                float2* o = rowo + 3 * (size_t)(ia + t);
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    float2 a = acc[c][t];
+                    if (diag && ia > 0) {
+                        two_sum_acc(a.x, a.y, o[c].x);
+                        a.y += o[c].y;
+                    }
+                    o[c] = a;
+                }
             }
         }
     }
@@ -1147,14 +837,61 @@ rpy_items_mixed_x2(const float4* __restrict__ hi, const float4* __restrict__ lo,
 
 // u = the sums over the slots of each element's system
 __global__ void __launch_bounds__(256)
-k_sum_items(int n3, int G, const double* __restrict__ part, const int* __restrict__ sys_of_blob,
+k_sum_items(int n3, int G, double scale, const double* __restrict__ part, const int* __restrict__ sys_of_blob,
             const int* __restrict__ sys_blob0, const int* __restrict__ sys_nb,
             const int* __restrict__ sys_nch, const long long* __restrict__ sys_poff,
             double* __restrict__ u) {
     __shared__ double sh[256];
-    const double a = slot_sum(blockIdx.x, G, n3, part, sys_of_blob, sys_blob0, sys_nb, sys_nch, sys_poff, sh);
+    const double a = slot_sum(blockIdx.x, G, scale, n3, part, sys_of_blob, sys_blob0, sys_nb, sys_nch, sys_poff, sh);
     const int t = blockIdx.x * (256 / G) + threadIdx.x;
     if (threadIdx.x < 256 / G && t < n3) u[t] = a;
+}
+
+// ---- stateless products ---------------------------------------------------
+static size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
+
+// The least scratch that a caller passes, for nt targets against n sources: a
+// packed copy of the positions and as many chunks of partial sums as give 4
+// blocks of 128 targets per SM.  (The cluster product needs none of it.)
+size_t least_workspace(int n, int nt, int precision) {
+    if (n <= 0 || nt <= 0) return 0;
+    const int want = 4 * num_sms();
+    const int tpt = precision == AM_MIXED && (nt + 2 * kThreads - 1) / (2 * kThreads) >= want ? 2 : 1;
+    const int tiles = (n + kTile - 1) / kTile;
+    const int tblocks = (nt + kThreads * tpt - 1) / (kThreads * tpt);
+    const int splits = std::max(1, std::min(tiles, (want + tblocks - 1) / tblocks));
+    const int chunk = (tiles + splits - 1) / splits * kTile;
+    const size_t pos = precision == AM_MIXED ? 2 * align256((size_t)n * sizeof(float4))
+                                             : align256((size_t)n * sizeof(double4_32a));
+    return pos + align256((size_t)((n + chunk - 1) / chunk) * 3 * nt * sizeof(double));
+}
+
+// The symmetric FP64 product of all n blobs: groups of 32-blob tiles.
+struct SymPlan {
+    SymSpan span;
+    int n_items = 0;
+    size_t bytes = 0;
+};
+static SymPlan sym_plan(int n) {
+    SymPlan p;
+    p.span.n = n;
+    p.span.T = 32 * sym_group_tiles(n);
+    p.span.ng = (n + p.span.T - 1) / p.span.T;
+    const int pairs = p.span.ng * (p.span.ng + 1) / 2;
+    p.span.splits = sym_step_splits(pairs);
+    p.n_items = pairs * p.span.splits;
+    p.bytes = align256((size_t)p.span.ng * p.span.splits * 3 * n * sizeof(double));
+    return p;
+}
+
+// FP64: from this many blobs on the symmetric product is the faster one.
+// Measured, cluster product against symmetric (us, free space / wall): 200
+// blobs 8.0 / 12.1 against 11.6 / 17.7, 300 blobs 16.9 / 31 against 12.3 / 17.2.
+constexpr int kSymFrom = 256;
+
+size_t product_workspace(int n, int precision) {
+    const size_t least = least_workspace(n, n, precision);
+    return precision == AM_FP64 && n >= kSymFrom ? std::max(least, sym_plan(n).bytes) : least;
 }
 
 template <class F>
@@ -1163,6 +900,65 @@ static int resident_grid(F kernel, int threads = kThreads) {
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, 0) != cudaSuccess || per <= 0)
         per = 4;
     return per * num_sms();
+}
+
+template <bool WALL>
+static void product_sym(const double* r, const double* lam, double* u, int n, const RpyParams& prm, const SymPlan& p,
+                        double* part, cudaStream_t st) {
+    static const int resident = resident_grid(k_sym_tiles<SymBlobPair<WALL>>, 32 * kSymWarps);  // asked for once
+    launch_dep(k_sym_tiles<SymBlobPair<WALL>>, dim3(std::min(resident, (p.n_items + kSymWarps - 1) / kSymWarps)),
+               dim3(32 * kSymWarps), 0, st, r, lam, part, (const SymItem*)nullptr, p.n_items, (int*)nullptr,
+               SymBlobPair<WALL>(rpy_consts<double>(prm)), (const int*)nullptr, p.span);
+    launch_dep(k_sum_slots, dim3((3 * n + 31) / 32), dim3(256), 0, st, (const double*)part, u, 3 * n,
+               p.span.ng * p.span.splits);
+    count_launch(2);
+}
+
+// Mixed: two targets per thread once groups of 64 targets in clusters of 8
+// give every SM two CTAs (2,432 targets); one target per thread spreads fewer
+// targets over more SMs.  Measured, one against two (us, wall): 853 rows of
+// 2,560 blobs 32.8 against 34.1, 1,666 of 5,000 43.6 against 56.7, 2,560 of 2,560
+// 38.7 against 37.9, 4,000 of 12,000 191 against 169, 60,000 of 60,000 9,423
+// against 8,849 (11,790 before, unpaired lanes over split sources).
+constexpr int kPairFrom = 2;
+template <bool WALL>
+static void product_mixed(const double* r, const double* lam, double* u, int n, int t0, int nt, const RpyParams& prm,
+                          char* work, cudaStream_t st) {
+    const RpyK<float> k = rpy_consts<float>(prm);
+    const int groups = (nt + 63) / 64;
+    if (groups * 8 < kPairFrom * num_sms()) {
+        launch_small_t<float, WALL>(r, lam, u, n, t0, nt, k, st);
+        return;
+    }
+    float4 *hi = reinterpret_cast<float4*>(work),
+           *lo = reinterpret_cast<float4*>(work + align256((size_t)n * sizeof(float4)));
+    launch_dep(k_pack_positions, dim3((n + 127) / 128), dim3(128), 0, st, r, hi, lo, n);
+    count_launch();
+    launch_cluster(k_rpy_small2<WALL>, groups, groups >= 4 * num_sms() ? 4 : 8, st, (const float4*)hi,
+                   (const float4*)lo, lam, u, n, t0, nt, k);
+}
+
+// u = rows t0 .. t0 + nt - 1 of M(r) lambda; `bytes` of scratch at work (at
+// least least_workspace; the symmetric product only where it holds its slots).
+cudaError_t product(const double* r, const double* lam, double* u, int n, int t0, int nt, double eta, double a,
+                    int wall, int precision, void* work, size_t bytes, cudaStream_t st) {
+    const RpyParams prm = make_params(eta, a);
+    if (precision == AM_MIXED) {
+        if (wall) product_mixed<true>(r, lam, u, n, t0, nt, prm, static_cast<char*>(work), st);
+        else product_mixed<false>(r, lam, u, n, t0, nt, prm, static_cast<char*>(work), st);
+        return cudaGetLastError();
+    }
+    if (nt == n && n >= kSymFrom) {
+        const SymPlan p = sym_plan(n);
+        if (bytes >= p.bytes) {
+            if (wall) product_sym<true>(r, lam, u, n, prm, p, static_cast<double*>(work), st);
+            else product_sym<false>(r, lam, u, n, prm, p, static_cast<double*>(work), st);
+            return cudaGetLastError();
+        }
+    }
+    if (wall) launch_small_t<double, true>(r, lam, u, n, t0, nt, rpy_consts<double>(prm), st);
+    else launch_small_t<double, false>(r, lam, u, n, t0, nt, rpy_consts<double>(prm), st);
+    return cudaGetLastError();
 }
 
 // resident blocks of the symmetric FP64 kernel
@@ -1197,7 +993,12 @@ int mobility_layout(am_handle* h, int tpt, int chunk, int tgroup, int sym) {
     if (h->cfg.precision != AM_MIXED) tpt = 1;
     if (h->per) chunk = std::max(1, h->Nb);  // the periodic product writes u in one piece
     if (h->per || (tpt == 2 && sym != 4)) sym = 0;  // paired lanes: tiles of 128 only
-    if (sym) chunk = 32 * sym;
+    // paired lanes: groups of tiles, at most kPairMaxGroups slots per system
+    int group = 1;
+    if (sym && tpt == 2)
+        for (int s = 0; s < S; ++s)
+            group = std::max(group, ((h->sys[s].Nb + 127) / 128 + kPairMaxGroups - 1) / kPairMaxGroups);
+    if (sym) chunk = 32 * sym * group;
     // targets per item: a block's targets, or (one target per thread) 32 or
     // 64 of them so that small systems spread over more SMs
     if (tpt == 2 || tgroup <= 0 || tgroup > kThreads || tgroup % 32) tgroup = kThreads * tpt;
@@ -1249,12 +1050,15 @@ int mobility_layout(am_handle* h, int tpt, int chunk, int tgroup, int sym) {
     std::vector<SymItem> sitems;
     if (sym) {
         for (int s = 0; s < S; ++s)
-            sym_append_items(sitems, s, h->sys_blob0[s], h->sys[s].Nb, 3, sym, splits, poff[s]);
+            sym_append_items(sitems, s, h->sys_blob0[s], h->sys[s].Nb, 3, sym * group, splits, poff[s]);
     }
     cudaStream_t st = h->stream;
     if (h->d_sym_items) cudaFree(h->d_sym_items);
     h->d_sym_items = nullptr;
     h->n_sym = 0;
+    if (sym && tpt == 2 && !h->d_lf &&
+        cudaMalloc(reinterpret_cast<void**>(&h->d_lf), std::max(h->Nb, 1) * sizeof(float4)) != cudaSuccess)
+        return 1;
     if (!sitems.empty()) {
         if (cudaMalloc(&h->d_sym_items, sitems.size() * sizeof(SymItem)) != cudaSuccess ||
             cudaMemcpyAsync(h->d_sym_items, sitems.data(), sitems.size() * sizeof(SymItem), cudaMemcpyHostToDevice,
@@ -1308,6 +1112,7 @@ int mobility_layout(am_handle* h, int tpt, int chunk, int tgroup, int sym) {
 // The partial sums of u = M lambda for all systems (mode: the handle's
 // precision, FP64 or double-float).
 void launch_items(am_handle* h, const double* lam, int mode, const int* active) {
+    h->mv_pairs = false;
     if (h->per) {  // FP32 wave part for the mixed operator; FP64 for FP64 and double-float requests
         launch_periodic(h, lam, mode == kOpMixed || (mode == kOpHandle && h->cfg.precision == AM_MIXED));
         return;
@@ -1325,10 +1130,10 @@ void launch_items(am_handle* h, const double* lam, int mode, const int* active) 
         const dim3 grid(h->mv_gridsym), block(32 * kSymWarps);
         if (h->cfg.wall)
             launch_dep(k_sym_tiles<SymBlobPair<true>>, grid, block, 0, st, (const double*)h->d_r3, lam, h->d_mv, si,
-                       h->n_sym, h->d_item_counter, SymBlobPair<true>{k}, active);
+                       h->n_sym, h->d_item_counter, SymBlobPair<true>(k), active, SymSpan{});
         else
             launch_dep(k_sym_tiles<SymBlobPair<false>>, grid, block, 0, st, (const double*)h->d_r3, lam, h->d_mv, si,
-                       h->n_sym, h->d_item_counter, SymBlobPair<false>{k}, active);
+                       h->n_sym, h->d_item_counter, SymBlobPair<false>(k), active, SymSpan{});
     } else if (fp64) {
         const RpyK<double> k = rpy_consts<double>(h->prm);
         if (h->cfg.wall)
@@ -1340,13 +1145,18 @@ void launch_items(am_handle* h, const double* lam, int mode, const int* active) 
     } else if (h->n_sym > 0 && h->sym_splits == 1) {
         const RpyK<float> k = rpy_consts<float>(h->prm);
         const SymItem* si = static_cast<const SymItem*>(h->d_sym_items);
-        const int th = h->mv_tpt == 2 || h->sym_nsub > 1 ? kThreads : 32;
+        const int th = h->sym_nsub > 1 ? kThreads : 32;
+        if (h->mv_tpt == 2) {  // forces as floats, slots as float pairs
+            launch_dep(k_pack_forces, dim3((h->Nb + 127) / 128), dim3(128), 0, st, lam, h->d_lf, h->Nb);
+            count_launch();
+            h->mv_pairs = true;
+        }
 #define AM_SYM32(W, N)                                                                                      \
     launch_dep(rpy_sym_mixed<W, N>, dim3(h->mv_gridsym32), dim3(th), 0, st, h->d_rhi, h->d_rlo, lam, h->d_mv, si, \
                h->n_sym, h->d_item_counter, k, active)
 #define AM_SYM32X2(W)                                                                                         \
-    launch_dep(rpy_sym_mixed_x2<W>, dim3(h->mv_gridsym32), dim3(kThreads), 0, st, h->d_rhi, h->d_rlo, lam, h->d_mv, \
-               si, h->n_sym, h->d_item_counter, k, active)
+    launch_dep(rpy_sym_mixed_x2<W>, dim3(h->mv_gridsym32), dim3(kThreads), 0, st, h->d_rhi, h->d_rlo,                \
+               (const float4*)h->d_lf, h->d_mv, si, h->n_sym, h->d_item_counter, k, active)
         if (h->cfg.wall) {
             if (h->mv_tpt == 2) AM_SYM32X2(true);
             else if (h->sym_nsub == 1) AM_SYM32(true, 1);
@@ -1382,7 +1192,7 @@ void launch_items(am_handle* h, const double* lam, int mode, const int* active) 
 void launch_sum_items(am_handle* h, double* u) {
     if (h->Nb <= 0) return;
     const int G = h->mv_sum_groups, per = 256 / G;
-    k_sum_items<<<(3 * h->Nb + per - 1) / per, 256, 0, h->stream>>>(3 * h->Nb, G, h->d_mv, h->d_sys_of_blob,
+    k_sum_items<<<(3 * h->Nb + per - 1) / per, 256, 0, h->stream>>>(3 * h->Nb, G, slot_scale(h), h->d_mv, h->d_sys_of_blob,
                                                                     h->d_sys_blob0, h->d_sys_nb, h->d_sys_nch,
                                                                     h->d_sys_poff, u);
     count_launch();
@@ -1426,9 +1236,9 @@ int mobility_autotune(am_handle* h) {
     }
     // The symmetric product: on tiles of 32, 64 and 128 blobs while its
     // partial sums (one slot per tile of the system) stay within 1 GiB (FP64,
-    // and mixed with one target per lane); mixed in paired lanes on tiles
-    // of 128 while they stay within a quarter of the free device memory
-    // (24 GB for 360,000 blobs)
+    // and mixed with one target per lane); mixed in paired lanes on groups
+    // of 128-blob tiles while they stay within a quarter of the free device
+    // memory (1.4 GB for 360,000 blobs)
     for (int nsub : {1, 2, 4}) {
         long long slots = 0;
         for (const auto& r : h->sys) slots += (long long)((r.Nb + 32 * nsub - 1) / (32 * nsub)) * 3 * r.Nb;
@@ -1438,7 +1248,8 @@ int mobility_autotune(am_handle* h) {
         size_t free_b = 0, total_b = 0;
         if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) free_b = 0;
         long long slots = 0;
-        for (const auto& r : h->sys) slots += (long long)((r.Nb + 127) / 128) * 3 * r.Nb;
+        for (const auto& r : h->sys)
+            slots += std::min<long long>((r.Nb + 127) / 128, kPairMaxGroups) * 3 * r.Nb;
         if ((double)slots * 8.0 <= 0.25 * (double)free_b) cand.push_back({2, 128, 0, 4});
     }
     cudaStream_t st = h->stream;

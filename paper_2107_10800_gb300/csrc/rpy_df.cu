@@ -172,11 +172,14 @@ __device__ __forceinline__ df df_shfl(df x, int src) {
     return df{__shfl_sync(0xffffffffu, x.h, src), __shfl_sync(0xffffffffu, x.l, src)};
 }
 
-// Symmetric double-float product on the handle's tile pairs of 128 blobs
+// Symmetric double-float product on the handle's items of 128-blob tiles
 // (the scheme of k_sym_tiles: 32 x 32 warp tiles, the source's column sum
-// carried lane to lane, steps 1..16 on the diagonal of a diagonal item);
-// warp-tile sums in double-float, added in FP64 across warps in a fixed
-// order.
+// carried lane to lane, steps 1..16 on the diagonal of a tile against
+// itself; groups of tiles walked tile pair by tile pair); warp-tile sums in
+// double-float, added in FP64 across warps and tiles in a fixed order.  As a
+// policy of k_sym_tiles, whose warps stage their own sources, it was slower
+// (36,000 wall blobs 20.0 against 17.5 ms): splitting doubles into floats is
+// FP64 work, here done once per 128 x 128 tile pair.
 template <bool WALL>
 __global__ void __launch_bounds__(kThreads)
 rpy_sym_df(const float4* __restrict__ hi, const float4* __restrict__ lo, const double* __restrict__ lam,
@@ -194,8 +197,14 @@ rpy_sym_df(const float4* __restrict__ hi, const float4* __restrict__ lo, const d
         __syncthreads();
         const int itn = s_item;
         if (itn >= n_items) break;
-        const SymItem m = items[itn];
-        const bool diag = m.ti == m.tj;
+        const SymItem g = items[itn];
+        for (int ia = 0; ia < g.ni; ia += T)
+        for (int jb = g.ti == g.tj ? ia : 0; jb < g.nj; jb += T) {
+        SymItem m = g;  // the tile pair
+        m.i0 += ia; m.ni = min(T, g.ni - ia);
+        m.j0 += jb; m.nj = min(T, g.nj - jb);
+        const bool diag = m.i0 == m.j0;
+        __syncthreads();
         {
             const int q = threadIdx.x;
             const bool oi = q < m.ni, oj = q < m.nj;
@@ -268,6 +277,9 @@ rpy_sym_df(const float4* __restrict__ hi, const float4* __restrict__ lo, const d
         __syncthreads();
         double* rowo = part + m.poff + (long long)m.tj * m.n3 + 3 * (long long)(m.i0 - m.tbase);
         double* colo = part + m.poff + (long long)m.ti * m.n3 + 3 * (long long)(m.j0 - m.tbase);
+        // the first tile pair to reach a row or column of the item writes it
+        // (rows of a diagonal item after their columns), later ones add
+        const bool row_first = g.ti == g.tj ? ia == 0 && jb == 0 : jb == 0, col_first = ia == 0;
         {
             const int t = threadIdx.x, a = t >> 5, l = t & 31;
             if (t < m.ni) {
@@ -279,15 +291,22 @@ rpy_sym_df(const float4* __restrict__ hi, const float4* __restrict__ lo, const d
                     for (int a2 = 0; a2 < NSUB; ++a2) {
                         sx += vp[a2 * NSUB + a][l][0]; sy += vp[a2 * NSUB + a][l][1]; sz += vp[a2 * NSUB + a][l][2];
                     }
-                rowo[3 * t] = k.A1 * sx; rowo[3 * t + 1] = k.A1 * sy; rowo[3 * t + 2] = k.A1 * sz;
+                double* o = rowo + 3 * t;
+                o[0] = row_first ? k.A1 * sx : fma(k.A1, sx, o[0]);
+                o[1] = row_first ? k.A1 * sy : fma(k.A1, sy, o[1]);
+                o[2] = row_first ? k.A1 * sz : fma(k.A1, sz, o[2]);
             }
             if (!diag && t < m.nj) {
                 double sx = 0.0, sy = 0.0, sz = 0.0;
                 for (int a2 = 0; a2 < NSUB; ++a2) {
                     sx += vp[a2 * NSUB + a][l][0]; sy += vp[a2 * NSUB + a][l][1]; sz += vp[a2 * NSUB + a][l][2];
                 }
-                colo[3 * t] = k.A1 * sx; colo[3 * t + 1] = k.A1 * sy; colo[3 * t + 2] = k.A1 * sz;
+                double* o = colo + 3 * t;
+                o[0] = col_first ? k.A1 * sx : fma(k.A1, sx, o[0]);
+                o[1] = col_first ? k.A1 * sy : fma(k.A1, sy, o[1]);
+                o[2] = col_first ? k.A1 * sz : fma(k.A1, sz, o[2]);
             }
+        }
         }
     }
     item_queue_done(counter);

@@ -77,7 +77,7 @@ __global__ void k_sb_ctphi(int M, const int* __restrict__ blo, const int* __rest
 // (1/s taken as 0 at r = 0, where every term but the self mobilities
 // vanishes).  FP64-issue-bound: about 90 FP64 operations per unordered pair
 // (136 per ordered pair in the one-direction form with its divisions).
-struct SymSpherePair {
+struct SymSpherePair : SymFp64 {
     static constexpr int kMinBlocks = 20;
     static constexpr int NC = 6;  // (force, torque) in, (velocity, rotation) out
     RpyK<double> k;
@@ -262,11 +262,16 @@ void sb_layout_free(am_handle* h) {
 // 90 operations per unordered pair).
 void sb_mobility(am_handle* h, const double* g, double* v) {
     const double a = h->cfg.blob_radius, a3 = a * a * a, a4 = a3 * a;
-    const SymSpherePair pr{rpy_consts<double>(h->prm), 1.0 / a, 0.5 / a3, 1.0 / a3, 9.0 / (32.0 * a4),
-                           -3.0 / (64.0 * a4 * a)};
+    SymSpherePair pr;
+    pr.k = rpy_consts<double>(h->prm);
+    pr.ia = 1.0 / a;
+    pr.h_a3 = 0.5 / a3;
+    pr.i_a3 = 1.0 / a3;
+    pr.n9_a4 = 9.0 / (32.0 * a4);
+    pr.n3_a5 = -3.0 / (64.0 * a4 * a);
     launch_dep(k_sym_tiles<SymSpherePair>, dim3(h->sb_grid), dim3(32 * kSymWarps), 0, h->stream,
                (const double*)h->d_q, g, h->d_sbpart, static_cast<const SymItem*>(h->d_sb_items), h->n_sb_items,
-               h->d_item_counter, pr, (const int*)nullptr);
+               h->d_item_counter, pr, (const int*)nullptr, SymSpan{});
     k_sb_sum<<<nb(6LL * h->M, 32), 256, 0, h->stream>>>(6 * h->M, h->d_sys_of_elem, h->d_sys_body_off, h->d_sb_poff,
                                                         h->d_sb_nslots, h->d_sbpart, v);
     count_launch(2);

@@ -1,6 +1,8 @@
-// Symmetric FP64 products on 32 x 32 warp tiles: u = N g for a symmetric
-// pair tensor N (N_ji = N_ij^T), each unordered pair evaluated once and
-// applied in both directions.
+// Symmetric products on 32 x 32 warp tiles: u = N g for a symmetric pair
+// tensor N (N_ji = N_ij^T), each unordered pair evaluated once and applied in
+// both directions.  The pair's arithmetic is a policy: FP64 here and in
+// single_blob.cu, double-float in rpy_df.cu; a tile's sums are in that
+// arithmetic, the sums over tiles in FP64.
 //
 // A warp takes a tile of 32 targets, one per lane, against 32 sources staged
 // in its own shared memory: at step t lane l meets source (l + t) mod 32, the
@@ -30,6 +32,7 @@
 #include "rpy_pair.cuh"
 
 #include <algorithm>
+#include <type_traits>
 #include <vector>
 
 namespace am {
@@ -39,13 +42,25 @@ namespace am {
 // 22 to 25 resident blocks per SM such a launch is one wave.
 constexpr int kSymWarps = 1;
 constexpr int kSymMaxGroups = 96;  // most groups (partial-sum slots) per system
+// the same for the paired-lane product, whose items run one per block of four
+// warps: about 12,000 items keep the last wave of a large product short
+constexpr int kPairMaxGroups = 160;
+
+// Values of the FP64 policies.
+struct SymFp64 {
+    using V = double;
+    static __device__ __forceinline__ double ld(double x) { return x; }
+    static __device__ __forceinline__ double to(double x) { return x; }
+    static __device__ __forceinline__ double shfl(double x, int lane) { return __shfl_sync(0xffffffffu, x, lane); }
+};
 
 // The blob mobility (3 components), free space or wall; sums in units of A1.
 template <bool WALL>
-struct SymBlobPair {
+struct SymBlobPair : SymFp64 {
     static constexpr int NC = 3;
     static constexpr int kMinBlocks = WALL ? 22 : 20;  // 80 and 96 registers, no spills
     RpyK<double> k;
+    explicit SymBlobPair(const RpyK<double>& q) : k(q) {}
     __device__ __forceinline__ double scale() const { return k.A1; }
     __device__ __forceinline__ void both(const double* xi, const double* xj, const double* l, const double* m,
                                          double* u, double* v) const {
@@ -68,28 +83,56 @@ struct SymBlobPair {
     }
 };
 
+// The items of one system of n without a list: groups of T, ng of them, the
+// steps split `splits` ways (items as sym_append_items makes them, poff = 0).
+struct SymSpan {
+    int n = 0, T = 32, ng = 0, splits = 1;
+};
+
+__device__ __forceinline__ SymItem sym_span_item(const SymSpan& sp, int nc, int idx) {
+    const int k = idx % sp.splits, p = idx / sp.splits;
+    // row a of the upper triangle starts at a ng - a (a - 1) / 2
+    const float w = 2.f * sp.ng + 1.f;
+    int a = (int)((w - sqrtf(fmaxf(0.f, w * w - 8.f * p))) * 0.5f);
+    a = max(0, min(a, sp.ng - 1));
+    while (a > 0 && a * sp.ng - a * (a - 1) / 2 > p) --a;
+    while ((a + 1) * sp.ng - (a + 1) * a / 2 <= p) ++a;
+    const int b = a + p - (a * sp.ng - a * (a - 1) / 2);
+    SymItem m;
+    m.i0 = a * sp.T; m.ni = min(sp.T, sp.n - m.i0);
+    m.j0 = b * sp.T; m.nj = min(sp.T, sp.n - m.j0);
+    m.tbase = 0; m.sys = 0;
+    m.ti = a * sp.splits + k; m.tj = b * sp.splits + k;
+    m.poff = 0; m.n3 = nc * sp.n;
+    m.steps = (32 * k / sp.splits) | (32 * (k + 1) / sp.splits) << 8;
+    return m;
+}
+
 // x: positions, g: NC values per target, both indexed by the items' blob (or
 // body) numbers; part: the slots.  counter[0]: next item, counter[1]: blocks
-// finished.
+// finished (NULL: warp w takes items w, w + warps, ..).  items NULL: those of
+// `span`.
 template <class Pair>
 __global__ void __launch_bounds__(32 * kSymWarps, Pair::kMinBlocks)
 k_sym_tiles(const double* __restrict__ x, const double* __restrict__ g, double* __restrict__ part,
             const SymItem* __restrict__ items, int n_items, int* __restrict__ counter, Pair pr,
-            const int* __restrict__ active) {
+            const int* __restrict__ active, SymSpan span) {
     dep_wait();
+    using V = typename Pair::V;
     constexpr int NC = Pair::NC;
-    __shared__ double sx[kSymWarps][3 + NC][32];
+    constexpr bool kFp64 = std::is_same_v<V, double>;
+    __shared__ V sx[kSymWarps][3 + NC][32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    double(*src)[32] = sx[warp];
+    V(*src)[32] = sx[warp];
+    const int warps = (int)gridDim.x * kSymWarps;
     for (int round = 0;; ++round) {
-        int itn = 0;
-        if (round == 0)
-            itn = blockIdx.x + warp * gridDim.x;  // the first items spread over the SMs
-        else if (lane == 0)
-            itn = (int)gridDim.x * kSymWarps + atomicAdd(counter, 1);
-        itn = __shfl_sync(0xffffffffu, itn, 0);
+        int itn = blockIdx.x + warp * gridDim.x + round * warps;  // the first items spread over the SMs
+        if (counter && round > 0) {  // taken only when the warp is free: no item waits for a busy one
+            if (lane == 0) itn = warps + atomicAdd(counter, 1);
+            itn = __shfl_sync(0xffffffffu, itn, 0);
+        }
         if (itn >= n_items) break;
-        const SymItem m = items[itn];
+        const SymItem m = items ? items[itn] : sym_span_item(span, NC, itn);
         const bool diag = m.ti == m.tj;
         double* rowo = part + m.poff + (long long)m.tj * m.n3 + NC * (long long)(m.i0 - m.tbase);
         double* colo = part + m.poff + (long long)m.ti * m.n3 + NC * (long long)(m.j0 - m.tbase);
@@ -104,14 +147,15 @@ k_sym_tiles(const double* __restrict__ x, const double* __restrict__ g, double* 
         for (int ia = 0; ia < m.ni; ia += 32) {
             const int t = ia + lane;
             const bool ti_ok = t < m.ni;
-            double xi[3] = {0.0, 0.0, 1.0}, mu[NC], u[NC];
+            V xi[3], mu[NC], u[NC];
+            double U[NC];  // sums over tiles (FP64 policies keep them in u)
 #pragma unroll
-            for (int c = 0; c < NC; ++c) mu[c] = u[c] = 0.0;
-            if (ti_ok) {
+            for (int c = 0; c < 3; ++c) xi[c] = Pair::ld(ti_ok ? x[3 * (size_t)(m.i0 + t) + c] : 1.0);
 #pragma unroll
-                for (int c = 0; c < 3; ++c) xi[c] = x[3 * (size_t)(m.i0 + t) + c];
-#pragma unroll
-                for (int c = 0; c < NC; ++c) mu[c] = g[NC * (size_t)(m.i0 + t) + c];
+            for (int c = 0; c < NC; ++c) {
+                mu[c] = Pair::ld(ti_ok ? g[NC * (size_t)(m.i0 + t) + c] : 0.0);
+                u[c] = Pair::ld(0.0);
+                U[c] = 0.0;
             }
             for (int jb = diag ? ia : 0; jb < m.nj; jb += 32) {
                 const bool self_tile = diag && jb == ia;
@@ -120,21 +164,24 @@ k_sym_tiles(const double* __restrict__ x, const double* __restrict__ g, double* 
                     const int q = jb + lane;
                     const bool ok = q < m.nj;
 #pragma unroll
-                    for (int c = 0; c < 3; ++c) src[c][lane] = ok ? x[3 * (size_t)(m.j0 + q) + c] : 1.0;
+                    for (int c = 0; c < 3; ++c) src[c][lane] = Pair::ld(ok ? x[3 * (size_t)(m.j0 + q) + c] : 1.0);
 #pragma unroll
-                    for (int c = 0; c < NC; ++c) src[3 + c][lane] = ok ? g[NC * (size_t)(m.j0 + q) + c] : 0.0;
+                    for (int c = 0; c < NC; ++c) src[3 + c][lane] = Pair::ld(ok ? g[NC * (size_t)(m.j0 + q) + c] : 0.0);
                 }
                 __syncwarp();
-                double v[NC];
+                V v[NC];
 #pragma unroll
-                for (int c = 0; c < NC; ++c) v[c] = 0.0;
+                for (int c = 0; c < NC; ++c) {
+                    v[c] = Pair::ld(0.0);
+                    if (!kFp64) u[c] = Pair::ld(0.0);
+                }
 #pragma unroll 1
                 for (int step = s0; step < s1; ++step) {
                     const int q = (lane + step) & 31;
                     const bool ok = ti_ok && jb + q < m.nj &&
                                     (!self_tile || (step >= 1 && (step < 16 || (step == 16 && lane < 16))));
                     if (ok) {
-                        double xj[3], l[NC];
+                        V xj[3], l[NC];
 #pragma unroll
                         for (int c = 0; c < 3; ++c) xj[c] = src[c][q];
 #pragma unroll
@@ -145,20 +192,27 @@ k_sym_tiles(const double* __restrict__ x, const double* __restrict__ g, double* 
                     }
                     // hand the column sum to the lane that meets this source next
 #pragma unroll
-                    for (int c = 0; c < NC; ++c) v[c] = __shfl_sync(0xffffffffu, v[c], (lane + 1) & 31);
+                    for (int c = 0; c < NC; ++c) v[c] = Pair::shfl(v[c], (lane + 1) & 31);
                 }
                 // lane l now holds the column sum of source (l + s1) mod 32
                 if (self_tile) {
 #pragma unroll
-                    for (int c = 0; c < NC; ++c) u[c] += __shfl_sync(0xffffffffu, v[c], (lane - s1) & 31);
+                    for (int c = 0; c < NC; ++c) {
+                        const V t = Pair::shfl(v[c], (lane - s1) & 31);
+                        if constexpr (kFp64) u[c] += t; else U[c] += Pair::to(t);
+                    }
                 } else {
                     const int q = jb + ((lane + s1) & 31);
                     if (q < m.nj) {
                         double* o = colo + NC * (size_t)q;
 #pragma unroll
-                        for (int c = 0; c < NC; ++c) o[c] = ia == 0 ? scale * v[c] : fma(scale, v[c], o[c]);
+                        for (int c = 0; c < NC; ++c)
+                            o[c] = ia == 0 ? scale * Pair::to(v[c]) : fma(scale, Pair::to(v[c]), o[c]);
                     }
                 }
+#pragma unroll
+                for (int c = 0; c < NC; ++c)
+                    if (!kFp64) U[c] += Pair::to(u[c]);
             }
             // the rows of a diagonal item also hold the column sums of its
             // earlier target tiles
@@ -166,11 +220,14 @@ k_sym_tiles(const double* __restrict__ x, const double* __restrict__ g, double* 
             if (ti_ok) {
                 double* o = rowo + NC * (size_t)t;
 #pragma unroll
-                for (int c = 0; c < NC; ++c) o[c] = diag && ia > 0 ? fma(scale, u[c], o[c]) : scale * u[c];
+                for (int c = 0; c < NC; ++c) {
+                    const double a = kFp64 ? Pair::to(u[c]) : U[c];
+                    o[c] = diag && ia > 0 ? fma(scale, a, o[c]) : scale * a;
+                }
             }
         }
     }
-    item_queue_done(counter);
+    if (counter) item_queue_done(counter);
 }
 
 // Tiles per group of a system of n: at most kSymMaxGroups groups.
