@@ -189,6 +189,7 @@ struct am_handle {
     int* d_sys_of_elem = nullptr;                 // n: system of each unknown
     int *d_chunk_start = nullptr, *d_chunk_end = nullptr, *d_sys_chunk_off = nullptr;
     int nchunks = 0;
+    void* d_chunk_info = nullptr;                 // int4 per chunk (k_arn_step)
     int* d_sys_of_blob = nullptr;                 // Nb
     int* d_sys_body_off = nullptr;                // S + 1: first body of each system
     int *d_sys_blob0 = nullptr, *d_sys_nb = nullptr, *d_sys_nch = nullptr;
@@ -196,8 +197,10 @@ struct am_handle {
     // batched GMRES scalars (per system)
     double *d_Hs = nullptr, *d_css = nullptr, *d_sns = nullptr, *d_gs = nullptr, *d_coefs = nullptr,
            *d_xis = nullptr, *d_bnorm_s = nullptr, *d_beta_s = nullptr, *d_inv_s = nullptr,
-           *d_tol_s = nullptr, *d_sysred = nullptr, *d_hcols = nullptr;
+           *d_tol_s = nullptr, *d_sysred = nullptr, *d_hcols = nullptr, *d_carry = nullptr;
     int *d_active = nullptr, *d_kdone = nullptr;
+    int* d_step_sync = nullptr;  // S arrival counts of the fused Arnoldi step
+    bool step_fused = false;
     int* d_arn_cnt = nullptr;  // S + 1 arrival counts of the fused Arnoldi step kernels
     int* d_pcb_cnt = nullptr;  // M arrival counts of the preconditioner apply (per body)
     int chunk_len = 1024, chunk_threads = 256;  // dot-product chunk length, threads per chunk block

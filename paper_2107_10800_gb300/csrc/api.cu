@@ -155,11 +155,13 @@ void free_solver(am_handle* h) {
     dfree(&h->d_Hm); dfree(&h->d_cs); dfree(&h->d_sn); dfree(&h->d_g); dfree(&h->d_coef);
     dfree(&h->d_xi); dfree(&h->d_part); dfree(&h->d_npart);
     dfree(&h->d_sys_of_elem); dfree(&h->d_sys_of_blob); dfree(&h->d_sys_body_off); dfree(&h->d_chunk_start); dfree(&h->d_chunk_end);
+    if (h->d_chunk_info) cudaFree(h->d_chunk_info);
+    h->d_chunk_info = nullptr;
     dfree(&h->d_sys_chunk_off); dfree(&h->d_Hs); dfree(&h->d_css); dfree(&h->d_sns); dfree(&h->d_gs);
-    dfree(&h->d_coefs); dfree(&h->d_xis); dfree(&h->d_hcols); dfree(&h->d_bnorm_s); dfree(&h->d_beta_s);
+    dfree(&h->d_coefs); dfree(&h->d_xis); dfree(&h->d_hcols); dfree(&h->d_carry); dfree(&h->d_bnorm_s); dfree(&h->d_beta_s);
     dfree(&h->d_inv_s); dfree(&h->d_tol_s); dfree(&h->d_sysred); dfree(&h->d_active); dfree(&h->d_kdone);
     dfree(&h->d_sys_blob0); dfree(&h->d_sys_nb); dfree(&h->d_sys_nch); dfree(&h->d_sys_poff);
-    dfree(&h->d_item_counter); dfree(&h->d_arn_cnt);
+    dfree(&h->d_item_counter); dfree(&h->d_arn_cnt); dfree(&h->d_step_sync);
     if (h->d_items) cudaFree(h->d_items);
     h->d_items = nullptr;
     h->n_items = 0;
@@ -721,16 +723,18 @@ int build_system_maps(am_handle* h) {
     CK(dalloc(&h->d_sys_of_elem, n)); CK(dalloc(&h->d_sys_of_blob, h->Nb));
     CK(dalloc(&h->d_chunk_start, cs.size())); CK(dalloc(&h->d_chunk_end, ce.size()));
     CK(dalloc(&h->d_sys_chunk_off, S + 1));
+    CK(cudaMalloc(&h->d_chunk_info, std::max<size_t>(cs.size(), 1) * sizeof(int4)));
     CK(dalloc(&h->d_Hs, (size_t)S * (m + 1) * m)); CK(dalloc(&h->d_css, (size_t)S * m));
     CK(dalloc(&h->d_sns, (size_t)S * m)); CK(dalloc(&h->d_gs, (size_t)S * (m + 1)));
     CK(dalloc(&h->d_coefs, (size_t)S * (m + 1))); CK(dalloc(&h->d_xis, (size_t)S * (m + 1)));
-    CK(dalloc(&h->d_hcols, (size_t)S * (m + 1)));
+    CK(dalloc(&h->d_hcols, (size_t)S * (m + 1))); CK(dalloc(&h->d_carry, S));
     CK(dalloc(&h->d_bnorm_s, S)); CK(dalloc(&h->d_beta_s, S)); CK(dalloc(&h->d_inv_s, S));
     CK(dalloc(&h->d_tol_s, S)); CK(dalloc(&h->d_sysred, 4 * (size_t)S + 16));
     CK(dalloc(&h->d_active, S)); CK(dalloc(&h->d_kdone, S));
-    CK(dalloc(&h->d_arn_cnt, S + 1));
+    CK(dalloc(&h->d_arn_cnt, S + 1)); CK(dalloc(&h->d_step_sync, S));
     CK(cudaMemsetAsync(h->d_arn_cnt, 0, (S + 1) * sizeof(int), st));
-    CK(dalloc(&h->d_part, (size_t)(m + 1) * std::max(1, h->nchunks)));
+    h->step_fused = am::step_fits(h, coff.data());
+    CK(dalloc(&h->d_part, 2 * (size_t)(m + 2) * std::max(1, h->nchunks)));
     CK(dalloc(&h->d_npart, std::max(h->nchunks, 4 * am::num_sms() + 64)));
     std::vector<int> b0(S), nb(S), bo(S + 1, h->M);
     for (int sI = 0; sI < S; ++sI) { b0[sI] = h->sys_blob0[sI]; nb[sI] = h->sys[sI].Nb; bo[sI] = h->sys_body0[sI]; }
@@ -744,6 +748,10 @@ int build_system_maps(am_handle* h) {
     CK(h2d(h->d_sys_of_blob, sys_of_blob.data(), h->Nb, st));
     CK(h2d(h->d_chunk_start, cs.data(), cs.size(), st));
     CK(h2d(h->d_chunk_end, ce.data(), ce.size(), st));
+    std::vector<int4> info(cs.size());
+    for (int sI = 0; sI < S; ++sI)
+        for (int c = coff[sI]; c < coff[sI + 1]; ++c) info[c] = make_int4(cs[c], ce[c], sI, coff[sI]);
+    CK(cudaMemcpyAsync(h->d_chunk_info, info.data(), info.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
     CK(h2d(h->d_sys_chunk_off, coff.data(), S + 1, st));
     CK(h2d(h->d_sys_blob0, b0.data(), S, st));
     CK(h2d(h->d_sys_nb, nb.data(), S, st));

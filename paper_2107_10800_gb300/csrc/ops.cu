@@ -184,9 +184,10 @@ __global__ void k_constraint_residual(int Nb, int M, int P, const int* __restric
                                       const double* __restrict__ lq, const double* __restrict__ B,
                                       const double* __restrict__ x, double* __restrict__ scal,
                                       int slot) {
-    __shared__ double sh[256];
+    __shared__ double sh[1024];
     const double* U = x + 3 * (size_t)Nb;
     double mx = 0.0;
+#pragma unroll 4
     for (int n = threadIdx.x; n < P; n += blockDim.x) {
         const double* up = U + 6 * bp[n];
         const double* uq = U + 6 * bq[n];
@@ -538,14 +539,16 @@ k_chunk_resid(const double* __restrict__ b, const double* __restrict__ Ax, doubl
     if (threadIdx.x == 0) npart[c] = a;
 }
 
-// out[s] = sqrt(sum of the system's chunk partials)
+// out[s] = sqrt(sum of the system's chunk partials), a warp per system
 __global__ void k_sys_norm(const double* __restrict__ npart, const int* __restrict__ coff, int S,
                            double* __restrict__ out) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    const int s = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (s >= S) return;
     double a = 0.0;
-    for (int c = coff[s]; c < coff[s + 1]; ++c) a += npart[c];
-    out[s] = sqrt(a);
+#pragma unroll 4
+    for (int c = coff[s] + lane; c < coff[s + 1]; c += 32) a += npart[c];
+    a = warp_sum(a);
+    if (lane == 0) out[s] = sqrt(a);
 }
 
 // out = min over systems (with b_s != 0) of |r_s| / |b_s|
@@ -567,16 +570,17 @@ __global__ void k_sys_minrel(int S, const double* __restrict__ beta, const doubl
 // Start of a restart cycle, one block: per system the relative residual
 // beta_s / ||b_s||; systems above tol are active, with v_0 scale 1/beta_s,
 // g = (beta_s, 0, ...), absolute stop threshold tol ||b_s||.  red[0] = max
-// relative residual (NaN if any is not finite), red[1] = active count.
+// relative residual (NaN if any is not finite, or a wait of an earlier step
+// ran out), red[1] = active count.
 __global__ void k_cycle_init(int S, int m, double tol, const double* __restrict__ beta,
                              const double* __restrict__ bnorm, int* __restrict__ active,
                              double* __restrict__ inv, double* __restrict__ g, int* __restrict__ kdone,
-                             double* __restrict__ tol_s, double* __restrict__ red) {
+                             double* __restrict__ tol_s, double* __restrict__ red, const int* __restrict__ flags) {
     __shared__ double smax[256];
     __shared__ int scnt[256];
     __shared__ int sbad[256];
     double mx = 0.0;
-    int cnt = 0, bad = 0;
+    int cnt = 0, bad = *flags & kFlagStepWait ? 1 : 0;
     for (int s = threadIdx.x; s < S; s += blockDim.x) {
         const double bn = bnorm[s], be = beta[s];
         const double rel = bn > 0.0 ? be / bn : 0.0;
@@ -627,44 +631,106 @@ __global__ void k_mask_sys(double* __restrict__ v, int n, const int* __restrict_
         if (!active[sys_of[i]]) v[i] = 0.0;
 }
 
-// Per active system, with a = |w_s|^2: H column j, Givens rotations, the
-// residual estimate; a system stops (kdone = j + 1) when the estimate
-// reaches its threshold or the step breaks down.  inv[s] = 1/|w_s| (0 if
-// stopped).
-__device__ __forceinline__ void finish_one(int s, int j, int m, const double* __restrict__ hcol, double a,
-                                           double* __restrict__ H, double* __restrict__ cs,
-                                           double* __restrict__ sn, double* __restrict__ g,
+// The running entry of the column hc under the earlier rotations,
+// c_{i+1} = -sn_i c_i + cs_i hc_{i+1}, by one warp: lane l composes the maps of
+// entries l E .. l E + E - 1, a scan over the lanes composes the rest.  The
+// rotated entries go to h (if not NULL); returns c_j in every lane.
+__device__ __forceinline__ double rotate_warp(int j, const double* __restrict__ cs, const double* __restrict__ sn,
+                                              const double* hc, double* h) {
+    constexpr int kMax = 7;  // 7 x 32 >= 200
+    const int lane = threadIdx.x & 31, E = (j + 31) / 32;
+    double A = 1.0, B = 0.0, sp[kMax], ss[kMax];
+#pragma unroll
+    for (int e = 0; e < kMax; ++e) {
+        const int i = lane * E + e;
+        const bool ok = e < E && i < j;
+        sp[e] = ok ? cs[i] * hc[i + 1] : 0.0;
+        ss[e] = ok ? -sn[i] : 1.0;
+        if (ok) {
+            A *= ss[e];
+            B = fma(ss[e], B, sp[e]);
+        }
+    }
+    for (int o = 1; o < 32; o <<= 1) {  // (A, B) after the lanes up to this one
+        const double a = __shfl_up_sync(0xffffffffu, A, o), b = __shfl_up_sync(0xffffffffu, B, o);
+        if (lane >= o) {
+            B = fma(A, b, B);
+            A *= a;
+        }
+    }
+    const double c0 = hc[0];
+    const double end = fma(__shfl_sync(0xffffffffu, A, 31), c0, __shfl_sync(0xffffffffu, B, 31));
+    const double a = __shfl_up_sync(0xffffffffu, A, 1), b = __shfl_up_sync(0xffffffffu, B, 1);
+    double c = lane ? fma(a, c0, b) : c0;
+    if (h) {
+#pragma unroll
+        for (int e = 0; e < kMax; ++e) {
+            const int i = lane * E + e;
+            if (e < E && i < j) {
+                h[i] = fma(cs[i], c, sn[i] * hc[i + 1]);
+                c = fma(ss[e], c, sp[e]);
+            }
+        }
+    }
+    return end;
+}
+
+// The end of a system's step from the running entry of the rotated column j,
+// a = |w_s|^2 and the residual so far g0: the new rotation, the column's last
+// entry and the residual estimate; the system stops when the estimate reaches
+// its threshold or the step breaks down.  inv = 1/|w_s| (0 if stopped).
+struct StepEnd {
+    double cc, sg, d, g0, g1, inv;
+    bool stop;
+};
+__device__ __forceinline__ StepEnd step_end(double carry, double a, double g0, double tol) {
+    StepEnd e;
+    double nrm, rn;
+    e.cc = 1.0;
+    e.sg = 0.0;
+    const double d2 = fma(carry, carry, a);
+    if (a > 1e-280 && d2 < 1e280) {
+        rn = rsqrt(a);
+        nrm = a * rn;
+        const double rd = rsqrt(d2);
+        e.d = d2 * rd;
+        e.cc = carry * rd;
+        e.sg = nrm * rd;
+    } else {  // squares out of range
+        nrm = sqrt(a);
+        rn = nrm > 0.0 ? 1.0 / nrm : 0.0;
+        e.d = hypot(carry, nrm);
+        if (e.d > 0.0) { e.cc = carry / e.d; e.sg = nrm / e.d; }
+    }
+    e.g1 = -e.sg * g0;
+    e.g0 = e.cc * g0;
+    e.stop = !(fabs(e.g1) > tol) || nrm == 0.0;
+    e.inv = (!e.stop && nrm > 0.0) ? rn : 0.0;
+    return e;
+}
+__device__ __forceinline__ void step_store(const StepEnd& e, int s, int j, int m, double* __restrict__ H,
+                                           double* __restrict__ cs, double* __restrict__ sn, double* __restrict__ g,
+                                           int* __restrict__ active, int* __restrict__ kdone,
+                                           double* __restrict__ inv) {
+    const int m1 = m + 1;
+    double* h = H + ((size_t)s * m + j) * m1;
+    cs[(size_t)s * m + j] = e.cc;
+    sn[(size_t)s * m + j] = e.sg;
+    h[j] = e.d;
+    h[j + 1] = 0.0;
+    g[(size_t)s * m1 + j] = e.g0;
+    g[(size_t)s * m1 + j + 1] = e.g1;
+    inv[s] = e.inv;
+    if (e.stop) { active[s] = 0; kdone[s] = j + 1; }
+}
+
+// The same per system in the separate kernels, by one thread.
+__device__ __forceinline__ void finish_one(int s, int j, int m, double carry, double a, double* __restrict__ H,
+                                           double* __restrict__ cs, double* __restrict__ sn, double* __restrict__ g,
                                            int* __restrict__ active, int* __restrict__ kdone,
                                            const double* __restrict__ tol_s, double* __restrict__ inv) {
     if (!active[s]) { inv[s] = 0.0; return; }
-    const int m1 = m + 1;
-    const double nrm = sqrt(a);
-    double* h = H + ((size_t)s * m + j) * m1;
-    const double* hc = hcol + (size_t)s * m1;
-    double* css = cs + (size_t)s * m;
-    double* sns = sn + (size_t)s * m;
-    double* gs = g + (size_t)s * m1;
-    // the earlier rotations applied in order; only the running entry carries
-    // from one rotation to the next, the rest are loads and stores
-    double carry = hc[0];
-    for (int i = 0; i < j; ++i) {
-        const double b = hc[i + 1];
-        const double t = css[i] * carry + sns[i] * b;
-        carry = -sns[i] * carry + css[i] * b;
-        h[i] = t;
-    }
-    const double d = hypot(carry, nrm);
-    double cc = 1.0, sg = 0.0;
-    if (d > 0.0) { cc = carry / d; sg = nrm / d; }
-    css[j] = cc; sns[j] = sg;
-    h[j] = d;
-    h[j + 1] = 0.0;
-    gs[j + 1] = -sg * gs[j];
-    gs[j] = cc * gs[j];
-    const double est = fabs(gs[j + 1]);
-    const bool stop = !(est > tol_s[s]) || nrm == 0.0;
-    inv[s] = (!stop && nrm > 0.0) ? 1.0 / nrm : 0.0;
-    if (stop) { active[s] = 0; kdone[s] = j + 1; }
+    step_store(step_end(carry, a, g[(size_t)s * (m + 1) + j], tol_s[s]), s, j, m, H, cs, sn, g, active, kdone, inv);
 }
 
 // Advance j; the cycle ends when no system is active, at the restart length
@@ -672,28 +738,19 @@ __device__ __forceinline__ void finish_one(int s, int j, int m, const double* __
 // thread of the one block calls it.
 __device__ void loop_ctrl(ArnoldiCtrl* c, int* __restrict__ active, int* __restrict__ kdone, int S,
                           cudaGraphConditionalHandle hc, int in_graph) {
-    __shared__ int scnt[256];
-    __shared__ int s_stop;
-    const int j1 = c->j + 1;
-    int cnt = 0;
-    for (int s = threadIdx.x; s < S; s += blockDim.x) cnt += __ldcg(active + s);  // set by other blocks
-    scnt[threadIdx.x] = cnt;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) scnt[threadIdx.x] += scnt[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) s_stop = (scnt[0] == 0 || j1 >= c->m || c->it + 1 >= c->budget) ? 1 : 0;
-    __syncthreads();
-    if (s_stop)
+    const int j1 = c->j + 1, it1 = c->it + 1;
+    int any = 0;
+    for (int s = threadIdx.x; s < S; s += blockDim.x) any |= __ldcg(active + s);  // set by other blocks
+    const int stop = (!__syncthreads_or(any) || j1 >= c->m || it1 >= c->budget) ? 1 : 0;
+    if (stop)
         for (int s = threadIdx.x; s < S; s += blockDim.x)
             if (__ldcg(active + s)) { kdone[s] = j1; active[s] = 0; }
     __syncthreads();
     if (threadIdx.x == 0) {
-        c->it += 1;
+        c->it = it1;
         c->j = j1;
-        c->stop = s_stop;
-        if (in_graph) cudaGraphSetConditional(hc, s_stop ? 0u : 1u);
+        c->stop = stop;
+        if (in_graph) cudaGraphSetConditional(hc, stop ? 0u : 1u);
     }
 }
 
@@ -707,59 +764,123 @@ __device__ void loop_ctrl(ArnoldiCtrl* c, int* __restrict__ active, int* __restr
 // arithmetic and its order are those of separate dot, coefficient,
 // orthogonalisation, norm and step-end kernels.
 
-// part[k * nchunks + b] = <V_k, w> over chunk [c0, c1), k <= j (a warp per k)
-__device__ __forceinline__ void chunk_dots(const double* __restrict__ V, size_t ldv, const double* w, int c0,
-                                           int c1, int j, double* __restrict__ part, int nchunks, int b) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int k = wid; k <= j; k += nw) {
-        const double* v = V + (size_t)k * ldv;
-        double a = 0.0;
-        for (int i = c0 + lane; i < c1; i += 32) a = fma(v[i], w[i], a);
-        a = warp_sum(a);
-        if (lane == 0) part[(size_t)k * nchunks + b] = a;
+// The sums over the warp of U values per lane (U = 1, 2, 4 or 8): the sum of
+// a[u] is returned in lanes u 32/U .. (u + 1) 32/U - 1.  Halves are exchanged
+// while several values are left, so U sums take U - 1 + 5 - log2 U additions
+// instead of 5 U; an FP64 warp instruction costs 16 cycles of its SM.
+template <int U>
+__device__ __forceinline__ double warp_sums(double* a, int lane) {
+    int off = 16;
+#pragma unroll
+    for (int n = U / 2; n >= 1; n /= 2, off /= 2) {
+        const bool up = lane & off;
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+            const double send = up ? a[i] : a[i + n], keep = up ? a[i + n] : a[i];
+            a[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+        }
+    }
+    for (; off >= 1; off /= 2) a[0] += __shfl_xor_sync(0xffffffffu, a[0], off);
+    return a[0];
+}
+
+// Sums over i in [i0, i1) of x_k[i] y[i], x_k = x + k ld, k <= j, given to
+// out(k, sum): U consecutive k per warp at a time, their loads in flight
+// together (a warp per k waited for every load and reduction in turn).  y NULL:
+// the sums of x_k, read past the SM's own cache (other blocks' values).
+template <int U, class Out>
+__device__ __forceinline__ void rows_sums_u(const double* x, size_t ld, const double* y, int i0, int i1, int j,
+                                            int nw, Out out) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (int k0 = U * wid; k0 <= j; k0 += U * nw) {
+        double a[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) a[u] = 0.0;
+#pragma unroll(U == 8 ? 2 : 4)
+        for (int i = i0 + lane; i < i1; i += 32) {
+            const double yi = y ? y[i] : 1.0;
+            double v[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const double* p = x + (size_t)min(k0 + u, j) * ld + i;
+                v[u] = y ? *p : __ldcg(p);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) a[u] = y ? fma(v[u], yi, a[u]) : a[u] + v[u];
+        }
+        const double t = warp_sums<U>(a, lane);
+        const int k = k0 + lane / (32 / U);
+        if (lane % (32 / U) == 0 && k <= j) out(k, t);
     }
 }
 
-// coef[s][k] = sum over the system's chunks (a warp per k, its lanes over
-// the chunks); hcol[s][k] = (hcol +) coef
+// U so that eight warps share the j + 1 sums in one go (at most 8 each)
+template <class Out>
+__device__ __forceinline__ void rows_sums(const double* x, size_t ld, const double* y, int i0, int i1, int j,
+                                          Out out) {
+    constexpr int nw = 8;  // the first 256 threads of the block
+    const int per = (j + nw) / nw;
+    if (per <= 1) rows_sums_u<1>(x, ld, y, i0, i1, j, nw, out);
+    else if (per <= 2) rows_sums_u<2>(x, ld, y, i0, i1, j, nw, out);
+    else if (per <= 4) rows_sums_u<4>(x, ld, y, i0, i1, j, nw, out);
+    else rows_sums_u<8>(x, ld, y, i0, i1, j, nw, out);
+}
+
+// part[k * nchunks + b] = <V_k, w> over chunk [c0, c1), k <= j
+__device__ __forceinline__ void chunk_dots(const double* __restrict__ V, size_t ldv, const double* w, int c0,
+                                           int c1, int j, double* __restrict__ part, int nchunks, int b) {
+    rows_sums(V, ldv, w, c0, c1, j, [&](int k, double a) { part[(size_t)k * nchunks + b] = a; });
+}
+
+// coef[s][k] = sum over the system's chunks; hcol[s][k] = (hcol +) coef
 __device__ __forceinline__ void sys_coef(int s, const double* part, int nchunks, const int* __restrict__ coff,
                                          int m1, int j, double* __restrict__ coef, double* __restrict__ hcol,
                                          int accumulate) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int q0 = coff[s], q1 = coff[s + 1];
-    for (int k = wid; k <= j; k += nw) {
-        const double* pk = part + (size_t)k * nchunks;
-        double a = 0.0;
-        for (int q = q0 + lane; q < q1; q += 32) a += __ldcg(pk + q);  // other blocks' sums
-        a = warp_sum(a);
-        if (lane == 0) {
-            coef[(size_t)s * m1 + k] = a;
-            double* hc = hcol + (size_t)s * m1 + k;
-            *hc = accumulate ? *hc + a : a;
-        }
-    }
+    rows_sums(part, nchunks, nullptr, coff[s], coff[s + 1], j, [&](int k, double a) {
+        coef[(size_t)s * m1 + k] = a;
+        double* hc = hcol + (size_t)s * m1 + k;
+        *hc = accumulate ? *hc + a : a;
+    });
 }
 
 // w_i -= sum_{k <= j} coef[s][k] V_k,i over the chunk; returns the thread's
 // share of |w|^2 over the chunk (after the update).  When the chunk is
 // shorter than the block, the block's G = blockDim / len groups of len
 // threads each sum every G-th term of an element's sum (shorter dependent
-// FP64 chains), combined in shared memory (sh: blockDim doubles).
+// FP64 chains), combined in shared memory (sh: blockDim doubles).  Eight terms
+// at a time, loaded together, in two chains.
 __device__ __forceinline__ double chunk_orth(const double* __restrict__ V, size_t ldv, double* w, int c0,
                                              int c1, int j, const double* cf, int len, double* sh) {
-    const int per = min((int)blockDim.x, len);  // threads per group
-    const int G = blockDim.x / per;
+    constexpr int kT = 256;  // the threads that call it
+    const int per = min(kT, len);  // threads per group
+    const int G = kT / per;
     const int e = threadIdx.x % per, g = threadIdx.x / per;
     double a = 0.0;
     for (int i0 = c0; i0 < c1; i0 += per) {
         const int i = i0 + e;
         double p = 0.0;
-        if (i < c1)
-            for (int k = g; k <= j; k += G) p = fma(cf[k], V[(size_t)k * ldv + i], p);
-        if (G > 1) {
-            __syncthreads();
+        if (i < c1) {
+            double q = 0.0;
+            for (int k = g; k <= j; k += 8 * G) {
+                double v[8], c[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const int kk = min(k + u * G, j);
+                    v[u] = V[(size_t)kk * ldv + i];
+                    c[u] = k + u * G <= j ? cf[kk] : 0.0;
+                }
+#pragma unroll
+                for (int u = 0; u < 8; u += 2) {
+                    if (k + u * G <= j) p = fma(c[u], v[u], p);
+                    if (k + (u + 1) * G <= j) q = fma(c[u + 1], v[u + 1], q);
+                }
+            }
+            p += q;
+        }
+        if (G > 1) {  // a barrier of these 256 threads
+            asm volatile("bar.sync 1, 256;" ::: "memory");
             sh[threadIdx.x] = p;
-            __syncthreads();
+            asm volatile("bar.sync 1, 256;" ::: "memory");
             if (g == 0)
                 for (int q = 1; q < G; ++q) p += sh[q * per + e];
         }
@@ -804,26 +925,44 @@ k_arn_orth_dots(const double* __restrict__ V, size_t ldv, double* __restrict__ w
 }
 
 // second pass: orthogonalisation and |w|^2; per system the step end
-// (finish_one), then the loop control
+// (finish_one), then the loop control.  Blocks nch .. nch + S - 1 rotate the
+// systems' new columns meanwhile (their coefficients are complete).
 __global__ void __launch_bounds__(256)
 k_arn_orth_finish(const double* __restrict__ V, size_t ldv, double* __restrict__ w, const int* __restrict__ cs,
                   const int* __restrict__ ce, const int* __restrict__ sys_of, const int* __restrict__ coff, int clen,
-                  double* __restrict__ npart, int m1, const double* __restrict__ coef,
+                  double* __restrict__ npart, int nch, int m1, const double* __restrict__ coef,
                   const double* __restrict__ hcol, int* __restrict__ cnt, int S, int m, double* __restrict__ H,
                   double* __restrict__ csv, double* __restrict__ snv, double* __restrict__ g,
-                  int* __restrict__ active, int* __restrict__ kdone, const double* __restrict__ tol_s,
-                  double* __restrict__ inv, ArnoldiCtrl* c, cudaGraphConditionalHandle hc, int in_graph) {
+                  double* __restrict__ carry, int* __restrict__ active, int* __restrict__ kdone,
+                  const double* __restrict__ tol_s, double* __restrict__ inv, ArnoldiCtrl* c,
+                  cudaGraphConditionalHandle hc, int in_graph) {
     dep_wait();
     __shared__ double sh[256];
-    const int j = c->j, b = blockIdx.x, c0 = cs[b], c1 = ce[b], s = sys_of[c0];
-    double a = chunk_orth(V, ldv, w, c0, c1, j, coef + (size_t)s * m1, clen, sh);
-    a = block_sum(a, sh);
-    if (threadIdx.x == 0) npart[b] = a;
-    if (arrive_last(cnt, s, coff[s + 1] - coff[s])) {
-        double w2 = 0.0;
-        for (int q = coff[s] + threadIdx.x; q < coff[s + 1]; q += blockDim.x) w2 += __ldcg(npart + q);
-        w2 = block_sum(w2, sh);
-        if (threadIdx.x == 0) finish_one(s, j, m, hcol, w2, H, csv, snv, g, active, kdone, tol_s, inv);
+    const int j = c->j, b = blockIdx.x;
+    int s;
+    if (b < nch) {
+        const int c0 = cs[b], c1 = ce[b];
+        s = sys_of[c0];
+        double a = chunk_orth(V, ldv, w, c0, c1, j, coef + (size_t)s * m1, clen, sh);
+        a = block_sum(a, sh);
+        if (threadIdx.x == 0) npart[b] = a;
+    } else {
+        s = b - nch;
+        if (active[s] && threadIdx.x < 32) {
+            const double e = rotate_warp(j, csv + (size_t)s * m, snv + (size_t)s * m, hcol + (size_t)s * m1,
+                                         H + ((size_t)s * m + j) * m1);
+            if (threadIdx.x == 0) carry[s] = e;
+        }
+    }
+    if (arrive_last(cnt, s, coff[s + 1] - coff[s] + 1)) {
+        if (threadIdx.x < 32) {
+            double w2 = 0.0;
+#pragma unroll 4
+            for (int q = coff[s] + threadIdx.x; q < coff[s + 1]; q += 32) w2 += __ldcg(npart + q);
+            w2 = warp_sum(w2);
+            if (threadIdx.x == 0)
+                finish_one(s, j, m, __ldcg(carry + s), w2, H, csv, snv, g, active, kdone, tol_s, inv);
+        }
         if (arrive_last(cnt, S, S)) loop_ctrl(c, active, kdone, S, hc, in_graph);
     }
 }
@@ -843,20 +982,211 @@ __global__ void k_next_basis(const double* __restrict__ w, double* __restrict__ 
     }
 }
 
-// xi_s = H_s(0:k, 0:k)^-1 g_s(0:k), k = kdone[s]  (one thread per system)
-__global__ void k_hess_solve_sys(const double* __restrict__ H, const double* __restrict__ g,
-                                 const int* __restrict__ kdone, double* __restrict__ xi, int S, int m) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+// ---- the whole step in one cooperative kernel ------------------------------
+// The steps of k_arn_dots .. k_next_basis for systems of a moderate number of
+// chunks, one block per chunk, all blocks resident.  Where the separate kernels
+// end, the blocks of a system meet at a counter: after the dots of either
+// pass.  Behind it every block adds the system's partial sums itself (a few
+// kilobytes of the L2), rotates the column and finds the residual estimate
+// itself, so nothing travels back; the system's first block writes the
+// results.  The norm needs no third meeting: with c the second pass's
+// coefficients |w - V c|^2 = |w|^2 - |c|^2, and c is the orthogonality error of
+// the first pass; if it is not small against w (a breakdown), the blocks meet
+// once more for the sum of the squares.  Eight warps hold the chunk of w (in
+// shared memory); a ninth forms |w|^2, the rotations and the step's end
+// meanwhile.  Latency-bound: an FP64 multiply-add takes about 100 cycles here,
+// a load from the L2 about 700, and the four kernels spent 27 to 30 us on launches,
+// first loads and serial sums.
+// sync[s] counts arrivals of system s since the start of the cycle: meeting b
+// (0, 1, 2) of step `it` waits for (3 it + b + 1) times its blocks.  The wait is
+// bounded; a wait that runs out sets kFlagStepWait and the kernel goes on to
+// its end.
+constexpr int kStepThreads = 288;
+constexpr int kStepSpins = 1 << 21;  // about a second
+
+__device__ __forceinline__ void sys_arrive(int* cnt) {  // after a barrier of the block
+    asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(cnt) : "memory");
+}
+__device__ __forceinline__ void sys_barrier(int* cnt, int target, int* flags) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        sys_arrive(cnt);
+        int n = 0, v;
+        do {
+            asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(cnt) : "memory");
+        } while (v < target && ++n < kStepSpins);
+        if (v < target) atomicOr(flags, kFlagStepWait);
+    }
+    __syncthreads();
+}
+
+struct StepArgs {
+    double* V;
+    size_t ldv;
+    const double* w;
+    const double* z;
+    double *Z, *vj;
+    const int4* info;  // per chunk: first and last element, system, first chunk of the system
+    const int* coff;
+    double *part, *npart;
+    int nch, m, S, clen;
+    double *H, *csv, *snv, *g;
+    int *active, *kdone;
+    const double* tol_s;
+    double* inv;
+    int *sync, *cnt, *flags;
+    ArnoldiCtrl* c;
+    cudaGraphConditionalHandle hc;
+    int in_graph;
+};
+
+__global__ void __launch_bounds__(kStepThreads)
+k_arn_step(StepArgs a) {
+    dep_wait();
+    __shared__ double ws[1024];                // the chunk of w
+    __shared__ double sh[256], red[64];
+    __shared__ double cf[200], hc[200];        // coefficients of a pass, of the column
+    __shared__ double s_cs[200], s_sn[200];
+    __shared__ double s_inv;
+    __shared__ int s_exact;
+    const int b = blockIdx.x, m1 = a.m + 1;
+    const int4 ci = a.info[b];
+    const int j = a.c->j, it = a.c->it;
+    const int c0 = ci.x, len = ci.y - ci.x, s = ci.z, q0 = ci.w, q1 = a.coff[s + 1], nb = q1 - q0;
+    const int lane = threadIdx.x & 31;
+    const bool vec = threadIdx.x < 256;  // the eight warps that hold the chunk
+    const bool first = b == q0;
+    if (a.active[s]) {
+        double g0 = 0.0, tol = 0.0;
+        if (vec) {
+            double* Zj = a.Z + (size_t)j * a.ldv;
+            for (int i = threadIdx.x; i < len; i += 256) {
+                ws[i] = a.w[c0 + i];
+                Zj[c0 + i] = a.z[c0 + i];
+            }
+        } else {
+            g0 = a.g[(size_t)s * m1 + j];
+            tol = a.tol_s[s];
+            for (int i = lane; i < j; i += 32) {
+                s_cs[i] = a.csv[(size_t)s * a.m + i];
+                s_sn[i] = a.snv[(size_t)s * a.m + i];
+            }
+        }
+        __syncthreads();
+        const double* V = a.V + c0;  // the chunk's columns
+        double sq = 0.0, n1 = 0.0;
+        for (int pass = 0; pass < 2; ++pass) {
+            double* part = a.part + (size_t)pass * (m1 + 1) * a.nch;
+            if (vec) {
+                rows_sums(V, a.ldv, ws, 0, len, j, [&](int k, double t) { part[(size_t)k * a.nch + b] = t; });
+            } else if (pass) {  // |w|^2 as row j + 1
+                double t = 0.0;
+                for (int i = lane; i < len; i += 32) t = fma(ws[i], ws[i], t);
+                t = warp_sum(t);
+                if (lane == 0) part[(size_t)(j + 1) * a.nch + b] = t;
+            }
+            sys_barrier(a.sync + s, nb * (3 * it + pass + 1), a.flags);
+            if (vec) {
+                rows_sums(part, a.nch, nullptr, q0, q1, j, [&](int k, double t) {
+                    cf[k] = t;
+                    hc[k] = pass ? hc[k] + t : t;
+                });
+            } else if (pass) {
+                for (int q = q0 + lane; q < q1; q += 32) n1 += __ldcg(part + (size_t)(j + 1) * a.nch + q);
+                n1 = warp_sum(n1);
+            }
+            __syncthreads();
+            if (vec) {
+                sq = chunk_orth(V, a.ldv, ws, 0, len, j, cf, a.clen, sh);
+            } else if (pass) {
+                double c2 = 0.0;
+                for (int k = lane; k <= j; k += 32) c2 = fma(cf[k], cf[k], c2);
+                c2 = warp_sum(c2);
+                const double carry = rotate_warp(j, s_cs, s_sn, hc,
+                                                 first ? a.H + ((size_t)s * a.m + j) * m1 : nullptr);
+                if (lane == 0) {
+                    const bool exact = !(c2 < 1e-6 * n1);
+                    s_exact = exact;
+                    if (!exact) {
+                        const StepEnd e = step_end(carry, n1 - c2, g0, tol);
+                        s_inv = e.inv;
+                        if (first) step_store(e, s, j, a.m, a.H, a.csv, a.snv, a.g, a.active, a.kdone, a.inv);
+                    }
+                    red[0] = carry;
+                }
+            }
+            __syncthreads();
+        }
+        if (s_exact) {  // the same in every block of the system
+            const double carry = red[0];
+            __syncthreads();
+            double t = warp_sum(sq);
+            if (vec && lane == 0) red[threadIdx.x >> 5] = t;
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                t = red[0];
+                for (int q = 1; q < 8; ++q) t += red[q];
+                a.npart[b] = t;
+            }
+            sys_barrier(a.sync + s, nb * (3 * it + 3), a.flags);
+            if (!vec) {
+                t = 0.0;
+                for (int q = q0 + lane; q < q1; q += 32) t += __ldcg(a.npart + q);
+                t = warp_sum(t);
+                if (lane == 0) {
+                    const StepEnd e = step_end(carry, t, g0, tol);
+                    s_inv = e.inv;
+                    if (first) step_store(e, s, j, a.m, a.H, a.csv, a.snv, a.g, a.active, a.kdone, a.inv);
+                }
+            }
+            __syncthreads();
+        } else if (threadIdx.x == 0) {
+            sys_arrive(a.sync + s);  // the third count of the step
+        }
+        const double inv = s_inv;
+        double* Vn = a.V + (size_t)(j + 1) * a.ldv;
+        for (int i = threadIdx.x; i < len; i += kStepThreads) {
+            const double t = inv * ws[i];
+            Vn[c0 + i] = t;
+            a.vj[c0 + i] = t;
+        }
+    }
+    if (first && arrive_last(a.cnt, a.S, a.S)) loop_ctrl(a.c, a.active, a.kdone, a.S, a.hc, a.in_graph);
+}
+
+// xi_s = H_s(0:k, 0:k)^-1 g_s(0:k), k = kdone[s], a warp per system: back
+// substitution by columns, lane l holding entries l, l + 32, .. (restart <= 200).
+// One thread per system, a chain of loads and subtractions per entry, took
+// 30 to 150 us.
+__global__ void __launch_bounds__(128)
+k_hess_solve_sys(const double* __restrict__ H, const double* __restrict__ g, const int* __restrict__ kdone,
+                 double* __restrict__ xi, int S, int m) {
+    const int s = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (s >= S) return;
+    constexpr int E = 7;  // 7 x 32 >= 200 entries
     const int k = kdone[s], m1 = m + 1;
     const double* Hs = H + (size_t)s * m * m1;
     const double* gs = g + (size_t)s * m1;
     double* xs = xi + (size_t)s * m1;
-    for (int i = k - 1; i >= 0; --i) {
-        double a = gs[i];
-        for (int q = i + 1; q < k; ++q) a -= Hs[(size_t)q * m1 + i] * xs[q];
-        const double d = Hs[(size_t)i * m1 + i];
-        xs[i] = d != 0.0 ? a / d : 0.0;
+    double a[E], inv[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const int i = lane + 32 * e;
+        a[e] = i < k ? gs[i] : 0.0;
+        const double d = i < k ? Hs[(size_t)i * m1 + i] : 0.0;
+        inv[e] = d != 0.0 ? 1.0 / d : 0.0;
+    }
+#pragma unroll
+    for (int eo = E - 1; eo >= 0; --eo) {
+        if (32 * eo >= k) continue;
+        for (int l = min(31, k - 1 - 32 * eo); l >= 0; --l) {  // column c = 32 eo + l
+            const double* col = Hs + (size_t)(32 * eo + l) * m1;
+            const double x = __shfl_sync(0xffffffffu, a[eo] * inv[eo], l);
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+                if (e < eo || (e == eo && lane < l)) a[e] = fma(-x, col[lane + 32 * e], a[e]);
+        }
+        if (lane + 32 * eo < k) xs[lane + 32 * eo] = a[eo] * inv[eo];
     }
 }
 
@@ -1004,7 +1334,7 @@ static void read_scal(am_handle* h, int count) {
 // per-system 2-norms of v into out (S doubles, device)
 static void sys_norms(am_handle* h, const double* v, double* out) {
     k_chunk_sq<<<h->nchunks, 256, 0, h->stream>>>(v, h->d_chunk_start, h->d_chunk_end, h->d_npart);
-    k_sys_norm<<<nblk(h->S, 128), 128, 0, h->stream>>>(h->d_npart, h->d_sys_chunk_off, h->S, out);
+    k_sys_norm<<<nblk(h->S, 4), 128, 0, h->stream>>>(h->d_npart, h->d_sys_chunk_off, h->S, out);
     count_launch(2);
 }
 
@@ -1013,7 +1343,7 @@ static void sys_norms(am_handle* h, const double* v, double* out) {
 static void sys_residual(am_handle* h, const double* b, const double* x, double* r, double* out, int mode) {
     op_apply(h, x, h->d_w, mode);
     k_chunk_resid<<<h->nchunks, 256, 0, h->stream>>>(b, h->d_w, r, h->d_chunk_start, h->d_chunk_end, h->d_npart);
-    k_sys_norm<<<nblk(h->S, 128), 128, 0, h->stream>>>(h->d_npart, h->d_sys_chunk_off, h->S, out);
+    k_sys_norm<<<nblk(h->S, 4), 128, 0, h->stream>>>(h->d_npart, h->d_sys_chunk_off, h->S, out);
     count_launch(2);
 }
 
@@ -1085,20 +1415,51 @@ static void issue_arnoldi_step(am_handle* h, bool fp64, cudaGraphConditionalHand
     pc_apply(h, h->d_vj, h->d_zj);  // vj = V[j], written with V[j]
     // the input of a stopped system is zero: its product skips the pairs
     op_apply(h, h->d_zj, h->d_w, fp64, S > 1 ? h->d_active : nullptr);
+    if (h->step_fused) {
+        const StepArgs a{h->d_V, ldv, h->d_w, h->d_zj, h->d_Z, h->d_vj, static_cast<const int4*>(h->d_chunk_info),
+                         h->d_sys_chunk_off, h->d_part, h->d_npart, nch, m, S, h->chunk_len,
+                         h->d_Hs, h->d_css, h->d_sns, h->d_gs, h->d_active, h->d_kdone, h->d_tol_s, h->d_inv_s,
+                         h->d_step_sync, h->d_arn_cnt, h->d_flags, h->d_ctrl, hc, in_graph ? 1 : 0};
+        cudaLaunchConfig_t lc = {};
+        cudaLaunchAttribute at[2];
+        at[0].id = cudaLaunchAttributeCooperative;
+        at[0].val.cooperative = 1;
+        at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[1].val.programmaticStreamSerializationAllowed = 1;
+        lc.gridDim = dim3(nch);
+        lc.blockDim = dim3(kStepThreads);
+        lc.stream = s;
+        lc.attrs = at;
+        lc.numAttrs = 2;
+        cudaLaunchKernelEx(&lc, k_arn_step, a);
+        count_launch();
+        return;
+    }
     launch_dep(k_arn_dots, dim3(nch), dim3(ct), 0, s, h->d_V, ldv, h->d_w, h->d_zj, h->d_Z, h->d_chunk_start,
                h->d_chunk_end, h->d_sys_of_elem, h->d_sys_chunk_off, h->d_part, nch, m1, h->d_coefs, h->d_hcols,
                h->d_arn_cnt, h->d_ctrl);
     launch_dep(k_arn_orth_dots, dim3(nch), dim3(ct), 0, s, h->d_V, ldv, h->d_w, h->d_chunk_start, h->d_chunk_end,
                h->d_sys_of_elem, h->d_sys_chunk_off, h->chunk_len, h->d_part, nch, m1, h->d_coefs, h->d_hcols,
                h->d_arn_cnt, h->d_ctrl);
-    launch_dep(k_arn_orth_finish, dim3(nch), dim3(ct), 0, s, h->d_V, ldv, h->d_w, h->d_chunk_start, h->d_chunk_end,
-               h->d_sys_of_elem, h->d_sys_chunk_off, h->chunk_len, h->d_npart, m1, h->d_coefs, h->d_hcols,
-               h->d_arn_cnt, S, m, h->d_Hs, h->d_css, h->d_sns, h->d_gs, h->d_active, h->d_kdone, h->d_tol_s,
-               h->d_inv_s, h->d_ctrl, hc, in_graph ? 1 : 0);
+    launch_dep(k_arn_orth_finish, dim3(nch + S), dim3(ct), 0, s, h->d_V, ldv, h->d_w, h->d_chunk_start,
+               h->d_chunk_end, h->d_sys_of_elem, h->d_sys_chunk_off, h->chunk_len, h->d_npart, nch, m1, h->d_coefs,
+               h->d_hcols, h->d_arn_cnt, S, m, h->d_Hs, h->d_css, h->d_sns, h->d_gs, h->d_carry, h->d_active,
+               h->d_kdone, h->d_tol_s, h->d_inv_s, h->d_ctrl, hc, in_graph ? 1 : 0);
     // j has advanced: V[j] = w / |w_s| and the next step's input
     launch_dep(k_next_basis, dim3(nb), dim3(256), 0, s, h->d_w, h->d_V, ldv, n, h->d_sys_of_elem, h->d_inv_s,
                h->d_ctrl, h->d_vj, 1);
     count_launch(4);
+}
+
+// The whole step in one kernel where its blocks are all resident (two of 256
+// threads per SM at most, so that the waits are short) and a system's partial
+// sums are few enough for every block to add them
+bool step_fits(const am_handle* h, const int* chunk_off) {
+    int per = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_arn_step, kStepThreads, 0) != cudaSuccess) return false;
+    int most = 0;
+    for (int s = 0; s < h->S; ++s) most = std::max(most, chunk_off[s + 1] - chunk_off[s]);
+    return h->nchunks <= std::min(per, 4) * num_sms() && most <= 160;
 }
 
 // The graph of one Arnoldi cycle: a WHILE node whose body is one step,
@@ -1180,7 +1541,7 @@ static int gmres(am_handle* h, const double* rhs, double* x, double tol, bool fp
     while (true) {
         sys_residual(h, rhs, x, h->d_V, h->d_beta_s, fp64);
         k_cycle_init<<<1, 256, 0, s>>>(S, m, tol, h->d_beta_s, h->d_bnorm_s, h->d_active, h->d_inv_s, h->d_gs,
-                                       h->d_kdone, h->d_tol_s, h->d_scal);
+                                       h->d_kdone, h->d_tol_s, h->d_scal, h->d_flags);
         count_launch();
         read_scal(h, 2);
         *rel = h->h_scal[0];
@@ -1191,6 +1552,7 @@ static int gmres(am_handle* h, const double* rhs, double* x, double tol, bool fp
         ++*cycles;
         k_scale_sys<<<nb, 256, 0, s>>>(h->d_V, n, h->d_sys_of_elem, h->d_inv_s, h->d_vj);
         k_ctrl_init<<<1, 1, 0, s>>>(h->d_ctrl, budget - it, m, 0.0);
+        cudaMemsetAsync(h->d_step_sync, 0, S * sizeof(int), s);
         count_launch(2);
         if (use_graph) {
             cudaGraphLaunch(h->gexec[gi], s);
@@ -1206,7 +1568,7 @@ static int gmres(am_handle* h, const double* rhs, double* x, double tol, bool fp
             } while (!h->h_ctrl->stop);
         }
         it += h->h_ctrl->it;
-        k_hess_solve_sys<<<nblk(S, 128), 128, 0, s>>>(h->d_Hs, h->d_gs, h->d_kdone, h->d_xis, S, m);
+        k_hess_solve_sys<<<nblk(S, 4), 128, 0, s>>>(h->d_Hs, h->d_gs, h->d_kdone, h->d_xis, S, m);
         k_combine_sys<<<nb, 256, 0, s>>>(h->d_Z, ldv, h->d_xis, h->d_kdone, h->d_sys_of_elem, n, m1, h->d_t);
         k_axpy<<<nb, 256, 0, s>>>(x, h->d_t, n, 1.0);
         count_launch(3);
@@ -1290,7 +1652,7 @@ int solve(am_handle* h, am_step_stats* st) {
             }
             accurate = res64 && !updated;
             k_cycle_init<<<1, 256, 0, s>>>(h->S, h->restart, tol, be_out, bn_out, h->d_active,
-                                           h->d_inv_s, h->d_gs, h->d_kdone, h->d_tol_s, h->d_scal);
+                                           h->d_inv_s, h->d_gs, h->d_kdone, h->d_tol_s, h->d_scal, h->d_flags);
             count_launch();
             if (!res64) {
                 k_sys_minrel<<<1, 256, 0, s>>>(h->S, be_out, bn_out, h->d_scal + 2);
@@ -1301,7 +1663,7 @@ int solve(am_handle* h, am_step_stats* st) {
                     accurate = true;
                     sys_residual(h, h->d_b, h->d_x, h->d_rir, be_out, kOpDF);
                     k_cycle_init<<<1, 256, 0, s>>>(h->S, h->restart, tol, be_out, bn_out, h->d_active,
-                                                   h->d_inv_s, h->d_gs, h->d_kdone, h->d_tol_s, h->d_scal);
+                                                   h->d_inv_s, h->d_gs, h->d_kdone, h->d_tol_s, h->d_scal, h->d_flags);
                     count_launch();
                 }
             }
@@ -1347,7 +1709,7 @@ int solve(am_handle* h, am_step_stats* st) {
         }
     }
     if (h->P) {
-        k_constraint_residual<<<1, 256, 0, h->stream>>>(h->Nb, h->M, h->P, h->d_bp, h->d_bq, h->d_lp,
+        k_constraint_residual<<<1, 1024, 0, h->stream>>>(h->Nb, h->M, h->P, h->d_bp, h->d_bq, h->d_lp,
                                                         h->d_lq, h->d_B, h->d_x, h->d_scal, 6);
         count_launch();
         read_scal(h, 7);
@@ -1358,6 +1720,10 @@ int solve(am_handle* h, am_step_stats* st) {
     st->iterations = it;
     st->restarts = cycles;
     st->rel_residual = rel;
+    if (!(rel == rel) && (take_flags(h) & kFlagStepWait)) {
+        h->err = "a wait of the Arnoldi step ran out";
+        return AM_ERR_CUDA;
+    }
     return (rel <= tol) ? AM_OK : AM_ERR_NOT_CONVERGED;
 }
 

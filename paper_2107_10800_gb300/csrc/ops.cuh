@@ -8,6 +8,7 @@ namespace am {
 constexpr int kFlagWall = 1;        // a blob centre at or below height a
 constexpr int kFlagSingular = 2;    // a body block of M or N~ not SPD
 constexpr int kFlagCorrection = 4;  // correction normal equations not SPD
+constexpr int kFlagStepWait = 1 << 9;  // a wait of the fused Arnoldi step ran out
 constexpr int kFlagTensor = 1 << 8; // a tensor-core (tcgen05) wait timed out (tc_gemm.cuh)
 // Bound on the relative error of the mixed mobility product, |(M32 - M) l|
 // <= kMixedProductError |M32 l| (20 times the largest measured, 4.7e-7 at
@@ -37,6 +38,9 @@ void combine_vectors(am_handle* h, double* x, const double* const* v, const doub
 // Solve A x = b (d_b, d_x in the handle; d_x holds the initial guess).
 // Returns AM_OK or AM_ERR_NOT_CONVERGED; fills iteration fields of st.
 int solve(am_handle* h, am_step_stats* st);
+// Whether the Arnoldi step runs as one kernel (chunk_off: first chunk of each
+// system, S + 1 values)
+bool step_fits(const am_handle* h, const int* chunk_off);
 // Euler update + reconstruction + correction (Sec. 4.3) from the solution
 // in d_x; writes the new q, theta into the handle.
 int advance(am_handle* h, double dt, am_step_stats* st);
