@@ -100,8 +100,10 @@ bool host_inverse(std::vector<double>& A, int n) {
 
 // Order of the per-body or per-articulated-body preconditioner builds:
 // matrices of at most two 32-row tiles (rows[i] <= 64) first, one CTA each,
-// then the larger ones, built by clusters of cs CTAs: cs doubles (up to 8)
-// while the larger ones' clusters still fit twice the SM count.
+// then the larger ones, built by clusters of cs CTAs (1, 2, 4 or 8).  The
+// builds are bound by the SMs' arithmetic, so cs is the one that loads the
+// busiest SM least, in matrices: ceil(n cs / SMs) / cs, and a few percent more
+// for each doubling (every CTA factors the diagonal tiles).
 void split_for_build(const std::vector<int>& rows, std::vector<int>& list, int& n_small, int& cs) {
     const int n = (int)rows.size();
     list.clear();
@@ -110,9 +112,13 @@ void split_for_build(const std::vector<int>& rows, std::vector<int>& list, int& 
     n_small = (int)list.size();
     for (int i = 0; i < n; ++i)
         if (rows[i] > 2 * 32) list.push_back(i);
-    const long long large = n - n_small;
+    const long long large = n - n_small, sms = am::num_sms();
     cs = 1;
-    while (cs < 8 && large > 0 && large * cs * 2 <= 2LL * am::num_sms()) cs *= 2;
+    double best = 1e300;
+    for (int c = 1, d = 0; c <= 8 && large > 0; c *= 2, ++d) {
+        const double load = (double)((large * c + sms - 1) / sms) / c * (1.0 + 0.03 * d);
+        if (load < best) { best = load; cs = c; }
+    }
 }
 
 void free_links(am_handle* h) {
