@@ -9,6 +9,26 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
+// The sums over the warp of U values per lane (U = 1, 2, 4 or 8): the sum of
+// a[u] is returned in lanes u 32/U .. (u + 1) 32/U - 1.  Halves are exchanged
+// while several values are left, so U sums take U - 1 + 5 - log2 U additions
+// instead of 5 U; an FP64 warp instruction costs 16 cycles of its SM.
+template <int U>
+__device__ __forceinline__ double warp_sums(double* a, int lane) {
+    int off = 16;
+#pragma unroll
+    for (int n = U / 2; n >= 1; n /= 2, off /= 2) {
+        const bool up = lane & off;
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+            const double send = up ? a[i] : a[i + n], keep = up ? a[i + n] : a[i];
+            a[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+        }
+    }
+    for (; off >= 1; off /= 2) a[0] += __shfl_xor_sync(0xffffffffu, a[0], off);
+    return a[0];
+}
+
 // Sum over the block; every thread gets the result.  sh: >= 33 doubles.
 __device__ __forceinline__ double block_sum(double v, double* sh) {
     v = warp_sum(v);

@@ -764,26 +764,6 @@ __device__ void loop_ctrl(ArnoldiCtrl* c, int* __restrict__ active, int* __restr
 // arithmetic and its order are those of separate dot, coefficient,
 // orthogonalisation, norm and step-end kernels.
 
-// The sums over the warp of U values per lane (U = 1, 2, 4 or 8): the sum of
-// a[u] is returned in lanes u 32/U .. (u + 1) 32/U - 1.  Halves are exchanged
-// while several values are left, so U sums take U - 1 + 5 - log2 U additions
-// instead of 5 U; an FP64 warp instruction costs 16 cycles of its SM.
-template <int U>
-__device__ __forceinline__ double warp_sums(double* a, int lane) {
-    int off = 16;
-#pragma unroll
-    for (int n = U / 2; n >= 1; n /= 2, off /= 2) {
-        const bool up = lane & off;
-#pragma unroll
-        for (int i = 0; i < n; ++i) {
-            const double send = up ? a[i] : a[i + n], keep = up ? a[i + n] : a[i];
-            a[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
-        }
-    }
-    for (; off >= 1; off /= 2) a[0] += __shfl_xor_sync(0xffffffffu, a[0], off);
-    return a[0];
-}
-
 // Sums over i in [i0, i1) of x_k[i] y[i], x_k = x + k ld, k <= j, given to
 // out(k, sum): U consecutive k per warp at a time, their loads in flight
 // together (a warp per k waited for every load and reduction in turn).  y NULL:

@@ -45,6 +45,7 @@
 #include <vector>
 
 #include "am_internal.cuh"
+#include "dev_util.cuh"
 #include "ops.cuh"
 #include "rpy_pair.cuh"
 
@@ -90,6 +91,8 @@ struct PeriodicPlan {
     int* d_code = nullptr;                  // per pair: neighbour cell << 26 | source sorted index
     double4_32a* d_rprev = nullptr;         // positions of the last binning
     int* d_moved = nullptr;                 // set when a blob moved since d_rprev
+    double* d_win = nullptr;                // FP64 window weights of the pose (Nb x 3 x P)
+    int* d_win0 = nullptr;                  // first grid point per axis (Nb x 3)
     bool valid = false;  // pair blocks of the current pose are in place
 };
 
@@ -649,17 +652,164 @@ k_per_gather(int Nb, SpreadGeom g, const double4_32a* __restrict__ spos, const i
     }
 }
 
+// ---- FP64 grid transfer: a warp per blob --------------------------------------
+// GB300 issues an FP64 warp instruction every 16 cycles per SM, so both
+// transfers are bound by how many of them a blob takes.  The lanes own the
+// blob's P^2 grid columns (x fastest: neighbouring lanes on neighbouring grid
+// points) in ceil(P^2 / 32) rounds and walk z; the window weights, whose
+// exponentials cost as much as a fifth of the transfer, are formed once per
+// pose (k_per_window).  Per blob at P = 11 the gather takes about 150 FP64
+// warp instructions for the field and 9 per 32 real-space pairs; lanes on one
+// column row and two blobs side by side took 240 and 9 per 22, and 70 for the
+// weights.
+
+// win[3 P p + d P + l]: weight of grid point i0 + l of axis d for the blob at
+// sorted position p, win0[3 p + d] = i0 wrapped into [0, M)
+__global__ void k_per_window(int Nb, SpreadGeom g, const double4_32a* __restrict__ spos, double* __restrict__ win,
+                             int* __restrict__ win0) {
+    const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const int per = 3 * g.P;
+    if (t >= (long long)Nb * per) return;
+    const int p = (int)(t / per), q = (int)(t % per), d = q / g.P, l = q % g.P;
+    const double4_32a r = spos[p];
+    const double x = d == 0 ? r.x : d == 1 ? r.y : r.z;
+    int idx;
+    double w;
+    axis_weight(x, d, g, l, idx, w);
+    win[t] = w;
+    if (l == 0) win0[3 * (size_t)p + d] = idx;
+}
+
+// The lane's columns of one blob: weights wx wy and offsets iy Mx + ix (round
+// r: column lane + 32 r), and the blob's z weights and first layer.
+template <int P>
+struct BlobColumns {
+    static constexpr int R = (P * P + 31) / 32;
+    double wxy[R];
+    int off[R];
+    bool ok[R];
+    double wz;  // of layer `lane`
+    int iz0;
+    __device__ __forceinline__ BlobColumns(const SpreadGeom& g, const double* __restrict__ win,
+                                           const int* __restrict__ win0, int p, int lane) {
+        const double* w = win + (size_t)3 * P * p;
+        const int ix0 = win0[3 * (size_t)p], iy0 = win0[3 * (size_t)p + 1];
+        iz0 = win0[3 * (size_t)p + 2];
+        wz = lane < P ? w[2 * P + lane] : 0.0;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int c = lane + 32 * r, cy = c / P, cx = c - cy * P;
+            ok[r] = c < P * P;
+            int ix = ix0 + cx, iy = iy0 + cy;
+            if (ix >= g.M[0]) ix -= g.M[0];
+            if (iy >= g.M[1]) iy -= g.M[1];
+            off[r] = ok[r] ? iy * g.M[0] + ix : 0;
+            wxy[r] = ok[r] ? w[cx] * w[P + cy] : 0.0;
+        }
+    }
+    __device__ __forceinline__ long long layer(const SpreadGeom& g, int pz) const {
+        int iz = iz0 + pz;
+        if (iz >= g.M[2]) iz -= g.M[2];
+        return (long long)iz * g.M[1] * g.M[0];
+    }
+};
+
+template <int P>
+__global__ void __launch_bounds__(128)
+k_per_spread64(int Nb, SpreadGeom g, const double* __restrict__ win, const int* __restrict__ win0,
+               const int* __restrict__ order, const double* __restrict__ lam, double* __restrict__ grid,
+               long long ngrid) {
+    const int p = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    if (p >= Nb) return;
+    const BlobColumns<P> b(g, win, win0, p, lane);
+    const double* f = lam + 3 * (size_t)order[p];
+    const double fx = f[0], fy = f[1], fz = f[2];
+    constexpr int R = BlobColumns<P>::R;
+    double ax[R], ay[R], az[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) { ax[r] = b.wxy[r] * fx; ay[r] = b.wxy[r] * fy; az[r] = b.wxy[r] * fz; }
+#pragma unroll 1
+    for (int pz = 0; pz < P; ++pz) {
+        const double wz = __shfl_sync(0xffffffffu, b.wz, pz);
+        double* q = grid + b.layer(g, pz);
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            if (b.ok[r]) {
+                atomicAdd(q + b.off[r], wz * ax[r]);
+                atomicAdd(q + ngrid + b.off[r], wz * ay[r]);
+                atomicAdd(q + 2 * ngrid + b.off[r], wz * az[r]);
+            }
+    }
+}
+
+// u_i = the real-space row of the blob plus the interpolated field; sums in a
+// fixed order (lane-strided rows and columns, then the warp's reduction)
+template <int P>
+__global__ void __launch_bounds__(128)
+k_per_gather64(int Nb, SpreadGeom g, const double* __restrict__ win, const int* __restrict__ win0,
+               const int* __restrict__ order, const long long* __restrict__ row, const int* __restrict__ nbr,
+               const double* __restrict__ blk, long long cap, const double* __restrict__ lam,
+               const double* __restrict__ grid, long long ngrid, double* __restrict__ out) {
+    const int p = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    if (p >= Nb) return;
+    double u[4] = {0.0, 0.0, 0.0, 0.0};
+    const long long e1 = row[p + 1];
+#pragma unroll 2
+    for (long long e = row[p] + lane; e < e1; e += 32) {
+        const double* l = lam + 3 * (size_t)nbr[e];
+        const double lx = l[0], ly = l[1], lz = l[2];
+        const double m00 = blk[e], m01 = blk[cap + e], m02 = blk[2 * cap + e];
+        const double m11 = blk[3 * cap + e], m12 = blk[4 * cap + e], m22 = blk[5 * cap + e];
+        u[0] = fma(m00, lx, fma(m01, ly, fma(m02, lz, u[0])));
+        u[1] = fma(m01, lx, fma(m11, ly, fma(m12, lz, u[1])));
+        u[2] = fma(m02, lx, fma(m12, ly, fma(m22, lz, u[2])));
+    }
+    const BlobColumns<P> b(g, win, win0, p, lane);
+    constexpr int R = BlobColumns<P>::R;
+    double vx[R], vy[R], vz[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) vx[r] = vy[r] = vz[r] = 0.0;
+#pragma unroll 1
+    for (int pz = 0; pz < P; ++pz) {
+        const double wz = __shfl_sync(0xffffffffu, b.wz, pz);
+        const double* q = grid + b.layer(g, pz);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            vx[r] = fma(wz, __ldg(q + b.off[r]), vx[r]);
+            vy[r] = fma(wz, __ldg(q + ngrid + b.off[r]), vy[r]);
+            vz[r] = fma(wz, __ldg(q + 2 * ngrid + b.off[r]), vz[r]);
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        u[0] = fma(b.wxy[r], vx[r], u[0]);
+        u[1] = fma(b.wxy[r], vy[r], u[1]);
+        u[2] = fma(b.wxy[r], vz[r], u[2]);
+    }
+    const double t = warp_sums<4>(u, lane);  // of u[c] in lanes 8 c .. 8 c + 7
+    if (lane % 8 == 0 && lane < 24) out[3 * (size_t)order[p] + lane / 8] = t;
+}
+
 template <class T, int P>
 void launch_window(int Nb, const SpreadGeom& g, const PeriodicPlan* p, const Wave& w, const T* blk,
                    const double* lam, double* out, bool spread, cudaStream_t s) {
-    const int per_block = 8 * (32 / P);  // blobs per 256-thread block (lane_map)
-    const int nb = (Nb + per_block - 1) / per_block;
     T* grid = static_cast<T*>(w.grid);
-    if (spread)
-        k_per_spread<T, P><<<nb, 256, 0, s>>>(Nb, g, p->d_spos, p->d_order, lam, grid, w.ngrid);
-    else
-        k_per_gather<T, P><<<nb, 256, 0, s>>>(Nb, g, p->d_spos, p->d_order, p->d_row, p->d_nbr, blk, p->cap, lam,
-                                              grid, w.ngrid, out);
+    if constexpr (sizeof(T) == 8) {
+        const int nb = (Nb + 3) / 4;  // four warps a block, one blob each
+        if (spread)
+            k_per_spread64<P><<<nb, 128, 0, s>>>(Nb, g, p->d_win, p->d_win0, p->d_order, lam, grid, w.ngrid);
+        else
+            k_per_gather64<P><<<nb, 128, 0, s>>>(Nb, g, p->d_win, p->d_win0, p->d_order, p->d_row, p->d_nbr, blk,
+                                                 p->cap, lam, grid, w.ngrid, out);
+    } else {
+        const int per_block = 8 * (32 / P);  // blobs per 256-thread block (lane_map)
+        const int nb = (Nb + per_block - 1) / per_block;
+        if (spread)
+            k_per_spread<T, P><<<nb, 256, 0, s>>>(Nb, g, p->d_spos, p->d_order, lam, grid, w.ngrid);
+        else
+            k_per_gather<T, P><<<nb, 256, 0, s>>>(Nb, g, p->d_spos, p->d_order, p->d_row, p->d_nbr, blk, p->cap, lam,
+                                                  grid, w.ngrid, out);
+    }
 }
 
 // window widths 4 .. 16 (tolerances 1e-3 .. 1e-15)
@@ -739,7 +889,7 @@ void free_plan(PeriodicPlan* p) {
     free_wave(p->w32);
     void* ptrs[] = {p->d_tab,  p->d_cell_start, p->d_cell_fill, p->d_cell_of, p->d_order, p->d_spos,
                     p->d_sposf, p->d_row,     p->d_nbr,       p->d_blk,     p->d_scan,  p->d_code,
-                    p->d_rprev, p->d_moved,   p->d_blk32};
+                    p->d_rprev, p->d_moved,   p->d_blk32,     p->d_win,   p->d_win0};
     for (void* q : ptrs)
         if (q) cudaFree(q);
     delete p;
@@ -951,7 +1101,8 @@ int periodic_setup(am_handle* h) {
     bool ok = dalloc(&p->d_tab, p->ntab) && dalloc(&p->d_cell_start, p->ncell + 1) &&
               dalloc(&p->d_cell_fill, p->ncell) && dalloc(&p->d_cell_of, Nb) && dalloc(&p->d_order, Nb) &&
               dalloc(&p->d_spos, Nb) && dalloc(&p->d_sposf, Nb) && dalloc(&p->d_row, Nb + 1) &&
-              dalloc(&p->d_scan, nscan) && dalloc(&p->d_rprev, Nb) && dalloc(&p->d_moved, 1);
+              dalloc(&p->d_scan, nscan) && dalloc(&p->d_rprev, Nb) && dalloc(&p->d_moved, 1) &&
+              dalloc(&p->d_win, (size_t)3 * P * Nb) && dalloc(&p->d_win0, 3 * (size_t)Nb);
     if (!ok) {
         cudaGetLastError();
         h->err = "periodic mobility: device allocation failed";
@@ -1084,8 +1235,10 @@ int periodic_bin(am_handle* h) {
         k_per_blk32<<<8 * num_sms(), 256, 0, s>>>(p->d_blk, p->d_blk32, p->cap, nnz);
         count_launch();
     }
+    k_per_window<<<(int)(((long long)Nb * 3 * p->w64.P + 255) / 256), 256, 0, s>>>(Nb, spread_geom(p->w64), p->d_spos,
+                                                                                   p->d_win, p->d_win0);
     cudaMemcpyAsync(p->d_rprev, h->d_r4, Nb * sizeof(double4_32a), cudaMemcpyDeviceToDevice, s);
-    count_launch(3);
+    count_launch(4);
     p->nnz = nnz;
     h->per_nnz = nnz;
     if (cudaGetLastError() != cudaSuccess) {
