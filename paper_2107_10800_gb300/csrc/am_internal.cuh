@@ -270,6 +270,7 @@ struct am_handle {
     int* d_perm = nullptr; long long* d_perm_off = nullptr;
     double *d_pc_w = nullptr, *d_pc_Uhat = nullptr;
     bool pc_valid = false;
+    int pc_small_cs = 0;  // cluster size of the one-launch apply (0: three kernels)
 
     // device: solver vectors
     double *d_b = nullptr, *d_x = nullptr, *d_t = nullptr,

@@ -339,7 +339,11 @@ k_pca_build(const int* __restrict__ asm_list, const int* __restrict__ asm_link_o
 
 // ------------------------------------------------------------- apply ---
 // Work item it: body pcw_body[it], rows pcw_chunk[it]*32 .. +32.  128 threads:
-// lane = row within the chunk, warp = quarter of the columns.
+// lane = row within the chunk, warp = quarter of the columns.  r1 is staged in
+// shared memory in the storage precision: converting it at every use is FP64
+// work (16 cycles of the SM per warp instruction) and was half of the time in
+// FP32 (36,000 blobs, bodies of up to 600 rows: 105 us, now 45; the 144 MB of
+// factors take 22 at the copy rate).
 template <class T>
 __global__ void __launch_bounds__(128)
 k_pc_ap1(const int* __restrict__ pcw_body, const int* __restrict__ pcw_chunk,
@@ -348,67 +352,69 @@ k_pc_ap1(const int* __restrict__ pcw_body, const int* __restrict__ pcw_chunk,
          double* __restrict__ w, double* __restrict__ ytp, int Nb, const int* __restrict__ pcw_off,
          const double* __restrict__ Nt, double* __restrict__ Uhat, int* __restrict__ body_cnt) {
     dep_wait();
+    constexpr int kStage = 1024;  // entries of r1 staged at a time
+    __shared__ T rs[kStage];
     __shared__ double red[4][kRows];
-    __shared__ double yred[4][6];
     const int it = blockIdx.x;
     const int b = pcw_body[it];
     const int i0 = blob_off[b];
     const int m = 3 * (blob_off[b + 1] - i0);
     const int lane = threadIdx.x & 31, part = threadIdx.x >> 5;
     const int row = pcw_chunk[it] * kRows + lane;
-    const T* A = minv + moff[b];
     const double* r1 = r + 3 * (size_t)i0;
-    double s = 0.0;
-    if (row < m) {
-        // eight independent loads in flight per thread, four partial sums
-        T acc[4] = {0, 0, 0, 0};
-        int k = part;
-        for (; k + 28 < m; k += 32) {
-            T av[8], rv[8];
+    // eight independent loads in flight per thread, four partial sums
+    T acc[4] = {0, 0, 0, 0};
+    for (int c0 = 0; c0 < m; c0 += kStage) {
+        const int cn = min(kStage, m - c0);
+        __syncthreads();
+        for (int k = threadIdx.x; k < cn; k += blockDim.x) rs[k] = (T)r1[c0 + k];
+        __syncthreads();
+        if (row < m) {
+            const T* A = minv + moff[b] + (size_t)c0 * m + row;
+            int k = part;
+            for (; k + 28 < cn; k += 32) {
+                T av[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                av[u] = A[(size_t)(k + 4 * u) * m + row];
-                rv[u] = (T)r1[k + 4 * u];
+                for (int u = 0; u < 8; ++u) av[u] = A[(size_t)(k + 4 * u) * m];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) acc[u & 3] = fma(av[u], rs[k + 4 * u], acc[u & 3]);
             }
+            for (; k < cn; k += 4) acc[0] = fma(A[(size_t)k * m], rs[k], acc[0]);
+        }
+    }
+    red[part][lane] = (double)((acc[0] + acc[1]) + (acc[2] + acc[3]));
+    if (part == 3) {  // partial Y^T r1 over this chunk's rows
+        double yv[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+        if (row < m) {
+            const T* Yr = Y + 18 * (size_t)i0 + 6 * (size_t)row;
+            const double ri = r1[row];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) acc[u & 3] = fma(av[u], rv[u], acc[u & 3]);
+            for (int c = 0; c < 6; ++c) yv[c] = (double)Yr[c] * ri;
         }
-        for (; k < m; k += 4) acc[0] = fma(A[(size_t)k * m + row], (T)r1[k], acc[0]);
-        s = (double)((acc[0] + acc[1]) + (acc[2] + acc[3]));
+        const double t = warp_sums<8>(yv, lane);  // of column c in lanes 4 c .. 4 c + 3
+        if (lane % 4 == 0 && lane < 24) ytp[6 * (size_t)it + lane / 4] = t;
     }
-    red[part][lane] = s;
-    // partial Y^T r1 over this chunk's rows (warp `part` takes columns part, part+4)
-    double yv[6] = {0, 0, 0, 0, 0, 0};
-    if (part == 0 && row < m) {
-        const T* Yr = Y + 18 * (size_t)i0 + 6 * (size_t)row;
-        const double ri = r1[row];
-        for (int c = 0; c < 6; ++c) yv[c] = (double)Yr[c] * ri;
-    }
-    if (part == 0)
-        for (int c = 0; c < 6; ++c) {
-            const double t = warp_sum(yv[c]);
-            if (lane == 0) yred[0][c] = t;
-        }
     __syncthreads();
-    if (part == 0) {
-        if (row < m) w[3 * (size_t)i0 + row] = red[0][lane] + red[1][lane] + red[2][lane] + red[3][lane];
-        if (lane < 6) ytp[6 * (size_t)it + lane] = yred[0][lane];
-    }
-    // the body's last item: U^_b = N~_b (-r2_b - sum of the body's Y^T r1 partials)
+    if (part == 0 && row < m) w[3 * (size_t)i0 + row] = red[0][lane] + red[1][lane] + red[2][lane] + red[3][lane];
+    // the body's last item: U^_b = N~_b (-r2_b - sum of the body's Y^T r1
+    // partials): lane 6 g + c adds every fifth partial of column c
     if (arrive_last(body_cnt, b, pcw_off[b + 1] - pcw_off[b]) && part == 0) {
+        const int c = lane % 6, g = lane / 6;
         double v = 0.0;
-        if (lane < 6) {
-            v = -r[3 * (size_t)Nb + 6 * (size_t)b + lane];
-            for (int q = pcw_off[b]; q < pcw_off[b + 1]; ++q) v -= __ldcg(ytp + 6 * (size_t)q + lane);
-        }
+        if (g < 5)
+            for (int q = pcw_off[b] + g; q < pcw_off[b + 1]; q += 5) v += __ldcg(ytp + 6 * (size_t)q + c);
+        double s = 0.0;
+#pragma unroll
+        for (int q = 0; q < 5; ++q) s += __shfl_sync(0xffffffffu, v, 6 * q + c);
+        v = lane < 6 ? -r[3 * (size_t)Nb + 6 * (size_t)b + lane] - s : 0.0;
         double vv[6];
 #pragma unroll
-        for (int c = 0; c < 6; ++c) vv[c] = __shfl_sync(0xffffffffu, v, c);
+        for (int q = 0; q < 6; ++q) vv[q] = __shfl_sync(0xffffffffu, v, q);
         if (lane < 6) {
             const double* N = Nt + 36 * (size_t)b + 6 * lane;
             double t = 0.0;
 #pragma unroll
-            for (int c = 0; c < 6; ++c) t += N[c] * vv[c];
+            for (int q = 0; q < 6; ++q) t += N[q] * vv[q];
             Uhat[6 * (size_t)b + lane] = t;
         }
     }
@@ -444,7 +450,7 @@ k_pc_ap2(int Nb, int M, const int* __restrict__ pca_asm, const int* __restrict__
     dep_wait();
     constexpr int kStage = 1024;  // entries of c staged in shared memory at a time
     __shared__ double red[4][kRows];
-    __shared__ double cs[kStage];
+    __shared__ T cs[kStage];
     const int it = blockIdx.x;
     const int a = pca_asm[it];
     const int L0 = asm_link_off[a];
@@ -465,9 +471,9 @@ k_pc_ap2(int Nb, int M, const int* __restrict__ pca_asm, const int* __restrict__
                 double wp[3], wq[3];
                 cross3(up + 3, lp + 3 * n, wp);
                 cross3(uq + 3, lq + 3 * n, wq);
-                cs[k] = r[3 * (size_t)Nb + 6 * (size_t)M + 3 * n + x] - (up[x] + wp[x] - uq[x] - wq[x]);
+                cs[k] = (T)(r[3 * (size_t)Nb + 6 * (size_t)M + 3 * n + x] - (up[x] + wp[x] - uq[x] - wq[x]));
             } else {
-                cs[k] = cbuf[3 * n + x];
+                cs[k] = (T)cbuf[3 * n + x];
             }
         }
         __syncthreads();
@@ -479,9 +485,9 @@ k_pc_ap2(int Nb, int M, const int* __restrict__ pca_asm, const int* __restrict__
 #pragma unroll
                 for (int u = 0; u < 8; ++u) gv[u] = Gc[(size_t)(k + 4 * u) * m];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) acc[u & 3] = fma(gv[u], (T)cs[k + 4 * u], acc[u & 3]);
+                for (int u = 0; u < 8; ++u) acc[u & 3] = fma(gv[u], cs[k + 4 * u], acc[u & 3]);
             }
-            for (; k < cn; k += 4) acc[0] = fma(Gc[(size_t)k * m], (T)cs[k], acc[0]);
+            for (; k < cn; k += 4) acc[0] = fma(Gc[(size_t)k * m], cs[k], acc[0]);
         }
     }
     const double s = row < m ? (double)((acc[0] + acc[1]) + (acc[2] + acc[3])) : 0.0;
@@ -509,7 +515,7 @@ k_pc_ap3(int Nb, int M, const int* __restrict__ pcw_body, const int* __restrict_
     if (threadIdx.x < 32) {
         // (C^T phi)_b: the body's link ends spread over the lanes of warp 0
         const int lane = threadIdx.x;
-        double f[6] = {0, 0, 0, 0, 0, 0};
+        double f[8] = {0, 0, 0, 0, 0, 0, 0, 0};
         for (int k = bl_off[b] + lane; k < bl_off[b + 1]; k += 32) {
             const int e = bl_idx[k];
             const int n = e >> 1;
@@ -520,13 +526,15 @@ k_pc_ap3(int Nb, int M, const int* __restrict__ pcw_body, const int* __restrict_
             cross3(l, ph, t);
             for (int x = 0; x < 3; ++x) { f[x] += sg * ph[x]; f[3 + x] += sg * t[x]; }
         }
+        const double fs = warp_sums<8>(f, lane);  // of component c in lanes 4 c .. 4 c + 3
+        double fc[6];
 #pragma unroll
-        for (int c = 0; c < 6; ++c) f[c] = warp_sum(f[c]);
+        for (int c = 0; c < 6; ++c) fc[c] = __shfl_sync(0xffffffffu, fs, 4 * c);
         if (lane < 6) {
             const double* N = Nt + 36 * (size_t)b + 6 * lane;
             double s = Uhat[6 * (size_t)b + lane];
 #pragma unroll
-            for (int c = 0; c < 6; ++c) s += N[c] * f[c];
+            for (int c = 0; c < 6; ++c) s += N[c] * fc[c];
             sU[lane] = s;
             if (pcw_chunk[it] == 0) z[3 * (size_t)Nb + 6 * (size_t)b + lane] = s;
         }
@@ -540,6 +548,171 @@ k_pc_ap3(int Nb, int M, const int* __restrict__ pcw_body, const int* __restrict_
         double s = w[3 * (size_t)i0 + row];
         for (int c = 0; c < 6; ++c) s = fma((double)Yr[c], sU[c], s);
         z[3 * (size_t)i0 + row] = s;
+    }
+}
+
+// The whole apply for handles of small articulated bodies (pc_small_fits): one
+// cluster per articulated body, a warp per body, one launch instead of three
+// (the problem is block-diagonal over articulated bodies).  With n the body's
+// rows (at most 64), lane l of the warp takes rows l and, when n > 32, the
+// remaining rows with several lanes sharing each: an FP64 warp instruction
+// costs 16 cycles of its SM however few lanes take part.  Every CTA forms c and
+// phi of its articulated body itself (at most 64 rows of G~), so the cluster
+// meets once.  Bound by chains of FP64 and L2 latency.  Measured, three kernels
+// against this one: 4 chains of 8 bodies of 12 blobs in FP64 18.3 us against
+// 15.8; 16 systems of 500 to 4,000 blobs in FP32 57 us
+// against 22.
+constexpr int kSmallRows = 64;
+template <class T>
+__global__ void __launch_bounds__(256)
+k_pc_small(int Nb, int M, const int* __restrict__ asm_body_off, const int* __restrict__ asm_body_idx,
+           const int* __restrict__ asm_link_off, const int* __restrict__ asm_link_idx,
+           const int* __restrict__ blob_off, const T* __restrict__ minv, const long long* __restrict__ moff,
+           const T* __restrict__ Y, const double* __restrict__ Nt, const T* __restrict__ G,
+           const long long* __restrict__ goff, const int* __restrict__ bp, const int* __restrict__ bq,
+           const double* __restrict__ lp, const double* __restrict__ lq, const int* __restrict__ bl_off,
+           const int* __restrict__ bl_idx, const int* __restrict__ link_local, const double* __restrict__ r,
+           double* __restrict__ w, double* __restrict__ Uhat, double* __restrict__ z) {
+    dep_wait();
+    __shared__ double cs[kSmallRows], phis[kSmallRows];
+    __shared__ T ct[kSmallRows];
+    __shared__ T red[8][kSmallRows];
+    const ClusterTeam team;
+    const int a = blockIdx.x / team.size();
+    const int B0 = asm_body_off[a], Ma = asm_body_off[a + 1] - B0;
+    const int L0 = asm_link_off ? asm_link_off[a] : 0, mg = asm_link_off ? 3 * (asm_link_off[a + 1] - L0) : 0;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int wg = team.rank() * 8 + wid, W = team.size() * 8;
+    // w = M~^-1 r1 and U^ = N~ (-r2 - Y^T r1)
+    for (int q = wg; q < Ma; q += W) {
+        const int b = asm_body_idx[B0 + q], i0 = blob_off[b], m = 3 * (blob_off[b + 1] - i0);
+        const double* r1 = r + 3 * (size_t)i0;
+        const T* A = minv + moff[b];
+        const double ra = lane < m ? r1[lane] : 0.0, rb = 32 + lane < m ? r1[32 + lane] : 0.0;
+        const T ta = (T)ra, tb = (T)rb;
+        T acc0 = 0, acc1 = 0;
+        for (int k = 0; k < m; k += 8) {  // rows 0 .. 31
+            T av[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) av[u] = k + u < m && lane < m ? A[(size_t)(k + u) * m + lane] : (T)0;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const T x = __shfl_sync(0xffffffffu, (k + u) & 32 ? tb : ta, (k + u) & 31);
+                if (k + u < m) {
+                    if (u & 1) acc1 = fma(av[u], x, acc1);
+                    else acc0 = fma(av[u], x, acc0);
+                }
+            }
+        }
+        if (lane < m) w[3 * (size_t)i0 + lane] = (double)(acc0 + acc1);
+        if (m > 32) {  // the remaining rows: `per` lanes on each column, 32 / per columns at a time
+            const int rest = m - 32;
+            int per = 1;
+            while (per < rest) per *= 2;
+            const int row = 32 + lane % per, k0 = lane / per, step = 32 / per;
+            T t = 0;
+#pragma unroll 4
+            for (int k = 0; k < m; k += step) {
+                const int kk = k + k0;
+                const T xa = __shfl_sync(0xffffffffu, ta, kk & 31), xb = __shfl_sync(0xffffffffu, tb, kk & 31);
+                if (kk < m && row < m) t = fma(A[(size_t)kk * m + row], kk & 32 ? xb : xa, t);
+            }
+            for (int o = per; o < 32; o *= 2) t += __shfl_xor_sync(0xffffffffu, t, o);
+            if (lane < rest) w[3 * (size_t)i0 + 32 + lane] = (double)t;
+        }
+        double yv[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+        if (lane < m) {
+            const T* Yr = Y + 18 * (size_t)i0 + 6 * lane;
+#pragma unroll
+            for (int c = 0; c < 6; ++c) yv[c] = (double)Yr[c] * ra;
+        }
+        if (32 + lane < m) {
+            const T* Yr = Y + 18 * (size_t)i0 + 6 * (32 + lane);
+#pragma unroll
+            for (int c = 0; c < 6; ++c) yv[c] = fma((double)Yr[c], rb, yv[c]);
+        }
+        const double ys = warp_sums<8>(yv, lane);  // of column c in lanes 4 c .. 4 c + 3
+        const double v = -(lane < 24 ? r[3 * (size_t)Nb + 6 * (size_t)b + lane / 4] : 0.0) - ys;
+        // U^ = N~ v: lane 4 c + g takes columns g and g + 4 of row c
+        const double* N = Nt + 36 * (size_t)b;
+        const int c = lane >> 2, g = lane & 3;
+        const double v0 = __shfl_sync(0xffffffffu, v, 4 * g), v1 = __shfl_sync(0xffffffffu, v, 4 * ((g + 4) % 6));
+        double t = c < 6 ? N[6 * c + g] * v0 : 0.0;
+        if (c < 6 && g < 2) t = fma(N[6 * c + g + 4], v1, t);
+        t += __shfl_xor_sync(0xffffffffu, t, 1);
+        t += __shfl_xor_sync(0xffffffffu, t, 2);
+        if (c < 6 && g == 0) Uhat[6 * (size_t)b + c] = t;
+    }
+    team.sync();
+    // c = r3 - C U^ and phi = G~ c
+    for (int k = threadIdx.x; k < mg; k += blockDim.x) {
+        const int n = asm_link_idx[L0 + k / 3], x = k % 3, x1 = x == 2 ? 0 : x + 1, x2 = x == 0 ? 2 : x - 1;
+        const double* up = Uhat + 6 * (size_t)bp[n];
+        const double* uq = Uhat + 6 * (size_t)bq[n];
+        const double *l1 = lp + 3 * (size_t)n, *l2 = lq + 3 * (size_t)n;
+        // component x of u_p + omega_p x l_p - u_q - omega_q x l_q
+        const double cp = __ldcg(up + x) + (__ldcg(up + 3 + x1) * l1[x2] - __ldcg(up + 3 + x2) * l1[x1]);
+        const double cq = __ldcg(uq + x) + (__ldcg(uq + 3 + x1) * l2[x2] - __ldcg(uq + 3 + x2) * l2[x1]);
+        cs[k] = r[3 * (size_t)Nb + 6 * (size_t)M + 3 * (size_t)n + x] - (cp - cq);
+        ct[k] = (T)cs[k];
+    }
+    __syncthreads();
+    if (mg) {
+        const T* Ga = G + goff[a];
+        for (int row = lane; row < mg; row += 32) {  // warp w: columns w, w + 8, ..
+            T t = 0;
+#pragma unroll 8
+            for (int k = wid; k < mg; k += 8) t = fma(Ga[(size_t)k * mg + row], ct[k], t);
+            red[wid][row] = t;
+        }
+        __syncthreads();
+        if (threadIdx.x < mg) {
+            double t = 0.0;
+            for (int q = 0; q < 8; ++q) t += (double)red[q][threadIdx.x];
+            phis[threadIdx.x] = t;
+            if (team.rank() == 0) {
+                const int n = asm_link_idx[L0 + threadIdx.x / 3];
+                z[3 * (size_t)Nb + 6 * (size_t)M + 3 * (size_t)n + threadIdx.x % 3] = t;
+            }
+        }
+        __syncthreads();
+    }
+    // U = U^ + N~ C^T phi; lambda = w + Y U
+    for (int q = wg; q < Ma; q += W) {
+        const int b = asm_body_idx[B0 + q], i0 = blob_off[b], m = 3 * (blob_off[b + 1] - i0);
+        double f[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+        if (mg)
+            for (int k = bl_off[b] + lane; k < bl_off[b + 1]; k += 32) {
+                const int e = bl_idx[k], n = e >> 1;
+                const double sg = (e & 1) ? -1.0 : 1.0;
+                const double* l = (e & 1) ? lq + 3 * (size_t)n : lp + 3 * (size_t)n;
+                const double* ph = phis + 3 * link_local[n];
+                const double p0 = sg * ph[0], p1 = sg * ph[1], p2 = sg * ph[2];
+                f[0] += p0; f[1] += p1; f[2] += p2;
+                f[3] = fma(l[1], p2, fma(-l[2], p1, f[3]));
+                f[4] = fma(l[2], p0, fma(-l[0], p2, f[4]));
+                f[5] = fma(l[0], p1, fma(-l[1], p0, f[5]));
+            }
+        const double fs = mg ? warp_sums<8>(f, lane) : 0.0;
+        const double* N = Nt + 36 * (size_t)b;
+        const int c = lane >> 2, g = lane & 3;
+        const double f0 = __shfl_sync(0xffffffffu, fs, 4 * g), f1 = __shfl_sync(0xffffffffu, fs, 4 * ((g + 4) % 6));
+        double t = c < 6 ? N[6 * c + g] * f0 : 0.0;
+        if (c < 6 && g < 2) t = fma(N[6 * c + g + 4], f1, t);
+        t += __shfl_xor_sync(0xffffffffu, t, 1);
+        t += __shfl_xor_sync(0xffffffffu, t, 2);
+        if (c < 6) t += __ldcg(Uhat + 6 * (size_t)b + c);
+        if (c < 6 && g == 0) z[3 * (size_t)Nb + 6 * (size_t)b + c] = t;
+        double u[6];
+#pragma unroll
+        for (int x = 0; x < 6; ++x) u[x] = __shfl_sync(0xffffffffu, t, 4 * x);
+        for (int row = lane; row < m; row += 32) {
+            const T* Yr = Y + 18 * (size_t)i0 + 6 * row;
+            double v = __ldcg(w + 3 * (size_t)i0 + row);
+#pragma unroll
+            for (int x = 0; x < 6; ++x) v = fma((double)Yr[x], u[x], v);
+            z[3 * (size_t)i0 + row] = v;
+        }
     }
 }
 
@@ -587,6 +760,21 @@ static void pca_build_t(am_handle* h, double tol) {
                     (const long long*)h->d_perm_off, h->d_G_rank, tol);
 }
 
+// Whether every articulated body is small enough for k_pc_small, and the
+// cluster size: a warp per body, as many CTAs as spread them over the SMs.  The
+// line at 64 rows is where a lane would get a third row and one warp would walk
+// more than 32 KB of factors; larger bodies keep a CTA per 32 rows.
+static int pc_small_size(const am_handle* h) {
+    if (h->sb || h->per || h->NA == 0) return 0;
+    if (3 * h->max_body_blobs > kSmallRows || (h->P && 3 * h->max_asm_links > kSmallRows)) return 0;
+    int most = 0;
+    for (int a = 0; a < h->NA; ++a) most = std::max(most, h->asm_body_off[a + 1] - h->asm_body_off[a]);
+    if (most > 64) return 0;
+    int cs = 1;
+    while (cs < 8 && cs < most && 2LL * cs * h->NA <= num_sms()) cs *= 2;
+    return cs;
+}
+
 template <class T>
 static void pc_build_t(am_handle* h, double tol) {
     cudaStream_t s = h->stream;
@@ -629,6 +817,7 @@ void pc_build(am_handle* h) {
     // arrival counts of the apply's per-body reductions (each completing
     // block zeroes its own; zeroed here as well, outside any graph)
     if (h->d_pcb_cnt) cudaMemsetAsync(h->d_pcb_cnt, 0, std::max(h->M, 1) * sizeof(int), h->stream);
+    h->pc_small_cs = pc_small_size(h);
     if (h->sb) {
         sb_pc_build(h);
         if (h->P) pca_build_t<double>(h, 1e-11);
@@ -645,6 +834,31 @@ void pc_build(am_handle* h) {
 template <class T>
 static void pc_apply_t(am_handle* h, const double* r, double* z) {
     cudaStream_t s = h->stream;
+    if (h->pc_small_cs) {
+        cudaLaunchConfig_t lc = {};
+        cudaLaunchAttribute at[2];
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[0].val.programmaticStreamSerializationAllowed = 1;
+        at[1].id = cudaLaunchAttributeClusterDimension;
+        at[1].val.clusterDim.x = (unsigned)h->pc_small_cs;
+        at[1].val.clusterDim.y = 1;
+        at[1].val.clusterDim.z = 1;
+        lc.gridDim = dim3((unsigned)(h->NA * h->pc_small_cs));
+        lc.blockDim = dim3(256);
+        lc.stream = s;
+        lc.attrs = at;
+        lc.numAttrs = 2;
+        cudaLaunchKernelEx(&lc, k_pc_small<T>, h->Nb, h->M, (const int*)h->d_asm_body_off,
+                           (const int*)h->d_asm_body_idx, h->P ? (const int*)h->d_asm_link_off : (const int*)nullptr,
+                           (const int*)h->d_asm_link_idx, (const int*)h->d_blob_off, (const T*)h->d_minv,
+                           (const long long*)h->d_minv_off, (const T*)h->d_Y, (const double*)h->d_Nt,
+                           (const T*)h->d_G, (const long long*)h->d_G_off, (const int*)h->d_bp, (const int*)h->d_bq,
+                           (const double*)h->d_lp, (const double*)h->d_lq, (const int*)h->d_body_link_off,
+                           (const int*)h->d_body_link_idx, (const int*)h->d_link_local, r, h->d_pc_w, h->d_pc_Uhat,
+                           z);
+        count_launch();
+        return;
+    }
     // w and Y^T r1 per (body, chunk) item; the body's last item forms U^
     launch_dep(k_pc_ap1<T>, dim3(h->n_pcw), dim3(128), 0, s, h->d_pcw_body, h->d_pcw_chunk, h->d_blob_off,
                (const T*)h->d_minv, h->d_minv_off, (const T*)h->d_Y, r, h->d_pc_w, h->d_ytp, h->Nb, h->d_pcw_off,
