@@ -1234,9 +1234,10 @@ static void timing_mark(am_handle* h) {
     cudaEventRecord(h->tev[h->tev_used++], h->stream);
 }
 
-static void mobility_partial(am_handle* h, const double* lam, int mode, const int* active = nullptr) {
+static void mobility_partial(am_handle* h, const double* lam, int mode, const int* active = nullptr,
+                             bool packed = false) {
     timing_mark(h);
-    launch_items(h, lam, mode, active);
+    launch_items(h, lam, mode, active, packed);
     timing_mark(h);
     long long pairs = h->per_nnz;  // periodic: the real-space pairs
     if (!h->per)
@@ -1249,12 +1250,12 @@ void mobility_apply(am_handle* h, const double* lam, double* u, int mode) {
     launch_sum_items(h, u);
 }
 
-void op_apply(am_handle* h, const double* y, double* out, int mode, const int* active) {
+void op_apply(am_handle* h, const double* y, double* out, int mode, const int* active, bool packed) {
     if (h->sb) {
         sb_op_apply(h, y, out);
         return;
     }
-    mobility_partial(h, y, mode, active);
+    mobility_partial(h, y, mode, active, packed);
     // The body sums are bound by FP64 issue (16 cycles of its SM for every
     // warp instruction, however few lanes take part) and by latency: few
     // bodies take a warp each, spread over the SMs; many share a warp, each
@@ -1392,9 +1393,10 @@ static void issue_arnoldi_step(am_handle* h, bool fp64, cudaGraphConditionalHand
     const int n = h->n, m = h->restart, m1 = m + 1, S = h->S;
     const size_t ldv = (size_t)h->ldv;
     const int nb = red_blocks(n), nch = h->nchunks, ct = h->chunk_threads;
-    pc_apply(h, h->d_vj, h->d_zj);  // vj = V[j], written with V[j]
+    const bool packed = !h->sb && symmetric_mixed(h, fp64 ? kOpFP64 : kOpHandle);
+    pc_apply(h, h->d_vj, h->d_zj, packed ? h->d_lf : nullptr);  // vj = V[j], written with V[j]
     // the input of a stopped system is zero: its product skips the pairs
-    op_apply(h, h->d_zj, h->d_w, fp64, S > 1 ? h->d_active : nullptr);
+    op_apply(h, h->d_zj, h->d_w, fp64, S > 1 ? h->d_active : nullptr, packed);
     if (h->step_fused) {
         const StepArgs a{h->d_V, ldv, h->d_w, h->d_zj, h->d_Z, h->d_vj, static_cast<const int4*>(h->d_chunk_info),
                          h->d_sys_chunk_off, h->d_part, h->d_npart, nch, m, S, h->chunk_len,

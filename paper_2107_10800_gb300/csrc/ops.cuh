@@ -24,12 +24,15 @@ void launch_geometry(am_handle* h);
 // out = A y (Eq. linear_system) with the mobility product of `mode`.
 // active: per-system flags (device); systems with flag 0 get a zero
 // mobility product without its pair arithmetic (nullptr: all systems)
-void op_apply(am_handle* h, const double* y, double* out, int mode, const int* active = nullptr);
+// packed: d_lf already holds the forces of y as floats
+void op_apply(am_handle* h, const double* y, double* out, int mode, const int* active = nullptr,
+              bool packed = false);
 // Blob mobility product only: u = M lambda (3Nb).
 void mobility_apply(am_handle* h, const double* lam, double* u, int mode);
 // Block-diagonal preconditioner (Sec. 3.1): build at the current pose, apply.
 void pc_build(am_handle* h);
-void pc_apply(am_handle* h, const double* r, double* z);
+// lf: the forces of z as floats as well (handles of multi-blob bodies)
+void pc_apply(am_handle* h, const double* r, double* z, float4* lf = nullptr);
 // Project the U block of x onto C U = B with the preconditioner
 // (x += P~^-1 (0, 0, B - C U)).
 void project_constraints(am_handle* h, double* x);
@@ -48,7 +51,9 @@ int advance(am_handle* h, double dt, am_step_stats* st);
 // tpt targets per thread and source chunks (0 = automatic), their launch,
 // the sum of the partials, and the autotuner that picks (tpt, chunk).
 int mobility_layout(am_handle* h, int tpt, int chunk, int tgroup = 0, int sym = 0);
-void launch_items(am_handle* h, const double* lam, int mode, const int* active = nullptr);
+void launch_items(am_handle* h, const double* lam, int mode, const int* active = nullptr, bool packed = false);
+// whether the product of this mode is the symmetric mixed one (its forces: d_lf)
+bool symmetric_mixed(const am_handle* h, int mode);
 int df_resident_grid(bool wall);
 int sym_df_resident_grid(bool wall);
 void launch_items_df(am_handle* h, const double* lam);

@@ -499,17 +499,21 @@ k_pc_ap2(int Nb, int M, const int* __restrict__ pca_asm, const int* __restrict__
     }
 }
 
-// U_b = U^_b + N~_b (C^T phi)_b;  lambda rows = w + Y U
+// U_b = U^_b + N~_b (C^T phi)_b;  lambda rows = w + Y U, also as floats to lf
+// when given.  A block per 128 rows (every fourth chunk): each block forms U_b
+// for itself, which is more FP64 work than its rows.
 template <class T>
 __global__ void __launch_bounds__(128)
 k_pc_ap3(int Nb, int M, const int* __restrict__ pcw_body, const int* __restrict__ pcw_chunk,
          const int* __restrict__ blob_off, const T* __restrict__ Y, const double* __restrict__ Nt,
          const double* __restrict__ w, const double* __restrict__ Uhat,
          const int* __restrict__ bl_off, const int* __restrict__ bl_idx,
-         const double* __restrict__ lp, const double* __restrict__ lq, double* __restrict__ z) {
+         const double* __restrict__ lp, const double* __restrict__ lq, double* __restrict__ z,
+         float* __restrict__ lf) {
     dep_wait();
     __shared__ double sU[6];
     const int it = blockIdx.x;
+    if (pcw_chunk[it] % 4) return;
     const int b = pcw_body[it];
     const double* phi = z + 3 * (size_t)Nb + 6 * (size_t)M;
     if (threadIdx.x < 32) {
@@ -543,15 +547,16 @@ k_pc_ap3(int Nb, int M, const int* __restrict__ pcw_body, const int* __restrict_
     const int i0 = blob_off[b];
     const int m = 3 * (blob_off[b + 1] - i0);
     const int row = pcw_chunk[it] * kRows + threadIdx.x;
-    if (threadIdx.x < kRows && row < m) {
+    if (row < m) {
         const T* Yr = Y + 18 * (size_t)i0 + 6 * (size_t)row;
         double s = w[3 * (size_t)i0 + row];
         for (int c = 0; c < 6; ++c) s = fma((double)Yr[c], sU[c], s);
         z[3 * (size_t)i0 + row] = s;
+        if (lf) lf[4 * (size_t)(i0 + row / 3) + row % 3] = (float)s;
     }
 }
 
-// The whole apply for handles of small articulated bodies (pc_small_fits): one
+// The whole apply for handles of small articulated bodies (pc_small_size): one
 // cluster per articulated body, a warp per body, one launch instead of three
 // (the problem is block-diagonal over articulated bodies).  With n the body's
 // rows (at most 64), lane l of the warp takes rows l and, when n > 32, the
@@ -572,7 +577,7 @@ k_pc_small(int Nb, int M, const int* __restrict__ asm_body_off, const int* __res
            const long long* __restrict__ goff, const int* __restrict__ bp, const int* __restrict__ bq,
            const double* __restrict__ lp, const double* __restrict__ lq, const int* __restrict__ bl_off,
            const int* __restrict__ bl_idx, const int* __restrict__ link_local, const double* __restrict__ r,
-           double* __restrict__ w, double* __restrict__ Uhat, double* __restrict__ z) {
+           double* __restrict__ w, double* __restrict__ Uhat, double* __restrict__ z, float* __restrict__ lf) {
     dep_wait();
     __shared__ double cs[kSmallRows], phis[kSmallRows];
     __shared__ T ct[kSmallRows];
@@ -712,6 +717,7 @@ k_pc_small(int Nb, int M, const int* __restrict__ asm_body_off, const int* __res
 #pragma unroll
             for (int x = 0; x < 6; ++x) v = fma((double)Yr[x], u[x], v);
             z[3 * (size_t)i0 + row] = v;
+            if (lf) lf[4 * (size_t)(i0 + row / 3) + row % 3] = (float)v;
         }
     }
 }
@@ -832,7 +838,7 @@ void pc_build(am_handle* h) {
 }
 
 template <class T>
-static void pc_apply_t(am_handle* h, const double* r, double* z) {
+static void pc_apply_t(am_handle* h, const double* r, double* z, float* lf) {
     cudaStream_t s = h->stream;
     if (h->pc_small_cs) {
         cudaLaunchConfig_t lc = {};
@@ -855,7 +861,7 @@ static void pc_apply_t(am_handle* h, const double* r, double* z) {
                            (const T*)h->d_G, (const long long*)h->d_G_off, (const int*)h->d_bp, (const int*)h->d_bq,
                            (const double*)h->d_lp, (const double*)h->d_lq, (const int*)h->d_body_link_off,
                            (const int*)h->d_body_link_idx, (const int*)h->d_link_local, r, h->d_pc_w, h->d_pc_Uhat,
-                           z);
+                           z, lf);
         count_launch();
         return;
     }
@@ -873,19 +879,19 @@ static void pc_apply_t(am_handle* h, const double* r, double* z) {
     }
     launch_dep(k_pc_ap3<T>, dim3(h->n_pcw), dim3(128), 0, s, h->Nb, h->M, h->d_pcw_body, h->d_pcw_chunk,
                h->d_blob_off, (const T*)h->d_Y, h->d_Nt, h->d_pc_w, h->d_pc_Uhat, h->d_body_link_off,
-               h->d_body_link_idx, h->d_lp, h->d_lq, z);
+               h->d_body_link_idx, h->d_lp, h->d_lq, z, lf);
     count_launch();
 }
 
-void pc_apply(am_handle* h, const double* r, double* z) {
+void pc_apply(am_handle* h, const double* r, double* z, float4* lf) {
     if (h->sb) {
         sb_pc_apply(h, r, z);
         return;
     }
     if (h->pc32)
-        pc_apply_t<float>(h, r, z);
+        pc_apply_t<float>(h, r, z, reinterpret_cast<float*>(lf));
     else
-        pc_apply_t<double>(h, r, z);
+        pc_apply_t<double>(h, r, z, reinterpret_cast<float*>(lf));
 }
 
 }  // namespace am

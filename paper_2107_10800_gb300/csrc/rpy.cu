@@ -425,39 +425,47 @@ __device__ __forceinline__ void pair2_sym(float2 dx, float2 dy, float2 dz, float
     vz = fma2(P1, dmxy, fma2(M33, mz, vz));
 }
 
-// Symmetric mixed product on tiles of 128 blobs: items are pairs of groups of
-// whole tiles, walked tile pair by tile pair.  Warp w holds 64 targets of tile
-// I, two per lane in the lanes of float2 registers (targets 64 (w & 1) + l and
-// + 32), and takes source sub-tiles 2 (w >> 1) and 2 (w >> 1) + 1 of tile J (32
-// sources each).  At step t lane l meets source (l + t) mod 32 of the sub-tile
-// with both targets; the source's column sum (the two targets' contributions
-// added) moves one lane per step as in k_sym_tiles.  Differences from the hi
-// parts, with the lo parts added within a quarter of the target's largest
-// coordinate (as rpy_items_mixed_x2).  FP32 sums over at most 64 terms (a
-// warp's sources for u, its targets for v), added across warps and tiles to
-// compensated (hi, lo) float pairs in a fixed order: the targets' in shared
-// memory, the sources' in the item's slots, which hold such pairs in units of
-// A1.  No FP64 work: sums and forces folded through the FP64 pipe (2 lanes per
-// SM and cycle) cost a tenth of the kernel.  A tile against itself meets every
+// Symmetric mixed product on tiles of T = 32, 64 or 128 blobs, in blocks of T
+// threads: items are pairs of groups of whole tiles, walked tile pair by tile
+// pair.  A team of LW lanes (a half-warp for T = 32, else a warp) holds 2 LW
+// targets of tile I, two per lane in the lanes of float2 registers, and takes
+// H source sub-tiles of LW sources of tile J.  At step t lane l meets source
+// (l + t + 1) mod LW of the sub-tile with both targets (a blob meets itself
+// last: the self term is the largest of its sum); the source's column sum
+// (the two targets' contributions added) moves one lane per step as in
+// k_sym_tiles.  Differences from the hi parts, with the lo parts added within a
+// quarter of the target's largest coordinate (as rpy_items_mixed_x2).  FP32
+// sums over the LW H sources a team meets (u) and its LW target pairs (v),
+// added across teams and tiles to compensated (hi, lo) float pairs in a fixed
+// order: the targets' in shared memory, the sources' in the item's slots, which
+// hold such pairs in units of A1.  No FP64 work: sums and forces folded through
+// the FP64 pipe (2 lanes per SM and cycle) cost a tenth of the kernel on tiles
+// of 128 and nearly half on tiles of 64.  A tile against itself meets every
 // ordered pair (the self term included) and drops the column sums: a second,
 // one-direction form of the pair in the loop cost 6 to 12 % by its code size.
-template <bool WALL>
-__global__ void __launch_bounds__(kThreads, 4)
-rpy_sym_mixed_x2(const float4* __restrict__ hi, const float4* __restrict__ lo, const float4* __restrict__ lf,
+// Bound by FP32 issue on large systems; the small tiles spread systems of a few
+// thousand blobs over every SM and keep an item at 16 (T = 32) or 32 steps.
+// Tiles of 64 against one target per lane with FP64 sums: 16 free systems of
+// 500 to 4,000 blobs 71.5 -> 56 us, the 3,600-blob colony above a wall 22.5 ->
+// 17.1.  Free space: 24 warps per SM (80 registers) 54 us, 16 warps 57; wall:
+// 113 registers, fewer cost more than the warps bring (17.1, 17.7).
+template <bool WALL, int T>
+__global__ void __launch_bounds__(T, (WALL ? 512 : 768) / T)
+rpy_sym_mixed(const float4* __restrict__ hi, const float4* __restrict__ lo, const float4* __restrict__ lf,
                  double* __restrict__ part, const SymItem* __restrict__ items,
                  int n_items, int* __restrict__ counter, RpyK<float> k, const int* __restrict__ active) {
     dep_wait();
-    constexpr int T = 128;
+    constexpr int LW = T == 32 ? 16 : 32, NG = T / LW, H = T / (2 * LW);
     __shared__ float4 sq[3][T];   // sources: (-hx, -hx, -hy, -hy), (2hz, 2hz, lz, lz), (lx, lx, ly, ly)
     __shared__ float4 so[T];      // (-ox, -ox, -oy, -oy)
     __shared__ float2 soz[T];     // (-oz, -oz)
     __shared__ float2 acc[3][T];       // row sums of the tile's targets: (hi, lo)
-    __shared__ float up[4][3][64];     // row sums of each warp's 64 targets over a tile of sources
-    __shared__ float vp[4][2][3][32];  // column sums of each warp's two sub-tiles
+    __shared__ float up[NG][3][2 * LW];  // row sums of each team's targets over a tile of sources
+    __shared__ float vp[NG][H][3][LW];   // column sums of each team's sub-tiles
     __shared__ int s_item;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int th = warp & 1;            // target half of tile I
-    const int sb0 = 2 * (warp >> 1);    // the warp's first source sub-tile
+    const int team = threadIdx.x / LW, lane = threadIdx.x % LW;
+    const int th = team % H;             // the team's targets: part th of tile I
+    const int sb0 = H * (team / H);      // its first source sub-tile
     for (int round = 0;; ++round) {
         __syncthreads();
         if (threadIdx.x == 0) s_item = round == 0 ? (int)blockIdx.x : (int)gridDim.x + atomicAdd(counter, 1);
@@ -476,7 +484,7 @@ rpy_sym_mixed_x2(const float4* __restrict__ hi, const float4* __restrict__ lo, c
             continue;
         }
         for (int ia = 0; ia < m.ni; ia += T) {
-            const int t0 = ia + 64 * th + lane, t1 = t0 + 32;
+            const int t0 = ia + 2 * LW * th + lane, t1 = t0 + LW;
             const bool ok0 = t0 < m.ni, ok1 = t1 < m.ni;
             const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
             const float4 h0 = ok0 ? hi[m.i0 + t0] : make_float4(0.f, 0.f, 1.f, 0.f);
@@ -511,12 +519,12 @@ rpy_sym_mixed_x2(const float4* __restrict__ hi, const float4* __restrict__ lo, c
                 __syncthreads();
                 float2 ux = bc2(0.f), uy = bc2(0.f), uz = bc2(0.f);
 #pragma unroll 1
-                for (int sbi = 0; sbi < 2; ++sbi) {
+                for (int sbi = 0; sbi < H; ++sbi) {
                     const int sb = sb0 + sbi;
-                    float vx = 0.f, vy = 0.f, vz = 0.f;  // column sum of source 32 sb + ((lane + t) & 31)
+                    float vx = 0.f, vy = 0.f, vz = 0.f;  // column sum of source LW sb + (lane + t + 1) % LW
 #pragma unroll 2
-                    for (int t = 0; t < 32; ++t) {
-                        const int q = 32 * sb + ((lane + t) & 31);
+                    for (int t = 0; t < LW; ++t) {
+                        const int q = LW * sb + ((lane + t + 1) & (LW - 1));
                         const float4 v0 = sq[0][q], v1 = sq[1][q], v2 = sq[2][q];
                         const float2 h2 = make_float2(v1.x, v1.y);
                         float2 dx = add2(HX, make_float2(v0.x, v0.y));
@@ -541,37 +549,39 @@ rpy_sym_mixed_x2(const float4* __restrict__ hi, const float4* __restrict__ lo, c
                         vx += cx.x + cx.y;
                         vy += cy.x + cy.y;
                         vz += cz.x + cz.y;
-                        const int src = (lane + 1) & 31;
-                        vx = __shfl_sync(0xffffffffu, vx, src);
-                        vy = __shfl_sync(0xffffffffu, vy, src);
-                        vz = __shfl_sync(0xffffffffu, vz, src);
+                        const int src = (lane + 1) & (LW - 1);
+                        vx = __shfl_sync(0xffffffffu, vx, src, LW);
+                        vy = __shfl_sync(0xffffffffu, vy, src, LW);
+                        vz = __shfl_sync(0xffffffffu, vz, src, LW);
                     }
-                    vp[warp][sbi][0][lane] = vx;
-                    vp[warp][sbi][1][lane] = vy;
-                    vp[warp][sbi][2][lane] = vz;
+                    const int first = (lane + 1) & (LW - 1);
+                    vp[team][sbi][0][first] = vx;
+                    vp[team][sbi][1][first] = vy;
+                    vp[team][sbi][2][first] = vz;
                 }
-                up[warp][0][lane] = ux.x; up[warp][1][lane] = uy.x; up[warp][2][lane] = uz.x;
-                up[warp][0][32 + lane] = ux.y; up[warp][1][32 + lane] = uy.y; up[warp][2][32 + lane] = uz.y;
+                float (*uo)[2 * LW] = up[team];
+                uo[0][lane] = ux.x; uo[1][lane] = uy.x; uo[2][lane] = uz.x;
+                uo[0][LW + lane] = ux.y; uo[1][LW + lane] = uy.y; uo[2][LW + lane] = uz.y;
                 __syncthreads();
                 const int t = threadIdx.x;
-                {   // target t: half t >> 6, entry t & 63 of warps t >> 6 and + 2
-                    const int hh = t >> 6, j = t & 63;
+                {   // target t: part t / (2 LW), of the teams that hold it
+                    const int hh = t / (2 * LW), j = t % (2 * LW);
 #pragma unroll
                     for (int c = 0; c < 3; ++c) {
                         float2 a = acc[c][t];
-                        two_sum_acc(a.x, a.y, up[hh][c][j]);
-                        two_sum_acc(a.x, a.y, up[hh + 2][c][j]);
+#pragma unroll
+                        for (int g = 0; g < 2; ++g) two_sum_acc(a.x, a.y, up[hh + H * g][c][j]);
                         acc[c][t] = a;
                     }
                 }
-                if (!dtile && jb + t < m.nj) {  // source t: sub-tile sb = t >> 5 of warps 2 (sb >> 1) and + 1
-                    const int sb = t >> 5, l = t & 31, wa = 2 * (sb >> 1), si = sb & 1;
+                if (!dtile && jb + t < m.nj) {  // source t: sub-tile t / LW, of the teams that met it
+                    const int sb = t / LW, l = t % LW, wa = H * (sb / H), si = sb % H;
                     float2* o = colo + 3 * (size_t)(jb + t);
 #pragma unroll
                     for (int c = 0; c < 3; ++c) {
                         float2 a = ia == 0 ? bc2(0.f) : o[c];
-                        two_sum_acc(a.x, a.y, vp[wa][si][c][l]);
-                        two_sum_acc(a.x, a.y, vp[wa + 1][si][c][l]);
+#pragma unroll
+                        for (int g = 0; g < H; ++g) two_sum_acc(a.x, a.y, vp[wa + g][si][c][l]);
                         o[c] = a;
                     }
                 }
@@ -590,141 +600,6 @@ rpy_sym_mixed_x2(const float4* __restrict__ hi, const float4* __restrict__ lo, c
                     }
                     o[c] = a;
                 }
-            }
-        }
-    }
-    item_queue_done(counter);
-}
-
-// Symmetric mixed product on tiles of 32 NSUB blobs, one target per lane:
-// the scheme of k_sym_tiles (each unordered pair of a tile pair evaluated
-// once and applied in both directions, the column sums carried from lane
-// to lane, the diagonal warp tile on steps 1..16) with FP32 pair terms.
-// Differences are formed from the hi parts of the positions; within a
-// quarter of the target's largest coordinate the lo parts are added, as in
-// rpy_items_mixed.  A lane sums the 32 terms of a warp tile in FP32; the
-// warp-tile sums are added in FP64 in a fixed order.  Small tiles spread
-// systems of a few thousand blobs over every SM.
-template <bool WALL, int NSUB>
-__global__ void __launch_bounds__(NSUB == 1 ? 32 : 128)
-rpy_sym_mixed(const float4* __restrict__ hi, const float4* __restrict__ lo, const double* __restrict__ lam,
-              double* __restrict__ part, const SymItem* __restrict__ items, int n_items, int* __restrict__ counter,
-              RpyK<float> k, const int* __restrict__ active) {
-    dep_wait();
-    constexpr int T = 32 * NSUB;
-    constexpr int NW = NSUB == 1 ? 1 : 4;
-    constexpr int NWT = NSUB * NSUB;
-    __shared__ float4 hI[T], hJ[T];  // hi parts, .w = twice the height
-    __shared__ float4 oI[T], oJ[T];  // lo parts
-    __shared__ float4 lI[T], lJ[T];  // forces
-    __shared__ double up[NWT][32][3], vp[NWT][32][3];
-    __shared__ int s_item;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int round = 0;; ++round) {
-        __syncthreads();
-        if (threadIdx.x == 0) s_item = round == 0 ? (int)blockIdx.x : (int)gridDim.x + atomicAdd(counter, 1);
-        __syncthreads();
-        const int itn = s_item;
-        if (itn >= n_items) break;
-        const SymItem m = items[itn];
-        const bool diag = m.ti == m.tj;
-        double* rowo = part + m.poff + (long long)m.tj * m.n3 + 3 * (long long)(m.i0 - m.tbase);
-        double* colo = part + m.poff + (long long)m.ti * m.n3 + 3 * (long long)(m.j0 - m.tbase);
-        if (active && !active[m.sys]) {  // a stopped system: zero partial sums
-            for (int q = threadIdx.x; q < 3 * m.ni; q += blockDim.x) rowo[q] = 0.0;
-            if (!diag)
-                for (int q = threadIdx.x; q < 3 * m.nj; q += blockDim.x) colo[q] = 0.0;
-            continue;
-        }
-        for (int q = threadIdx.x; q < T; q += blockDim.x) {
-            const bool oi = q < m.ni, oj = q < m.nj;
-            float4 a = oi ? hi[m.i0 + q] : make_float4(0.f, 0.f, 1.f, 0.f);
-            a.w = 2.f * a.z;
-            hI[q] = a;
-            oI[q] = oi ? lo[m.i0 + q] : make_float4(0.f, 0.f, 0.f, 0.f);
-            lI[q] = oi ? make_float4((float)lam[3 * (size_t)(m.i0 + q)], (float)lam[3 * (size_t)(m.i0 + q) + 1],
-                                     (float)lam[3 * (size_t)(m.i0 + q) + 2], 0.f)
-                       : make_float4(0.f, 0.f, 0.f, 0.f);
-            float4 b = oj ? hi[m.j0 + q] : make_float4(0.f, 0.f, 1.f, 0.f);
-            b.w = 2.f * b.z;
-            hJ[q] = b;
-            oJ[q] = oj ? lo[m.j0 + q] : make_float4(0.f, 0.f, 0.f, 0.f);
-            lJ[q] = oj ? make_float4((float)lam[3 * (size_t)(m.j0 + q)], (float)lam[3 * (size_t)(m.j0 + q) + 1],
-                                     (float)lam[3 * (size_t)(m.j0 + q) + 2], 0.f)
-                       : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-        __syncthreads();
-        for (int wt = warp; wt < NWT; wt += NW) {
-            const int a = wt / NSUB, b = wt % NSUB;
-            float ux = 0.f, uy = 0.f, uz = 0.f, vx = 0.f, vy = 0.f, vz = 0.f;
-            if (!(diag && b < a)) {  // below the diagonal of a diagonal item: taken by (b, a)
-                const bool self_tile = diag && a == b;
-                const int t = 32 * a + lane;
-                const float4 xi = hI[t], xo = oI[t], mu = lI[t];
-                const float nr = 0.25f * fmaxf(fabsf(xi.x), fmaxf(fabsf(xi.y), fabsf(xi.z)));
-                const float near2 = nr * nr;
-                const bool ti_ok = t < m.ni;
-#pragma unroll 1
-                for (int step = 0; step < 32; ++step) {
-                    const int q = 32 * b + ((lane + step) & 31);
-                    const bool pair_ok = ti_ok && q < m.nj &&
-                                         (!self_tile || (step >= 1 && (step < 16 || (step == 16 && lane < 16))));
-                    if (pair_ok) {
-                        const float4 xj = hJ[q], l = lJ[q];
-                        float dx = xi.x - xj.x, dy = xi.y - xj.y, dz = xi.z - xj.z;
-                        float rxy2 = fmaf(dx, dx, dy * dy);
-                        float r2 = fmaf(dz, dz, rxy2);
-                        if (r2 < near2) {
-                            const float4 o = oJ[q];
-                            dx += xo.x - o.x;
-                            dy += xo.y - o.y;
-                            dz += xo.z - o.z;
-                            rxy2 = fmaf(dx, dx, dy * dy);
-                            r2 = fmaf(dz, dz, rxy2);
-                        }
-                        if (WALL)
-                            pair_wall_sym<float>(dx, dy, dz, rxy2, r2, xi.z + xj.z, xj.w, -xi.z, l.x, l.y, l.z, mu.x,
-                                                 mu.y, mu.z, k, ux, uy, uz, vx, vy, vz);
-                        else
-                            pair_free_sym<float>(dx, dy, dz, r2, l.x, l.y, l.z, mu.x, mu.y, mu.z, k, ux, uy, uz, vx,
-                                                 vy, vz);
-                    } else if (self_tile && step == 0 && ti_ok) {  // the self term
-                        if (WALL)
-                            pair_wall_r2<float>(0.f, 0.f, 0.f, 0.f, 0.f, xi.w, xi.w, -xi.z, mu.x, mu.y, mu.z, k, ux,
-                                                uy, uz);
-                        else
-                            pair_free<float>(0.f, 0.f, 0.f, mu.x, mu.y, mu.z, k, ux, uy, uz);
-                    }
-                    // hand the column sum to the lane that meets this source next
-                    const int src = (lane + 1) & 31;
-                    vx = __shfl_sync(0xffffffffu, vx, src);
-                    vy = __shfl_sync(0xffffffffu, vy, src);
-                    vz = __shfl_sync(0xffffffffu, vz, src);
-                }
-            }
-            up[wt][lane][0] = ux; up[wt][lane][1] = uy; up[wt][lane][2] = uz;
-            vp[wt][lane][0] = vx; vp[wt][lane][1] = vy; vp[wt][lane][2] = vz;
-        }
-        __syncthreads();
-        for (int t = threadIdx.x; t < T; t += blockDim.x) {
-            const int a = t >> 5, l = t & 31;
-            if (t < m.ni) {
-                double sx = 0.0, sy = 0.0, sz = 0.0;
-                for (int b = 0; b < NSUB; ++b) {
-                    sx += up[a * NSUB + b][l][0]; sy += up[a * NSUB + b][l][1]; sz += up[a * NSUB + b][l][2];
-                }
-                if (diag)
-                    for (int a2 = 0; a2 < NSUB; ++a2) {
-                        sx += vp[a2 * NSUB + a][l][0]; sy += vp[a2 * NSUB + a][l][1]; sz += vp[a2 * NSUB + a][l][2];
-                    }
-                rowo[3 * t] = k.A1 * sx; rowo[3 * t + 1] = k.A1 * sy; rowo[3 * t + 2] = k.A1 * sz;
-            }
-            if (!diag && t < m.nj) {
-                double sx = 0.0, sy = 0.0, sz = 0.0;
-                for (int a2 = 0; a2 < NSUB; ++a2) {
-                    sx += vp[a2 * NSUB + a][l][0]; sy += vp[a2 * NSUB + a][l][1]; sz += vp[a2 * NSUB + a][l][2];
-                }
-                colo[3 * t] = k.A1 * sx; colo[3 * t + 1] = k.A1 * sy; colo[3 * t + 2] = k.A1 * sz;
             }
         }
     }
@@ -967,27 +842,18 @@ static int sym_grid(bool wall) {
                 : resident_grid(k_sym_tiles<SymBlobPair<false>>, 32 * kSymWarps);
 }
 
-// resident blocks of the symmetric mixed kernel: paired lanes (tpt 2,
-// tiles of 128) or one target per lane (tiles of 32 nsub)
-static int sym_mixed_grid(bool wall, int tpt, int nsub) {
-    if (tpt == 2) return wall ? resident_grid(rpy_sym_mixed_x2<true>) : resident_grid(rpy_sym_mixed_x2<false>);
-    const int th = nsub == 1 ? 32 : 128;
-    if (wall) {
-        if (nsub == 1) return resident_grid(rpy_sym_mixed<true, 1>, th);
-        if (nsub == 2) return resident_grid(rpy_sym_mixed<true, 2>, th);
-        return resident_grid(rpy_sym_mixed<true, 4>, th);
-    }
-    if (nsub == 1) return resident_grid(rpy_sym_mixed<false, 1>, th);
-    if (nsub == 2) return resident_grid(rpy_sym_mixed<false, 2>, th);
-    return resident_grid(rpy_sym_mixed<false, 4>, th);
+// resident blocks of the symmetric mixed kernel on tiles of 32 nsub blobs
+static int sym_mixed_grid(bool wall, int nsub) {
+    if (nsub == 1) return wall ? resident_grid(rpy_sym_mixed<true, 32>, 32) : resident_grid(rpy_sym_mixed<false, 32>, 32);
+    if (nsub == 2) return wall ? resident_grid(rpy_sym_mixed<true, 64>, 64) : resident_grid(rpy_sym_mixed<false, 64>, 64);
+    return wall ? resident_grid(rpy_sym_mixed<true, 128>, 128) : resident_grid(rpy_sym_mixed<false, 128>, 128);
 }
 
 // Work items for tpt targets per thread and source chunks of `chunk` blobs
 // (0: choose so that the items fill the GPU); with sym = nsub > 0 also the
 // tile-pair items of the symmetric product on tiles of 32 nsub blobs, whose
 // partial-sum slots are the source chunks of that length (mixed handles:
-// paired lanes with tpt = 2 on tiles of 128, one target per lane with
-// tpt = 1).  Returns 0 on success.
+// groups of such tiles when tpt = 2).  Returns 0 on success.
 int mobility_layout(am_handle* h, int tpt, int chunk, int tgroup, int sym) {
     const int S = h->S;
     if (h->cfg.precision != AM_MIXED) tpt = 1;
@@ -1056,7 +922,7 @@ int mobility_layout(am_handle* h, int tpt, int chunk, int tgroup, int sym) {
     if (h->d_sym_items) cudaFree(h->d_sym_items);
     h->d_sym_items = nullptr;
     h->n_sym = 0;
-    if (sym && tpt == 2 && !h->d_lf &&
+    if (sym && !h->d_lf &&
         cudaMalloc(reinterpret_cast<void**>(&h->d_lf), std::max(h->Nb, 1) * sizeof(float4)) != cudaSuccess)
         return 1;
     if (!sitems.empty()) {
@@ -1068,7 +934,7 @@ int mobility_layout(am_handle* h, int tpt, int chunk, int tgroup, int sym) {
         h->sym_nsub = sym;
         h->sym_splits = splits;
         h->mv_gridsym = std::min(sym_grid(h->cfg.wall != 0), (h->n_sym + kSymWarps - 1) / kSymWarps);
-        h->mv_gridsym32 = std::min(sym_mixed_grid(h->cfg.wall != 0, tpt, sym), h->n_sym);
+        h->mv_gridsym32 = std::min(sym_mixed_grid(h->cfg.wall != 0, sym), h->n_sym);
         h->mv_gridsymdf = std::min(sym_df_resident_grid(h->cfg.wall != 0), h->n_sym);
     }
     if (h->d_items) cudaFree(h->d_items);
@@ -1109,9 +975,14 @@ int mobility_layout(am_handle* h, int tpt, int chunk, int tgroup, int sym) {
     return 0;
 }
 
+bool symmetric_mixed(const am_handle* h, int mode) {
+    return !h->per && (mode == kOpMixed || (mode == kOpHandle && h->cfg.precision == AM_MIXED)) && h->n_sym > 0 &&
+           h->sym_splits == 1;
+}
+
 // The partial sums of u = M lambda for all systems (mode: the handle's
-// precision, FP64 or double-float).
-void launch_items(am_handle* h, const double* lam, int mode, const int* active) {
+// precision, FP64, mixed or double-float).
+void launch_items(am_handle* h, const double* lam, int mode, const int* active, bool packed) {
     h->mv_pairs = false;
     if (h->per) {  // FP32 wave part for the mixed operator; FP64 for FP64 and double-float requests
         launch_periodic(h, lam, mode == kOpMixed || (mode == kOpHandle && h->cfg.precision == AM_MIXED));
@@ -1142,33 +1013,27 @@ void launch_items(am_handle* h, const double* lam, int mode, const int* active) 
         else
             launch_dep(rpy_items_f64<false>, dim3(h->mv_grid64), dim3(kThreads), 0, st, h->d_r4, lam, h->d_mv, items,
                        h->n_items, h->d_item_counter, k, active);
-    } else if (h->n_sym > 0 && h->sym_splits == 1) {
+    } else if (symmetric_mixed(h, mode)) {
         const RpyK<float> k = rpy_consts<float>(h->prm);
         const SymItem* si = static_cast<const SymItem*>(h->d_sym_items);
-        const int th = h->sym_nsub > 1 ? kThreads : 32;
-        if (h->mv_tpt == 2) {  // forces as floats, slots as float pairs
+        // forces as floats, slots as float pairs
+        if (!packed) {
             launch_dep(k_pack_forces, dim3((h->Nb + 127) / 128), dim3(128), 0, st, lam, h->d_lf, h->Nb);
             count_launch();
-            h->mv_pairs = true;
         }
-#define AM_SYM32(W, N)                                                                                      \
-    launch_dep(rpy_sym_mixed<W, N>, dim3(h->mv_gridsym32), dim3(th), 0, st, h->d_rhi, h->d_rlo, lam, h->d_mv, si, \
-               h->n_sym, h->d_item_counter, k, active)
-#define AM_SYM32X2(W)                                                                                         \
-    launch_dep(rpy_sym_mixed_x2<W>, dim3(h->mv_gridsym32), dim3(kThreads), 0, st, h->d_rhi, h->d_rlo,                \
+        h->mv_pairs = true;
+#define AM_SYM32(W, T)                                                                                     \
+    launch_dep(rpy_sym_mixed<W, T>, dim3(h->mv_gridsym32), dim3(T), 0, st, h->d_rhi, h->d_rlo,             \
                (const float4*)h->d_lf, h->d_mv, si, h->n_sym, h->d_item_counter, k, active)
         if (h->cfg.wall) {
-            if (h->mv_tpt == 2) AM_SYM32X2(true);
-            else if (h->sym_nsub == 1) AM_SYM32(true, 1);
-            else if (h->sym_nsub == 2) AM_SYM32(true, 2);
-            else AM_SYM32(true, 4);
+            if (h->sym_nsub == 1) AM_SYM32(true, 32);
+            else if (h->sym_nsub == 2) AM_SYM32(true, 64);
+            else AM_SYM32(true, 128);
         } else {
-            if (h->mv_tpt == 2) AM_SYM32X2(false);
-            else if (h->sym_nsub == 1) AM_SYM32(false, 1);
-            else if (h->sym_nsub == 2) AM_SYM32(false, 2);
-            else AM_SYM32(false, 4);
+            if (h->sym_nsub == 1) AM_SYM32(false, 32);
+            else if (h->sym_nsub == 2) AM_SYM32(false, 64);
+            else AM_SYM32(false, 128);
         }
-#undef AM_SYM32X2
 #undef AM_SYM32
     } else {
         const RpyK<float> k = rpy_consts<float>(h->prm);
@@ -1235,11 +1100,12 @@ int mobility_autotune(am_handle* h) {
         }
     }
     // The symmetric product: on tiles of 32, 64 and 128 blobs while its
-    // partial sums (one slot per tile of the system) stay within 1 GiB (FP64,
-    // and mixed with one target per lane); mixed in paired lanes on groups
-    // of 128-blob tiles while they stay within a quarter of the free device
-    // memory (1.4 GB for 360,000 blobs)
-    for (int nsub : {1, 2, 4}) {
+    // partial sums (one slot per tile of the system) stay within 1 GiB; mixed
+    // on groups of 128-blob tiles while they stay within a quarter of the free
+    // device memory (1.4 GB for 360,000 blobs).  Mixed product and sum, one
+    // system above a wall, tiles of 32 / 64 / 128: 2,000 blobs 22 / 33 / 53 us,
+    // 4,000 38 / 45 / 67, 8,000 122 / 113 / 144, 32,000 1,819 / 1,664 / 1,622
+    for (int nsub : mixed ? std::vector<int>{1, 2} : std::vector<int>{1, 2, 4}) {
         long long slots = 0;
         for (const auto& r : h->sys) slots += (long long)((r.Nb + 32 * nsub - 1) / (32 * nsub)) * 3 * r.Nb;
         if (slots * 8 <= (1LL << 30)) cand.push_back({1, 32 * nsub, 0, nsub});
@@ -1267,7 +1133,10 @@ int mobility_autotune(am_handle* h) {
     // per candidate: a warm-up product and sum, timed; a candidate whose
     // warm-up is already 50 % slower than the best (per product) stops there,
     // and products of more than 20 ms are taken from the warm-up alone (large
-    // systems, where the candidates cost seconds)
+    // systems, where the candidates cost seconds).  Mixed, tiles of 32 and 64
+    // have to be 5 % faster: the double-float product of a solve's residuals is
+    // symmetric on tiles of 128 only (17.5 ms against 28 at 36,000 wall blobs,
+    // one for about 50 mixed products)
     for (auto c : cand) {
         if (mobility_layout(h, c.tpt, c.chunk, c.tgroup, c.sym)) continue;
         cudaEventRecord(e0, st);
@@ -1289,6 +1158,7 @@ int mobility_autotune(am_handle* h) {
             cudaEventElapsedTime(&ms, e0, e1);
             ms *= 0.5f;
         }
+        if (mixed && (c.sym == 1 || c.sym == 2)) ms *= 1.05f;
         if (ms < best) { best = ms; pick = c; }
     }
     h->timing = timing;
