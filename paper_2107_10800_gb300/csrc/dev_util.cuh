@@ -75,32 +75,33 @@ __device__ __forceinline__ bool arrive_last(int* cnt, int idx, int total) {
 }
 
 // The sum of slots q, q + G, .. of one element (p: its value in slot 0, n
-// values per slot).  pairs: a slot value is a compensated (hi, lo) pair of
-// floats; they are added as such (a conversion is FP64 work).
-__device__ __forceinline__ double slot_run(const double* __restrict__ p, size_t n, int q, int ns, int G, bool pairs) {
-    if (pairs) {
-        const float2* f = reinterpret_cast<const float2*>(p);
-        float h = 0.f, l = 0.f;
-#pragma unroll 4
-        for (int c = q; c < ns; c += G) {
-            const float2 v = f[c * n];
-            two_sum_acc(h, l, v.x);
-            l += v.y;
-        }
-        return (double)h + (double)l;
-    }
+// values per slot).
+__device__ __forceinline__ double slot_run(const double* __restrict__ p, size_t n, int q, int ns, int G) {
     double a = 0.0;
 #pragma unroll 4
     for (int c = q; c < ns; c += G) a += p[c * n];
     return a;
 }
 
+// The same of compensated (hi, lo) pairs of floats, added as such: a
+// conversion is FP64 work.
+__device__ __forceinline__ void add_pair(float2& a, float2 v) {
+    two_sum_acc(a.x, a.y, v.x);
+    a.y += v.y;
+}
+__device__ __forceinline__ float2 slot_run_pairs(const float2* __restrict__ p, size_t n, int q, int ns, int G) {
+    float2 a = make_float2(0.f, 0.f);
+#pragma unroll 4
+    for (int c = q; c < ns; c += G) add_pair(a, p[c * n]);
+    return a;
+}
+
 // Element of u = M lambda from the partial sums, in a block of 256 threads for
 // 256 / G elements: G threads add the slots of an element's system (thread g
 // of them every G-th slot, then the G sums in order; the result is valid in
-// threads 0 .. 256 / G - 1, whose element is blk 256 / G + threadIdx.x).  G = 8
+// threads 0 .. 256 / G - 1, whose element is blk 256 / G + threadIdx.x).  G > 1
 // for many slots (consecutive threads still read consecutive doubles, and the
-// chain of dependent additions is an eighth of the slots), else 1.  scale !=
+// chain of dependent additions is a G-th of the slots).  scale !=
 // 0: the slots hold float pairs in units of it.  Every thread calls it; sh:
 // 256 doubles.
 __device__ __forceinline__ double slot_sum(int blk, int G, double scale, int n3, const double* __restrict__ part,
@@ -110,19 +111,32 @@ __device__ __forceinline__ double slot_sum(int blk, int G, double scale, int n3,
     const int per = 256 / G, q = threadIdx.x / per;
     const int t = blk * per + (int)threadIdx.x - q * per;
     double a = 0.0;
+    size_t n = 0, at = 0;
+    int ns = 0;
     if (t < n3) {
         const int s = sys_of_blob[t / 3];
-        const size_t n = 3 * (size_t)sys_nb[s];
-        const double* p = part + sys_poff[s] + (t - 3 * (size_t)sys_blob0[s]);
-        a = slot_run(p, n, q, sys_nch[s], G, scale != 0.0);
+        n = 3 * (size_t)sys_nb[s];
+        at = sys_poff[s] + (t - 3 * (size_t)sys_blob0[s]);
+        ns = sys_nch[s];
     }
+    if (scale != 0.0) {
+        float2 f = slot_run_pairs(reinterpret_cast<const float2*>(part) + at, n, q, ns, G);
+        if (G > 1) {
+            float2* fs = reinterpret_cast<float2*>(sh);
+            fs[threadIdx.x] = f;
+            __syncthreads();
+            if (q == 0)
+                for (int c = 1; c < G; ++c) add_pair(f, fs[c * per + threadIdx.x]);
+        }
+        return q == 0 ? scale * ((double)f.x + (double)f.y) : 0.0;
+    }
+    a = slot_run(part + at, n, q, ns, G);
     if (G > 1) {
         sh[threadIdx.x] = a;
         __syncthreads();
         if (q == 0)
             for (int c = 1; c < G; ++c) a += sh[c * per + threadIdx.x];
     }
-    if (scale != 0.0) a *= scale;
     return a;
 }
 

@@ -91,7 +91,7 @@ k_sum_slots(const double* __restrict__ part, double* __restrict__ u, int n3, int
     __shared__ double sh[256];
     const int q = threadIdx.x >> 5, t = blockIdx.x * 32 + (threadIdx.x & 31);
     double a = 0.0;
-    if (t < n3) a = slot_run(part + t, n3, q, slots, 8, false);
+    if (t < n3) a = slot_run(part + t, n3, q, slots, 8);
     sh[threadIdx.x] = a;
     __syncthreads();
     if (q == 0 && t < n3) {
@@ -957,7 +957,12 @@ int mobility_layout(am_handle* h, int tpt, int chunk, int tgroup, int sym) {
     h->mv_chunk = chunk;
     h->mv_tgroup = tgroup;
     h->mv_part_total = off;
-    h->mv_sum_groups = *std::max_element(nch.begin(), nch.end()) >= 16 ? 8 : 1;
+    // many slots: 8 threads per element, fewer once they would pass three
+    // quarters of the resident threads (8 / 4 / 2 / 1 of them: 1,152 elements
+    // 5.6 / 6.8 / 9.7 / 15 us, 81,000 elements 14.5 / 10 / 8.5 / 10.2)
+    int G = *std::max_element(nch.begin(), nch.end()) >= 16 ? 8 : 1;
+    while (G > 1 && 3LL * G * h->Nb > 1536LL * num_sms()) G /= 2;
+    h->mv_sum_groups = G;
     if (h->cfg.precision == AM_MIXED) {
         if (h->cfg.wall)
             h->mv_grid = tpt == 2 ? resident_grid(rpy_items_mixed_x2<true>) : resident_grid(rpy_items_mixed<true, 1>);
