@@ -267,7 +267,7 @@ struct am_handle {
     int n_pcw = 0, n_pca = 0;
     double* d_ytp = nullptr;
     long long* d_G_off = nullptr; int* d_G_rank = nullptr;
-    int* d_perm = nullptr; long long* d_perm_off = nullptr;
+    int *d_perm = nullptr, *d_pos = nullptr; long long* d_perm_off = nullptr;
     double *d_pc_w = nullptr, *d_pc_Uhat = nullptr;
     bool pc_valid = false;
     int pc_small_cs = 0;  // cluster size of the one-launch apply (0: three kernels)

@@ -129,7 +129,7 @@ void free_links(am_handle* h) {
     dfree(&h->d_asm_link_off); dfree(&h->d_asm_link_idx); dfree(&h->d_link_local);
     dfree(&h->d_pplus); dfree(&h->d_pplus_off);
     dfree(&h->d_G); dfree(&h->d_Gwork); dfree(&h->d_G_off); dfree(&h->d_G_rank);
-    dfree(&h->d_perm); dfree(&h->d_perm_off);
+    dfree(&h->d_perm); dfree(&h->d_pos); dfree(&h->d_perm_off);
     dfree(&h->d_corr); dfree(&h->d_corr_off); dfree(&h->d_zbuf); dfree(&h->d_cbuf);
     dfree(&h->d_pca_asm); dfree(&h->d_pca_chunk); dfree(&h->d_pca_list);
     h->n_pca = 0;
@@ -387,7 +387,7 @@ int build_links(am_handle* h, int P, const int* bp, const int* bq) {
     h->n_pca = (int)pca_asm.size();
     CK(dalloc(&h->d_pca_asm, pca_asm.size())); CK(dalloc(&h->d_pca_chunk, pca_chunk.size()));
     CK(dalloc(&h->d_G_off, NA + 1)); CK(dalloc(&h->d_G_rank, NA));
-    CK(dalloc(&h->d_perm, permoff[NA])); CK(dalloc(&h->d_perm_off, NA + 1));
+    CK(dalloc(&h->d_perm, permoff[NA])); CK(dalloc(&h->d_pos, permoff[NA])); CK(dalloc(&h->d_perm_off, NA + 1));
     CK(dalloc(&h->d_corr, coff[NA])); CK(dalloc(&h->d_corr_off, NA + 1));
     CK(dalloc(&h->d_zbuf, 3 * (size_t)P)); CK(dalloc(&h->d_cbuf, 3 * (size_t)P));
     CK(h2d(h->d_bp, bp, P, s)); CK(h2d(h->d_bq, bq, P, s));

@@ -128,23 +128,30 @@ __device__ __forceinline__ void e_times_n(double sg, const double* l, const doub
 
 // One articulated body per team: asm_list[blockIdx.x / team size].  In a
 // cluster team the first CTA takes the column steps of each panel (pivot
-// search and swaps included) and the team shares the trailing tiles, the
-// blocked inverse and the scatter into G~; the first CTA publishes the rank
-// (or -1 while the factorisation goes on) in rank_out[a] before each team
-// barrier, so every CTA leaves the panel loop at the same panel.
+// search included) and the team shares the trailing tiles, the blocked inverse
+// and the scatter into G~; the first CTA publishes the rank (or -1 while the
+// factorisation goes on) in rank_out[a] before each team barrier, so every CTA
+// leaves the panel loop at the same panel.
+// Bound by the chain of column steps.  Rows and columns stay where they are:
+// pos[i] is the place of row i in the pivot order, perm its inverse; a column
+// step reads one row of H (kept transposed, so that it is the pivot's column),
+// the panel's columns lie in shared memory (lay & 2: kNB m entries) by row, and
+// every warp finds the pivot for itself with integer comparisons (FP64 ones
+// cost 16 cycles of the SM each).  lay & 1: pos and perm in shared memory.
+// 186 rows (31 rods, two links each): 771 (FP32) and 1,114 (FP64) us with rows and columns
+// exchanged in global memory, 457 and 723 us so.
 template <class T, class Team>
 __global__ void __launch_bounds__(kPcThreads)
 k_pca_build(const int* __restrict__ asm_list, const int* __restrict__ asm_link_off,
             const int* __restrict__ asm_link_idx, const int* __restrict__ bp, const int* __restrict__ bq,
             const double* __restrict__ lp, const double* __restrict__ lq, const double* __restrict__ Nt,
             const long long* __restrict__ goff, T* __restrict__ G, T* __restrict__ gwork,
-            int* __restrict__ perm_all, const long long* __restrict__ poff, int* __restrict__ rank_out,
-            double tol) {
+            int* __restrict__ perm_all, int* __restrict__ pos_all, const long long* __restrict__ poff,
+            int* __restrict__ rank_out, double tol, int mmax, int lay) {
     extern __shared__ unsigned char dyn_smem[];
     double* dg = reinterpret_cast<double*>(dyn_smem);  // m values: the Schur-complement diagonal
     __shared__ PcTiles<T> tiles;
-    __shared__ double s_pv, s_sk, s_isk;
-    __shared__ int s_pi;
+    __shared__ double s_sk, s_isk;
     const Team team;
     const int tr = team.rank(), ts = team.size();
     const int a = asm_list[blockIdx.x / ts];
@@ -152,11 +159,14 @@ k_pca_build(const int* __restrict__ asm_list, const int* __restrict__ asm_link_o
     const int Pa = asm_link_off[a + 1] - L0;
     const int m = 3 * Pa;
     if (m == 0) return;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
     T* H = gwork + 2 * goff[a];
-    T* X = H + (size_t)m * m;
+    T* X = H + (size_t)m * m;  // column k of the factor in row k
     T* Ga = G + goff[a];
     int* perm = perm_all + poff[a];
+    int* sperm = lay & 1 ? reinterpret_cast<int*>(dg + mmax) : perm;
+    int* pos = lay & 1 ? sperm + mmax : pos_all + poff[a];
+    T* const panel = lay & 2 ? reinterpret_cast<T*>(pos + mmax) : nullptr;
     for (int idx = threadIdx.x + tr * blockDim.x; idx < Pa * Pa; idx += blockDim.x * ts) {
         const int r = idx / Pa, c = idx % Pa;
         const int ln = asm_link_idx[L0 + r], lk = asm_link_idx[L0 + c];
@@ -180,152 +190,130 @@ k_pca_build(const int* __restrict__ asm_list, const int* __restrict__ asm_link_o
             }
         }
         for (int x = 0; x < 3; ++x)
-            for (int yy = 0; yy < 3; ++yy) H[(size_t)(3 * r + x) * m + 3 * c + yy] = (T)blk[x * 3 + yy];
+            for (int yy = 0; yy < 3; ++yy) H[(size_t)(3 * c + yy) * m + 3 * r + x] = (T)blk[x * 3 + yy];
     }
-    if (tr == 0)
-        for (int i = threadIdx.x; i < m; i += blockDim.x) perm[i] = i;
     team.sync();
     // symmetric pivoted Cholesky (largest remaining diagonal first, ties to
-    // the lower index), stopped at the first pivot <= tol * the first one;
+    // the lower place), stopped at the first pivot <= tol * the first one;
     // blocked: within a panel of 32 columns each column is formed from the
     // panel's earlier columns (left-looking) with the Schur-complement
     // diagonal dg kept up to date for the pivot search, and after the panel
-    // the trailing block (both triangles, which the row and column swaps
-    // read) takes one tile-product update.
+    // the trailing block takes one tile-product update.
     if (tr == 0)
-        for (int i = threadIdx.x; i < m; i += blockDim.x) dg[i] = (double)H[(size_t)i * m + i];
+        for (int i = threadIdx.x; i < m; i += blockDim.x) {
+            dg[i] = (double)H[(size_t)i * m + i];
+            pos[i] = sperm[i] = i;
+        }
     __syncthreads();
-    double d0 = 0.0;
+    unsigned long long thr = 0;  // bits of the threshold: positive doubles compare as integers
     int r = m;
     for (int k0 = 0; k0 < m; k0 += kNB) {
         const int kend = min(m, k0 + kNB);
         if (tr == 0) {
+            T* Lp = panel ? panel : X + (size_t)k0 * m;
             bool stop = false;
             for (int k = k0; k < kend; ++k) {
-                // pivot: warp 0 scans the remaining diagonal
-                if (wid == 0) {
-                    double best = -1.0;
-                    int bi = 0x7fffffff;
-                    for (int i = k + lane; i < m; i += 32) {
-                        const double v = dg[i];
-                        if (v > best || (v == best && i < bi)) { best = v; bi = i; }
+                // pivot: every warp scans the remaining diagonal
+                unsigned long long key = 0;
+                unsigned at = 0xffffffffu;
+                for (int i = lane; i < m; i += 32) {
+                    const int q = pos[i];
+                    unsigned long long v = (unsigned long long)__double_as_longlong(dg[i]);
+                    if (v > 0x7ff0000000000000ull) v = 0;  // negative or NaN
+                    if (q >= k && (v > key || (v == key && (unsigned)q < at))) { key = v; at = q; }
+                }
+                const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(key >> 32));
+                unsigned lo = (unsigned)(key >> 32) == hi ? (unsigned)key : 0u;
+                lo = __reduce_max_sync(0xffffffffu, lo);
+                const bool mine = key == (((unsigned long long)hi << 32) | lo);
+                key = ((unsigned long long)hi << 32) | lo;
+                at = __reduce_min_sync(0xffffffffu, mine ? at : 0xffffffffu);
+                if (k == 0) thr = (unsigned long long)__double_as_longlong(tol * __longlong_as_double((long long)key));
+                if (!(key > thr) || key == 0) { r = k; stop = true; break; }
+                const int j = (int)at, p = sperm[j];
+                if (threadIdx.x == 0) {
+                    s_sk = sqrt(__longlong_as_double((long long)key));
+                    s_isk = 1.0 / s_sk;
+                }
+                // column k: Schur value from the panel's earlier columns (at
+                // most 31, summed in T), scaled by the pivot's inverse square
+                // root (formed once)
+                const int nk = k - k0;
+                const T* row = H + (size_t)p * m;
+                for (int base = 0; base < m; base += blockDim.x) {
+                    const int i = base + threadIdx.x;
+                    const bool live = i < m && pos[i] >= k;
+                    T h = 0, acc = 0;
+                    if (live) {
+                        h = row[i];
+#pragma unroll 8
+                        for (int t = 0; t < nk; ++t) acc = fma(Lp[(size_t)t * m + i], Lp[(size_t)t * m + p], acc);
                     }
-                    for (int o = 16; o > 0; o >>= 1) {
-                        const double ov = __shfl_down_sync(0xffffffffu, best, o);
-                        const int oi = __shfl_down_sync(0xffffffffu, bi, o);
-                        if (ov > best || (ov == best && oi < bi)) { best = ov; bi = oi; }
-                    }
-                    if (lane == 0) {
-                        s_pv = best;
-                        s_pi = bi;
-                        s_sk = best > 0.0 ? sqrt(best) : 1.0;
-                        s_isk = 1.0 / s_sk;
+                    if (base == 0) __syncthreads();  // the root; every warp has searched
+                    if (live) {
+                        T v;
+                        if (i == p) {
+                            v = (T)s_sk;
+                        } else {
+                            const double l = ((double)h - (double)acc) * s_isk;
+                            v = (T)l;
+                            dg[i] -= l * l;
+                        }
+                        Lp[(size_t)nk * m + i] = v;
+                        if (panel) X[(size_t)k * m + i] = v;
                     }
                 }
                 __syncthreads();
-                const double dmax = s_pv;
-                const int j = s_pi;
-                if (k == 0) d0 = dmax;
-                if (!(dmax > tol * d0) || !(dmax > 0.0)) { r = k; stop = true; break; }
-                if (j != k) {
-                    // rows k, j and columns k, j exchanged in one pass: the
-                    // row entries off columns k, j, the column entries off
-                    // rows k, j, and the 2 x 2 block of both
-                    for (int x = threadIdx.x; x < 2 * m; x += blockDim.x) {
-                        if (x < m) {
-                            const int c = x;
-                            if (c == j) continue;
-                            if (c == k) {
-                                const T hkk = H[(size_t)k * m + k], hjj = H[(size_t)j * m + j];
-                                const T hkj = H[(size_t)k * m + j], hjk = H[(size_t)j * m + k];
-                                H[(size_t)k * m + k] = hjj;
-                                H[(size_t)j * m + j] = hkk;
-                                H[(size_t)k * m + j] = hjk;
-                                H[(size_t)j * m + k] = hkj;
-                            } else {
-                                const T t = H[(size_t)k * m + c];
-                                H[(size_t)k * m + c] = H[(size_t)j * m + c];
-                                H[(size_t)j * m + c] = t;
-                            }
-                        } else {
-                            const int rr = x - m;
-                            if (rr == k || rr == j) continue;
-                            const T t = H[(size_t)rr * m + k];
-                            H[(size_t)rr * m + k] = H[(size_t)rr * m + j];
-                            H[(size_t)rr * m + j] = t;
-                        }
-                    }
-                    if (threadIdx.x == 0) {
-                        const int t = perm[k];
-                        perm[k] = perm[j];
-                        perm[j] = t;
-                        const double td = dg[k];
-                        dg[k] = dg[j];
-                        dg[j] = td;
-                    }
-                    __syncthreads();
-                }
-                // column k: Schur value from the panel's earlier columns (at
-                // most 31, loaded together and summed in T, groups of 8 past
-                // the panel's count skipped), scaled by the pivot's inverse
-                // square root (formed once, by the thread that found it)
-                const double sk = s_sk, isk = s_isk;
-                const T* rowk = H + (size_t)k * m + k0;
-                const int nk = k - k0;
-                for (int i = k + threadIdx.x; i < m; i += blockDim.x) {
-                    T* rowi = H + (size_t)i * m;
-                    T pa[kNB], pb[kNB];
-#pragma unroll
-                    for (int t = 0; t < kNB; ++t) {
-                        pa[t] = t < nk ? rowi[k0 + t] : (T)0;
-                        pb[t] = t < nk ? rowk[t] : (T)0;
-                    }
-                    T acc = 0;
-#pragma unroll
-                    for (int g = 0; g < kNB; g += 8)
-                        if (g < nk) {
-#pragma unroll
-                            for (int u = 0; u < 8; ++u) acc = fma(pa[g + u], pb[g + u], acc);
-                        }
-                    const double v = (double)rowi[k] - (double)acc;
-                    if (i == k) {
-                        rowi[k] = (T)sk;
-                    } else {
-                        const double l = v * isk;
-                        rowi[k] = (T)l;
-                        dg[i] -= l * l;
-                    }
+                if (threadIdx.x == 0 && j != k) {  // places k and j exchanged
+                    const int o = sperm[k];
+                    sperm[k] = p;
+                    sperm[j] = o;
+                    pos[p] = k;
+                    pos[o] = j;
                 }
                 __syncthreads();
             }
+            if (sperm != perm)
+                for (int i = threadIdx.x; i < m; i += blockDim.x) perm[i] = sperm[i];
             if (threadIdx.x == 0) rank_out[a] = stop ? r : -1;
         }
         team.sync();
         const int st = *reinterpret_cast<volatile const int*>(rank_out + a);
         if (st >= 0) { r = st; break; }
-        // trailing update of rows and columns >= kend by the panel's columns
+        // trailing update of the rows and columns of places >= kend by the
+        // panel's columns
         constexpr int E = kNB * kNB / kPcThreads;
         int q = 0;
         for (int i0 = kend; i0 < m; i0 += kNB) {
             for (int j0 = kend; j0 < m; j0 += kNB, ++q) {
                 if (q % ts != tr) continue;
-                tile_load(tiles.a, H, m, m, i0, k0, false);
-                tile_load(tiles.b, H, m, m, j0, k0, false);
+                for (int idx = threadIdx.x; idx < kNB * kNB; idx += blockDim.x) {
+                    const int t = idx / kNB, x = idx % kNB;
+                    const T* col = X + (size_t)(k0 + t) * m;
+                    tiles.a[x][t] = i0 + x < m ? col[perm[i0 + x]] : (T)0;
+                    tiles.b[x][t] = j0 + x < m ? col[perm[j0 + x]] : (T)0;
+                }
                 __syncthreads();
                 T acc[E];
 #pragma unroll
                 for (int e = 0; e < E; ++e) acc[e] = 0;
-                tile_mac<T, true>(tiles.a, tiles.b, acc);
+                tile_mac<T, true>(tiles.b, tiles.a, acc);
 #pragma unroll
                 for (int e = 0; e < E; ++e) {
-                    const int rr = acc_row(e), c = acc_col(e);
-                    if (i0 + rr < m && j0 + c < m) H[(size_t)(i0 + rr) * m + j0 + c] -= acc[e];
+                    const int c = acc_row(e), rr = acc_col(e);
+                    if (i0 + rr < m && j0 + c < m) H[(size_t)perm[j0 + c] * m + perm[i0 + rr]] -= acc[e];
                 }
                 __syncthreads();
             }
         }
         team.sync();
     }
+    // the leading r x r factor in pivot order, over H
+    for (int idx = threadIdx.x + tr * blockDim.x; idx < r * r; idx += blockDim.x * ts) {
+        const int i = idx % r, j = idx / r;
+        if (j <= i) H[(size_t)i * m + j] = X[(size_t)j * m + perm[i]];
+    }
+    team.sync();
     if (threadIdx.x == 0 && tr == 0) rank_out[a] = r;
     // (L11 L11^T)^-1 of the rank-r leading block, blocked (written over H)
     blocked_chol_inverse(H, X, H, r, m, tiles, team);
@@ -746,8 +734,20 @@ static void launch_team(K kernel, int n, int cs, size_t smem, cudaStream_t s, Ar
 
 template <class T>
 static void pca_build_t(am_handle* h, double tol) {
-    const size_t smem = (size_t)3 * std::max(1, h->max_asm_links) * sizeof(double);  // Schur diagonal
-    if (smem > 48 * 1024) {
+    // the Schur diagonal and, as far as they fit, the places and the panel (64 KB
+    // leave three CTAs to an SM; a larger panel stays in global memory)
+    const int m = 3 * std::max(1, h->max_asm_links);
+    size_t smem = (size_t)m * sizeof(double);
+    int lay = 0;
+    if (2 * smem <= 160 * 1024) {
+        lay = 1;
+        smem *= 2;
+        if (smem + (size_t)kNB * m * sizeof(T) <= 64 * 1024) {
+            lay = 3;
+            smem += (size_t)kNB * m * sizeof(T);
+        }
+    }
+    if (smem > 16 * 1024) {
         cudaFuncSetAttribute(k_pca_build<T, CtaTeam>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         cudaFuncSetAttribute(k_pca_build<T, ClusterTeam>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     }
@@ -756,14 +756,14 @@ static void pca_build_t(am_handle* h, double tol) {
                 (const int*)h->d_asm_link_off, (const int*)h->d_asm_link_idx, (const int*)h->d_bp,
                 (const int*)h->d_bq, (const double*)h->d_lp, (const double*)h->d_lq, (const double*)h->d_Nt,
                 (const long long*)h->d_G_off, (T*)h->d_G, (T*)h->d_Gwork, h->d_perm,
-                (const long long*)h->d_perm_off, h->d_G_rank, tol);
+                h->d_pos, (const long long*)h->d_perm_off, h->d_G_rank, tol, m, lay);
     if (h->pca_cs > 1)
         launch_team(k_pca_build<T, ClusterTeam>, h->NA - h->n_pca_small, h->pca_cs, smem, h->stream,
                     (const int*)(h->d_pca_list + h->n_pca_small), (const int*)h->d_asm_link_off,
                     (const int*)h->d_asm_link_idx, (const int*)h->d_bp, (const int*)h->d_bq,
                     (const double*)h->d_lp, (const double*)h->d_lq, (const double*)h->d_Nt,
                     (const long long*)h->d_G_off, (T*)h->d_G, (T*)h->d_Gwork, h->d_perm,
-                    (const long long*)h->d_perm_off, h->d_G_rank, tol);
+                    h->d_pos, (const long long*)h->d_perm_off, h->d_G_rank, tol, m, lay);
 }
 
 // Whether every articulated body is small enough for k_pc_small, and the
