@@ -443,12 +443,18 @@ __device__ __forceinline__ void pair2_sym(float2 dx, float2 dy, float2 dz, float
 // of 128 and nearly half on tiles of 64.  A tile against itself meets every
 // ordered pair (the self term included) and drops the column sums: a second,
 // one-direction form of the pair in the loop cost 6 to 12 % by its code size.
-// Bound by FP32 issue on large systems; the small tiles spread systems of a few
-// thousand blobs over every SM and keep an item at 16 (T = 32) or 32 steps.
-// Tiles of 64 against one target per lane with FP64 sums: 16 free systems of
-// 500 to 4,000 blobs 71.5 -> 56 us, the 3,600-blob colony above a wall 22.5 ->
-// 17.1.  Free space: 24 warps per SM (80 registers) 54 us, 16 warps 57; wall:
-// 113 registers, fewer cost more than the warps bring (17.1, 17.7).
+// Bound by issue and the FP32 pipe (32,000 wall blobs: issue slots 60 %, FP32
+// pipe 65 % busy); the small tiles spread systems of a few thousand blobs over
+// every SM and keep an item at 16 (T = 32) or 32 steps.  Sources are staged once
+// per value and doubled in registers: staged as ready pairs they took twice the
+// shared-memory wavefronts.  Every sub-tile lies twice in a row, so that a
+// lane's index needs no wrap and the loads of four steps share an address.
+// Tiles of 128 at 32,000 blobs, free / wall: 998 / 1,590 us with both pairs and
+// wrap, 937 / 1,568 without pairs, 911 / 1,493 now.  Tiles of 64 against one
+// target per lane with FP64 sums: 16 free systems of 500 to 4,000 blobs 71.5 ->
+// 54 us, the 2,560-blob colony above a wall 22.5 -> 16.7.  Free space: 24 warps
+// per SM (80 registers) take 5 % less time than 16; wall: 113 registers, fewer
+// cost more than the warps bring (17.1 us, 17.7).
 template <bool WALL, int T>
 __global__ void __launch_bounds__(T, (WALL ? 512 : 768) / T)
 rpy_sym_mixed(const float4* __restrict__ hi, const float4* __restrict__ lo, const float4* __restrict__ lf,
@@ -456,9 +462,10 @@ rpy_sym_mixed(const float4* __restrict__ hi, const float4* __restrict__ lo, cons
                  int n_items, int* __restrict__ counter, RpyK<float> k, const int* __restrict__ active) {
     dep_wait();
     constexpr int LW = T == 32 ? 16 : 32, NG = T / LW, H = T / (2 * LW);
-    __shared__ float4 sq[3][T];   // sources: (-hx, -hx, -hy, -hy), (2hz, 2hz, lz, lz), (lx, lx, ly, ly)
-    __shared__ float4 so[T];      // (-ox, -ox, -oy, -oy)
-    __shared__ float2 soz[T];     // (-oz, -oz)
+    // sources, every sub-tile twice in a row (a lane's index then never wraps)
+    __shared__ float4 sq[2 * T];             // (-hx, -hy, 2hz, lx)
+    __shared__ float2 sl[2 * T], so[2 * T];  // (ly, lz), (-ox, -oy)
+    __shared__ float soz[2 * T];             // -oz
     __shared__ float2 acc[3][T];       // row sums of the tile's targets: (hi, lo)
     __shared__ float up[NG][3][2 * LW];  // row sums of each team's targets over a tile of sources
     __shared__ float vp[NG][H][3][LW];   // column sums of each team's sub-tiles
@@ -510,11 +517,14 @@ rpy_sym_mixed(const float4* __restrict__ hi, const float4* __restrict__ lo, cons
                     const int i = m.j0 + jb + q;
                     const float4 h = ok ? hi[i] : make_float4(0.f, 0.f, 1.f, 0.f);
                     const float4 o = ok ? lo[i] : none, f = ok ? lf[i] : none;
-                    sq[0][q] = make_float4(-h.x, -h.x, -h.y, -h.y);
-                    sq[1][q] = make_float4(2.f * h.z, 2.f * h.z, f.z, f.z);
-                    sq[2][q] = make_float4(f.x, f.x, f.y, f.y);
-                    so[q] = make_float4(-o.x, -o.x, -o.y, -o.y);
-                    soz[q] = make_float2(-o.z, -o.z);
+                    const int at = q + (q / LW) * LW;
+#pragma unroll
+                    for (int c = 0; c <= LW; c += LW) {
+                        sq[at + c] = make_float4(-h.x, -h.y, 2.f * h.z, f.x);
+                        sl[at + c] = make_float2(f.y, f.z);
+                        so[at + c] = make_float2(-o.x, -o.y);
+                        soz[at + c] = -o.z;
+                    }
                 }
                 __syncthreads();
                 float2 ux = bc2(0.f), uy = bc2(0.f), uz = bc2(0.f);
@@ -522,29 +532,28 @@ rpy_sym_mixed(const float4* __restrict__ hi, const float4* __restrict__ lo, cons
                 for (int sbi = 0; sbi < H; ++sbi) {
                     const int sb = sb0 + sbi;
                     float vx = 0.f, vy = 0.f, vz = 0.f;  // column sum of source LW sb + (lane + t + 1) % LW
-#pragma unroll 2
+#pragma unroll 4
                     for (int t = 0; t < LW; ++t) {
-                        const int q = LW * sb + ((lane + t + 1) & (LW - 1));
-                        const float4 v0 = sq[0][q], v1 = sq[1][q], v2 = sq[2][q];
-                        const float2 h2 = make_float2(v1.x, v1.y);
-                        float2 dx = add2(HX, make_float2(v0.x, v0.y));
-                        float2 dy = add2(HY, make_float2(v0.z, v0.w));
+                        const int q = 2 * LW * sb + lane + 1 + t;
+                        const float4 v = sq[q];
+                        const float2 l = sl[q];
+                        const float2 h2 = bc2(v.z);
+                        float2 dx = add2(HX, bc2(v.x));
+                        float2 dy = add2(HY, bc2(v.y));
                         float2 dz = fma2(h2, bc2(-0.5f), HZ);
                         const float2 Rz = fma2(h2, bc2(0.5f), HZ);
                         float2 rxy2 = fma2(dx, dx, mul2(dy, dy));
                         float2 r2 = fma2(dz, dz, rxy2);
                         if (r2.x < near2x || r2.y < near2y) {
-                            const float4 o = so[q];
-                            dx = add2(dx, add2(LX, make_float2(o.x, o.y)));
-                            dy = add2(dy, add2(LY, make_float2(o.z, o.w)));
-                            dz = add2(dz, add2(LZ, soz[q]));
+                            const float2 o = so[q];
+                            dx = add2(dx, add2(LX, bc2(o.x)));
+                            dy = add2(dy, add2(LY, bc2(o.y)));
+                            dz = add2(dz, add2(LZ, bc2(soz[q])));
                             rxy2 = fma2(dx, dx, mul2(dy, dy));
                             r2 = fma2(dz, dz, rxy2);
                         }
-                        const float2 lxs = make_float2(v2.x, v2.y), lys = make_float2(v2.z, v2.w),
-                                     lzs = make_float2(v1.z, v1.w);
                         float2 cx = bc2(0.f), cy = bc2(0.f), cz = bc2(0.f);
-                        pair2_sym<WALL>(dx, dy, dz, rxy2, r2, Rz, h2, NX3, lxs, lys, lzs, MX, MY, MZ, k, ux, uy, uz,
+                        pair2_sym<WALL>(dx, dy, dz, rxy2, r2, Rz, h2, NX3, bc2(v.w), bc2(l.x), bc2(l.y), MX, MY, MZ, k, ux, uy, uz,
                                         cx, cy, cz);
                         vx += cx.x + cx.y;
                         vy += cy.x + cy.y;
@@ -1108,8 +1117,8 @@ int mobility_autotune(am_handle* h) {
     // partial sums (one slot per tile of the system) stay within 1 GiB; mixed
     // on groups of 128-blob tiles while they stay within a quarter of the free
     // device memory (1.4 GB for 360,000 blobs).  Mixed product and sum, one
-    // system above a wall, tiles of 32 / 64 / 128: 2,000 blobs 22 / 33 / 53 us,
-    // 4,000 38 / 45 / 67, 8,000 122 / 113 / 144, 32,000 1,819 / 1,664 / 1,622
+    // system above a wall, tiles of 32 / 64 / 128: 2,000 blobs 21 / 32 / 51 us,
+    // 4,000 36 / 43 / 63, 8,000 117 / 112 / 130, 32,000 1,757 / 1,608 / 1,510
     for (int nsub : mixed ? std::vector<int>{1, 2} : std::vector<int>{1, 2, 4}) {
         long long slots = 0;
         for (const auto& r : h->sys) slots += (long long)((r.Nb + 32 * nsub - 1) / (32 * nsub)) * 3 * r.Nb;
