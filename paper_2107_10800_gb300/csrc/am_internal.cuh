@@ -259,7 +259,11 @@ struct am_handle {
     // body preconditioner build: bodies of <= 64 rows first (n_pcb_small),
     // then the larger ones, built by clusters of pcb_cs CTAs when pcb_cs > 1
     int* d_pcb_list = nullptr;
-    int n_pcb_small = 0, pcb_cs = 1;
+    int n_pcb = 0, n_pcb_small = 0, pcb_cs = 1;
+    // bodies rotated from a body of their shape instead: (body, that body,
+    // first blob, blobs) per block
+    int4* d_pcb_copy = nullptr;
+    int n_pcb_copy = 0;
     // the same for the articulated-body build (by 3 x links rows)
     int* d_pca_list = nullptr;
     int n_pca_small = 0, pca_cs = 1;

@@ -9,6 +9,7 @@
 #include <cstring>
 #include <numeric>
 #include <string>
+#include <unordered_map>
 #include <vector>
 
 namespace am {
@@ -121,6 +122,44 @@ void split_for_build(const std::vector<int>& rows, std::vector<int>& list, int& 
     }
 }
 
+// For every body the first one of its shape (the same blobs in the body frame,
+// bit for bit), whose preconditioner blocks are rotated to it.  Above a wall a
+// block depends on the pose, and while the bodies fit the SMs at once (small
+// ones a CTA each, large ones eight) all are built in the time of one: then
+// every body is its own.  Of dependent links the factorisation of the link
+// block keeps the same number, but which of equal ones is a matter of rounding.
+std::vector<int> same_shapes(bool wall, int M, const int* off, const double* rho) {
+    std::vector<int> first(M);
+    long long small = 0, large = 0;
+    for (int p = 0; p < M; ++p) {
+        first[p] = p;
+        ++(3 * (off[p + 1] - off[p]) <= 2 * 32 ? small : large);
+    }
+    if (wall || (small <= am::num_sms() && 8 * large <= am::num_sms())) return first;
+    std::unordered_map<unsigned long long, std::vector<int>> seen;
+    for (int p = 0; p < M; ++p) {
+        const size_t n = 3 * (size_t)(off[p + 1] - off[p]);
+        if (n == 0) continue;
+        const double* x = rho + 3 * (size_t)off[p];
+        unsigned long long key = n;
+        for (size_t i = 0; i < n; ++i) {
+            unsigned long long bits;
+            std::memcpy(&bits, x + i, 8);
+            key = (key ^ bits) * 0x9e3779b97f4a7c15ull;
+            key ^= key >> 29;
+        }
+        std::vector<int>& same = seen[key];
+        for (int q : same)
+            if (off[q + 1] - off[q] == off[p + 1] - off[p] &&
+                std::memcmp(rho + 3 * (size_t)off[q], x, n * sizeof(double)) == 0) {
+                first[p] = q;
+                break;
+            }
+        if (first[p] == p) same.push_back(p);
+    }
+    return first;
+}
+
 void free_links(am_handle* h) {
     dfree(&h->d_bp); dfree(&h->d_bq); dfree(&h->d_dlp); dfree(&h->d_dlq);
     dfree(&h->d_dlpd); dfree(&h->d_dlqd); dfree(&h->d_dlp1); dfree(&h->d_dlq1);
@@ -145,7 +184,8 @@ void free_bodies(am_handle* h) {
     dfree(&h->d_minv); dfree(&h->d_pcwork); dfree(&h->d_Y); dfree(&h->d_Nt); dfree(&h->d_minv_off);
     dfree(&h->d_pc_w); dfree(&h->d_pc_Uhat); dfree(&h->d_mv); dfree(&h->d_lf);
     dfree(&h->d_pcw_body); dfree(&h->d_pcw_chunk); dfree(&h->d_pcw_off); dfree(&h->d_ytp); dfree(&h->d_pcb_cnt);
-    dfree(&h->d_pcb_list);
+    dfree(&h->d_pcb_list); dfree(&h->d_pcb_copy);
+    h->n_pcb = h->n_pcb_copy = 0;
     h->n_pcb_small = 0;
     h->pcb_cs = 1;
     h->n_pcw = 0;
@@ -657,10 +697,25 @@ int build_layout(am_handle* h, int M, int Nb, int NA, int maxb, const double* q,
         pcw_off[p + 1] = (int)pcw_body.size();
     }
     h->n_pcw = (int)pcw_body.size();
-    std::vector<int> pcb_rows(M), pcb_list;
-    for (int p = 0; p < M; ++p) pcb_rows[p] = 3 * (blob_offset[p + 1] - blob_offset[p]);
+    const std::vector<int> shape = same_shapes(h->cfg.wall != 0, M, blob_offset, rho);
+    std::vector<int> pcb_rows, pcb_list, built;
+    std::vector<int4> pcb_copy;
+    for (int p = 0; p < M; ++p) {
+        const int n = blob_offset[p + 1] - blob_offset[p];
+        if (shape[p] == p) {
+            built.push_back(p);
+            pcb_rows.push_back(3 * n);
+            continue;
+        }
+        const int step = std::min(n, std::max(1, 2048 / n));  // about eight blob pairs per thread
+        for (int i = 0; i < n; i += step) pcb_copy.push_back(make_int4(p, shape[p], i, std::min(step, n - i)));
+    }
     split_for_build(pcb_rows, pcb_list, h->n_pcb_small, h->pcb_cs);
-    CK(dalloc(&h->d_pcb_list, std::max(M, 1)));
+    for (int& p : pcb_list) p = built[p];
+    h->n_pcb = (int)built.size();
+    h->n_pcb_copy = (int)pcb_copy.size();
+    CK(dalloc(&h->d_pcb_list, std::max(h->n_pcb, 1)));
+    CK(dalloc(&h->d_pcb_copy, std::max(h->n_pcb_copy, 1)));
     CK(dalloc(&h->d_pcw_body, pcw_body.size())); CK(dalloc(&h->d_pcw_chunk, pcw_chunk.size()));
     CK(dalloc(&h->d_pcw_off, M + 1)); CK(dalloc(&h->d_ytp, 6 * pcw_body.size()));
     CK(dalloc(&h->d_pcb_cnt, M));
@@ -684,7 +739,8 @@ int build_layout(am_handle* h, int M, int Nb, int NA, int maxb, const double* q,
     CK(h2d(h->d_asm_body_idx, h->asm_body_idx.data(), M, s));
     CK(h2d(h->d_body_local, body_local.data(), M, s));
     CK(h2d(h->d_minv_off, moff.data(), M + 1, s));
-    if (M) CK(h2d(h->d_pcb_list, pcb_list.data(), M, s));
+    if (M) CK(h2d(h->d_pcb_list, pcb_list.data(), h->n_pcb, s));
+    if (h->n_pcb_copy) CK(h2d(h->d_pcb_copy, pcb_copy.data(), h->n_pcb_copy, s));
     CK(h2d(h->d_pcw_body, pcw_body.data(), pcw_body.size(), s));
     CK(h2d(h->d_pcw_chunk, pcw_chunk.data(), pcw_chunk.size(), s));
     CK(h2d(h->d_pcw_off, pcw_off.data(), M + 1, s));

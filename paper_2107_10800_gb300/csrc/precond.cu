@@ -5,7 +5,8 @@
 // inverse by blocked Cholesky, blocked triangular inverse and X^T X on 32 x 32
 // shared-memory tiles, Y_p = (M^(pp))^-1 K_p, S_p = K_p^T Y_p and
 // N~_p = S_p^-1 (a body of more than two tiles takes a cluster of CTAs when
-// such bodies are too few to fill the GPU).  Per articulated body a (one
+// such bodies are too few to fill the GPU; of many bodies of one shape, away
+// from a wall, one is built and the others are rotated from it).  Per articulated body a (one
 // block): H_a = C_a N~_a C_a^T and its generalised inverse G~_a
 // (Eq. block_diag_const_res) by symmetric pivoted Cholesky (32-column panels,
 // then the blocked inverse of the rank-r factor):
@@ -113,6 +114,68 @@ k_pcb_build(const int* __restrict__ body_list, const int* __restrict__ blob_off,
         double S[36];
         for (int k = 0; k < 36; ++k) S[k] = sh[k];
         if (!spd6_inverse(S, Nt + 36 * (size_t)b)) atomicOr(flags, kFlagSingular);
+    }
+}
+
+// Q X Q^T of the 3 x 3 block X, rows ld entries apart
+template <class T>
+__device__ __forceinline__ void rotate_block(const T* q, const T* X, T* out, size_t ld) {
+    T t[9];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        const T x0 = X[j], x1 = X[ld + j], x2 = X[2 * ld + j];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) t[3 * i + j] = q[3 * i] * x0 + q[3 * i + 1] * x1 + q[3 * i + 2] * x2;
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+            out[i * ld + j] = t[3 * i] * q[3 * j] + t[3 * i + 1] * q[3 * j + 1] + t[3 * i + 2] * q[3 * j + 2];
+}
+
+// Blocks of bodies that are rotations of a built one (without a wall M^(pp)
+// turns with the body): with Q the rotation between them every 3 x 3 block of
+// (M^(pp))^-1, Y and N~ becomes Q X Q^T.  Item: (body, built body, first blob,
+// blobs).  Bound by FP64 issue (54 multiply-adds per blob pair) and the write of
+// the factors; a factorisation costs m / 2 multiply-adds per entry.  216 bodies
+// of 600 rows and 3,456 of 30 in FP64: every body built 56.5 ms, two built and
+// the others rotated 7.1 + 1.05 ms; 2,240 bodies of 36 rows in FP32: 586 us,
+// 105 + 27.
+template <class T>
+__global__ void __launch_bounds__(256)
+k_pcb_copy(const int4* __restrict__ items, const int* __restrict__ blob_off, const double* __restrict__ theta,
+           const long long* __restrict__ moff, T* __restrict__ minv, T* __restrict__ Y, double* __restrict__ Nt) {
+    __shared__ double Q[9];
+    const int4 it = items[blockIdx.x];
+    const int b = it.x, a = it.y;
+    if (threadIdx.x < 3) {  // column c of R_b R_a^T
+        const int c = threadIdx.x;
+        const double *ta = theta + 4 * (size_t)a, *tb = theta + 4 * (size_t)b;
+        double x, y, z, ox, oy, oz;
+        quat_rotate_inv(ta[0], ta[1], ta[2], ta[3], c == 0, c == 1, c == 2, x, y, z);
+        quat_rotate(tb[0], tb[1], tb[2], tb[3], x, y, z, ox, oy, oz);
+        Q[c] = ox; Q[3 + c] = oy; Q[6 + c] = oz;
+    }
+    __syncthreads();
+    T q[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) q[k] = (T)Q[k];
+    const int n = blob_off[b + 1] - blob_off[b];
+    const size_t m = 3 * (size_t)n;
+    const T* A = minv + moff[a];
+    T* B = minv + moff[b];
+    for (int idx = threadIdx.x; idx < it.w * n; idx += blockDim.x) {
+        const size_t at = 3 * (size_t)(it.z + idx / n) * m + 3 * (idx % n);
+        rotate_block(q, A + at, B + at, m);
+    }
+    for (int idx = threadIdx.x; idx < 2 * it.w; idx += blockDim.x) {
+        const size_t at = 18 * (size_t)(it.z + idx / 2) + 3 * (idx % 2);
+        rotate_block(q, Y + 18 * (size_t)blob_off[a] + at, Y + 18 * (size_t)blob_off[b] + at, 6);
+    }
+    if (it.z == 0 && threadIdx.x < 4) {
+        const size_t at = 18 * (size_t)(threadIdx.x / 2) + 3 * (threadIdx.x % 2);
+        rotate_block(Q, Nt + 36 * (size_t)a + at, Nt + 36 * (size_t)b + at, 6);
     }
 }
 
@@ -788,17 +851,22 @@ static void pc_build_t(am_handle* h, double tol) {
     // routines assume that block size)
     // bodies of one or two 32-row tiles one CTA each; larger bodies one
     // cluster of pcb_cs CTAs each when they are too few to fill the GPU
-    const int n_one = h->pcb_cs > 1 ? h->n_pcb_small : h->M;
+    const int n_one = h->pcb_cs > 1 ? h->n_pcb_small : h->n_pcb;
     launch_team(k_pcb_build<T, CtaTeam>, n_one, 1, 0, s, (const int*)h->d_pcb_list, (const int*)h->d_blob_off,
                 (const double4_32a*)h->d_r4, (const double4_32a*)h->d_d4, (const long long*)h->d_minv_off,
                 (T*)h->d_minv, (T*)h->d_pcwork, (T*)h->d_Y, h->d_Nt, rpy_consts<T>(h->prm), h->cfg.wall,
                 h->d_flags);
     if (h->pcb_cs > 1)
-        launch_team(k_pcb_build<T, ClusterTeam>, h->M - h->n_pcb_small, h->pcb_cs, 0, s,
+        launch_team(k_pcb_build<T, ClusterTeam>, h->n_pcb - h->n_pcb_small, h->pcb_cs, 0, s,
                     (const int*)(h->d_pcb_list + h->n_pcb_small), (const int*)h->d_blob_off,
                     (const double4_32a*)h->d_r4, (const double4_32a*)h->d_d4, (const long long*)h->d_minv_off,
                     (T*)h->d_minv, (T*)h->d_pcwork, (T*)h->d_Y, h->d_Nt, rpy_consts<T>(h->prm),
                     h->cfg.wall, h->d_flags);
+    if (h->n_pcb_copy) {
+        k_pcb_copy<T><<<h->n_pcb_copy, 256, 0, s>>>(h->d_pcb_copy, h->d_blob_off, h->d_theta, h->d_minv_off,
+                                                    (T*)h->d_minv, (T*)h->d_Y, h->d_Nt);
+        count_launch();
+    }
     if (h->P) pca_build_t<T>(h, tol);
 }
 
