@@ -616,8 +616,8 @@ k_pc_ap3(int Nb, int M, const int* __restrict__ pcw_body, const int* __restrict_
 // phi of its articulated body itself (at most 64 rows of G~), so the cluster
 // meets once.  Bound by chains of FP64 and L2 latency.  Measured, three kernels
 // against this one: 4 chains of 8 bodies of 12 blobs in FP64 18.3 us against
-// 15.8; 16 systems of 500 to 4,000 blobs in FP32 57 us
-// against 22.
+// 14.0 (15.8 with a chain's bodies on the warps of one SM); 16 systems of 500 to
+// 4,000 blobs in FP32 57 us against 22.
 constexpr int kSmallRows = 64;
 template <class T>
 __global__ void __launch_bounds__(256)
@@ -638,7 +638,7 @@ k_pc_small(int Nb, int M, const int* __restrict__ asm_body_off, const int* __res
     const int B0 = asm_body_off[a], Ma = asm_body_off[a + 1] - B0;
     const int L0 = asm_link_off ? asm_link_off[a] : 0, mg = asm_link_off ? 3 * (asm_link_off[a + 1] - L0) : 0;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int wg = team.rank() * 8 + wid, W = team.size() * 8;
+    const int wg = wid * team.size() + team.rank(), W = team.size() * 8;  // bodies spread over the SMs first
     // w = M~^-1 r1 and U^ = N~ (-r2 - Y^T r1)
     for (int q = wg; q < Ma; q += W) {
         const int b = asm_body_idx[B0 + q], i0 = blob_off[b], m = 3 * (blob_off[b + 1] - i0);
