@@ -798,28 +798,47 @@ static void product_sym(const double* r, const double* lam, double* u, int n, co
     count_launch(2);
 }
 
-// Mixed: two targets per thread once groups of 64 targets in clusters of 8
-// give every SM two CTAs (2,432 targets); one target per thread spreads fewer
-// targets over more SMs.  Measured, one against two (us, wall): 853 rows of
-// 2,560 blobs 32.8 against 34.1, 1,666 of 5,000 43.6 against 56.7, 2,560 of 2,560
-// 38.7 against 37.9, 4,000 of 12,000 191 against 169, 60,000 of 60,000 9,423
-// against 8,849 (11,790 before, unpaired lanes over split sources).
-constexpr int kPairFrom = 2;
+// the sum of the parts of a cluster product, if there are several
+static void sum_parts(const double* part, double* u, int nt, int parts, cudaStream_t st) {
+    if (parts == 1) return;
+    launch_dep(k_sum_slots, dim3((3 * nt + 31) / 32), dim3(256), 0, st, part, u, 3 * nt, parts);
+    count_launch();
+}
+
+// Mixed: one target per thread, which splits the positions itself (FP64 work,
+// repeated for every group), or two targets per thread on positions split by a
+// launch before: by the time that small_shape expects.
 template <bool WALL>
 static void product_mixed(const double* r, const double* lam, double* u, int n, int t0, int nt, const RpyParams& prm,
-                          char* work, cudaStream_t st) {
+                          char* work, size_t bytes, cudaStream_t st) {
     const RpyK<float> k = rpy_consts<float>(prm);
-    const int groups = (nt + 63) / 64;
-    if (groups * 8 < kPairFrom * num_sms()) {
-        launch_small_t<float, WALL>(r, lam, u, n, t0, nt, k, st);
+    const size_t packed = 2 * align256((size_t)n * sizeof(float4)), slot = 3 * (size_t)nt * sizeof(double);
+    const SmallShape one = small_shape(n, nt, bytes / slot, {16, 32, 1, 8, false, WALL ? 0.060 : 0.040, 0.25, 0.3});
+    const SmallShape two = small_shape(n, nt, (bytes - packed) / slot, {32, 32, 2, 5, false, WALL ? 0.100 : 0.062, 0.4, 0.15});
+    if (one.us <= two.us + 3.0) {
+        double* out = one.parts > 1 ? reinterpret_cast<double*>(work) : u;
+        launch_small_t<float, WALL>(r, lam, out, n, t0, nt, one, k, st);
+        sum_parts(out, u, nt, one.parts, st);
         return;
     }
     float4 *hi = reinterpret_cast<float4*>(work),
            *lo = reinterpret_cast<float4*>(work + align256((size_t)n * sizeof(float4)));
     launch_dep(k_pack_positions, dim3((n + 127) / 128), dim3(128), 0, st, r, hi, lo, n);
     count_launch();
-    launch_cluster(k_rpy_small2<WALL>, groups, groups >= 4 * num_sms() ? 4 : 8, st, (const float4*)hi,
-                   (const float4*)lo, lam, u, n, t0, nt, k);
+    double* out = two.parts > 1 ? reinterpret_cast<double*>(work + packed) : u;
+    launch_cluster(k_rpy_small2<WALL>, (nt + 63) / 64 * two.parts, two.cs, st, (const float4*)hi, (const float4*)lo,
+                   lam, out, n, t0, nt, two.parts, k);
+    sum_parts(out, u, nt, two.parts, st);
+}
+
+template <bool WALL>
+static void product_small(const double* r, const double* lam, double* u, int n, int t0, int nt, const RpyParams& prm,
+                          char* work, size_t bytes, cudaStream_t st) {
+    const SmallShape s = small_shape(n, nt, bytes / (3 * (size_t)nt * sizeof(double)),
+                                     {8, 32, 1, 8, true, WALL ? 2.0 : 0.95, WALL ? 2.0 : 1.0, 0.1});
+    double* out = s.parts > 1 ? reinterpret_cast<double*>(work) : u;
+    launch_small_t<double, WALL>(r, lam, out, n, t0, nt, s, rpy_consts<double>(prm), st);
+    sum_parts(out, u, nt, s.parts, st);
 }
 
 // u = rows t0 .. t0 + nt - 1 of M(r) lambda; `bytes` of scratch at work (at
@@ -828,8 +847,8 @@ cudaError_t product(const double* r, const double* lam, double* u, int n, int t0
                     int wall, int precision, void* work, size_t bytes, cudaStream_t st) {
     const RpyParams prm = make_params(eta, a);
     if (precision == AM_MIXED) {
-        if (wall) product_mixed<true>(r, lam, u, n, t0, nt, prm, static_cast<char*>(work), st);
-        else product_mixed<false>(r, lam, u, n, t0, nt, prm, static_cast<char*>(work), st);
+        if (wall) product_mixed<true>(r, lam, u, n, t0, nt, prm, static_cast<char*>(work), bytes, st);
+        else product_mixed<false>(r, lam, u, n, t0, nt, prm, static_cast<char*>(work), bytes, st);
         return cudaGetLastError();
     }
     if (nt == n && n >= kSymFrom) {
@@ -840,8 +859,8 @@ cudaError_t product(const double* r, const double* lam, double* u, int n, int t0
             return cudaGetLastError();
         }
     }
-    if (wall) launch_small_t<double, true>(r, lam, u, n, t0, nt, rpy_consts<double>(prm), st);
-    else launch_small_t<double, false>(r, lam, u, n, t0, nt, rpy_consts<double>(prm), st);
+    if (wall) product_small<true>(r, lam, u, n, t0, nt, prm, static_cast<char*>(work), bytes, st);
+    else product_small<false>(r, lam, u, n, t0, nt, prm, static_cast<char*>(work), bytes, st);
     return cudaGetLastError();
 }
 

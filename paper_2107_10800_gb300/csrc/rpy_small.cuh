@@ -1,21 +1,25 @@
-// One-direction blob mobility product of few targets on thread-block
-// clusters: u = M lambda in a single launch, without partial sums in memory.
+// One-direction blob mobility product of a range of targets: u = M lambda on
+// thread-block clusters in a single launch, or, for more work, on single CTAs
+// with slots for parts of the sources.
 //
 // A cluster takes a group of G targets (G = 8, 16 or 32) and splits the
 // sources over its CTAs (at most 8); in a CTA of 128 threads thread t holds
 // target t mod G and meets every (128 / G)-th source of the CTA's share from
 // t / G on, staged in shared memory 128 at a time.  The 128 / G sums of a
 // target are added in the CTA, the CTAs' sums by the first one through
-// distributed shared memory, both in a fixed order.
+// distributed shared memory, both in a fixed order.  With several parts every
+// cluster takes one part of the sources and writes the part's slot (3 nt
+// doubles); the slots are added afterwards.
 //
 // What bounds it and why this split: 384 free blobs are 147,456 pairs of 28
 // FP64 operations, 6.4 us if all 152 SMs work (2 FP64 multiply-adds per SM
 // and cycle); blocks of 128 targets and 128 sources gave 200 blobs to 4 SMs
-// (172 us with its three launches; here 8.0 us).  G and the cluster size are
-// chosen for the least work on the busiest SM (small_shape); positions are
-// read as they are, so the product needs no packing launch, no workspace and
-// no second launch for the sums.  The row ranges of a sharded suspension take
-// it at every size: 5,003 rows of 20,011 free blobs FP64 6.28 -> 5.39 ms.
+// (172 us with its three launches; here 8.0 us).  G, the cluster size and the
+// parts are chosen by the expected time (small_shape); positions are read as
+// they are, so a small product needs no packing launch, no workspace and no
+// second launch for the sums.  The row ranges of a sharded suspension take it
+// at every size: 5,003 rows of 20,011 free blobs FP64 6.28 -> 5.04 ms, 949 rows
+// of 7,594 wall blobs FP64 1.27 -> 0.84 ms, mixed 54 -> 45 us.
 //
 // FP32 pair terms (T = float) as in rpy_items_mixed: differences from the hi
 // parts, lo parts added within a quarter of the target's largest coordinate;
@@ -30,6 +34,7 @@
 #include "rpy_pair2.cuh"
 
 #include <algorithm>
+#include <cmath>
 
 namespace am {
 
@@ -81,20 +86,22 @@ struct SmallTile<float> {
 template <class T, bool WALL, int G>
 __global__ void __launch_bounds__(kSmallThreads)
 k_rpy_small(const double* __restrict__ r, const double* __restrict__ lam, double* __restrict__ u, int n, int t0,
-            int nt, RpyK<T> k) {
+            int nt, int parts, RpyK<T> k) {
     dep_wait();
     constexpr int NS = kSmallThreads / G;
     __shared__ SmallTile<T> tile;
     __shared__ double red[NS][3][G];
     __shared__ double own[3 * G];
     const int rank = (int)cluster_rank(), cs = (int)cluster_size();
-    const int group = blockIdx.x / cs;
+    const int group = blockIdx.x / cs / parts, part = blockIdx.x / cs % parts;
     const int e = threadIdx.x % G, sub = threadIdx.x / G;
     const int it = group * G + e;  // target within the rows
     // whole blocks of kSumBlock sources per CTA
     const int nb = (n + kSumBlock - 1) / kSumBlock;
-    const int j0 = kSumBlock * (int)((long long)nb * rank / cs);
-    const int j1 = min(n, kSumBlock * (int)((long long)nb * (rank + 1) / cs));
+    const int piece = part * cs + rank, pieces = parts * cs;
+    const int j0 = kSumBlock * (int)((long long)nb * piece / pieces);
+    const int j1 = min(n, kSumBlock * (int)((long long)nb * (piece + 1) / pieces));
+    u += (size_t)part * 3 * nt;
     double x = 0.0, y = 0.0, z = 1.0;
     if (it < nt) {
         const double* p = r + 3 * (size_t)(t0 + it);
@@ -201,7 +208,7 @@ k_rpy_small(const double* __restrict__ r, const double* __restrict__ lam, double
 template <bool WALL>
 __global__ void __launch_bounds__(kSmallThreads, 5)
 k_rpy_small2(const float4* __restrict__ hi, const float4* __restrict__ lo, const double* __restrict__ lam,
-              double* __restrict__ u, int n, int t0, int nt, RpyK<float> k) {
+              double* __restrict__ u, int n, int t0, int nt, int parts, RpyK<float> k) {
     dep_wait();
     constexpr int NS = kSmallThreads / 32;
     __shared__ float4 sq[3][kSmallTile];  // (-hx, -hx, -hy, -hy), (2hz, 2hz, lz, lz), (lx, lx, ly, ly)
@@ -210,11 +217,13 @@ k_rpy_small2(const float4* __restrict__ hi, const float4* __restrict__ lo, const
     __shared__ double red[NS][3][64];
     __shared__ double own[3 * 64];
     const int rank = (int)cluster_rank(), cs = (int)cluster_size();
-    const int group = blockIdx.x / cs;
+    const int group = blockIdx.x / cs / parts, part = blockIdx.x / cs % parts;
     const int lane = threadIdx.x & 31, sub = threadIdx.x >> 5;
     const int nb = (n + kSumBlock - 1) / kSumBlock;
-    const int j0 = kSumBlock * (int)((long long)nb * rank / cs);
-    const int j1 = min(n, kSumBlock * (int)((long long)nb * (rank + 1) / cs));
+    const int piece = part * cs + rank, pieces = parts * cs;
+    const int j0 = kSumBlock * (int)((long long)nb * piece / pieces);
+    const int j1 = min(n, kSumBlock * (int)((long long)nb * (piece + 1) / pieces));
+    u += (size_t)part * 3 * nt;
     float4 h0 = make_float4(0.f, 0.f, 1.f, 0.f), h1 = h0, o0 = make_float4(0.f, 0.f, 0.f, 0.f), o1 = o0;
     const int i0 = 64 * group + lane, i1 = i0 + 32;
     if (i0 < nt) { h0 = hi[t0 + i0]; o0 = lo[t0 + i0]; }
@@ -294,23 +303,51 @@ k_rpy_small2(const float4* __restrict__ hi, const float4* __restrict__ lo, const
     if (cs > 1) cluster_sync_all();
 }
 
-// Targets per cluster and CTAs per cluster for nt targets against n sources:
-// the shape with the least work on the busiest SM, CTAs dealt out evenly
-// (a CTA also costs about 64 pairs per thread of staging and reduction).
-struct SmallShape { int G, cs; };
-inline SmallShape small_shape(int n, int nt, bool fp64) {
-    SmallShape best{32, 1};
-    double cost = 1e300;
-    for (int G : {32, 16, 8}) {
-        if (G < 16 && !fp64) continue;  // a tile of 128 sources has 8 blocks of 16
-        for (int cs = 1; cs <= 8; ++cs) {
-            const long long ctas = (long long)((nt + G - 1) / G) * cs;
-            const long long per_sm = (ctas + num_sms() - 1) / num_sms();
-            const long long share = (n + cs - 1) / cs;  // sources per CTA
-            const long long ns = kSmallThreads / G;
-            const double c = (double)per_sm * ((double)((share + ns - 1) / ns) + 4.0);
-            if (c < cost) { cost = c; best = {G, cs}; }
-        }
+// Targets per CTA or cluster, CTAs per cluster and parts of the sources with
+// slots of their own (at most `slots`; the sum is another launch) for nt targets
+// against n sources, by the time (us) that they should take.  While all CTAs are
+// resident the busiest SM's work counts (FP32: over the share of the pipe that so
+// few CTAs keep busy; one CTA fills the FP64 pipe), beyond that the mean and most
+// of a CTA more.  Clusters are not dealt out evenly (949 rows of 7,594 blobs, 150
+// CTAs in clusters of 5: two on many of the 152 SMs, twice the time), so where
+// they are not few they count as a less busy pipe.  Small products come out as
+// one launch of clusters, large ones as single CTAs, 20 to 50 an SM.  Measured,
+// FP64 wall, 2,135 rows of 17,086 blobs: one launch, 3.5 to 7 CTAs an SM, 5.18
+// ms; parts, 10.6 4.77, 21 4.71, 56 (32 parts of groups of 8) 4.59; mixed, 4,271
+// rows: 3.5 CTAs 242 us, 7 225, 21 205.
+struct SmallCost {
+    int g_min, g_max, per_thread, resident;  // targets per CTA: G x per_thread; CTAs an SM holds
+    bool fp64;
+    double pair, start, stage;  // us: a pair per thread of a CTA, a CTA, the staging of 128 sources
+};
+struct SmallShape {
+    int G = 32, cs = 1, parts = 1;
+    double us = 1e300;
+};
+inline SmallShape small_shape(int n, int nt, long long slots, const SmallCost& c) {
+    SmallShape best;
+    for (int parts : {1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 48}) {
+        if (parts > 1 && (parts > slots || n / parts < 2 * kSmallTile)) break;
+        const double sum = parts > 1 ? 5.0 + 1.2e-5 * parts * (double)nt : 0.0;
+        for (int G = c.g_max; G >= c.g_min; G /= 2)
+            for (int cs = 1; cs <= 8; ++cs) {
+                if (parts > 1 && n / (parts * cs) < 2 * kSmallTile) break;
+                const long long ctas = (long long)((nt + G * c.per_thread - 1) / (G * c.per_thread)) * cs * parts;
+                const double mean = (double)ctas / num_sms(), most = std::ceil(mean);
+                double load, start = c.start;
+                if (cs == 1) {
+                    const double busy = c.fp64 || most > 3.0 ? 1.0 : most > 2.0 ? 0.9 : most > 1.0 ? 0.76 : 0.47;
+                    load = most <= c.resident ? (most > 1.0 ? 1.04 : 1.0) * most / busy : mean + 0.7;
+                } else {
+                    const double busy = c.fp64 && mean <= 0.9 ? 0.8 : std::max(0.4, std::min(1.0, 0.15 + 0.25 * mean));
+                    load = (mean > 1.0 ? most * (0.99 + 0.01 * cs) + 0.25 : 1.0) / busy;
+                    start = 4.0 * c.pair;
+                }
+                const double share = (double)((n + parts * cs - 1) / (parts * cs));
+                const double us =
+                    load * (std::ceil(share * G / kSmallThreads) * c.pair + start + share / kSmallTile * c.stage) + sum;
+                if (us < best.us) best = {G, cs, parts, us};
+            }
     }
     return best;
 }
@@ -336,13 +373,13 @@ inline void launch_cluster(K kernel, int groups, int cs, cudaStream_t st, Args..
 }
 
 template <class T, bool WALL>
-inline void launch_small_t(const double* r, const double* lam, double* u, int n, int t0, int nt, const RpyK<T>& k,
-                           cudaStream_t st) {
-    const SmallShape s = small_shape(n, nt, sizeof(T) == 8);
-    const int groups = (nt + s.G - 1) / s.G;
-    if (s.G == 32) launch_cluster(k_rpy_small<T, WALL, 32>, groups, s.cs, st, r, lam, u, n, t0, nt, k);
-    else if (s.G == 16) launch_cluster(k_rpy_small<T, WALL, 16>, groups, s.cs, st, r, lam, u, n, t0, nt, k);
-    else if constexpr (sizeof(T) == 8) launch_cluster(k_rpy_small<T, WALL, 8>, groups, s.cs, st, r, lam, u, n, t0, nt, k);
+inline void launch_small_t(const double* r, const double* lam, double* u, int n, int t0, int nt, const SmallShape& s,
+                           const RpyK<T>& k, cudaStream_t st) {
+    const int cl = (nt + s.G - 1) / s.G * s.parts;
+    if (s.G == 32) launch_cluster(k_rpy_small<T, WALL, 32>, cl, s.cs, st, r, lam, u, n, t0, nt, s.parts, k);
+    else if (s.G == 16) launch_cluster(k_rpy_small<T, WALL, 16>, cl, s.cs, st, r, lam, u, n, t0, nt, s.parts, k);
+    else if constexpr (sizeof(T) == 8)
+        launch_cluster(k_rpy_small<T, WALL, 8>, cl, s.cs, st, r, lam, u, n, t0, nt, s.parts, k);
 }
 
 }  // namespace am
