@@ -41,9 +41,9 @@ L2_FLUSH_BYTES = 512 << 20  # > 129 MB L2
 # with the tile fixed (profile_cases colony --host-steps --tile T;
 # dram__bytes_read.sum + dram__bytes_write.sum); absent where no capture of
 # the kernel as it now stands exists
-TRAFFIC_BYTES = {("fp64", 32): 337152, ("fp64", 64): 219648}
+TRAFFIC_BYTES = {("fp64", 32): 309504, ("fp64", 64): 193792}
 # flop per unordered pair of the symmetric FP64 wall product (see run_ours)
-SYM_WALL_FLOP_PER_UNORDERED_PAIR = 126
+SYM_WALL_FLOP_PER_UNORDERED_PAIR = 114
 
 
 def parse():
@@ -253,7 +253,7 @@ def matvec_at_scale(torch, binding, W, stream, fp32_peak, fp64_peak):
         pairs = float(n) * n
         out[key] = {"blobs": n, "ms": t * 1e3, "pairs_per_s": pairs / t,
                     "tflops": pairs * fpp / t / 1e12, "frac_of_fma_peak": pairs * fpp / t / peak,
-                    "kernel": {"mixed": "rpy_items_mixed_x2<wall>", "mixed_symmetric": "rpy_sym_mixed_x2<wall>",
+                    "kernel": {"mixed": "rpy_items_mixed_x2<wall>", "mixed_symmetric": "rpy_sym_mixed<wall>, tiles of 128",
                                "fp64": "rpy_items_f64<wall>", "fp64_symmetric": "k_sym_tiles<SymBlobPair<wall>>, tiles of 128"}[key]}
     return out
 
@@ -810,7 +810,7 @@ def run_ours(args):
     layout = solver.mobility_layout()
     if layout[3] > 0:
         # symmetric FP64 product: each unordered pair evaluated once and applied
-        # both ways, 126 flop per unordered pair (FMA = 2, rsqrt = 1, counted
+        # both ways, 114 flop per unordered pair (FMA = 2, rsqrt = 1, counted
         # from pair_wall_sym and the pair's distances) against 2 x 119
         kname = "k_sym_tiles<SymBlobPair<wall>>, tiles of %d" % layout[3]
         executed = nb * (nb + 1) / 2 * SYM_WALL_FLOP_PER_UNORDERED_PAIR / avg_launch_s
@@ -825,7 +825,7 @@ def run_ours(args):
                 "kernel": kname, "layout": list(layout),
                 "executed_tflops": executed / 1e12, "executed_frac": executed / peak,
                 "algorithmic_vs_executed": "achieved counts N^2 pairs x 119 flop per launch; the symmetric "
-                                           "kernel executes N(N+1)/2 x 126, so frac can exceed the FP64 "
+                                           "kernel executes N(N+1)/2 x 114, so frac can exceed the FP64 "
                                            "pipe's busy fraction" if layout[3] > 0 else None,
                 "flop_per_pair": fpp, "pairs_per_launch": nb * nb,
                 "launch_ms": avg_launch_s * 1e3, "launches": mob_launches,
