@@ -327,7 +327,8 @@ AM_API int am_apply_precond(am_handle* h, const double* r, double* z);
  * at z = 0 (wall = 1; every r_z must exceed a, not checked here).
  *   d_r        3n doubles, blob centres
  *   d_lambda   3n doubles, blob forces
- *   d_u        3n doubles, output velocities (overwritten)
+ *   d_u        3n doubles, output velocities (overwritten); may share
+ *              memory with d_r and d_lambda
  *   precision  AM_FP64 or AM_MIXED
  *   d_work     scratch of am_rpy_matvec_workspace(n, precision) bytes,
  *              256-byte aligned; contents are overwritten.  At least
@@ -346,7 +347,8 @@ AM_API size_t am_rpy_matvec_workspace(int n, int precision);
 /* Rows row0 .. row0 + nrows - 1 of the product u = M(r) lambda against all
  * n sources: the local step of a suspension sharded by blobs over several
  * GPUs, after the positions and forces of all shards have been gathered.
- *   d_r, d_lambda  3n doubles (all blobs, device); d_u  3 nrows doubles
+ *   d_r, d_lambda  3n doubles (all blobs, device); d_u  3 nrows doubles,
+ *                  which may lie in them
  *   d_work         at least am_rpy_matvec_rows_workspace(n, nrows,
  *                  precision) bytes, 256-byte aligned
  * Otherwise as am_rpy_matvec (with row0 = 0 and nrows = n the two agree).
@@ -363,7 +365,8 @@ AM_API size_t am_rpy_matvec_rows_workspace(int n, int nrows, int precision);
  * callback, or a process whose device memory is owned by a pool it must
  * not grow.  The caller still passes inputs and outputs (d_r, d_lambda,
  * d_u, n, eta, a, wall, precision and stream mean what they mean for
- * am_rpy_matvec); the scratch lives in a fixed device array of
+ * am_rpy_matvec, and d_u may share memory with the inputs); the scratch
+ * lives in a fixed device array of
  * AM_NOALLOC_SCRATCH_BYTES inside the library, which every GPU that loads
  * the library holds until the process exits.
  *  - Limit: n must satisfy am_rpy_matvec_rows_workspace(n, n, precision) <=

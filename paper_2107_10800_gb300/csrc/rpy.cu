@@ -798,9 +798,18 @@ static void product_sym(const double* r, const double* lam, double* u, int n, co
     count_launch(2);
 }
 
-// the sum of the parts of a cluster product, if there are several
+// whether the output u (3 nt doubles) shares memory with v (3 n doubles)
+static bool shares(const double* u, size_t nt, const double* v, size_t n) {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(u), b = reinterpret_cast<uintptr_t>(v);
+    return a < b + 3 * n * sizeof(double) && b < a + 3 * nt * sizeof(double);
+}
+
+// A cluster product whose sources are in one part writes u while other CTAs of
+// the launch still read lambda and r.  Where u shares memory with them (`held`)
+// the part goes to a slot like several parts do; the least scratch holds one.
+// The sum of the parts, if they are in slots:
 static void sum_parts(const double* part, double* u, int nt, int parts, cudaStream_t st) {
-    if (parts == 1) return;
+    if (part == u) return;
     launch_dep(k_sum_slots, dim3((3 * nt + 31) / 32), dim3(256), 0, st, part, u, 3 * nt, parts);
     count_launch();
 }
@@ -810,13 +819,13 @@ static void sum_parts(const double* part, double* u, int nt, int parts, cudaStre
 // launch before: by the time that small_shape expects.
 template <bool WALL>
 static void product_mixed(const double* r, const double* lam, double* u, int n, int t0, int nt, const RpyParams& prm,
-                          char* work, size_t bytes, cudaStream_t st) {
+                          bool held, char* work, size_t bytes, cudaStream_t st) {
     const RpyK<float> k = rpy_consts<float>(prm);
     const size_t packed = 2 * align256((size_t)n * sizeof(float4)), slot = 3 * (size_t)nt * sizeof(double);
     const SmallShape one = small_shape(n, nt, bytes / slot, {16, 32, 1, 8, false, WALL ? 0.060 : 0.040, 0.25, 0.3});
     const SmallShape two = small_shape(n, nt, (bytes - packed) / slot, {32, 32, 2, 5, false, WALL ? 0.100 : 0.062, 0.4, 0.15});
     if (one.us <= two.us + 3.0) {
-        double* out = one.parts > 1 ? reinterpret_cast<double*>(work) : u;
+        double* out = one.parts > 1 || held ? reinterpret_cast<double*>(work) : u;
         launch_small_t<float, WALL>(r, lam, out, n, t0, nt, one, k, st);
         sum_parts(out, u, nt, one.parts, st);
         return;
@@ -825,7 +834,7 @@ static void product_mixed(const double* r, const double* lam, double* u, int n, 
            *lo = reinterpret_cast<float4*>(work + align256((size_t)n * sizeof(float4)));
     launch_dep(k_pack_positions, dim3((n + 127) / 128), dim3(128), 0, st, r, hi, lo, n);
     count_launch();
-    double* out = two.parts > 1 ? reinterpret_cast<double*>(work + packed) : u;
+    double* out = two.parts > 1 || held ? reinterpret_cast<double*>(work + packed) : u;
     launch_cluster(k_rpy_small2<WALL>, (nt + 63) / 64 * two.parts, two.cs, st, (const float4*)hi, (const float4*)lo,
                    lam, out, n, t0, nt, two.parts, k);
     sum_parts(out, u, nt, two.parts, st);
@@ -833,22 +842,25 @@ static void product_mixed(const double* r, const double* lam, double* u, int n, 
 
 template <bool WALL>
 static void product_small(const double* r, const double* lam, double* u, int n, int t0, int nt, const RpyParams& prm,
-                          char* work, size_t bytes, cudaStream_t st) {
+                          bool held, char* work, size_t bytes, cudaStream_t st) {
     const SmallShape s = small_shape(n, nt, bytes / (3 * (size_t)nt * sizeof(double)),
                                      {8, 32, 1, 8, true, WALL ? 2.0 : 0.95, WALL ? 2.0 : 1.0, 0.1});
-    double* out = s.parts > 1 ? reinterpret_cast<double*>(work) : u;
+    double* out = s.parts > 1 || held ? reinterpret_cast<double*>(work) : u;
     launch_small_t<double, WALL>(r, lam, out, n, t0, nt, s, rpy_consts<double>(prm), st);
     sum_parts(out, u, nt, s.parts, st);
 }
 
 // u = rows t0 .. t0 + nt - 1 of M(r) lambda; `bytes` of scratch at work (at
 // least least_workspace; the symmetric product only where it holds its slots).
+// u may share memory with r and lam: every route writes it in a launch of its
+// own then, after the last read of them.
 cudaError_t product(const double* r, const double* lam, double* u, int n, int t0, int nt, double eta, double a,
                     int wall, int precision, void* work, size_t bytes, cudaStream_t st) {
     const RpyParams prm = make_params(eta, a);
+    const bool held = shares(u, nt, lam, n) || shares(u, nt, r, n);
     if (precision == AM_MIXED) {
-        if (wall) product_mixed<true>(r, lam, u, n, t0, nt, prm, static_cast<char*>(work), bytes, st);
-        else product_mixed<false>(r, lam, u, n, t0, nt, prm, static_cast<char*>(work), bytes, st);
+        if (wall) product_mixed<true>(r, lam, u, n, t0, nt, prm, held, static_cast<char*>(work), bytes, st);
+        else product_mixed<false>(r, lam, u, n, t0, nt, prm, held, static_cast<char*>(work), bytes, st);
         return cudaGetLastError();
     }
     if (nt == n && n >= kSymFrom) {
@@ -859,8 +871,8 @@ cudaError_t product(const double* r, const double* lam, double* u, int n, int t0
             return cudaGetLastError();
         }
     }
-    if (wall) product_small<true>(r, lam, u, n, t0, nt, prm, static_cast<char*>(work), bytes, st);
-    else product_small<false>(r, lam, u, n, t0, nt, prm, static_cast<char*>(work), bytes, st);
+    if (wall) product_small<true>(r, lam, u, n, t0, nt, prm, held, static_cast<char*>(work), bytes, st);
+    else product_small<false>(r, lam, u, n, t0, nt, prm, held, static_cast<char*>(work), bytes, st);
     return cudaGetLastError();
 }
 
