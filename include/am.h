@@ -312,6 +312,17 @@ AM_API int am_set_mobility_layout(am_handle* h, int targets_per_thread, int sour
  * bodies). */
 AM_API int am_get_mobility_layout(am_handle* h, int* layout);
 
+/* Form of the Arnoldi step of the handle's solves:
+ *   0  one cooperative kernel where the systems are small enough, else
+ *      separate kernels (the default)
+ *   1  separate kernels
+ *   2  as 0, with the cooperative launch answered as a refused one is: the
+ *      solve goes on with the separate kernels
+ * A solve that has gone over to the separate kernels keeps them until the
+ * bodies or links change or this is called.  A testing aid, not in the paper.
+ * Errors: AM_ERR_ARG (unknown form). */
+AM_API int am_set_arnoldi_step(am_handle* h, int form);
+
 /* y -> A y for the full operator of Eq. linear_system at the current pose
  * (y and Ay: 3Nb + 6M + 3P, ordered (lambda, U, phi)). */
 AM_API int am_apply_operator(am_handle* h, const double* y, double* Ay);

@@ -67,6 +67,7 @@ SIGNATURES = {
     "am_apply_mobility": (ctypes.c_int, [_vp, _dp, _dp]),
     "am_apply_mobility_ex": (ctypes.c_int, [_vp, _dp, _dp, ctypes.c_int]),
     "am_set_mobility_layout": (ctypes.c_int, [_vp, ctypes.c_int, ctypes.c_int]),
+    "am_set_arnoldi_step": (ctypes.c_int, [_vp, ctypes.c_int]),
     "am_get_mobility_layout": (ctypes.c_int, [_vp, _ip]),
     "am_set_repulsion": (ctypes.c_int, [_vp, ctypes.c_double, ctypes.c_double, ctypes.c_double,
                                         ctypes.c_double, ctypes.c_double]),
@@ -357,6 +358,10 @@ class Solver:
     def set_mobility_layout(self, targets_per_thread, source_chunk=0):
         """Fix the all-pairs product layout (0 targets per thread: autotune)."""
         self._check(lib().am_set_mobility_layout(self.h, targets_per_thread, source_chunk))
+
+    def set_arnoldi_step(self, form):
+        """0 one kernel where it fits, 1 separate kernels, 2 a refused launch."""
+        self._check(lib().am_set_arnoldi_step(self.h, form))
 
     def apply_operator(self, y):
         ya, yp = _d(y, self.n)

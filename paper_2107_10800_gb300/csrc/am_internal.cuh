@@ -52,6 +52,9 @@ struct ArnoldiCtrl {
     double tol_abs; // stop when the residual estimate is <= tol_abs
 };
 
+// am_set_arnoldi_step
+enum { kStepAuto = 0, kStepSeparate = 1, kStepRefused = 2 };
+
 // One work item of the block-diagonal all-pairs product: targets [t0, t1)
 // against sources [j0, j1) of one system, partial sums at pbase.
 struct MvItem {
@@ -200,7 +203,9 @@ struct am_handle {
            *d_tol_s = nullptr, *d_sysred = nullptr, *d_hcols = nullptr, *d_carry = nullptr;
     int *d_active = nullptr, *d_kdone = nullptr;
     int* d_step_sync = nullptr;  // S arrival counts of the fused Arnoldi step
-    bool step_fused = false;
+    bool step_fits = false;   // whether the Arnoldi step can run as one kernel
+    bool step_fused = false;  // whether it does
+    int step_form = 0;        // am_set_arnoldi_step
     int* d_arn_cnt = nullptr;  // S + 1 arrival counts of the fused Arnoldi step kernels
     int* d_pcb_cnt = nullptr;  // M arrival counts of the preconditioner apply (per body)
     int chunk_len = 1024, chunk_threads = 256;  // dot-product chunk length, threads per chunk block

@@ -795,7 +795,8 @@ int build_system_maps(am_handle* h) {
     CK(dalloc(&h->d_active, S)); CK(dalloc(&h->d_kdone, S));
     CK(dalloc(&h->d_arn_cnt, S + 1)); CK(dalloc(&h->d_step_sync, S));
     CK(cudaMemsetAsync(h->d_arn_cnt, 0, (S + 1) * sizeof(int), st));
-    h->step_fused = am::step_fits(h, coff.data());
+    h->step_fits = am::step_fits(h, coff.data());
+    h->step_fused = h->step_fits && h->step_form != am::kStepSeparate;
     CK(dalloc(&h->d_part, 2 * (size_t)(m + 2) * std::max(1, h->nchunks)));
     CK(dalloc(&h->d_npart, std::max(h->nchunks, 4 * am::num_sms() + 64)));
     std::vector<int> b0(S), nb(S), bo(S + 1, h->M);
@@ -1450,6 +1451,16 @@ extern "C" AM_API int am_set_mobility_layout(am_handle* h, int targets_per_threa
     if (am::mobility_layout(h, targets_per_thread, source_chunk))
         return set_err(h, AM_ERR_CUDA, "am_set_mobility_layout: device allocation failed");
     h->mv_tuned = true;
+    return AM_OK;
+}
+
+extern "C" AM_API int am_set_arnoldi_step(am_handle* h, int form) {
+    if (!h) return AM_ERR_ARG;
+    if (form < am::kStepAuto || form > am::kStepRefused)
+        return set_err(h, AM_ERR_ARG, "am_set_arnoldi_step: unknown form");
+    h->step_form = form;
+    h->step_fused = h->step_fits && form != am::kStepSeparate;
+    h->layout_gen++;  // captured steps may be of another form
     return AM_OK;
 }
 

@@ -1387,8 +1387,10 @@ int line_initial(am_handle* h, double* x, const double* xp) {
 // One Arnoldi step of flexible GMRES for every system at once, with the step
 // index in device memory: z = P^-1 V[j] (stored in Z[j]), w = A z, CGS2 with
 // per-system coefficients, per-system Givens updates and stopping,
-// V[j+1] = w / |w_s|, then the loop control.
-static void issue_arnoldi_step(am_handle* h, bool fp64, cudaGraphConditionalHandle hc, bool in_graph) {
+// V[j+1] = w / |w_s|, then the loop control.  Returns the status of the launch
+// that advances the control block (a cooperative launch can be refused where
+// others are not).
+static cudaError_t issue_arnoldi_step(am_handle* h, bool fp64, cudaGraphConditionalHandle hc, bool in_graph) {
     cudaStream_t s = h->stream;
     const int n = h->n, m = h->restart, m1 = m + 1, S = h->S;
     const size_t ldv = (size_t)h->ldv;
@@ -1413,9 +1415,10 @@ static void issue_arnoldi_step(am_handle* h, bool fp64, cudaGraphConditionalHand
         lc.stream = s;
         lc.attrs = at;
         lc.numAttrs = 2;
-        cudaLaunchKernelEx(&lc, k_arn_step, a);
+        const cudaError_t e = h->step_form == kStepRefused ? cudaErrorCooperativeLaunchTooLarge
+                                                           : cudaLaunchKernelEx(&lc, k_arn_step, a);
         count_launch();
-        return;
+        return e;
     }
     launch_dep(k_arn_dots, dim3(nch), dim3(ct), 0, s, h->d_V, ldv, h->d_w, h->d_zj, h->d_Z, h->d_chunk_start,
                h->d_chunk_end, h->d_sys_of_elem, h->d_sys_chunk_off, h->d_part, nch, m1, h->d_coefs, h->d_hcols,
@@ -1423,21 +1426,26 @@ static void issue_arnoldi_step(am_handle* h, bool fp64, cudaGraphConditionalHand
     launch_dep(k_arn_orth_dots, dim3(nch), dim3(ct), 0, s, h->d_V, ldv, h->d_w, h->d_chunk_start, h->d_chunk_end,
                h->d_sys_of_elem, h->d_sys_chunk_off, h->chunk_len, h->d_part, nch, m1, h->d_coefs, h->d_hcols,
                h->d_arn_cnt, h->d_ctrl);
-    launch_dep(k_arn_orth_finish, dim3(nch + S), dim3(ct), 0, s, h->d_V, ldv, h->d_w, h->d_chunk_start,
-               h->d_chunk_end, h->d_sys_of_elem, h->d_sys_chunk_off, h->chunk_len, h->d_npart, nch, m1, h->d_coefs,
-               h->d_hcols, h->d_arn_cnt, S, m, h->d_Hs, h->d_css, h->d_sns, h->d_gs, h->d_carry, h->d_active,
-               h->d_kdone, h->d_tol_s, h->d_inv_s, h->d_ctrl, hc, in_graph ? 1 : 0);
+    const cudaError_t e = launch_dep(
+        k_arn_orth_finish, dim3(nch + S), dim3(ct), 0, s, h->d_V, ldv, h->d_w, h->d_chunk_start, h->d_chunk_end,
+        h->d_sys_of_elem, h->d_sys_chunk_off, h->chunk_len, h->d_npart, nch, m1, h->d_coefs, h->d_hcols, h->d_arn_cnt,
+        S, m, h->d_Hs, h->d_css, h->d_sns, h->d_gs, h->d_carry, h->d_active, h->d_kdone, h->d_tol_s, h->d_inv_s,
+        h->d_ctrl, hc, in_graph ? 1 : 0);
     // j has advanced: V[j] = w / |w_s| and the next step's input
     launch_dep(k_next_basis, dim3(nb), dim3(256), 0, s, h->d_w, h->d_V, ldv, n, h->d_sys_of_elem, h->d_inv_s,
                h->d_ctrl, h->d_vj, 1);
     count_launch(4);
+    return e;
 }
 
-// The whole step in one kernel where its blocks are all resident (two of 256
-// threads per SM at most, so that the waits are short) and a system's partial
-// sums are few enough for every block to add them
+// The whole step in one kernel where its blocks are all resident (at most four
+// of kStepThreads per SM) and a system's partial sums are few enough for every
+// block to add them
 bool step_fits(const am_handle* h, const int* chunk_off) {
-    int per = 0;
+    int per = 0, dev = 0, coop = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop)
+        return false;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_arn_step, kStepThreads, 0) != cudaSuccess) return false;
     int most = 0;
     for (int s = 0; s < h->S; ++s) most = std::max(most, chunk_off[s + 1] - chunk_off[s]);
@@ -1476,9 +1484,9 @@ static bool ensure_graph(am_handle* h, bool fp64) {
     bool ok = cudaStreamBeginCaptureToGraph(h->stream, body, nullptr, nullptr, 0,
                                             cudaStreamCaptureModeThreadLocal) == cudaSuccess;
     if (ok) {
-        issue_arnoldi_step(h, fp64, hc, true);
+        const cudaError_t e = issue_arnoldi_step(h, fp64, hc, true);
         cudaGraph_t out = nullptr;
-        ok = cudaStreamEndCapture(h->stream, &out) == cudaSuccess;
+        ok = cudaStreamEndCapture(h->stream, &out) == cudaSuccess && e == cudaSuccess;
     }
     h->timing = timing;
     h->body_launches[gi] = g_launches.load() - l0;
@@ -1497,6 +1505,28 @@ static bool ensure_graph(am_handle* h, bool fp64) {
     return true;
 }
 
+// One restart cycle: the graph, or the steps launched from the host; its end in
+// h_ctrl.  Returns the error of a launch or of the stream.
+static cudaError_t run_cycle(am_handle* h, bool fp64, bool use_graph) {
+    cudaStream_t s = h->stream;
+    const int gi = fp64 ? 1 : 0;
+    cudaError_t e;
+    if (use_graph) {
+        if ((e = cudaGraphLaunch(h->gexec[gi], s)) != cudaSuccess) return e;
+        cudaMemcpyAsync(h->h_ctrl, h->d_ctrl, sizeof(ArnoldiCtrl), cudaMemcpyDeviceToHost, s);
+        if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
+        g_launches.fetch_add(h->body_launches[gi] * h->h_ctrl->it);
+        h->pairs += h->body_pairs[gi] * h->h_ctrl->it;
+        return cudaSuccess;
+    }
+    do {
+        if ((e = issue_arnoldi_step(h, fp64, 0, false)) != cudaSuccess) return e;
+        cudaMemcpyAsync(h->h_ctrl, h->d_ctrl, sizeof(ArnoldiCtrl), cudaMemcpyDeviceToHost, s);
+        if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
+    } while (!h->h_ctrl->stop);
+    return cudaSuccess;
+}
+
 // Flexible GMRES(m) (right preconditioning, x = x0 + Z xi with the stored
 // z_j = P^-1 v_j, so a preconditioner applied in FP32 is allowed), CGS2, for
 // all systems of the handle at once: each system has its own Krylov basis
@@ -1506,7 +1536,10 @@ static bool ensure_graph(am_handle* h, bool fp64) {
 // device as one graph launch (WHILE node over Arnoldi steps); with
 // per-kernel timing on, the same steps are launched from the host instead
 // (event records cannot live in a graph loop).  Returns the number of steps;
-// *rel = the largest final relative residual.
+// *rel = the largest final relative residual (NaN after a failed launch, which
+// the caller finds with cudaGetLastError).  A cycle whose one-kernel step is
+// refused is repeated with the separate kernels, which the handle then keeps
+// until its bodies or links change: x is updated only behind a cycle.
 static int gmres(am_handle* h, const double* rhs, double* x, double tol, bool fp64, int budget,
                  double* rel, int* cycles, double* rel0 = nullptr) {
     cudaStream_t s = h->stream;
@@ -1515,8 +1548,7 @@ static int gmres(am_handle* h, const double* rhs, double* x, double tol, bool fp
     const int nb = red_blocks(n);
     sys_norms(h, rhs, h->d_bnorm_s);
     cudaMemsetAsync(h->d_arn_cnt, 0, (S + 1) * sizeof(int), s);  // arrival counts of the step kernels
-    const bool use_graph = !h->timing && h->graphs_ok && ensure_graph(h, fp64);
-    const int gi = fp64 ? 1 : 0;
+    bool use_graph = !h->timing && h->graphs_ok && ensure_graph(h, fp64);
     int it = 0;
     *rel = 0.0;
     bool first = true;
@@ -1531,24 +1563,22 @@ static int gmres(am_handle* h, const double* rhs, double* x, double tol, bool fp
         first = false;
         const int n_active = (int)h->h_scal[1];
         if (n_active == 0 || it >= budget || !(*rel == *rel)) break;
-        ++*cycles;
         k_scale_sys<<<nb, 256, 0, s>>>(h->d_V, n, h->d_sys_of_elem, h->d_inv_s, h->d_vj);
         k_ctrl_init<<<1, 1, 0, s>>>(h->d_ctrl, budget - it, m, 0.0);
         cudaMemsetAsync(h->d_step_sync, 0, S * sizeof(int), s);
         count_launch(2);
-        if (use_graph) {
-            cudaGraphLaunch(h->gexec[gi], s);
-            cudaMemcpyAsync(h->h_ctrl, h->d_ctrl, sizeof(ArnoldiCtrl), cudaMemcpyDeviceToHost, s);
-            cudaStreamSynchronize(s);
-            g_launches.fetch_add(h->body_launches[gi] * h->h_ctrl->it);
-            h->pairs += h->body_pairs[gi] * h->h_ctrl->it;
-        } else {
-            do {
-                issue_arnoldi_step(h, fp64, 0, false);
-                cudaMemcpyAsync(h->h_ctrl, h->d_ctrl, sizeof(ArnoldiCtrl), cudaMemcpyDeviceToHost, s);
-                cudaStreamSynchronize(s);
-            } while (!h->h_ctrl->stop);
+        if (run_cycle(h, fp64, use_graph) != cudaSuccess) {
+            if (!h->step_fused) {
+                *rel = nan("");
+                break;
+            }
+            cudaGetLastError();  // refused; nothing else was lost
+            h->step_fused = false;
+            h->layout_gen++;  // captured steps are of the other form
+            use_graph = !h->timing && h->graphs_ok && ensure_graph(h, fp64);
+            continue;
         }
+        ++*cycles;
         it += h->h_ctrl->it;
         k_hess_solve_sys<<<nblk(S, 4), 128, 0, s>>>(h->d_Hs, h->d_gs, h->d_kdone, h->d_xis, S, m);
         k_combine_sys<<<nb, 256, 0, s>>>(h->d_Z, ldv, h->d_xis, h->d_kdone, h->d_sys_of_elem, n, m1, h->d_t);
@@ -1670,6 +1700,7 @@ int solve(am_handle* h, am_step_stats* st) {
             cudaMemsetAsync(h->d_dx, 0, h->n * sizeof(double), s);
             double rin = 0.0;
             it += gmres(h, h->d_rir, h->d_dx, tin, false, budget - it, &rin, &cycles);
+            if (cudaPeekAtLastError() != cudaSuccess) break;
             k_axpy<<<nb, 256, 0, s>>>(h->d_x, h->d_dx, h->n, 1.0);
             count_launch();
             updated = false;
