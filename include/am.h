@@ -318,6 +318,8 @@ AM_API int am_get_mobility_layout(am_handle* h, int* layout);
  *   1  separate kernels
  *   2  as 0, with the cooperative launch answered as a refused one is: the
  *      solve goes on with the separate kernels
+ *   3  as 0, with waits that end after one look: the solve goes on with the
+ *      separate kernels
  * A solve that has gone over to the separate kernels keeps them until the
  * bodies or links change or this is called.  A testing aid, not in the paper.
  * Errors: AM_ERR_ARG (unknown form). */

@@ -360,7 +360,8 @@ class Solver:
         self._check(lib().am_set_mobility_layout(self.h, targets_per_thread, source_chunk))
 
     def set_arnoldi_step(self, form):
-        """0 one kernel where it fits, 1 separate kernels, 2 a refused launch."""
+        """0 one kernel where it fits, 1 separate kernels, 2 a refused launch,
+        3 waits that run out."""
         self._check(lib().am_set_arnoldi_step(self.h, form))
 
     def apply_operator(self, y):

@@ -49,11 +49,12 @@ struct ArnoldiCtrl {
     int budget;     // steps allowed in this cycle
     int m;          // restart length
     int stop;       // set when the cycle ends
+    int late;       // a wait of the one-kernel step ran out: the cycle does not count
     double tol_abs; // stop when the residual estimate is <= tol_abs
 };
 
 // am_set_arnoldi_step
-enum { kStepAuto = 0, kStepSeparate = 1, kStepRefused = 2 };
+enum { kStepAuto = 0, kStepSeparate = 1, kStepRefused = 2, kStepLate = 3 };
 
 // One work item of the block-diagonal all-pairs product: targets [t0, t1)
 // against sources [j0, j1) of one system, partial sums at pbase.

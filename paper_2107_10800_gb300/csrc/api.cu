@@ -1456,7 +1456,7 @@ extern "C" AM_API int am_set_mobility_layout(am_handle* h, int targets_per_threa
 
 extern "C" AM_API int am_set_arnoldi_step(am_handle* h, int form) {
     if (!h) return AM_ERR_ARG;
-    if (form < am::kStepAuto || form > am::kStepRefused)
+    if (form < am::kStepAuto || form > am::kStepLate)
         return set_err(h, AM_ERR_ARG, "am_set_arnoldi_step: unknown form");
     h->step_form = form;
     h->step_fused = h->step_fits && form != am::kStepSeparate;

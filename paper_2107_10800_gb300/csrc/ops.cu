@@ -502,7 +502,7 @@ namespace am {
 // same kernels can run inside a CUDA-graph WHILE node without the host.
 
 __global__ void k_ctrl_init(ArnoldiCtrl* c, int budget, int m, double tol_abs) {
-    c->j = 0; c->it = 0; c->budget = budget; c->m = m; c->stop = 0; c->tol_abs = tol_abs;
+    c->j = 0; c->it = 0; c->budget = budget; c->m = m; c->stop = 0; c->late = 0; c->tol_abs = tol_abs;
 }
 
 // ---- per-system (batched) GMRES kernels ----------------------------------
@@ -570,17 +570,16 @@ __global__ void k_sys_minrel(int S, const double* __restrict__ beta, const doubl
 // Start of a restart cycle, one block: per system the relative residual
 // beta_s / ||b_s||; systems above tol are active, with v_0 scale 1/beta_s,
 // g = (beta_s, 0, ...), absolute stop threshold tol ||b_s||.  red[0] = max
-// relative residual (NaN if any is not finite, or a wait of an earlier step
-// ran out), red[1] = active count.
+// relative residual (NaN if any is not finite), red[1] = active count.
 __global__ void k_cycle_init(int S, int m, double tol, const double* __restrict__ beta,
                              const double* __restrict__ bnorm, int* __restrict__ active,
                              double* __restrict__ inv, double* __restrict__ g, int* __restrict__ kdone,
-                             double* __restrict__ tol_s, double* __restrict__ red, const int* __restrict__ flags) {
+                             double* __restrict__ tol_s, double* __restrict__ red) {
     __shared__ double smax[256];
     __shared__ int scnt[256];
     __shared__ int sbad[256];
     double mx = 0.0;
-    int cnt = 0, bad = *flags & kFlagStepWait ? 1 : 0;
+    int cnt = 0, bad = 0;
     for (int s = threadIdx.x; s < S; s += blockDim.x) {
         const double bn = bnorm[s], be = beta[s];
         const double rel = bn > 0.0 ? be / bn : 0.0;
@@ -734,8 +733,9 @@ __device__ __forceinline__ void finish_one(int s, int j, int m, double carry, do
 }
 
 // Advance j; the cycle ends when no system is active, at the restart length
-// or at the step budget (still-active systems then close at j + 1).  Every
-// thread of the one block calls it.
+// or at the step budget (still-active systems then close at j + 1), or when a
+// wait of the one-kernel step has run out (the cycle does not count then).
+// Every thread of the one block calls it.
 __device__ void loop_ctrl(ArnoldiCtrl* c, int* __restrict__ active, int* __restrict__ kdone, int S,
                           cudaGraphConditionalHandle hc, int in_graph) {
     const int j1 = c->j + 1, it1 = c->it + 1;
@@ -747,10 +747,11 @@ __device__ void loop_ctrl(ArnoldiCtrl* c, int* __restrict__ active, int* __restr
             if (__ldcg(active + s)) { kdone[s] = j1; active[s] = 0; }
     __syncthreads();
     if (threadIdx.x == 0) {
+        const int end = stop | __ldcg(&c->late);
         c->it = it1;
         c->j = j1;
-        c->stop = stop;
-        if (in_graph) cudaGraphSetConditional(hc, stop ? 0u : 1u);
+        c->stop = end;
+        if (in_graph) cudaGraphSetConditional(hc, end ? 0u : 1u);
     }
 }
 
@@ -979,23 +980,25 @@ __global__ void k_next_basis(const double* __restrict__ w, double* __restrict__ 
 // first loads and serial sums.
 // sync[s] counts arrivals of system s since the start of the cycle: meeting b
 // (0, 1, 2) of step `it` waits for (3 it + b + 1) times its blocks.  The wait is
-// bounded; a wait that runs out sets kFlagStepWait and the kernel goes on to
-// its end.
+// bounded, since a block may get its SM late where other streams hold it.  A
+// wait that runs out sets c->late, which ends the other waits and the cycle;
+// every block still arrives three times and goes on to its end.  Nothing of
+// such a cycle is used: gmres repeats it with the separate kernels.
 constexpr int kStepThreads = 288;
 constexpr int kStepSpins = 1 << 21;  // about a second
 
 __device__ __forceinline__ void sys_arrive(int* cnt) {  // after a barrier of the block
     asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(cnt) : "memory");
 }
-__device__ __forceinline__ void sys_barrier(int* cnt, int target, int* flags) {
+__device__ __forceinline__ void sys_barrier(int* cnt, int target, int* late, int spins) {
     __syncthreads();
     if (threadIdx.x == 0) {
         sys_arrive(cnt);
         int n = 0, v;
         do {
             asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(cnt) : "memory");
-        } while (v < target && ++n < kStepSpins);
-        if (v < target) atomicOr(flags, kFlagStepWait);
+        } while (v < target && ++n < spins && (n % 256 || !__ldcg(late)));
+        if (v < target) atomicOr(late, 1);
     }
     __syncthreads();
 }
@@ -1014,7 +1017,8 @@ struct StepArgs {
     int *active, *kdone;
     const double* tol_s;
     double* inv;
-    int *sync, *cnt, *flags;
+    int *sync, *cnt;
+    int spins;
     ArnoldiCtrl* c;
     cudaGraphConditionalHandle hc;
     int in_graph;
@@ -1065,7 +1069,7 @@ k_arn_step(StepArgs a) {
                 t = warp_sum(t);
                 if (lane == 0) part[(size_t)(j + 1) * a.nch + b] = t;
             }
-            sys_barrier(a.sync + s, nb * (3 * it + pass + 1), a.flags);
+            sys_barrier(a.sync + s, nb * (3 * it + pass + 1), &a.c->late, a.spins);
             if (vec) {
                 rows_sums(part, a.nch, nullptr, q0, q1, j, [&](int k, double t) {
                     cf[k] = t;
@@ -1108,7 +1112,7 @@ k_arn_step(StepArgs a) {
                 for (int q = 1; q < 8; ++q) t += red[q];
                 a.npart[b] = t;
             }
-            sys_barrier(a.sync + s, nb * (3 * it + 3), a.flags);
+            sys_barrier(a.sync + s, nb * (3 * it + 3), &a.c->late, a.spins);
             if (!vec) {
                 t = 0.0;
                 for (int q = q0 + lane; q < q1; q += 32) t += __ldcg(a.npart + q);
@@ -1403,7 +1407,8 @@ static cudaError_t issue_arnoldi_step(am_handle* h, bool fp64, cudaGraphConditio
         const StepArgs a{h->d_V, ldv, h->d_w, h->d_zj, h->d_Z, h->d_vj, static_cast<const int4*>(h->d_chunk_info),
                          h->d_sys_chunk_off, h->d_part, h->d_npart, nch, m, S, h->chunk_len,
                          h->d_Hs, h->d_css, h->d_sns, h->d_gs, h->d_active, h->d_kdone, h->d_tol_s, h->d_inv_s,
-                         h->d_step_sync, h->d_arn_cnt, h->d_flags, h->d_ctrl, hc, in_graph ? 1 : 0};
+                         h->d_step_sync, h->d_arn_cnt, h->step_form == kStepLate ? 1 : kStepSpins, h->d_ctrl, hc,
+                         in_graph ? 1 : 0};
         cudaLaunchConfig_t lc = {};
         cudaLaunchAttribute at[2];
         at[0].id = cudaLaunchAttributeCooperative;
@@ -1538,7 +1543,7 @@ static cudaError_t run_cycle(am_handle* h, bool fp64, bool use_graph) {
 // (event records cannot live in a graph loop).  Returns the number of steps;
 // *rel = the largest final relative residual (NaN after a failed launch, which
 // the caller finds with cudaGetLastError).  A cycle whose one-kernel step is
-// refused is repeated with the separate kernels, which the handle then keeps
+// refused, or a wait of which ran out, is repeated with the separate kernels, which the handle then keeps
 // until its bodies or links change: x is updated only behind a cycle.
 static int gmres(am_handle* h, const double* rhs, double* x, double tol, bool fp64, int budget,
                  double* rel, int* cycles, double* rel0 = nullptr) {
@@ -1555,7 +1560,7 @@ static int gmres(am_handle* h, const double* rhs, double* x, double tol, bool fp
     while (true) {
         sys_residual(h, rhs, x, h->d_V, h->d_beta_s, fp64);
         k_cycle_init<<<1, 256, 0, s>>>(S, m, tol, h->d_beta_s, h->d_bnorm_s, h->d_active, h->d_inv_s, h->d_gs,
-                                       h->d_kdone, h->d_tol_s, h->d_scal, h->d_flags);
+                                       h->d_kdone, h->d_tol_s, h->d_scal);
         count_launch();
         read_scal(h, 2);
         *rel = h->h_scal[0];
@@ -1567,12 +1572,13 @@ static int gmres(am_handle* h, const double* rhs, double* x, double tol, bool fp
         k_ctrl_init<<<1, 1, 0, s>>>(h->d_ctrl, budget - it, m, 0.0);
         cudaMemsetAsync(h->d_step_sync, 0, S * sizeof(int), s);
         count_launch(2);
-        if (run_cycle(h, fp64, use_graph) != cudaSuccess) {
-            if (!h->step_fused) {
-                *rel = nan("");
-                break;
-            }
-            cudaGetLastError();  // refused; nothing else was lost
+        const bool failed = run_cycle(h, fp64, use_graph) != cudaSuccess;
+        if (failed && !h->step_fused) {
+            *rel = nan("");
+            break;
+        }
+        if (failed || h->h_ctrl->late) {
+            if (failed) cudaGetLastError();  // refused; nothing else was lost
             h->step_fused = false;
             h->layout_gen++;  // captured steps are of the other form
             use_graph = !h->timing && h->graphs_ok && ensure_graph(h, fp64);
@@ -1664,7 +1670,7 @@ int solve(am_handle* h, am_step_stats* st) {
             }
             accurate = res64 && !updated;
             k_cycle_init<<<1, 256, 0, s>>>(h->S, h->restart, tol, be_out, bn_out, h->d_active,
-                                           h->d_inv_s, h->d_gs, h->d_kdone, h->d_tol_s, h->d_scal, h->d_flags);
+                                           h->d_inv_s, h->d_gs, h->d_kdone, h->d_tol_s, h->d_scal);
             count_launch();
             if (!res64) {
                 k_sys_minrel<<<1, 256, 0, s>>>(h->S, be_out, bn_out, h->d_scal + 2);
@@ -1675,7 +1681,7 @@ int solve(am_handle* h, am_step_stats* st) {
                     accurate = true;
                     sys_residual(h, h->d_b, h->d_x, h->d_rir, be_out, kOpDF);
                     k_cycle_init<<<1, 256, 0, s>>>(h->S, h->restart, tol, be_out, bn_out, h->d_active,
-                                                   h->d_inv_s, h->d_gs, h->d_kdone, h->d_tol_s, h->d_scal, h->d_flags);
+                                                   h->d_inv_s, h->d_gs, h->d_kdone, h->d_tol_s, h->d_scal);
                     count_launch();
                 }
             }
@@ -1733,10 +1739,6 @@ int solve(am_handle* h, am_step_stats* st) {
     st->iterations = it;
     st->restarts = cycles;
     st->rel_residual = rel;
-    if (!(rel == rel) && (take_flags(h) & kFlagStepWait)) {
-        h->err = "a wait of the Arnoldi step ran out";
-        return AM_ERR_CUDA;
-    }
     return (rel <= tol) ? AM_OK : AM_ERR_NOT_CONVERGED;
 }
 

@@ -8,7 +8,6 @@ namespace am {
 constexpr int kFlagWall = 1;        // a blob centre at or below height a
 constexpr int kFlagSingular = 2;    // a body block of M or N~ not SPD
 constexpr int kFlagCorrection = 4;  // correction normal equations not SPD
-constexpr int kFlagStepWait = 1 << 9;  // a wait of the fused Arnoldi step ran out
 constexpr int kFlagTensor = 1 << 8; // a tensor-core (tcgen05) wait timed out (tc_gemm.cuh)
 // Bound on the relative error of the mixed mobility product, |(M32 - M) l|
 // <= kMixedProductError |M32 l| (20 times the largest measured, 4.7e-7 at
