@@ -101,24 +101,57 @@ bool host_inverse(std::vector<double>& A, int n) {
 
 // Order of the per-body or per-articulated-body preconditioner builds:
 // matrices of at most two 32-row tiles (rows[i] <= 64) first, one CTA each,
-// then the larger ones, built by clusters of cs CTAs (1, 2, 4 or 8).  The
-// builds are bound by the SMs' arithmetic, so cs is the one that loads the
-// busiest SM least, in matrices: ceil(n cs / SMs) / cs, and a few percent more
-// for each doubling (every CTA factors the diagonal tiles).
-void split_for_build(const std::vector<int>& rows, std::vector<int>& list, int& n_small, int& cs) {
+// then the larger ones, built by clusters of cs CTAs (1, 2, 4 or 8): the cs of
+// the least expected time.
+//
+// A matrix of T tiles a side takes a time like serial / T^2 + 1 / cs: the
+// diagonal tiles or panels go one after the other (T of them) on every CTA or
+// the first, the T^3 tile products are shared.  Clusters stay within a GPC, so
+// that one CTA per SM holds SMs / 2 clusters of 2, but 0.95 SMs / 4 of 4 and
+// 0.85 SMs / 8 of 8.  Further layers of clusters share the SMs: each costs
+// `share` of the first while they are resident together, and a layer after
+// that begins anew.
+//
+// Measured with every cs, 5 to 608 matrices on 152 SMs (us): FP64 bodies of 600
+// rows, 200 of them: cs 1 73,200, 2 55,700, 4 59,300, 8 66,900; of 72 rows: 620,
+// 630, 1,110, 1,940; FP32 bodies of 600 rows, 60 of them: 9,050, 5,090, 3,740,
+// 4,610; 200 articulated bodies of 87 rows FP64: 900, 1,050, 1,360, 2,360.  Over
+// that sweep the rule's cs is within 3 % of the best in FP64 and 14 % in FP32 (300
+// bodies of 600 rows), and within 2 % of what doubling cs while all clusters fit
+// twice the SMs takes where it is not faster.
+struct BuildCost {
+    double serial, share;  // as above
+    int resident;          // CTAs an SM holds (registers)
+};
+constexpr BuildCost kBodyBuild[2] = {{10.0, 0.75, 3}, {50.0, 0.25, 3}};  // FP64, FP32
+constexpr BuildCost kLinkBuild[2] = {{15.0, 0.4, 2}, {15.0, 0.25, 2}};
+
+void split_for_build(const std::vector<int>& rows, const BuildCost& cost, std::vector<int>& list, int& n_small,
+                     int& cs) {
     const int n = (int)rows.size();
     list.clear();
     for (int i = 0; i < n; ++i)
         if (rows[i] <= 2 * 32) list.push_back(i);
     n_small = (int)list.size();
+    double work = 0.0;  // T^3, the mean of the larger ones
     for (int i = 0; i < n; ++i)
-        if (rows[i] > 2 * 32) list.push_back(i);
-    const long long large = n - n_small, sms = am::num_sms();
+        if (rows[i] > 2 * 32) {
+            list.push_back(i);
+            work += std::pow((rows[i] + 31) / 32, 3.0);
+        }
     cs = 1;
+    const int large = n - n_small;
+    if (large == 0) return;
+    const double serial = cost.serial / std::pow(work / large, 2.0 / 3.0);
     double best = 1e300;
-    for (int c = 1, d = 0; c <= 8 && large > 0; c *= 2, ++d) {
-        const double load = (double)((large * c + sms - 1) / sms) / c * (1.0 + 0.03 * d);
-        if (load < best) { best = load; cs = c; }
+    for (int c = 1; c <= 8; c *= 2) {
+        const double per_layer = am::num_sms() / c * (c == 8 ? 0.85 : c == 4 ? 0.95 : 1.0);
+        const int layers = (int)std::ceil(large / std::max(1.0, std::floor(per_layer)));
+        const int waves = layers / cost.resident, rest = layers % cost.resident;
+        const double load = waves * (1.0 + cost.share * (cost.resident - 1)) +
+                            (rest ? 1.0 + cost.share * (rest - 1) : 0.0);
+        const double t = (serial + 1.0 / c) * load;
+        if (t < best) { best = t; cs = c; }
     }
 }
 
@@ -421,7 +454,7 @@ int build_links(am_handle* h, int P, const int* bp, const int* bq) {
         pca_rows[a] = m;
         for (int c = 0; c * 32 < m; ++c) { pca_asm.push_back(a); pca_chunk.push_back(c); }
     }
-    split_for_build(pca_rows, pca_list, h->n_pca_small, h->pca_cs);
+    split_for_build(pca_rows, kLinkBuild[h->pc32 && !h->sb], pca_list, h->n_pca_small, h->pca_cs);
     CK(dalloc(&h->d_pca_list, std::max(NA, 1)));
     if (NA) CK(h2d(h->d_pca_list, pca_list.data(), NA, s));
     h->n_pca = (int)pca_asm.size();
@@ -710,7 +743,7 @@ int build_layout(am_handle* h, int M, int Nb, int NA, int maxb, const double* q,
         const int step = std::min(n, std::max(1, 2048 / n));  // about eight blob pairs per thread
         for (int i = 0; i < n; i += step) pcb_copy.push_back(make_int4(p, shape[p], i, std::min(step, n - i)));
     }
-    split_for_build(pcb_rows, pcb_list, h->n_pcb_small, h->pcb_cs);
+    split_for_build(pcb_rows, kBodyBuild[h->pc32], pcb_list, h->n_pcb_small, h->pcb_cs);
     for (int& p : pcb_list) p = built[p];
     h->n_pcb = (int)built.size();
     h->n_pcb_copy = (int)pcb_copy.size();
