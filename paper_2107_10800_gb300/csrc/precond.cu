@@ -610,7 +610,7 @@ k_pc_ap3(int Nb, int M, const int* __restrict__ pcw_body, const int* __restrict_
 // The whole apply for handles of small articulated bodies (pc_small_size): one
 // cluster per articulated body, a warp per body, one launch instead of three
 // (the problem is block-diagonal over articulated bodies).  With n the body's
-// rows (at most 64), lane l of the warp takes rows l and, when n > 32, the
+// rows (at most 36), lane l of the warp takes rows l and, when n > 32, the
 // remaining rows with several lanes sharing each: an FP64 warp instruction
 // costs 16 cycles of its SM however few lanes take part.  Every CTA forms c and
 // phi of its articulated body itself (at most 64 rows of G~), so the cluster
@@ -618,7 +618,7 @@ k_pc_ap3(int Nb, int M, const int* __restrict__ pcw_body, const int* __restrict_
 // against this one: 4 chains of 8 bodies of 12 blobs in FP64 18.3 us against
 // 14.0 (15.8 with a chain's bodies on the warps of one SM); 16 systems of 500 to
 // 4,000 blobs in FP32 57 us against 22.
-constexpr int kSmallRows = 64;
+constexpr int kSmallRows = 64, kSmallBodyRows = 36;
 template <class T>
 __global__ void __launch_bounds__(256)
 k_pc_small(int Nb, int M, const int* __restrict__ asm_body_off, const int* __restrict__ asm_body_idx,
@@ -630,7 +630,7 @@ k_pc_small(int Nb, int M, const int* __restrict__ asm_body_off, const int* __res
            const int* __restrict__ bl_idx, const int* __restrict__ link_local, const double* __restrict__ r,
            double* __restrict__ w, double* __restrict__ Uhat, double* __restrict__ z, float* __restrict__ lf) {
     dep_wait();
-    __shared__ double cs[kSmallRows], phis[kSmallRows];
+    __shared__ double phis[kSmallRows];
     __shared__ T ct[kSmallRows];
     __shared__ T red[8][kSmallRows];
     const ClusterTeam team;
@@ -709,8 +709,7 @@ k_pc_small(int Nb, int M, const int* __restrict__ asm_body_off, const int* __res
         // component x of u_p + omega_p x l_p - u_q - omega_q x l_q
         const double cp = __ldcg(up + x) + (__ldcg(up + 3 + x1) * l1[x2] - __ldcg(up + 3 + x2) * l1[x1]);
         const double cq = __ldcg(uq + x) + (__ldcg(uq + 3 + x1) * l2[x2] - __ldcg(uq + 3 + x2) * l2[x1]);
-        cs[k] = r[3 * (size_t)Nb + 6 * (size_t)M + 3 * (size_t)n + x] - (cp - cq);
-        ct[k] = (T)cs[k];
+        ct[k] = (T)(r[3 * (size_t)Nb + 6 * (size_t)M + 3 * (size_t)n + x] - (cp - cq));
     }
     __syncthreads();
     if (mg) {
@@ -830,12 +829,18 @@ static void pca_build_t(am_handle* h, double tol) {
 }
 
 // Whether every articulated body is small enough for k_pc_small, and the
-// cluster size: a warp per body, as many CTAs as spread them over the SMs.  The
-// line at 64 rows is where a lane would get a third row and one warp would walk
-// more than 32 KB of factors; larger bodies keep a CTA per 32 rows.
+// cluster size: a warp per body, as many CTAs as spread them over the SMs.
+// Measured against the three kernels, per GMRES iteration: bodies of 12 rows 2
+// to 5 us less, of 36 rows 4 less to 1 more, of 42 rows 1 to 4 more, of 54 to 63
+// rows 4 to 10 more (one warp walks a body's factors; the three kernels have a
+// CTA per 32 rows).  Each articulated body has a CTA of eight warps: of one
+// body each, 600 of them 3 us less, 800 3 more, 3,000 10 more; of two, 600 4 to 8
+// less, 1,500 5 to 11 more; of four, 1,500 no more.  Periodic handles, whose
+// iterations take milliseconds, keep the three kernels that they were measured with.
 static int pc_small_size(const am_handle* h) {
     if (h->sb || h->per || h->NA == 0) return 0;
-    if (3 * h->max_body_blobs > kSmallRows || (h->P && 3 * h->max_asm_links > kSmallRows)) return 0;
+    if (3 * h->max_body_blobs > kSmallBodyRows || (h->P && 3 * h->max_asm_links > kSmallRows)) return 0;
+    if (h->NA > 4 * num_sms() && h->M < 4 * h->NA) return 0;
     int most = 0;
     for (int a = 0; a < h->NA; ++a) most = std::max(most, h->asm_body_off[a + 1] - h->asm_body_off[a]);
     if (most > 64) return 0;
