@@ -158,17 +158,21 @@ void split_for_build(const std::vector<int>& rows, const BuildCost& cost, std::v
 // For every body the first one of its shape (the same blobs in the body frame,
 // bit for bit), whose preconditioner blocks are rotated to it.  Above a wall a
 // block depends on the pose, and while the bodies fit the SMs at once (small
-// ones a CTA each, large ones eight) all are built in the time of one: then
-// every body is its own.  Of dependent links the factorisation of the link
+// ones a CTA each, in FP32 three to an SM, large ones eight) all are built in
+// about the time of one: then every body is its own.  Small ones, all built
+// against rotated (us, the rotation's own launch included): FP64, 12 blobs, 120
+// bodies 297 / 308, 160 382 / 310; FP32, 4 blobs, 450 134 / 149, 600 211 / 156, 12
+// blobs, 300 188 / 194, 450 202 / 194, 600 301 / 193.  Of dependent links the factorisation of the link
 // block keeps the same number, but which of equal ones is a matter of rounding.
-std::vector<int> same_shapes(bool wall, int M, const int* off, const double* rho) {
+std::vector<int> same_shapes(bool wall, bool fp32, int M, const int* off, const double* rho) {
     std::vector<int> first(M);
     long long small = 0, large = 0;
     for (int p = 0; p < M; ++p) {
         first[p] = p;
         ++(3 * (off[p + 1] - off[p]) <= 2 * 32 ? small : large);
     }
-    if (wall || (small <= am::num_sms() && 8 * large <= am::num_sms())) return first;
+    const long long sms = am::num_sms();
+    if (wall || (small <= (fp32 ? 3 : 1) * sms && 8 * large <= sms)) return first;
     std::unordered_map<unsigned long long, std::vector<int>> seen;
     for (int p = 0; p < M; ++p) {
         const size_t n = 3 * (size_t)(off[p + 1] - off[p]);
@@ -730,7 +734,7 @@ int build_layout(am_handle* h, int M, int Nb, int NA, int maxb, const double* q,
         pcw_off[p + 1] = (int)pcw_body.size();
     }
     h->n_pcw = (int)pcw_body.size();
-    const std::vector<int> shape = same_shapes(h->cfg.wall != 0, M, blob_offset, rho);
+    const std::vector<int> shape = same_shapes(h->cfg.wall != 0, h->pc32, M, blob_offset, rho);
     std::vector<int> pcb_rows, pcb_list, built;
     std::vector<int4> pcb_copy;
     for (int p = 0; p < M; ++p) {

@@ -1,7 +1,9 @@
-"""Which way the preconditioner is applied: in one launch, or in two (bodies
+"""Which way the preconditioner is built and applied.  Blocks: every body's
+built, or, of many bodies of one shape in free space, one built and the others
+rotated from it in another launch.  Apply: in one launch, or in two (bodies
 without links) where bodies are larger or too many articulated bodies have few
 bodies each; the lines and the times on both sides stand beside the rules in
-precond.cu.  Told by the launches of one am_apply_precond; the results against
+api.cu and precond.cu.  Told by the launches of one am_apply_precond; the results against
 handles of one articulated body, FP64 1e-11, FP32 factors 1e-4 of the largest
 entry."""
 import numpy as np
@@ -61,3 +63,13 @@ def check(M, blobs, per, precision, wall, launches):
     (20, 4, 4, 4, 1)])
 def test_apply_in_one_launch_or_two(sms, sm, rest, blobs, per, apply, precision):
     check(sm * sms + rest, blobs, per, precision, 1, 3 + apply)
+
+
+@pytest.mark.parametrize("precision, sm, rest, blobs, rotated", [
+    ("fp64", 1, 0, 4, 0), ("fp64", 1, 1, 4, 1), ("mixed", 1, 1, 4, 0), ("mixed", 3, 0, 12, 0), ("mixed", 3, 1, 4, 1),
+    ("mixed", 3, 1, 12, 1), ("mixed", 0, 19, 25, 0), ("mixed", 0, 20, 25, 1)])
+def test_blocks_built_or_rotated(sms, precision, sm, rest, blobs, rotated):
+    if sm == 0 and sms // 8 != 19:
+        pytest.skip("the line of large bodies lies elsewhere")
+    # 25 blobs: 75 rows, applied in two launches
+    check(sm * sms + rest, blobs, 1, precision, 0, 3 + rotated + (1 if blobs <= 12 else 2))
