@@ -209,7 +209,7 @@ struct am_handle {
     int step_form = 0;        // am_set_arnoldi_step
     int* d_arn_cnt = nullptr;  // S + 1 arrival counts of the fused Arnoldi step kernels
     int* d_pcb_cnt = nullptr;  // M arrival counts of the preconditioner apply (per body)
-    int chunk_len = 1024, chunk_threads = 256;  // dot-product chunk length, threads per chunk block
+    int chunk_len = 1024;  // dot-product chunk length
     // all-pairs work items (block-diagonal over systems) and their queue
     void* d_items = nullptr;
     int n_items = 0;

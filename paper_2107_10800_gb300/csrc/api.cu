@@ -796,12 +796,11 @@ int build_system_maps(am_handle* h) {
     // Chunk length: about n / (4 x SMs), rounded up to a power of two in
     // 64 .. 1024, so that the FP64 dot products and orthogonalisation of a
     // small system still spread over all SMs (GB300 has 2 FP64 FMAs per SM
-    // per cycle); the chunk kernels run 256 threads a block.
+    // per cycle).
     const long long per = ((long long)n + 4LL * am::num_sms() - 1) / (4LL * am::num_sms());
     int clen = 64;
     while (clen < per && clen < 1024) clen *= 2;
     h->chunk_len = clen;
-    h->chunk_threads = 256;
     for (int sI = 0; sI < S; ++sI) {
         const am_sys_rec& r = h->sys[sI];
         const int segs[3][2] = {{3 * h->sys_blob0[sI], 3 * (h->sys_blob0[sI] + r.Nb)},

@@ -765,6 +765,10 @@ __device__ void loop_ctrl(ArnoldiCtrl* c, int* __restrict__ active, int* __restr
 // arithmetic and its order are those of separate dot, coefficient,
 // orthogonalisation, norm and step-end kernels.
 
+// threads that share a chunk: the block of the separate kernels, the first eight
+// warps of the one-kernel step
+constexpr int kChunkThreads = 256;
+
 // Sums over i in [i0, i1) of x_k[i] y[i], x_k = x + k ld, k <= j, given to
 // out(k, sum): U consecutive k per warp at a time, their loads in flight
 // together (a warp per k waited for every load and reduction in turn).  y NULL:
@@ -799,7 +803,7 @@ __device__ __forceinline__ void rows_sums_u(const double* x, size_t ld, const do
 template <class Out>
 __device__ __forceinline__ void rows_sums(const double* x, size_t ld, const double* y, int i0, int i1, int j,
                                           Out out) {
-    constexpr int nw = 8;  // the first 256 threads of the block
+    constexpr int nw = kChunkThreads / 32;  // the first warps of the block
     const int per = (j + nw) / nw;
     if (per <= 1) rows_sums_u<1>(x, ld, y, i0, i1, j, nw, out);
     else if (per <= 2) rows_sums_u<2>(x, ld, y, i0, i1, j, nw, out);
@@ -832,7 +836,7 @@ __device__ __forceinline__ void sys_coef(int s, const double* part, int nchunks,
 // at a time, loaded together, in two chains.
 __device__ __forceinline__ double chunk_orth(const double* __restrict__ V, size_t ldv, double* w, int c0,
                                              int c1, int j, const double* cf, int len, double* sh) {
-    constexpr int kT = 256;  // the threads that call it
+    constexpr int kT = kChunkThreads;  // the threads that call it
     const int per = min(kT, len);  // threads per group
     const int G = kT / per;
     const int e = threadIdx.x % per, g = threadIdx.x / per;
@@ -858,10 +862,10 @@ __device__ __forceinline__ double chunk_orth(const double* __restrict__ V, size_
             }
             p += q;
         }
-        if (G > 1) {  // a barrier of these 256 threads
-            asm volatile("bar.sync 1, 256;" ::: "memory");
+        if (G > 1) {  // a barrier of these threads
+            asm volatile("bar.sync 1, %0;" ::"n"(kT) : "memory");
             sh[threadIdx.x] = p;
-            asm volatile("bar.sync 1, 256;" ::: "memory");
+            asm volatile("bar.sync 1, %0;" ::"n"(kT) : "memory");
             if (g == 0)
                 for (int q = 1; q < G; ++q) p += sh[q * per + e];
         }
@@ -876,7 +880,7 @@ __device__ __forceinline__ double chunk_orth(const double* __restrict__ V, size_
 
 // Z[j] = z (flexible GMRES keeps the preconditioned vectors); first CGS
 // pass: dots and coefficients
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kChunkThreads)
 k_arn_dots(const double* __restrict__ V, size_t ldv, const double* __restrict__ w,
            const double* __restrict__ z, double* __restrict__ Z, const int* __restrict__ cs,
            const int* __restrict__ ce, const int* __restrict__ sys_of, const int* __restrict__ coff,
@@ -891,13 +895,13 @@ k_arn_dots(const double* __restrict__ V, size_t ldv, const double* __restrict__ 
 }
 
 // first CGS pass: orthogonalisation; second pass: dots and coefficients
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kChunkThreads)
 k_arn_orth_dots(const double* __restrict__ V, size_t ldv, double* __restrict__ w, const int* __restrict__ cs,
                 const int* __restrict__ ce, const int* __restrict__ sys_of, const int* __restrict__ coff, int clen,
                 double* __restrict__ part, int nchunks, int m1, double* __restrict__ coef,
                 double* __restrict__ hcol, int* __restrict__ cnt, const ArnoldiCtrl* __restrict__ c) {
     dep_wait();
-    __shared__ double sh[256];
+    __shared__ double sh[kChunkThreads];
     const int j = c->j, b = blockIdx.x, c0 = cs[b], c1 = ce[b], s = sys_of[c0];
     chunk_orth(V, ldv, w, c0, c1, j, coef + (size_t)s * m1, clen, sh);
     __syncthreads();  // the chunk of w is updated before its dots
@@ -908,7 +912,7 @@ k_arn_orth_dots(const double* __restrict__ V, size_t ldv, double* __restrict__ w
 // second pass: orthogonalisation and |w|^2; per system the step end
 // (finish_one), then the loop control.  Blocks nch .. nch + S - 1 rotate the
 // systems' new columns meanwhile (their coefficients are complete).
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kChunkThreads)
 k_arn_orth_finish(const double* __restrict__ V, size_t ldv, double* __restrict__ w, const int* __restrict__ cs,
                   const int* __restrict__ ce, const int* __restrict__ sys_of, const int* __restrict__ coff, int clen,
                   double* __restrict__ npart, int nch, int m1, const double* __restrict__ coef,
@@ -918,7 +922,7 @@ k_arn_orth_finish(const double* __restrict__ V, size_t ldv, double* __restrict__
                   const double* __restrict__ tol_s, double* __restrict__ inv, ArnoldiCtrl* c,
                   cudaGraphConditionalHandle hc, int in_graph) {
     dep_wait();
-    __shared__ double sh[256];
+    __shared__ double sh[kChunkThreads];
     const int j = c->j, b = blockIdx.x;
     int s;
     if (b < nch) {
@@ -984,7 +988,7 @@ __global__ void k_next_basis(const double* __restrict__ w, double* __restrict__ 
 // wait that runs out sets c->late, which ends the other waits and the cycle;
 // every block still arrives three times and goes on to its end.  Nothing of
 // such a cycle is used: gmres repeats it with the separate kernels.
-constexpr int kStepThreads = 288;
+constexpr int kStepThreads = kChunkThreads + 32;
 constexpr int kStepSpins = 1 << 21;  // about a second
 
 __device__ __forceinline__ void sys_arrive(int* cnt) {  // after a barrier of the block
@@ -1028,7 +1032,7 @@ __global__ void __launch_bounds__(kStepThreads)
 k_arn_step(StepArgs a) {
     dep_wait();
     __shared__ double ws[1024];                // the chunk of w
-    __shared__ double sh[256], red[64];
+    __shared__ double sh[kChunkThreads], red[64];
     __shared__ double cf[200], hc[200];        // coefficients of a pass, of the column
     __shared__ double s_cs[200], s_sn[200];
     __shared__ double s_inv;
@@ -1038,13 +1042,13 @@ k_arn_step(StepArgs a) {
     const int j = a.c->j, it = a.c->it;
     const int c0 = ci.x, len = ci.y - ci.x, s = ci.z, q0 = ci.w, q1 = a.coff[s + 1], nb = q1 - q0;
     const int lane = threadIdx.x & 31;
-    const bool vec = threadIdx.x < 256;  // the eight warps that hold the chunk
+    const bool vec = threadIdx.x < kChunkThreads;  // the eight warps that hold the chunk
     const bool first = b == q0;
     if (a.active[s]) {
         double g0 = 0.0, tol = 0.0;
         if (vec) {
             double* Zj = a.Z + (size_t)j * a.ldv;
-            for (int i = threadIdx.x; i < len; i += 256) {
+            for (int i = threadIdx.x; i < len; i += kChunkThreads) {
                 ws[i] = a.w[c0 + i];
                 Zj[c0 + i] = a.z[c0 + i];
             }
@@ -1109,7 +1113,7 @@ k_arn_step(StepArgs a) {
             __syncthreads();
             if (threadIdx.x == 0) {
                 t = red[0];
-                for (int q = 1; q < 8; ++q) t += red[q];
+                for (int q = 1; q < kChunkThreads / 32; ++q) t += red[q];
                 a.npart[b] = t;
             }
             sys_barrier(a.sync + s, nb * (3 * it + 3), &a.c->late, a.spins);
@@ -1398,7 +1402,7 @@ static cudaError_t issue_arnoldi_step(am_handle* h, bool fp64, cudaGraphConditio
     cudaStream_t s = h->stream;
     const int n = h->n, m = h->restart, m1 = m + 1, S = h->S;
     const size_t ldv = (size_t)h->ldv;
-    const int nb = red_blocks(n), nch = h->nchunks, ct = h->chunk_threads;
+    const int nb = red_blocks(n), nch = h->nchunks, ct = kChunkThreads;
     const bool packed = !h->sb && symmetric_mixed(h, fp64 ? kOpFP64 : kOpHandle);
     pc_apply(h, h->d_vj, h->d_zj, packed ? h->d_lf : nullptr);  // vj = V[j], written with V[j]
     // the input of a stopped system is zero: its product skips the pairs
