@@ -60,10 +60,12 @@ extern "C" {
 
 /* ---- precision of the blob mobility product --------------------------- */
 #define AM_FP64  0   /* every operation in FP64                              */
-#define AM_MIXED 1   /* pair terms in FP32, per-target sums in FP64; the
-                        outer residual of the refinement with double-float
-                        pair terms (AM_DF64); Arnoldi and constraint algebra
-                        in FP64                                              */
+#define AM_MIXED 1   /* pair terms in FP32, summed in FP32 over 16 to 64 of
+                        them, those sums added in FP64 or as compensated
+                        pairs of floats (48 bits); the outer residual of the
+                        refinement with double-float pair terms (AM_DF64);
+                        preconditioner matrices in FP32; Arnoldi and
+                        constraint algebra in FP64                           */
 #define AM_DF64  2   /* pair terms in double-float arithmetic (pairs of
                         floats, ~2^-44 relative), sums in FP64: only as the
                         arithmetic of am_apply_mobility_ex                   */
@@ -364,7 +366,9 @@ AM_API size_t am_rpy_matvec_workspace(int n, int precision);
  *                  which may lie in them
  *   d_work         at least am_rpy_matvec_rows_workspace(n, nrows,
  *                  precision) bytes, 256-byte aligned
- * Otherwise as am_rpy_matvec (with row0 = 0 and nrows = n the two agree).
+ * Otherwise as am_rpy_matvec (with row0 = 0 and nrows = n the two agree to
+ * rounding; neither depends on scheduling, but the order of the sums depends
+ * on the shape of the call and, in am_rpy_matvec, on the scratch).
  * Errors: AM_ERR_ARG (rows outside 0 .. n - 1 and as am_rpy_matvec),
  * AM_ERR_CUDA. */
 AM_API int am_rpy_matvec_rows(const double* d_r, const double* d_lambda, double* d_u, int n,

@@ -66,11 +66,12 @@ struct MvItem {
     int sys, pad;     // system index
 };
 
-// One item of the symmetric products: tiles I (targets) and J (sources)
-// of T = 32 NSUB blobs of one system with I <= J; the pairs between them are
-// evaluated once and give the rows of I (slot J) and the columns of J (slot
-// I); the diagonal item (I = J) takes each unordered pair of its tile once
-// and writes rows and columns together.
+// One item of the symmetric products: tiles or groups of tiles I (targets) and J
+// (sources) of one system with I <= J; the pairs between them are evaluated once
+// and give the rows of I (slot J) and the columns of J (slot I).  In the
+// diagonal item (I = J) a tile against itself gives its rows only: each
+// unordered pair once, with the columns added to them (FP64, double-float), or
+// every ordered pair (mixed).
 struct SymItem {
     int i0, ni, j0, nj;     // first blob and count of tile I and of tile J
     int tbase, sys;         // first blob of the system, system

@@ -1,7 +1,8 @@
 // am_rpy_matvec_noalloc: the blob mobility product for callers that cannot
 // allocate device memory.  The same product as am_rpy_matvec with a fixed
 // device array of this file as its scratch: the symmetric product where its
-// partial sums fit in it, else the cluster product, which needs none.
+// partial sums fit in it, else the cluster product, which keeps the slots of
+// its parts there and, in mixed precision, the split positions.
 #include "am_internal.cuh"
 
 #include <string>

@@ -4,10 +4,10 @@
 // Build, per body p (one block): M^(pp) from the pair tensors, its explicit
 // inverse by blocked Cholesky, blocked triangular inverse and X^T X on 32 x 32
 // shared-memory tiles, Y_p = (M^(pp))^-1 K_p, S_p = K_p^T Y_p and
-// N~_p = S_p^-1 (a body of more than two tiles takes a cluster of CTAs when
-// such bodies are too few to fill the GPU; of many bodies of one shape, away
-// from a wall, one is built and the others are rotated from it).  Per articulated body a (one
-// block): H_a = C_a N~_a C_a^T and its generalised inverse G~_a
+// N~_p = S_p^-1 (bodies of more than two tiles take clusters of CTAs where that
+// is expected to be faster; of many bodies of one shape, away from a wall, one is
+// built and the others are rotated from it).  Per articulated body a (one
+// block or cluster): H_a = C_a N~_a C_a^T and its generalised inverse G~_a
 // (Eq. block_diag_const_res) by symmetric pivoted Cholesky (32-column panels,
 // then the blocked inverse of the rank-r factor):
 // H(perm) = L L^T with L of rank r gives
@@ -796,8 +796,10 @@ static void launch_team(K kernel, int n, int cs, size_t smem, cudaStream_t s, Ar
 
 template <class T>
 static void pca_build_t(am_handle* h, double tol) {
-    // the Schur diagonal and, as far as they fit, the places and the panel (64 KB
-    // leave three CTAs to an SM; a larger panel stays in global memory)
+    // the Schur diagonal and, as far as they fit, the places and the panel.  64 KB
+    // beside the tiles leave an SM the two CTAs that its registers allow (4,000
+    // articulated bodies of 6 rows beside one of 9, 87, 177 or 417 rows: 615 us in
+    // FP64, 420 in FP32, whatever the longest); a larger panel stays in global memory
     const int m = 3 * std::max(1, h->max_asm_links);
     size_t smem = (size_t)m * sizeof(double);
     int lay = 0;
@@ -855,7 +857,7 @@ static void pc_build_t(am_handle* h, double tol) {
     // one block of kPcThreads per body and per articulated body (the tile
     // routines assume that block size)
     // bodies of one or two 32-row tiles one CTA each; larger bodies one
-    // cluster of pcb_cs CTAs each when they are too few to fill the GPU
+    // cluster of pcb_cs CTAs each
     const int n_one = h->pcb_cs > 1 ? h->n_pcb_small : h->n_pcb;
     launch_team(k_pcb_build<T, CtaTeam>, n_one, 1, 0, s, (const int*)h->d_pcb_list, (const int*)h->d_blob_off,
                 (const double4_32a*)h->d_r4, (const double4_32a*)h->d_d4, (const long long*)h->d_minv_off,

@@ -453,7 +453,8 @@ __device__ __forceinline__ void pair2_sym(float2 dx, float2 dy, float2 dz, float
 // wrap, 937 / 1,568 without pairs, 911 / 1,493 now.  Tiles of 64 against one
 // target per lane with FP64 sums: 16 free systems of 500 to 4,000 blobs 71.5 ->
 // 54 us, the 2,560-blob colony above a wall 22.5 -> 16.7.  Free space: 24 warps
-// per SM (80 registers) take 5 % less time than 16; wall: 113 registers, fewer
+// per SM (80 registers, 12 bytes a thread spilled) take 5 % less time than 16;
+// wall: 113 registers, fewer
 // cost more than the warps bring (17.1 us, 17.7).
 template <bool WALL, int T>
 __global__ void __launch_bounds__(T, (WALL ? 512 : 768) / T)
@@ -734,9 +735,11 @@ k_sum_items(int n3, int G, double scale, const double* __restrict__ part, const 
 // ---- stateless products ---------------------------------------------------
 static size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
 
-// The least scratch that a caller passes, for nt targets against n sources: a
-// packed copy of the positions and as many chunks of partial sums as give 4
-// blocks of 128 targets per SM.  (The cluster product needs none of it.)
+// The least scratch that a caller passes, for nt targets against n sources: room
+// for a packed copy of the positions (the mixed product with two targets per
+// thread splits them there) and for as many slots of partial sums as chunks of
+// sources would give 4 blocks of 128 targets per SM, one at least.  The cluster
+// product takes as many parts as there are slots for, or none.
 size_t least_workspace(int n, int nt, int precision) {
     if (n <= 0 || nt <= 0) return 0;
     const int want = 4 * num_sms();

@@ -19,7 +19,7 @@
 // they are, so a small product needs no packing launch, no workspace and no
 // second launch for the sums.  The row ranges of a sharded suspension take it
 // at every size: 5,003 rows of 20,011 free blobs FP64 6.28 -> 5.04 ms, 949 rows
-// of 7,594 wall blobs FP64 1.27 -> 0.93 ms, mixed 54 -> 44 us.
+// of 7,594 wall blobs FP64 1.27 -> 0.96 ms, mixed 54 -> 40 us.
 //
 // FP32 pair terms (T = float) as in rpy_items_mixed: differences from the hi
 // parts, lo parts added within a quarter of the target's largest coordinate;

@@ -38,8 +38,9 @@
 namespace am {
 
 // One warp per block: the blocks of a launch then spread evenly over the SMs
-// whatever their number (2,560 blobs make 3,240 items, 21.3 per SM), and at
-// 22 to 25 resident blocks per SM such a launch is one wave.
+// whatever their number (2,560 blobs make 3,240 items, 21.3 per SM).  An SM holds
+// 25 of them above a wall (78 registers) and 21 in free space (95): such a
+// launch is one wave, or one and a few items.
 constexpr int kSymWarps = 1;
 constexpr int kSymMaxGroups = 96;  // most groups (partial-sum slots) per system
 // the same for the paired-lane product, whose items run one per block of four
@@ -58,7 +59,7 @@ struct SymFp64 {
 template <bool WALL>
 struct SymBlobPair : SymFp64 {
     static constexpr int NC = 3;
-    static constexpr int kMinBlocks = WALL ? 22 : 20;  // 80 and 96 registers, no spills
+    static constexpr int kMinBlocks = WALL ? 22 : 20;  // 78 and 95 registers, no spills
     RpyK<double> k;
     explicit SymBlobPair(const RpyK<double>& q) : k(q) {}
     __device__ __forceinline__ double scale() const { return k.A1; }
