@@ -539,16 +539,22 @@ k_chunk_resid(const double* __restrict__ b, const double* __restrict__ Ax, doubl
     if (threadIdx.x == 0) npart[c] = a;
 }
 
-// out[s] = sqrt(sum of the system's chunk partials), a warp per system
-__global__ void k_sys_norm(const double* __restrict__ npart, const int* __restrict__ coff, int S,
+// out[s] = sqrt(sum of the system's chunk partials), L = 32 or 1 threads per
+// system: a thread where systems have few chunks (20,000 systems of two: 19.5
+// and 4 us)
+__global__ void k_sys_norm(const double* __restrict__ npart, const int* __restrict__ coff, int S, int L,
                            double* __restrict__ out) {
-    const int s = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, s = t / L, lane = t % L;
     if (s >= S) return;
     double a = 0.0;
 #pragma unroll 4
-    for (int c = coff[s] + lane; c < coff[s + 1]; c += 32) a += npart[c];
-    a = warp_sum(a);
+    for (int c = coff[s] + lane; c < coff[s + 1]; c += L) a += npart[c];
+    if (L == 32) a = warp_sum(a);
     if (lane == 0) out[s] = sqrt(a);
+}
+static void launch_sys_norm(const am_handle* h, double* out) {
+    const int L = h->nchunks > 8 * h->S ? 32 : 1;
+    k_sys_norm<<<(int)((1LL * h->S * L + 127) / 128), 128, 0, h->stream>>>(h->d_npart, h->d_sys_chunk_off, h->S, L, out);
 }
 
 // out = min over systems (with b_s != 0) of |r_s| / |b_s|
@@ -764,6 +770,14 @@ __device__ void loop_ctrl(ArnoldiCtrl* c, int* __restrict__ active, int* __restr
 // control.  The completing block zeroes its count for the next use.  The
 // arithmetic and its order are those of separate dot, coefficient,
 // orthogonalisation, norm and step-end kernels.
+//
+// Two forms (separate_few in issue_arnoldi_step).  Many chunks: eight blocks to
+// an SM hide the latency, so 32 registers a thread; with 76 (rows_sums and the
+// rotation unbounded) 5,000 systems of 24 blobs took 749 us an iteration, now 520,
+// 1,000 of 96 300 and 250, 24 of about 3,000 500 and 478.  At most four short
+// chunks to an SM: latency per block counts, rows_sums keeps several rows in
+// flight and the registers are given (chains of 5,800 to 9,600 blobs: 2 to 5 %
+// less per iteration than the other form).
 
 // threads that share a chunk: the block of the separate kernels, the first eight
 // warps of the one-kernel step
@@ -811,10 +825,23 @@ __device__ __forceinline__ void rows_sums(const double* x, size_t ld, const doub
     else rows_sums_u<8>(x, ld, y, i0, i1, j, nw, out);
 }
 
-// part[k * nchunks + b] = <V_k, w> over chunk [c0, c1), k <= j
+// part[k * nchunks + b] = <V_k, w> over chunk [c0, c1), k <= j: rows_sums for
+// few chunks, else a warp per k (FEW: separate_few)
+template <bool FEW>
 __device__ __forceinline__ void chunk_dots(const double* __restrict__ V, size_t ldv, const double* w, int c0,
                                            int c1, int j, double* __restrict__ part, int nchunks, int b) {
-    rows_sums(V, ldv, w, c0, c1, j, [&](int k, double a) { part[(size_t)k * nchunks + b] = a; });
+    if (FEW) {
+        rows_sums(V, ldv, w, c0, c1, j, [&](int k, double a) { part[(size_t)k * nchunks + b] = a; });
+        return;
+    }
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (int k = wid; k <= j; k += kChunkThreads / 32) {
+        const double* v = V + (size_t)k * ldv;
+        double a = 0.0;
+        for (int i = c0 + lane; i < c1; i += 32) a = fma(v[i], w[i], a);
+        a = warp_sum(a);
+        if (lane == 0) part[(size_t)k * nchunks + b] = a;
+    }
 }
 
 // coef[s][k] = sum over the system's chunks; hcol[s][k] = (hcol +) coef
@@ -832,9 +859,37 @@ __device__ __forceinline__ void sys_coef(int s, const double* part, int nchunks,
 // share of |w|^2 over the chunk (after the update).  When the chunk is
 // shorter than the block, the block's G = blockDim / len groups of len
 // threads each sum every G-th term of an element's sum (shorter dependent
-// FP64 chains), combined in shared memory (sh: blockDim doubles).  Eight terms
-// at a time, loaded together, in two chains.
+// FP64 chains), combined in shared memory (sh: blockDim doubles).
 __device__ __forceinline__ double chunk_orth(const double* __restrict__ V, size_t ldv, double* w, int c0,
+                                             int c1, int j, const double* cf, int len, double* sh) {
+    const int per = min(kChunkThreads, len);  // threads per group
+    const int G = kChunkThreads / per;
+    const int e = threadIdx.x % per, g = threadIdx.x / per;
+    double a = 0.0;
+    for (int i0 = c0; i0 < c1; i0 += per) {
+        const int i = i0 + e;
+        double p = 0.0;
+        if (i < c1)
+            for (int k = g; k <= j; k += G) p = fma(cf[k], V[(size_t)k * ldv + i], p);
+        if (G > 1) {
+            __syncthreads();
+            sh[threadIdx.x] = p;
+            __syncthreads();
+            if (g == 0)
+                for (int q = 1; q < G; ++q) p += sh[q * per + e];
+        }
+        if (g == 0 && i < c1) {
+            const double v = w[i] - p;
+            w[i] = v;
+            a = fma(v, v, a);
+        }
+    }
+    return a;
+}
+
+// The same in the one-kernel step, whose blocks are few to an SM: eight terms
+// at a time, loaded together, in two chains.
+__device__ __forceinline__ double chunk_orth_ahead(const double* __restrict__ V, size_t ldv, double* w, int c0,
                                              int c1, int j, const double* cf, int len, double* sh) {
     constexpr int kT = kChunkThreads;  // the threads that call it
     const int per = min(kT, len);  // threads per group
@@ -880,7 +935,8 @@ __device__ __forceinline__ double chunk_orth(const double* __restrict__ V, size_
 
 // Z[j] = z (flexible GMRES keeps the preconditioned vectors); first CGS
 // pass: dots and coefficients
-__global__ void __launch_bounds__(kChunkThreads)
+template <bool FEW>
+__global__ void __launch_bounds__(kChunkThreads, FEW ? 3 : 8)
 k_arn_dots(const double* __restrict__ V, size_t ldv, const double* __restrict__ w,
            const double* __restrict__ z, double* __restrict__ Z, const int* __restrict__ cs,
            const int* __restrict__ ce, const int* __restrict__ sys_of, const int* __restrict__ coff,
@@ -890,12 +946,13 @@ k_arn_dots(const double* __restrict__ V, size_t ldv, const double* __restrict__ 
     const int j = c->j, b = blockIdx.x, c0 = cs[b], c1 = ce[b], s = sys_of[c0];
     double* zc = Z + (size_t)j * ldv;
     for (int i = c0 + threadIdx.x; i < c1; i += blockDim.x) zc[i] = z[i];
-    chunk_dots(V, ldv, w, c0, c1, j, part, nchunks, b);
+    chunk_dots<FEW>(V, ldv, w, c0, c1, j, part, nchunks, b);
     if (arrive_last(cnt, s, coff[s + 1] - coff[s])) sys_coef(s, part, nchunks, coff, m1, j, coef, hcol, 0);
 }
 
 // first CGS pass: orthogonalisation; second pass: dots and coefficients
-__global__ void __launch_bounds__(kChunkThreads)
+template <bool FEW>
+__global__ void __launch_bounds__(kChunkThreads, FEW ? 3 : 8)
 k_arn_orth_dots(const double* __restrict__ V, size_t ldv, double* __restrict__ w, const int* __restrict__ cs,
                 const int* __restrict__ ce, const int* __restrict__ sys_of, const int* __restrict__ coff, int clen,
                 double* __restrict__ part, int nchunks, int m1, double* __restrict__ coef,
@@ -905,14 +962,15 @@ k_arn_orth_dots(const double* __restrict__ V, size_t ldv, double* __restrict__ w
     const int j = c->j, b = blockIdx.x, c0 = cs[b], c1 = ce[b], s = sys_of[c0];
     chunk_orth(V, ldv, w, c0, c1, j, coef + (size_t)s * m1, clen, sh);
     __syncthreads();  // the chunk of w is updated before its dots
-    chunk_dots(V, ldv, w, c0, c1, j, part, nchunks, b);
+    chunk_dots<FEW>(V, ldv, w, c0, c1, j, part, nchunks, b);
     if (arrive_last(cnt, s, coff[s + 1] - coff[s])) sys_coef(s, part, nchunks, coff, m1, j, coef, hcol, 1);
 }
 
 // second pass: orthogonalisation and |w|^2; per system the step end
 // (finish_one), then the loop control.  Blocks nch .. nch + S - 1 rotate the
 // systems' new columns meanwhile (their coefficients are complete).
-__global__ void __launch_bounds__(kChunkThreads)
+template <bool FEW>
+__global__ void __launch_bounds__(kChunkThreads, FEW ? 5 : 8)
 k_arn_orth_finish(const double* __restrict__ V, size_t ldv, double* __restrict__ w, const int* __restrict__ cs,
                   const int* __restrict__ ce, const int* __restrict__ sys_of, const int* __restrict__ coff, int clen,
                   double* __restrict__ npart, int nch, int m1, const double* __restrict__ coef,
@@ -1085,7 +1143,7 @@ k_arn_step(StepArgs a) {
             }
             __syncthreads();
             if (vec) {
-                sq = chunk_orth(V, a.ldv, ws, 0, len, j, cf, a.clen, sh);
+                sq = chunk_orth_ahead(V, a.ldv, ws, 0, len, j, cf, a.clen, sh);
             } else if (pass) {
                 double c2 = 0.0;
                 for (int k = lane; k <= j; k += 32) c2 = fma(cf[k], cf[k], c2);
@@ -1161,8 +1219,11 @@ k_hess_solve_sys(const double* __restrict__ H, const double* __restrict__ g, con
     for (int e = 0; e < E; ++e) {
         const int i = lane + 32 * e;
         a[e] = i < k ? gs[i] : 0.0;
-        const double d = i < k ? Hs[(size_t)i * m1 + i] : 0.0;
-        inv[e] = d != 0.0 ? 1.0 / d : 0.0;
+        inv[e] = 0.0;
+        if (32 * e < k) {  // an FP64 division of every block of 32, needed or not, took 75 us for 20,000 systems
+            const double d = i < k ? Hs[(size_t)i * m1 + i] : 0.0;
+            if (d != 0.0) inv[e] = 1.0 / d;
+        }
     }
 #pragma unroll
     for (int eo = E - 1; eo >= 0; --eo) {
@@ -1323,7 +1384,7 @@ static void read_scal(am_handle* h, int count) {
 // per-system 2-norms of v into out (S doubles, device)
 static void sys_norms(am_handle* h, const double* v, double* out) {
     k_chunk_sq<<<h->nchunks, 256, 0, h->stream>>>(v, h->d_chunk_start, h->d_chunk_end, h->d_npart);
-    k_sys_norm<<<nblk(h->S, 4), 128, 0, h->stream>>>(h->d_npart, h->d_sys_chunk_off, h->S, out);
+    launch_sys_norm(h, out);
     count_launch(2);
 }
 
@@ -1332,7 +1393,7 @@ static void sys_norms(am_handle* h, const double* v, double* out) {
 static void sys_residual(am_handle* h, const double* b, const double* x, double* r, double* out, int mode) {
     op_apply(h, x, h->d_w, mode);
     k_chunk_resid<<<h->nchunks, 256, 0, h->stream>>>(b, h->d_w, r, h->d_chunk_start, h->d_chunk_end, h->d_npart);
-    k_sys_norm<<<nblk(h->S, 4), 128, 0, h->stream>>>(h->d_npart, h->d_sys_chunk_off, h->S, out);
+    launch_sys_norm(h, out);
     count_launch(2);
 }
 
@@ -1403,6 +1464,7 @@ static cudaError_t issue_arnoldi_step(am_handle* h, bool fp64, cudaGraphConditio
     const int n = h->n, m = h->restart, m1 = m + 1, S = h->S;
     const size_t ldv = (size_t)h->ldv;
     const int nb = red_blocks(n), nch = h->nchunks, ct = kChunkThreads;
+    const bool separate_few = h->chunk_len <= 64 && nch <= 4 * num_sms();
     const bool packed = !h->sb && symmetric_mixed(h, fp64 ? kOpFP64 : kOpHandle);
     pc_apply(h, h->d_vj, h->d_zj, packed ? h->d_lf : nullptr);  // vj = V[j], written with V[j]
     // the input of a stopped system is zero: its product skips the pairs
@@ -1429,15 +1491,15 @@ static cudaError_t issue_arnoldi_step(am_handle* h, bool fp64, cudaGraphConditio
         count_launch();
         return e;
     }
-    launch_dep(k_arn_dots, dim3(nch), dim3(ct), 0, s, h->d_V, ldv, h->d_w, h->d_zj, h->d_Z, h->d_chunk_start,
+    launch_dep(separate_few ? k_arn_dots<true> : k_arn_dots<false>, dim3(nch), dim3(ct), 0, s, h->d_V, ldv, h->d_w, h->d_zj, h->d_Z, h->d_chunk_start,
                h->d_chunk_end, h->d_sys_of_elem, h->d_sys_chunk_off, h->d_part, nch, m1, h->d_coefs, h->d_hcols,
                h->d_arn_cnt, h->d_ctrl);
-    launch_dep(k_arn_orth_dots, dim3(nch), dim3(ct), 0, s, h->d_V, ldv, h->d_w, h->d_chunk_start, h->d_chunk_end,
+    launch_dep(separate_few ? k_arn_orth_dots<true> : k_arn_orth_dots<false>, dim3(nch), dim3(ct), 0, s, h->d_V, ldv, h->d_w, h->d_chunk_start, h->d_chunk_end,
                h->d_sys_of_elem, h->d_sys_chunk_off, h->chunk_len, h->d_part, nch, m1, h->d_coefs, h->d_hcols,
                h->d_arn_cnt, h->d_ctrl);
     const cudaError_t e = launch_dep(
-        k_arn_orth_finish, dim3(nch + S), dim3(ct), 0, s, h->d_V, ldv, h->d_w, h->d_chunk_start, h->d_chunk_end,
-        h->d_sys_of_elem, h->d_sys_chunk_off, h->chunk_len, h->d_npart, nch, m1, h->d_coefs, h->d_hcols, h->d_arn_cnt,
+        separate_few ? k_arn_orth_finish<true> : k_arn_orth_finish<false>, dim3(nch + S), dim3(ct), 0, s, h->d_V, ldv,
+        h->d_w, h->d_chunk_start, h->d_chunk_end, h->d_sys_of_elem, h->d_sys_chunk_off, h->chunk_len, h->d_npart, nch, m1, h->d_coefs, h->d_hcols, h->d_arn_cnt,
         S, m, h->d_Hs, h->d_css, h->d_sns, h->d_gs, h->d_carry, h->d_active, h->d_kdone, h->d_tol_s, h->d_inv_s,
         h->d_ctrl, hc, in_graph ? 1 : 0);
     // j has advanced: V[j] = w / |w_s| and the next step's input
