@@ -224,6 +224,7 @@ struct am_handle {
     // tile-pair items of the symmetric FP64 product (tiles of 32 sym_nsub blobs)
     void* d_sym_items = nullptr;
     int sym_splits = 1;  // items per tile pair, each with part of the steps (FP64 kernel only)
+    bool mv_tiny = false;  // tiles of 32 and every system a single one
     int n_sym = 0, sym_nsub = 0, mv_gridsym = 0, mv_gridsym32 = 0, mv_gridsymdf = 0;
 
     // host structure

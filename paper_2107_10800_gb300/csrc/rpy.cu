@@ -363,6 +363,67 @@ rpy_items_mixed(const float4* __restrict__ hi, const float4* __restrict__ lo,
     item_queue_done(counter);
 }
 
+// Systems of at most 32 blobs each, the whole of one in an item: a warp per
+// system, one target per lane, against every source in turn; pair terms, FP32
+// blocks and (hi, lo) sums as in rpy_items_mixed, no queue and no block
+// barriers.  rpy_sym_mixed spends 16 steps of two targets and two teams on a
+// tile however few its blobs are: 10,000 systems of 12 blobs 58 us (above a wall
+// 79), here 25 (29); 20,000 of 24 blobs 80 (115), here 68 (85).
+template <bool WALL>
+__global__ void __launch_bounds__(128)
+rpy_tiny_mixed(const float4* __restrict__ hi, const float4* __restrict__ lo, const double* __restrict__ lam,
+               double* __restrict__ part, const SymItem* __restrict__ items, int n_items, RpyK<float> k,
+               const int* __restrict__ active) {
+    dep_wait();
+    __shared__ float4 sh[4][32], so[4][32], sl[4][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, itn = 4 * (int)blockIdx.x + warp;
+    if (itn >= n_items) return;
+    const SymItem m = items[itn];
+    const bool ok = lane < m.ni;
+    double* out = part + m.poff + 3 * lane;
+    if (active && !active[m.sys]) {  // a stopped system: zero partial sums
+        if (ok) out[0] = out[1] = out[2] = 0.0;
+        return;
+    }
+    const int i = m.i0 + (ok ? lane : 0);
+    const float4 h0 = hi[i], o0 = lo[i];
+    sh[warp][lane] = make_float4(h0.x, h0.y, h0.z, 2.f * h0.z);  // .w: twice the height
+    so[warp][lane] = o0;
+    sl[warp][lane] = make_float4((float)lam[3 * (size_t)i], (float)lam[3 * (size_t)i + 1], (float)lam[3 * (size_t)i + 2], 0.f);
+    __syncwarp();
+    if (!ok) return;
+    const float nr = 0.25f * fmaxf(fabsf(h0.x), fmaxf(fabsf(h0.y), fabsf(h0.z)));
+    const float near2 = nr * nr;
+    float th[3] = {0.f, 0.f, 0.f}, tl[3] = {0.f, 0.f, 0.f};
+    for (int q0 = 0; q0 < m.ni; q0 += kSumBlock) {
+        const int qe = min(m.ni, q0 + kSumBlock);
+        float u[3] = {0.f, 0.f, 0.f};
+#pragma unroll 2
+        for (int q = q0; q < qe; ++q) {
+            const float4 h = sh[warp][q], l = sl[warp][q];
+            float dx = h0.x - h.x, dy = h0.y - h.y, dz = h0.z - h.z;
+            float rxy2 = fmaf(dx, dx, dy * dy);
+            float r2 = fmaf(dz, dz, rxy2);
+            if (r2 < near2) {
+                const float4 o = so[warp][q];
+                dx += o0.x - o.x;
+                dy += o0.y - o.y;
+                dz += o0.z - o.z;
+                rxy2 = fmaf(dx, dx, dy * dy);
+                r2 = fmaf(dz, dz, rxy2);
+            }
+            if (WALL)
+                pair_wall_r2<float>(dx, dy, dz, rxy2, r2, h0.z + h.z, h.w, -h0.z, l.x, l.y, l.z, k, u[0], u[1], u[2]);
+            else
+                pair_free_r2<float>(dx, dy, dz, r2, l.x, l.y, l.z, k, u[0], u[1], u[2]);
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) two_sum_acc(th[c], tl[c], u[c]);
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) out[c] = k.A1 * ((double)th[c] + (double)tl[c]);
+}
+
 // Both directions of a pair in paired FP32 lanes: u += M lambda_src for two
 // targets (the lanes), and v += M^T mu for the source from each target (v.x
 // from the first, v.y from the second; the caller adds them).  The
@@ -965,6 +1026,7 @@ int mobility_layout(am_handle* h, int tpt, int chunk, int tgroup, int sym) {
     if (h->d_sym_items) cudaFree(h->d_sym_items);
     h->d_sym_items = nullptr;
     h->n_sym = 0;
+    h->mv_tiny = false;
     if (sym && !h->d_lf &&
         cudaMalloc(reinterpret_cast<void**>(&h->d_lf), std::max(h->Nb, 1) * sizeof(float4)) != cudaSuccess)
         return 1;
@@ -976,6 +1038,7 @@ int mobility_layout(am_handle* h, int tpt, int chunk, int tgroup, int sym) {
         h->n_sym = (int)sitems.size();
         h->sym_nsub = sym;
         h->sym_splits = splits;
+        h->mv_tiny = sym == 1 && h->n_sym == S;  // every system a single tile, its steps not split
         h->mv_gridsym = std::min(sym_grid(h->cfg.wall != 0), (h->n_sym + kSymWarps - 1) / kSymWarps);
         h->mv_gridsym32 = std::min(sym_mixed_grid(h->cfg.wall != 0, sym), h->n_sym);
         h->mv_gridsymdf = std::min(sym_df_resident_grid(h->cfg.wall != 0), h->n_sym);
@@ -1025,7 +1088,7 @@ int mobility_layout(am_handle* h, int tpt, int chunk, int tgroup, int sym) {
 
 bool symmetric_mixed(const am_handle* h, int mode) {
     return !h->per && (mode == kOpMixed || (mode == kOpHandle && h->cfg.precision == AM_MIXED)) && h->n_sym > 0 &&
-           h->sym_splits == 1;
+           h->sym_splits == 1 && !h->mv_tiny;
 }
 
 // The partial sums of u = M lambda for all systems (mode: the handle's
@@ -1061,6 +1124,14 @@ void launch_items(am_handle* h, const double* lam, int mode, const int* active, 
         else
             launch_dep(rpy_items_f64<false>, dim3(h->mv_grid64), dim3(kThreads), 0, st, h->d_r4, lam, h->d_mv, items,
                        h->n_items, h->d_item_counter, k, active);
+    } else if (h->mv_tiny) {
+        const RpyK<float> k = rpy_consts<float>(h->prm);
+        const SymItem* si = static_cast<const SymItem*>(h->d_sym_items);
+        const dim3 grid((h->n_sym + 3) / 4), block(128);
+        if (h->cfg.wall)
+            launch_dep(rpy_tiny_mixed<true>, grid, block, 0, st, h->d_rhi, h->d_rlo, lam, h->d_mv, si, h->n_sym, k, active);
+        else
+            launch_dep(rpy_tiny_mixed<false>, grid, block, 0, st, h->d_rhi, h->d_rlo, lam, h->d_mv, si, h->n_sym, k, active);
     } else if (symmetric_mixed(h, mode)) {
         const RpyK<float> k = rpy_consts<float>(h->prm);
         const SymItem* si = static_cast<const SymItem*>(h->d_sym_items);
