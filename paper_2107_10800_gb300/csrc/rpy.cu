@@ -980,10 +980,10 @@ int mobility_layout(am_handle* h, int tpt, int chunk, int tgroup, int sym) {
         const long long per_item = std::max<long long>(pairs / want, (long long)kThreads * tpt * kTile);
         chunk = (int)std::max<long long>(kTile, per_item / (kThreads * tpt) / kTile * kTile);
     }
-    // few tile pairs (FP64, tiles of 32 or 64): their steps split over several
-    // items with slots of their own
+    // few tile pairs (FP64): their steps split over several items with slots of
+    // their own
     int splits = 1;
-    if ((sym == 1 || sym == 2) && h->cfg.precision == AM_FP64) {
+    if (sym && h->cfg.precision == AM_FP64) {
         long long tp = 0;
         for (int s = 0; s < S; ++s) {
             const long long nt = (h->sys[s].Nb + 32 * sym - 1) / (32 * sym);

@@ -408,7 +408,7 @@ void launch_items_df(am_handle* h, const double* lam) {
     cudaStream_t st = h->stream;  // the queue counter is zero (reset by the last launch's last block)
     const MvItem* items = static_cast<const MvItem*>(h->d_items);
     const RpyDf k = rpy_df_consts(h->prm);
-    if (h->n_sym > 0 && h->sym_nsub == 4) {  // tile pairs of 128: the symmetric double-float product
+    if (h->n_sym > 0 && h->sym_nsub == 4 && h->sym_splits == 1) {  // tile pairs of 128: the symmetric double-float product
         const SymItem* si = static_cast<const SymItem*>(h->d_sym_items);
         if (h->cfg.wall)
             rpy_sym_df<true><<<h->mv_gridsymdf, kThreads, 0, st>>>(h->d_rhi, h->d_rlo, lam, h->d_mv, si, h->n_sym,

@@ -2,7 +2,8 @@
 the step to larger ones: sizes around a block of 16 sources and the limit,
 systems of one size and of several, free space and wall, far from the origin,
 against the FP64 product with the bar of the mixed tests; and solves, in which
-systems stop one after the other."""
+systems stop one after the other.  FP64 handles on few tiles of 128, whose steps
+are split, beside tiles of 32."""
 import numpy as np
 import pytest
 
@@ -65,3 +66,13 @@ def test_solve(name, wall):
     ref = handle(SIZES[name], wall, "fp64", 32).solve()[0]
     # both within 1e-8 of their right side; a body's blob mobility is conditioned below 1e3
     assert np.abs(U - ref).max() <= 1e-5 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("wall", [0, 1])
+@pytest.mark.parametrize("sizes", [[[40, 40, 40]], [[130]], [[12]] * 5, [[100, 157], [3]]])
+def test_fp64_tiles_of_128(sizes, wall):
+    a, b = (handle(sizes, wall, "fp64", t) for t in (32, 128))
+    lam = np.random.default_rng(2).standard_normal((a.Nb, 3))
+    ref = a.apply_mobility(lam)
+    for arithmetic, tol in (("fp64", 1e-12), ("mixed", 1e-5), ("df64", 1e-11)):
+        assert np.abs(b.apply_mobility_ex(lam, arithmetic) - ref).max() <= tol * np.abs(ref).max()
